@@ -47,6 +47,7 @@ struct FieldSet {
     size_t spec_stride = 0;    // elements between spectra
     void *vext = nullptr, *tab = nullptr;
     void *tw[3] = {nullptr, nullptr, nullptr};
+    void *dmat[3] = {nullptr, nullptr, nullptr};   // derivative matrices of the tensor-core passes
     FftAxis ax[3];
     CgState *cs = nullptr;     // device CG state
     cudaGraphExec_t graph = nullptr;
@@ -194,6 +195,14 @@ template <typename T> ofdft_status upload_twiddles(ofdft_ctx *c, FieldSet &f, in
     // butterfly chains between the barriers of the fused z kernels)
     f.ax[axis] = fft_axis(n, f.tw[axis], (sizeof(T) == 8 && axis == 2) ? 4 : 8);
     f.ax[axis].twf = nbf ? (const void *)((const char *)f.tw[axis] + nb) : nullptr;
+    // double-float sets: digits of the derivative matrices
+    if (sizeof(T) == 8 && c->g.dd && !c->g.dws && c->fp.kind != 0 && tline_supported(n)) {
+        std::vector<uint16_t> img(tline_matrix_bytes(n) / 2);
+        f.ax[axis].dexp = tline_derivative_matrix(n, c->g.ds[axis] * n, img.data());
+        CK(cudaMallocAsync((void **)&f.dmat[axis], tline_matrix_bytes(n), c->st));
+        CK(cudaMemcpyAsync(f.dmat[axis], img.data(), tline_matrix_bytes(n), cudaMemcpyHostToDevice, c->st));
+        f.ax[axis].dmat = f.dmat[axis];
+    }
     return OFDFT_OK;
 }
 
@@ -261,7 +270,14 @@ EvalScalars unpack_sums(const double *h, bool fttf)
     return es;
 }
 
-int eval_kernel_count(const ofdft_ctx *c) { return c->fp.kind == 0 ? 6 : 11; }
+// Kernels of one evaluation (GGA: two launches instead of a pass per axis
+// and half for the axes taken on the tensor cores).
+int eval_kernel_count(const ofdft_ctx *c, const FieldSet &f)
+{
+    if (c->fp.kind == 0) return 6;
+    const int tc = (f.ax[0].dmat ? 1 : 0) + (f.ax[1].dmat ? 1 : 0);
+    return 11 - 2 * tc + (tc || f.ax[2].dmat ? 2 : 0);
+}
 
 // Enqueue one energy + potential evaluation at ph (or, with phi0 and dh, at the
 // trial phi0 cos + dh sin written into ph; angles from csd (two T values in
@@ -274,10 +290,12 @@ int eval_kernel_count(const ofdft_ctx *c) { return c->fp.kind == 0 ? 6 : 11; }
 //        -> y^-1 -> zfinal [C2R z, pointwise, potential, sums].
 // GGA:   the same Hartree path, and the gradient and divergence one axis at
 //        a time (the derivative along axis j needs transforms along j only):
-//        zfwd also writes d_z n; dline x, y: d_x n, d_y n (second to fourth
-//        spectra, used as real fields); pointwise: v_part and U_j over the
-//        derivatives; dline x, y: d_x U_x + d_y U_y into vout; zfinal_gga:
-//        v = v_HL - d_z U_z + v_part - (d_x U_x + d_y U_y), sums.
+//        d_x n, d_y n, d_z n into the second to fourth spectra, used as real
+//        fields; pointwise: v_part and U_j over the derivatives; d_x U_x,
+//        d_y U_y, d_z U_z in place; zfinal_gga: v = v_HL + v_part - their
+//        sum, sums.  Derivatives of double-float sets run on the tensor
+//        cores (one launch for all axes, from the field n that zfwd writes);
+//        other axes take dline along x and y, zfwd and zfinal_gga along z.
 template <typename T>
 ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const T *dh, double cth,
                           double sth, const void *csd, T *vout, bool keep_nG, double *sums,
@@ -297,11 +315,14 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
     const int nbx = xpass_blocks(g);
     const long long npairs = (long long)g.nx * g.ny / 2;
     double *pA = c->part, *pB = pA + 3 * nbx, *pC = pB + 6 * npairs;
+    // the tensor-core derivative passes read n as a field: it waits in the
+    // buffer that the pointwise stage overwrites with v_part
+    T *nf = !fttf && (ax.dmat || ay.dmat || az.dmat) ? (T *)f.vpart : nullptr;
     {
         TimerScope ts(c, TM_ZFWD, sizeof(T) == 4);
-        T *dz = fttf ? nullptr : d2;
-        if (phi0) launch_zfwd<T>(g, az, 2, nullptr, phi0, dh, (T)cth, (T)sth, csd, ph, s0, st, dz);
-        else launch_zfwd<T>(g, az, 1, nullptr, ph, nullptr, T(0), T(0), nullptr, nullptr, s0, st, dz);
+        T *dz = fttf || az.dmat ? nullptr : d2;
+        if (phi0) launch_zfwd<T>(g, az, 2, nullptr, phi0, dh, (T)cth, (T)sth, csd, ph, s0, st, dz, nf);
+        else launch_zfwd<T>(g, az, 1, nullptr, ph, nullptr, T(0), T(0), nullptr, nullptr, s0, st, dz, nf);
     }
     DBG("k_zfwd");
     // GGA: the Hartree chain (y, x, y^-1 on the first spectrum) needs only
@@ -340,13 +361,26 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
                                c->fp, tab, c->xc, vout, pC, st);
     } else {
         cudaStream_t s2nd = fork ? c->aux[1] : st;   // stream of each pair's second pass
-        {
+        // derivatives along the axes with a digit matrix: one launch on the
+        // tensor cores (each pass may write over its input)
+        const FftAxis *const tax[3] = {ax.dmat ? &ax : nullptr, ay.dmat ? &ay : nullptr, az.dmat ? &az : nullptr};
+        auto tline = [&](T *x, T *y, T *z) {
+            if constexpr (sizeof(T) == 8) {
+                if (!nf) return;
+                TimerScope ts(c, TM_DLINE, false);
+                const double *const in[3] = {x ? x : nf, y ? y : nf, z ? z : nf};
+                float2 *const out[3] = {(float2 *)d0, (float2 *)d1, (float2 *)d2};
+                launch_tline(g, tax, in, out, st);
+            }
+        };
+        tline(nullptr, nullptr, nullptr);
+        if (!ax.dmat) {
             TimerScope ts(c, TM_DLINE, sizeof(T) == 4);
-            launch_dline<T>(g, ax, 0, 0, 0, ph, d0, st);
+            launch_dline<T>(g, ax, 0, nf ? 1 : 0, 0, nf ? nf : ph, d0, st);
         }
-        {
+        if (!ay.dmat) {
             TimerScope ts(c, TM_DLINE, sizeof(T) == 4);
-            launch_dline<T>(g, ay, 1, 0, 0, ph, d1, s2nd);
+            launch_dline<T>(g, ay, 1, nf ? 1 : 0, 0, nf ? nf : ph, d1, s2nd);
         }
         if (fork) {
             CK(cudaEventRecord(c->fj[2], s2nd));
@@ -368,13 +402,15 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
             CK(cudaEventRecord(c->fj[3], st));
             CK(cudaStreamWaitEvent(s2nd, c->fj[3], 0));
         }
-        // d_y U_y into vout, d_x U_x in place over U_x (d0); the final z pass
-        // subtracts both
-        {
+        // d_x U_x and d_y U_y in place over U_x and U_y; the final z pass
+        // subtracts both (and d_z U_z, which it takes itself unless the
+        // tensor-core pass has)
+        tline(d0, d1, d2);
+        if (!ay.dmat) {
             TimerScope ts(c, TM_DLINE, sizeof(T) == 4);
-            launch_dline<T>(g, ay, 1, 1, 0, d1, vout, st);
+            launch_dline<T>(g, ay, 1, 1, 0, d1, d1, st);
         }
-        {
+        if (!ax.dmat) {
             TimerScope ts(c, TM_DLINE, sizeof(T) == 4);
             launch_dline<T>(g, ax, 0, 1, 0, d0, d0, s2nd);
         }
@@ -385,13 +421,13 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
         }
         DBG("k_dline (div W)");
         TimerScope ts(c, TM_ZFINAL, sizeof(T) == 4);
-        nbz = launch_zfinal_gga<T>(g, az, s0, d2, (const T *)f.vpart, vout, d0, ph, phi0, dh, (T)cth, (T)sth,
-                                   csd, vout, pC, st);
+        nbz = launch_zfinal_gga<T>(g, az, s0, az.dmat ? nullptr : d2, (const T *)f.vpart, d1, d0, d2, ph, phi0, dh,
+                                   (T)cth, (T)sth, csd, vout, pC, st);
     }
     DBG("k_zfinal");
     launch_reduce_eval(pA, nbx, pB, nbg, pC, nbz, !fttf, sums, st);
     DBG("k_reduce_eval");
-    c->launches += eval_kernel_count(c);
+    c->launches += eval_kernel_count(c, f);
     if (keep_nG && !fttf) {
         // n(G) for forces and stress: forward z, y, x of n into the second spectrum
         launch_zfwd<T>(g, az, 1, nullptr, ph, nullptr, T(0), T(0), nullptr, nullptr, s1, st);
@@ -829,10 +865,10 @@ ofdft_status minimize_start(ofdft_ctx *c, double gtol, int maxit)
 
 // Launches of one graph-driven minimisation: prologue, per outer iteration
 // (direction + update), per line-search trial (evaluation + controller).
-long long graph_launches(const ofdft_ctx *c, const CgState &h)
+long long graph_launches(const ofdft_ctx *c, const FieldSet &f, const CgState &h)
 {
-    return 8 + eval_kernel_count(c) + (long long)h.nouter * 9 +
-           (long long)(h.nevals - 1) * (eval_kernel_count(c) + 1);
+    return 8 + eval_kernel_count(c, f) + (long long)h.nouter * 9 +
+           (long long)(h.nevals - 1) * (eval_kernel_count(c, f) + 1);
 }
 
 ofdft_status finish_minimize(ofdft_ctx *c, bool graph, ofdft_stats &stats, EvalScalars &es);
@@ -859,13 +895,13 @@ ofdft_status finish_minimize(ofdft_ctx *c, bool graph, ofdft_stats &stats, EvalS
     stats.evaluations = h.nevals;
     stats.gnorm = h.gnorm;
     stats.status = h.status == kCgStagnated ? OFDFT_OK : h.status;
-    if (graph) c->launches += graph_launches(c, h);
+    if (graph) c->launches += graph_launches(c, c->f[0], h);
     if (mixed) {
         const CgState &l = *c->st_h[1];
         stats.iterations += l.it;
         stats.evaluations_lo = l.nevals;
         stats.evaluations += l.nevals;
-        if (graph) c->launches += graph_launches(c, l);
+        if (graph) c->launches += graph_launches(c, c->f[1], l);
     }
     es = unpack_sums(h.ev_acc, c->fp.kind == 0);
     if (h.status == OFDFT_ENUMERIC) return fail(c, OFDFT_ENUMERIC, "non-finite energy, gradient or norm");
@@ -1265,7 +1301,7 @@ ofdft_status forces_now(ofdft_ctx *c, EvalScalars &es)
 void free_fieldset(FieldSet &f, cudaStream_t st)
 {
     void *ptrs[] = {f.phi, f.phit, f.dhat, f.g, f.gprev, f.d, f.v, f.vt, f.vpart, f.spec, f.vext, f.tab,
-                    f.tw[0], f.tw[1], f.tw[2], f.cs};
+                    f.tw[0], f.tw[1], f.tw[2], f.dmat[0], f.dmat[1], f.dmat[2], f.cs};
     for (void *p : ptrs)
         if (p) cudaFreeAsync(p, st);
     if (f.graph) cudaGraphExecDestroy(f.graph);
@@ -1381,6 +1417,7 @@ ofdft_status alloc_ctx(ofdft_ctx *c)
         return fail(c, OFDFT_EINVAL, "grid too large for the shared-memory tiles");
     CK(set_field_smem_limits<double>(dyn));
     CK(set_field_smem_limits<float>(dyn));
+    CK(tline_smem_limits());
     CK(cudaStreamCreateWithFlags(&c->cap2, cudaStreamNonBlocking));
     for (cudaStream_t &a : c->aux) CK(cudaStreamCreateWithFlags(&a, cudaStreamNonBlocking));
     for (cudaEvent_t &e : c->fj) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -1416,6 +1453,8 @@ double footprint_bytes(const int grid[3], int nat, int precision)
     };
     double b = fieldset(8.0) + (precision == OFDFT_MIXED ? fieldset(4.0) : 0.0);
     b += N * 8;                                                        // phiprev
+    for (int a = 0; a < 3; ++a)                                        // derivative matrices
+        if (tline_supported(grid[a])) b += (double)tline_matrix_bytes(grid[a]);
     b += (3 * ny * std::ceil(K / 4) + 15 * (nx * ny / 2) + 64) * 8 + 64 * 8;  // partials, scalars
     b += nat * 11.0 * 8 + 32 + nat * (2 * nx + 2 * ny + 3 * K) * 16.0;  // ions, phase factors (+ double-float)
     b += nat * std::max(1216.0, (double)lpp_force_chunks_dd((long long)(nx * ny), nat)) * 3 * 8 + 16 * 8;   // force partials
@@ -1454,9 +1493,11 @@ struct Tuned {
 // twiddle tables do not depend on the schedule).
 void set_radix(FieldSet &f, int a, int m)
 {
-    const void *twf = f.ax[a].twf;
-    f.ax[a] = fft_axis(f.ax[a].n, f.ax[a].tw, m);
-    f.ax[a].twf = twf;
+    const FftAxis old = f.ax[a];
+    f.ax[a] = fft_axis(old.n, old.tw, m);
+    f.ax[a].twf = old.twf;
+    f.ax[a].dmat = old.dmat;
+    f.ax[a].dexp = old.dexp;
 }
 std::map<TuneKey, Tuned> g_tune;
 
@@ -1554,8 +1595,9 @@ template <typename T> ofdft_status autotune_set(ofdft_ctx *c, int k, int reps)
                 if (r != OFDFT_OK) return r;
             }
     }
-    // the derivative passes' tile width and threads together (GGA only)
-    if (c->fp.kind != 0) {
+    // the derivative passes' tile width and threads together (GGA only; the
+    // tensor-core form has one shape)
+    if (c->fp.kind != 0 && !(f.ax[0].dmat && f.ax[1].dmat)) {
         const GridInfo base = best;
         for (int dk : {4, 8, 16})
             for (int th : {64, 128, 256}) {

@@ -288,7 +288,7 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
         nbg = launch_pw<double>(g, d0, d1, d2, ph, T, fp, tab, xc, vpart, pB, false, st);
         launch_dline<double>(g, ax, 0, 1, 0, d0, v_dev, st);
         launch_dline<double>(g, ay, 1, 1, 1, d1, v_dev, st);
-        nbz = launch_zfinal_gga<double>(g, az, s0, d2, vpart, v_dev, nullptr, ph, nullptr, nullptr, 1.0, 0.0,
+        nbz = launch_zfinal_gga<double>(g, az, s0, d2, vpart, v_dev, nullptr, nullptr, ph, nullptr, nullptr, 1.0, 0.0,
                                         nullptr, v_dev, pC, st);
     }
     launch_reduce_eval(pA, nbx, pB, nbg, pC, nbz, !fttf, scal, st);

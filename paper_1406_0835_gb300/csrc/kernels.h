@@ -8,16 +8,30 @@ namespace ofdft {
 // ---- grid fields (kernels_fields.cu)
 // z pass, forward: n = phi^2 (mode 1), the trial rotation phi cos + dhat sin
 // written to phit (mode 2) or a plain field (mode 0), R2C along z into the
-// half spectrum out; with dz also d_z n into the real field dz.
+// half spectrum out; with dz also d_z n into the real field dz, with nout
+// also n.
 template <typename T>
 void launch_zfwd(const GridInfo &g, const FftAxis &az, int mode, const T *in, const T *phi,
                  const T *dhat, T c, T s, const void *cs, T *phit, cplx<T> *out, cudaStream_t st,
-                 T *dz = nullptr);
+                 T *dz = nullptr, T *nout = nullptr);
 // Derivative of a real field along grid axis 0 (x) or 1 (y) by 1-D
 // transforms along that axis: out (= or, acc != 0, +=) d f, f = phi^2 for
-// mode 0 and f = in for mode 1 (scale GridInfo::ds).
+// mode 0 and f = in for mode 1 (scale GridInfo::ds).  Derivative fields
+// (this out, zfwd's dz, zfinal_gga's div*) are double-float pairs in a
+// double-float grid (two binary32 words in a double's place).
 template <typename T>
 void launch_dline(const GridInfo &g, const FftAxis &fa, int axis, int mode, int acc, const T *in, T *out,
+                  cudaStream_t st);
+// Derivatives d f (f = in[a]) along the axes a whose ax[a] is not null, in
+// one launch on the tensor cores, written as double-float pairs; for axes
+// whose digit matrix is set (FftAxis::dmat).  out[a] may be in[a].
+// tline_derivative_matrix fills img (tline_matrix_bytes(n)) with the digits
+// of the derivative matrix times scale and returns its binary exponent.
+bool tline_supported(int n);
+size_t tline_matrix_bytes(int n);
+int tline_derivative_matrix(int n, double scale, uint16_t *img);
+cudaError_t tline_smem_limits();
+void launch_tline(const GridInfo &g, const FftAxis *const ax[3], const double *const in[3], float2 *const out[3],
                   cudaStream_t st);
 // Pointwise functional + XC: reads phi and the derivatives of n in d0..d2,
 // writes v_part and, over d0..d2, the fields U_j whose derivatives sum to
@@ -33,11 +47,11 @@ int launch_zfinal(const GridInfo &g, const FftAxis &az, bool fttf, const cplx<T>
                   const void *cs, T temp, const FuncParams &fp, const T *tab, int xc, T *vout,
                   double *part, cudaStream_t st);
 // z pass, final (GGA): v = v_HL - d_z U_z + v_part - div - div2 (div may
-// alias vout; div2 may be null).
+// alias vout; div2 may be null); with uz null, div3 stands for d_z U_z.
 template <typename T>
 int launch_zfinal_gga(const GridInfo &g, const FftAxis &az, const cplx<T> *dspec, const T *uz, const T *vpart,
-                      const T *div, const T *div2, const T *phit, const T *phi, const T *dhat, T c, T s,
-                      const void *cs, T *vout, double *part, cudaStream_t st);
+                      const T *div, const T *div2, const T *div3, const T *phit, const T *phi, const T *dhat, T c,
+                      T s, const void *cs, T *vout, double *part, cudaStream_t st);
 template <typename T>
 void launch_ypass(const GridInfo &g, const FftAxis &ay, bool inv, cplx<T> *data, int nfields,
                   long long fstride, cudaStream_t st);

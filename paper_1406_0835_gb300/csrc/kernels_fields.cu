@@ -59,6 +59,19 @@ template <> __device__ __forceinline__ double2 stc<DD>(ff::cf2 v)
 {
     return make_double2(ff::to_double(v.x), ff::to_double(v.y));
 }
+// Derivative fields between kernels of one evaluation: the double-float
+// kernels keep them as pairs (hi, lo) in the 8 bytes of a binary64, so that
+// neither side converts.
+template <typename PR> __device__ __forceinline__ typename KT<PR>::R ldp(typename KT<PR>::T x) { return x; }
+template <> __device__ __forceinline__ ff::f2 ldp<DD>(double x)
+{
+    return ff::f2(__int_as_float(__double2loint(x)), __int_as_float(__double2hiint(x)));
+}
+template <typename PR> __device__ __forceinline__ typename KT<PR>::T stp(typename KT<PR>::R x) { return x; }
+template <> __device__ __forceinline__ double stp<DD>(ff::f2 x)
+{
+    return __hiloint2double(__float_as_int(x.lo), __float_as_int(x.hi));
+}
 // grid constant in the computed type (binary64 value d, binary32 copy f,
 // double-float pair p)
 template <typename PR>
@@ -273,7 +286,7 @@ __global__ void OFDFT_FFT_BOUNDS k_zfwd(GridInfo g, FftAxis az, int P, const typ
                        const typename KT<PR>::T *__restrict__ phi, const typename KT<PR>::T *__restrict__ dhat,
                        typename KT<PR>::T c, typename KT<PR>::T s, const void *__restrict__ cs,
                        typename KT<PR>::T *__restrict__ phit, typename KT<PR>::C *__restrict__ out,
-                       typename KT<PR>::T *__restrict__ dzout)
+                       typename KT<PR>::T *__restrict__ dzout, typename KT<PR>::T *__restrict__ nout)
 {
     typedef typename KT<PR>::T T;
     typedef typename KT<PR>::R R;
@@ -305,6 +318,7 @@ __global__ void OFDFT_FFT_BOUNDS k_zfwd(GridInfo g, FftAxis az, int P, const typ
             phit[base + i] = str<PR>(ph);
             val = ph * ph;
         }
+        if (nout != nullptr) nout[base + i] = str<PR>(val);
         R *dstp = reinterpret_cast<R *>(&A[(line >> 1) * nz + e]);
         dstp[line & 1] = val;
     }
@@ -332,7 +346,7 @@ __global__ void OFDFT_FFT_BOUNDS k_zfwd(GridInfo g, FftAxis az, int P, const typ
         RowCol ro(nz);
         for (int i = threadIdx.x; i < 2 * nl * nz; i += blockDim.x, ro.next()) {
             const R *src = reinterpret_cast<const R *>(&Y[(ro.r >> 1) * nz + ro.c]);
-            dzout[base + i] = str<PR>(src[ro.r & 1]);
+            dzout[base + i] = stp<PR>(src[ro.r & 1]);
         }
     }
 }
@@ -724,11 +738,11 @@ __global__ void OFDFT_FFT_BOUNDS k_dline(GridInfo g, FftAxis fa, const typename 
         T2 o;
         if (ACC) {
             const T2 q = *p;
-            o.x = str<PR>(ldr<PR>(q.x) + y.x);
-            o.y = str<PR>(ldr<PR>(q.y) + y.y);
+            o.x = stp<PR>(ldp<PR>(q.x) + y.x);
+            o.y = stp<PR>(ldp<PR>(q.y) + y.y);
         } else {
-            o.x = str<PR>(y.x);
-            o.y = str<PR>(y.y);
+            o.x = stp<PR>(y.x);
+            o.y = stp<PR>(y.y);
         }
         *p = o;
     }
@@ -788,11 +802,11 @@ __global__ void OFDFT_FFT_BOUNDS k_dline_ws(GridInfo g, FftAxis fa, const typena
         T2 o;
         if (ACC) {
             const T2 q = *p;
-            o.x = str<PR>(ldr<PR>(q.x) + y.x);
-            o.y = str<PR>(ldr<PR>(q.y) + y.y);
+            o.x = stp<PR>(ldp<PR>(q.x) + y.x);
+            o.y = stp<PR>(ldp<PR>(q.y) + y.y);
         } else {
-            o.x = str<PR>(y.x);
-            o.y = str<PR>(y.y);
+            o.x = stp<PR>(y.x);
+            o.y = stp<PR>(y.y);
         }
         *p = o;
     }
@@ -836,7 +850,7 @@ __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB) k_pw(GridInfo
     const ff::f2 tcoef = is_dd<PR>() ? ff::f2(2.0 / OF_K23 * (double)temp) : ff::f2(0.0f, 0.0f);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < g.N;
          i += (long long)gridDim.x * blockDim.x) {
-        const R dj[3] = {ldr<PR>(d0[i]), ldr<PR>(d1[i]), ldr<PR>(d2[i])};
+        const R dj[3] = {ldp<PR>(d0[i]), ldp<PR>(d1[i]), ldp<PR>(d2[i])};
         R gr[3];
         if constexpr (TRI) {
             for (int a = 0; a < 3; ++a) gr[a] = bm[a] * dj[0] + bm[3 + a] * dj[1] + bm[6 + a] * dj[2];
@@ -906,14 +920,16 @@ __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB) k_pw(GridInfo
 // times i kt ds_z, added to the packed spectrum of v_HL, so one inverse
 // transform serves both) and div = d_x U_x + d_y U_y, given as one field or
 // as two (div + div2; div2 may be null).  div may alias vout (each point is
-// read before it is written, by the same thread).  Partials
+// read before it is written, by the same thread).  With uz null, d_z U_z is
+// given as the field div3 instead.  div, div2 and div3 are derivative fields
+// (ldp).  Partials
 // (as k_zfinal's GGA form): rows 0..5 zero, then sum phi^2 v, sum phi^2,
 // sum 2 phi v dphi/dtheta.
 template <typename PR>
 __global__ void OFDFT_FFT_BOUNDS k_zfinal_g(GridInfo g, FftAxis az, int P, const typename KT<PR>::C *__restrict__ dspec,
                            const typename KT<PR>::T *__restrict__ uz, const typename KT<PR>::T *__restrict__ vpart,
                            const typename KT<PR>::T *div, const typename KT<PR>::T *__restrict__ div2,
-                           const typename KT<PR>::T *__restrict__ phit,
+                           const typename KT<PR>::T *__restrict__ div3, const typename KT<PR>::T *__restrict__ phit,
                            const typename KT<PR>::T *__restrict__ phi, const typename KT<PR>::T *__restrict__ dhat,
                            typename KT<PR>::T c, typename KT<PR>::T s, const void *__restrict__ cs,
                            typename KT<PR>::T *vout, double *__restrict__ part)
@@ -931,24 +947,22 @@ __global__ void OFDFT_FFT_BOUNDS k_zfinal_g(GridInfo g, FftAxis az, int P, const
     const int nz = g.nz, K = g.K;
     CC *A = reinterpret_cast<CC *>(smraw);
     CC *B = A + P * nz;
-    CC *D = B + P * nz;
     const long long npairs = (long long)g.nx * g.ny / 2;
     const long long p0 = (long long)blockIdx.x * P;
     const int nl = (int)min((long long)P, npairs - p0);
     const long long obase = 2 * p0 * K;
     const long long rbase = 2 * p0 * nz;
     pack_c2r<PR>(dspec, obase, nl, nz, K, A);
-    {
+    CC *Z = B;
+    if (uz != nullptr) {
         RowCol rc(nz);
         for (int i = threadIdx.x; i < 2 * nl * nz; i += blockDim.x, rc.next()) {
             R *dst = reinterpret_cast<R *>(&B[(rc.r >> 1) * nz + rc.c]);
             dst[rc.r & 1] = ldr<PR>(uz[rbase + i]);
         }
-    }
-    __syncthreads();
-    CC *Z = fft_lines<CC, false>(B, D, az, nl, nz, 1, false);
-    const R sz = gcst<PR>(g.ds[2], g.dsf[2], g.ds2[2]);
-    {
+        __syncthreads();
+        Z = fft_lines<CC, false>(B, B + P * nz, az, nl, nz, 1, false);
+        const R sz = gcst<PR>(g.ds[2], g.dsf[2], g.ds2[2]);
         RowCol re(nz);
         for (int i = threadIdx.x; i < nl * nz; i += blockDim.x, re.next()) {
             const CC d = times_ik<CC, R>(Z[i], re.c, nz, sz);
@@ -964,8 +978,9 @@ __global__ void OFDFT_FFT_BOUNDS k_zfinal_g(GridInfo g, FftAxis az, int P, const
         const R dr = (rc.r & 1) ? d.y : d.x;
         const R ph = ldr<PR>(phit[rbase + i]);
         const R n = ph * ph;
-        R v = ldr<PR>(vpart[rbase + i]) + dr - ldr<PR>(div[rbase + i]);
-        if (div2 != nullptr) v = v - ldr<PR>(div2[rbase + i]);
+        R v = ldr<PR>(vpart[rbase + i]) + dr - ldp<PR>(div[rbase + i]);
+        if (div2 != nullptr) v = v - ldp<PR>(div2[rbase + i]);
+        if (uz == nullptr) v = v - ldp<PR>(div3[rbase + i]);
         vout[rbase + i] = str<PR>(v);
         acc[6] += n * v;
         acc[7] += n;
@@ -1025,7 +1040,7 @@ int threads_for(int work)
 // ---------------------------------------------------------------- launchers
 template <typename T>
 void launch_zfwd(const GridInfo &g, const FftAxis &az, int mode, const T *in, const T *phi,
-                 const T *dhat, T c, T s, const void *cs, T *phit, cplx<T> *out, cudaStream_t st, T *dz)
+                 const T *dhat, T c, T s, const void *cs, T *phit, cplx<T> *out, cudaStream_t st, T *dz, T *nout)
 {
     int P = zpairs_light(g);
     long long npairs = (long long)g.nx * g.ny / 2;
@@ -1033,9 +1048,9 @@ void launch_zfwd(const GridInfo &g, const FftAxis &az, int mode, const T *in, co
     size_t sm = 2 * (size_t)P * g.nz * sizeof(cplx<T>);
     int th = g.zth > 0 ? g.zth : threads_for(P * g.nz);
 #define CALL(PR)                                                                                              \
-    if (mode == 0) k_zfwd<PR, 0><<<blocks, th, sm, st>>>(g, az, P, in, phi, dhat, c, s, cs, phit, out, dz);     \
-    else if (mode == 1) k_zfwd<PR, 1><<<blocks, th, sm, st>>>(g, az, P, in, phi, dhat, c, s, cs, phit, out, dz); \
-    else k_zfwd<PR, 2><<<blocks, th, sm, st>>>(g, az, P, in, phi, dhat, c, s, cs, phit, out, dz)
+    if (mode == 0) k_zfwd<PR, 0><<<blocks, th, sm, st>>>(g, az, P, in, phi, dhat, c, s, cs, phit, out, dz, nout);     \
+    else if (mode == 1) k_zfwd<PR, 1><<<blocks, th, sm, st>>>(g, az, P, in, phi, dhat, c, s, cs, phit, out, dz, nout); \
+    else k_zfwd<PR, 2><<<blocks, th, sm, st>>>(g, az, P, in, phi, dhat, c, s, cs, phit, out, dz, nout)
     OFDFT_DISPATCH(T, g, CALL);
 #undef CALL
 }
@@ -1151,16 +1166,16 @@ int launch_zfinal(const GridInfo &g, const FftAxis &az, bool fttf, const cplx<T>
 
 template <typename T>
 int launch_zfinal_gga(const GridInfo &g, const FftAxis &az, const cplx<T> *dspec, const T *uz, const T *vpart,
-                      const T *div, const T *div2, const T *phit, const T *phi, const T *dhat, T c, T s,
-                      const void *cs, T *vout, double *part, cudaStream_t st)
+                      const T *div, const T *div2, const T *div3, const T *phit, const T *phi, const T *dhat, T c,
+                      T s, const void *cs, T *vout, double *part, cudaStream_t st)
 {
     int P = zpairs_light(g);
     long long npairs = (long long)g.nx * g.ny / 2;
     int blocks = (int)((npairs + P - 1) / P);
-    size_t sm = 3 * (size_t)P * g.nz * sizeof(cplx<T>);
+    size_t sm = (uz ? 3 : 2) * (size_t)P * g.nz * sizeof(cplx<T>);
     int th = g.zth > 0 ? g.zth : threads_for(P * g.nz);
 #define CALL(PR) \
-    k_zfinal_g<PR><<<blocks, th, sm, st>>>(g, az, P, dspec, uz, vpart, div, div2, phit, phi, dhat, c, s, cs, vout, \
+    k_zfinal_g<PR><<<blocks, th, sm, st>>>(g, az, P, dspec, uz, vpart, div, div2, div3, phit, phi, dhat, c, s, cs, vout, \
                                            part)
     OFDFT_DISPATCH(T, g, CALL);
 #undef CALL
@@ -1253,7 +1268,7 @@ template <typename T> cudaError_t set_field_smem_limits(size_t bytes)
 
 #define OFDFT_INST(T)                                                                              \
     template void launch_zfwd<T>(const GridInfo &, const FftAxis &, int, const T *, const T *,     \
-                                 const T *, T, T, const void *, T *, cplx<T> *, cudaStream_t, T *); \
+                                 const T *, T, T, const void *, T *, cplx<T> *, cudaStream_t, T *, T *); \
     template void launch_dline<T>(const GridInfo &, const FftAxis &, int, int, int, const T *, T *, \
                                   cudaStream_t);                                                  \
     template int launch_pw<T>(const GridInfo &, T *, T *, T *, const T *, T, const FuncParams &,   \
@@ -1264,7 +1279,8 @@ template <typename T> cudaError_t set_field_smem_limits(size_t bytes)
                                   cudaStream_t);                                                  \
     template int launch_zfinal_gga<T>(const GridInfo &, const FftAxis &, const cplx<T> *, const T *, \
                                       const T *, const T *, const T *, const T *, const T *,      \
-                                      const T *, T, T, const void *, T *, double *, cudaStream_t); \
+                                      const T *, const T *, T, T, const void *, T *, double *,     \
+                                      cudaStream_t);                                               \
     template void launch_ypass<T>(const GridInfo &, const FftAxis &, bool, cplx<T> *, int,         \
                                   long long, cudaStream_t);                                       \
     template int launch_xhl<T>(const GridInfo &, const FftAxis &, cplx<T> *, const cplx<T> *,      \

@@ -1,0 +1,522 @@
+// Derivatives along the grid axes on the tensor cores, exact to more than
+// the double-float transforms they replace.
+//
+// The spectral derivative along an axis of n points is a real circulant
+// matrix D (antisymmetric, D(j - l)), so a batch of lines is a contraction.
+// It is taken in integers.  With h = n/2 and the half-length sums and
+// differences s = x_lo + x_hi, d = x_lo - x_hi,
+//   e = De s,  o = Do d,  out_lo = e + o,  out_hi = e - o,
+//   De, Do = (D(j - l) +- D(j - l - h)) / 2      (h x h),
+// each line is scaled by the power of two of its largest magnitude to 53-bit
+// integers (binary64's own last place at that magnitude), the matrices are
+// rounded to 54-bit integers once, and both are cut into seven signed digits
+// of radix 256.  A digit is exact in f16, a product of two is at most 2^14,
+// and the sums over h <= 128 and up to seven digit pairs (two of them with a
+// leading digit, at most 64) stay below 2^24, so the f32 accumulators of
+// tcgen05.mma (kind::f16) hold exact integers.  Digit products of equal
+// weight share one accumulator: 7 accumulators, 28 products, the first
+// dropped weight about 2^-51 of the line's largest value times the largest
+// matrix entry.
+#include <math.h>
+
+#include <algorithm>
+
+#include "ffmath.cuh"
+#include "kernels.h"
+#include "tcgen.cuh"
+
+namespace ofdft {
+
+namespace {
+
+constexpr int kLines = 64;    // lines of a tile: the rows of one M = 64 accumulator
+constexpr int kDig = 7;       // digits of radix 256
+constexpr uint64_t kDigBias = 0x0080808080808080ull;   // + 128 per digit
+constexpr int kTlThreads = 640;   // converting and reading-out threads at most; one more warp issues the products
+constexpr int kMaxChunks = 3;     // column chunks of a matrix
+constexpr int kMaxUnits = 2 * kMaxChunks;
+
+// Shared-memory distance between 8-wide K chunks of the lines' digits: one
+// 16-byte row more than the 64 lines, so that threads that walk the chunks
+// of one line (z axis) store to different banks.
+constexpr uint32_t kALbo = (kLines + 1) * 16;
+
+// Sizes of the operands for an axis of n points.  The outputs come in column
+// chunks of up to 4 groups of 8 (their 7 accumulators then fit one product's
+// N <= 256); chunk c of e and of o are units 2c and 2c + 1 of the matrix,
+// which pass through nslot shared-memory slots.
+struct TlShape {
+    int h, np, nc;            // half length; padded to 8 (N); 8-wide K chunks (an even number)
+    int chunks, g;            // column chunks; groups of 8 in each (the last may have fewer)
+    int nslot;
+    uint32_t a_dig;           // bytes of one digit of a tile half
+    uint32_t unit;            // bytes of a slot (a full chunk's unit)
+    uint32_t cols;            // tensor-memory columns
+    uint32_t smem;
+};
+
+__host__ __device__ __forceinline__ int tl_width(const TlShape &s, int c) { return 8 * min(s.g, s.np / 8 - c * s.g); }
+__host__ __device__ __forceinline__ uint32_t tl_unit_bytes(const TlShape &s, int c)
+{
+    return (uint32_t)(s.nc * kDig * tl_width(s, c) * 16);
+}
+
+constexpr size_t kTlSmemMax = 227 * 1024 - 2048;   // static shared memory of the kernel beside it
+
+TlShape tl_shape(int n)
+{
+    TlShape s;
+    s.h = n / 2;
+    s.np = (s.h + 7) / 8 * 8;
+    s.nc = (s.h + 15) / 16 * 2;
+    const int groups = s.np / 8;
+    s.chunks = std::max((groups + 3) / 4, groups > 1 ? 2 : 1);
+    s.g = (groups + s.chunks - 1) / s.chunks;
+    s.a_dig = (uint32_t)s.nc * kALbo;
+    s.unit = (uint32_t)(s.nc * kDig * s.g * 128);
+    s.cols = 32;
+    while (s.cols < (uint32_t)(kDig * s.np)) s.cols *= 2;
+    const uint32_t a = 2 * kDig * s.a_dig;
+    s.nslot = a < kTlSmemMax ? (int)std::min<size_t>(2 * s.chunks, (kTlSmemMax - a) / s.unit) : 0;
+    s.smem = a + s.nslot * s.unit;
+    return s;
+}
+
+// One axis of a launch.
+struct TlJob {
+    TlShape sh;
+    int nlines, tiles, zlen;       // lines; tiles of 64; lines of one outer index (x, y: consecutive in memory)
+    int zaxis;                     // lines contiguous in memory
+    long long ostride, rstride;    // between outer indices; between a line's points
+    int mexp;
+    const unsigned char *mat;
+    const double *in;
+    float2 *out;
+};
+constexpr int kMaxJobs = 3;
+struct TlJobs {
+    TlJob job[kMaxJobs];
+    int count;
+};
+
+// x as an integer multiple of 2^(E - 52) (truncated towards zero), E the
+// exponent of the line's largest magnitude (at least -100, so that the
+// output's unit is a normal binary32); esh = biased E.
+__device__ __forceinline__ uint64_t to_fixed(double x, int esh)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const int sh = min(esh - (int)((hi >> 20) & 0x7ffu), 63);
+    const uint64_t m = (((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32) | lo) >> sh;
+    const int64_t s = (int64_t)((int32_t)hi >> 31);
+    return (m ^ (uint64_t)s) - (uint64_t)s;
+}
+
+__device__ __forceinline__ uint32_t digit_pair(uint32_t bytes, uint32_t sel)
+{
+    // (b, 0x64) is the f16 1024 + b; minus 1152 gives the digit b - 128 exactly
+    const uint32_t u = __byte_perm(bytes, 0x64646464u, sel);
+    uint32_t r;
+    asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(u), "r"(0xe480e480u));
+    return r;
+}
+
+// The seven digits (most significant first) of eight biased integers as
+// seven 16-byte rows of f16.
+__device__ __forceinline__ void store_digits(const uint64_t (&x)[8], unsigned char *dst, uint32_t dig_bytes)
+{
+    uint32_t w[kDig][4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const uint32_t l0 = (uint32_t)x[2 * p], l1 = (uint32_t)x[2 * p + 1];
+        const uint32_t h0 = (uint32_t)(x[2 * p] >> 32), h1 = (uint32_t)(x[2 * p + 1] >> 32);
+        const uint32_t t0 = __byte_perm(l0, l1, 0x5140), t1 = __byte_perm(l0, l1, 0x7362);
+        const uint32_t u0 = __byte_perm(h0, h1, 0x5140), u1 = __byte_perm(h0, h1, 0x7362);
+        w[6][p] = digit_pair(t0, 0x4140);
+        w[5][p] = digit_pair(t0, 0x4342);
+        w[4][p] = digit_pair(t1, 0x4140);
+        w[3][p] = digit_pair(t1, 0x4342);
+        w[2][p] = digit_pair(u0, 0x4140);
+        w[1][p] = digit_pair(u0, 0x4342);
+        w[0][p] = digit_pair(u1, 0x4140);
+    }
+#pragma unroll
+    for (int d = 0; d < kDig; ++d)
+        *reinterpret_cast<uint4 *>(dst + d * dig_bytes) = make_uint4(w[d][0], w[d][1], w[d][2], w[d][3]);
+}
+
+// The accumulators (exact integers in f32, below 2^24) summed with their
+// weights 256^-d, as an unnormalised pair (s, rounding errors of the sums of
+// weight 256^-3 and up; those below are under 2^-51 of the full scale).
+// Fast2Sum is exact here although its operands are not ordered: each
+// accumulator is an integer, hence a multiple of the last place of the
+// smaller-weight sum it meets (below 2^16).
+__device__ __forceinline__ ff::f2 combine(const float (&a)[kDig])
+{
+    constexpr float w = 1.0f / 256.0f;
+    float s = ff::ffma(ff::ffma(a[6], w, a[5]), w, a[4]);
+    float err = 0.0f;
+#pragma unroll
+    for (int d = 3; d >= 0; --d) {
+        const float t = ff::ffma(s, w, a[d]);           // w is a power of two: the product is exact
+        const float e = ff::ffma(s, w, -ff::fsub(t, a[d]));
+        err = d == 3 ? e : ff::ffma(err, w, e);
+        s = t;
+    }
+    return ff::f2(s, err);
+}
+
+// x + sgn y of two such pairs, normalised, times sc (a power of two).
+__device__ __forceinline__ float2 butterfly(ff::f2 x, ff::f2 y, float sgn, float sc)
+{
+    const float s = ff::ffma(sgn, y.hi, x.hi);
+    const float bb = ff::fsub(s, x.hi);
+    const float e = ff::fadd(ff::fsub(x.hi, ff::fsub(s, bb)), ff::ffma(sgn, y.hi, -bb));
+    const float l = ff::fadd(ff::ffma(sgn, y.lo, x.lo), e);
+    const ff::f2 r = ff::fast_two_sum(s, l);
+    return make_float2(r.hi * sc, r.lo * sc);
+}
+
+__device__ __forceinline__ void bar_arrive(int id, int count) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory"); }
+__device__ __forceinline__ void bar_sync(int id, int count) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory"); }
+
+// The issuing warp: for every unit of the matrix, digit i of the lines meets
+// digits 0 .. 6 - i of the unit, which lie side by side along N as their
+// accumulators i .. 6 do.  e accumulates in lanes 0-15 of each quarter of
+// the tensor memory, o in lanes 16-31.  KS: 16-wide K steps; unrolled, so
+// that the descriptors are built in uniform registers (with run-time loops
+// the products of n = 96 took 9,400 cycles to issue, from a single thread
+// 19,100; so they run at the tensor cores' rate, 0.46 cycles a column).
+template <int KS>
+__device__ __forceinline__ bool issue(const TlShape &sh, const unsigned char *mat, uint32_t full, uint32_t done, uint32_t sa,
+                                      uint32_t sb, uint32_t tmem, int nthreads)
+{
+    const int units = 2 * sh.chunks;
+    const uint32_t a_dig = sh.a_dig;
+    bool good = true;
+#pragma unroll 1
+    for (int u = 0; u < units; ++u) {
+        const int c = u >> 1, width = tl_width(sh, c);
+        good = tc::mbar_wait(full + 8 * u, 0) && good;
+        if (u < 2) bar_sync(1 + u, nthreads);     // the digits of s (u = 0), of d (u = 1)
+        tc::fence_after_sync();
+        const uint32_t blb = (uint32_t)(kDig * width) * 16;
+        const uint64_t a0 = tc::operand(sa + (u & 1) * kDig * a_dig, kALbo, 128);
+        const uint64_t b0 = tc::operand(sb + (u % sh.nslot) * sh.unit, blb, 128);
+        const uint32_t acc = tmem + ((uint32_t)(u & 1) << 20) + c * sh.g * 8 * kDig;
+#pragma unroll
+        for (int i = 0; i < kDig; ++i) {
+            const uint32_t idesc = tc::idesc_f16(kLines, (kDig - i) * width);
+#pragma unroll
+            for (int k = 0; k < KS; ++k)
+                tc::mma_f16(acc + i * width, a0 + ((i * a_dig + k * 2 * kALbo) >> 4), b0 + ((k * 2 * blb) >> 4), idesc,
+                            (i | k) != 0);
+        }
+        tc::mma_commit(done + 8 * u);
+        const int next = u - 1 + sh.nslot;        // the unit that takes over slot (u - 1)
+        if (u >= 1 && next < units) {
+            good = tc::mbar_wait(done + 8 * (u - 1), 0) && good;
+            if ((threadIdx.x & 31) == 0) {
+                const uint32_t bytes = tl_unit_bytes(sh, next >> 1);
+                tc::mbar_expect(full + 8 * next, bytes);
+                tc::bulk_load(sb + (next % sh.nslot) * sh.unit, mat + (size_t)next * sh.unit, bytes, full + 8 * next);
+            }
+            __syncwarp();
+        }
+    }
+    return good;
+}
+
+// out = d f along each job's axis, one block per tile of 64 lines.  out may
+// be in: a block reads its lines whole before it writes them.
+//
+// M = 64 because at 96^3 tiles of 128 lines would leave half the SMs idle
+// (144 tiles of 64 for 152 SMs).  Measured (GB300, in a graph): one axis at
+// 96^3 7.8 us (z 9.5), at 48^3 5.2 us; the double-float transforms took
+// about 19 us a pass at 96^3, of which a GGA evaluation had four and the
+// two z kernels half of theirs.  Of the 12,000 cycles of a tile the MMAs
+// are 6,000 (0.5-0.7 cycles a column, M = 64 runs at half rate), the
+// conversion 2,600, the load 1,500, the read-out 1,700 behind the last MMA;
+// instruction fetch is the largest stall, since each warp runs the code once.
+__global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_constant__ TlJobs jobs)
+{
+    extern __shared__ __align__(1024) unsigned char smraw[];
+    __shared__ __align__(8) uint64_t s_bar[2 * kMaxUnits];   // units of the matrix in place; their products done
+    __shared__ uint32_t s_tmem;
+    __shared__ uint32_t s_max[kLines];
+    __shared__ int s_bad;                          // a bounded wait ran out: the tile's output is NaN
+    int ji = 0, tile = blockIdx.x;
+    while (ji + 1 < jobs.count && tile >= jobs.job[ji].tiles) tile -= jobs.job[ji++].tiles;
+    const TlJob &jb = jobs.job[ji];
+    const TlShape &sh = jb.sh;
+    const int h = sh.h, nc = sh.nc, zaxis = jb.zaxis;
+    const uint32_t a_dig = sh.a_dig;
+    unsigned char *A = smraw, *B = smraw + 2 * kDig * (size_t)a_dig;
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const int nconv = blockDim.x - 32;             // the last warp issues the products
+    const uint32_t full = tc::smem_addr(s_bar), done = full + 8 * kMaxUnits;
+    const uint32_t sa = tc::smem_addr(A), sb = tc::smem_addr(B);
+    const long long rstride = jb.rstride;
+    if (tid >= nconv) {
+        const int units = 2 * sh.chunks;
+        if (tid == nconv) {
+            s_bad = 0;
+            for (int i = 0; i < 2 * kMaxUnits; ++i) tc::mbar_init(full + 8 * i, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            for (int u = 0; u < min(units, sh.nslot); ++u) {
+                const uint32_t bytes = tl_unit_bytes(sh, u >> 1);
+                tc::mbar_expect(full + 8 * u, bytes);
+                tc::bulk_load(sb + u * sh.unit, jb.mat + (size_t)u * sh.unit, bytes, full + 8 * u);
+            }
+        }
+        __syncwarp();
+        tc::tmem_alloc(tc::smem_addr(&s_tmem), sh.cols);
+        __syncwarp();
+        tc::fence_before_sync();
+        bar_arrive(4, blockDim.x);                 // barriers and tensor memory are there
+        const uint32_t tmem = __shfl_sync(0xffffffffu, *(volatile uint32_t *)&s_tmem, 0);
+        bool good;
+        switch (nc / 2) {
+        case 1: good = issue<1>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x); break;
+        case 2: good = issue<2>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x); break;
+        case 3: good = issue<3>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x); break;
+        case 4: good = issue<4>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x); break;
+        default: good = issue<5>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x); break;
+        }
+        if (!good) s_bad = 1;
+        __syncthreads();                           // every accumulator has been read
+        tc::fence_after_sync();
+        tc::tmem_dealloc(tmem, sh.cols);
+        return;
+    }
+
+    // thread = (line, K chunk): consecutive threads walk the lines of an x or
+    // y tile, the chunks of a z line, so that loads coalesce
+    const int row = zaxis ? tid / nc : tid & (kLines - 1);
+    const int chunk = zaxis ? tid - row * nc : tid >> 6;
+    const bool mine = tid < kLines * nc;           // (a shorter job may share the launch)
+    double v[16];
+    if (mine) {
+        const int line = tile * kLines + row;
+        const bool ok = line < jb.nlines;
+        const int outer = ok ? line / jb.zlen : 0, left = min(8, h - chunk * 8);
+        const double *src = jb.in + (ok ? outer * jb.ostride + (zaxis ? 0 : line - outer * jb.zlen) : 0) + chunk * 8 * rstride;
+        const double *srh = src + h * rstride;
+        if (ok && left == 8) {
+            if (zaxis && (h & 1) == 0) {           // 16-byte aligned halves
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const double2 x = reinterpret_cast<const double2 *>(src)[i], y = reinterpret_cast<const double2 *>(srh)[i];
+                    v[2 * i] = x.x;
+                    v[2 * i + 1] = x.y;
+                    v[8 + 2 * i] = y.x;
+                    v[8 + 2 * i + 1] = y.y;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    v[i] = src[i * rstride];
+                    v[8 + i] = srh[i * rstride];
+                }
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const bool in_line = ok && i < left;
+                v[i] = in_line ? src[i * rstride] : 0.0;
+                v[8 + i] = in_line ? srh[i * rstride] : 0.0;
+            }
+        }
+    }
+    if (tid < kLines) s_max[tid] = 0x39b00000u;    // 2^-100: the least exponent of the scale
+    bar_sync(3, nconv);
+    if (mine) {
+        uint32_t m = 0;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) m = max(m, (uint32_t)__double2hiint(v[i]) & 0x7fffffffu);
+        if (m > 0x39b00000u) atomicMax(&s_max[row], m);
+    }
+    bar_sync(3, nconv);
+    // digits of s, then of d: the products of e start in between
+    unsigned char *dsta = A + chunk * kALbo + row * 16;
+    uint64_t q[8];
+    if (mine) {
+        const int esh = (int)(s_max[row] >> 20);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint64_t x = to_fixed(v[i], esh), y = to_fixed(v[8 + i], esh);
+            q[i] = x + y + kDigBias;
+            v[i] = __longlong_as_double((long long)(x - y + kDigBias));
+        }
+        store_digits(q, dsta, a_dig);
+    }
+    tc::fence_async();
+    bar_arrive(1, blockDim.x);
+    if (mine) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) q[i] = (uint64_t)__double_as_longlong(v[i]);
+        store_digits(q, dsta + kDig * a_dig, a_dig);
+    }
+    tc::fence_async();
+    bar_arrive(2, blockDim.x);
+    bar_sync(4, blockDim.x);
+    tc::fence_after_sync();
+    const uint32_t tmem = s_tmem;
+
+    // read-out: a warp reads its quarter's 16 lines of e and of o
+    const int lane = tid & 31, half = lane >> 4, quarter = warp & 3, set = warp >> 2, nset = nconv >> 7;
+    const int r = quarter * 16 + (lane & 15);
+    const int ln = tile * kLines + r;
+    const bool w_ok = ln < jb.nlines;
+    const int ou = ln / jb.zlen;
+    float2 *dst = jb.out + (w_ok ? ou * jb.ostride + (zaxis ? 0 : ln - ou * jb.zlen) : 0) + (half ? h * rstride : 0);
+    const bool wide = zaxis && (h & 1) == 0;
+    const uint32_t m = s_max[r];
+    // weight 1 stands for 2^96 times the integers' units 2^(E - 52) and 2^-mexp
+    float sc = ff::pow2i((int)(m >> 20) - 1023 + 44 - jb.mexp);
+    if (m >= 0x47f00000u) sc = __uint_as_float(0x7fc00000u);   // 2^128 and beyond, inf, NaN
+    const float sgn = half ? -1.0f : 1.0f;
+#pragma unroll 1
+    for (int ch = 0; ch < sh.chunks; ++ch) {
+        const int width = tl_width(sh, ch), j0 = ch * sh.g * 8;
+        if (!tc::mbar_wait(done + 8 * (2 * ch + 1), 0) || *(volatile int *)&s_bad) sc = __uint_as_float(0x7fc00000u);
+        tc::fence_after_sync();
+        const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + j0 * kDig;
+#pragma unroll 1
+        for (int c0 = set * 8; c0 < width; c0 += nset * 8) {
+            float a[kDig][8];
+#pragma unroll
+            for (int d = 0; d < kDig; ++d) tc::tmem_ld8(acc + d * width + c0, a[d]);
+            tc::tmem_wait_ld();
+#pragma unroll
+            for (int d = 0; d < kDig; ++d) tc::pin8(a[d]);
+            float2 y[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                float t[kDig];
+#pragma unroll
+                for (int d = 0; d < kDig; ++d) t[d] = a[d][i];
+                const ff::f2 own = combine(t);
+                ff::f2 other;
+                other.hi = __shfl_xor_sync(0xffffffffu, own.hi, 16);
+                other.lo = __shfl_xor_sync(0xffffffffu, own.lo, 16);
+                y[i] = butterfly(other, own, sgn, sc);
+            }
+            const int j = j0 + c0;
+            float2 *p = dst + j * rstride;
+            if (w_ok && j + 8 <= h) {
+                if (wide) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        reinterpret_cast<float4 *>(p)[i] = make_float4(y[2 * i].x, y[2 * i].y, y[2 * i + 1].x, y[2 * i + 1].y);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) p[i * rstride] = y[i];
+                }
+            } else if (w_ok) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (j + i < h) p[i * rstride] = y[i];
+            }
+        }
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+}
+
+}  // namespace
+
+bool tline_supported(int n)
+{
+    const TlShape s = tl_shape(n);
+    return s.nslot >= 2 && kDig * s.np <= 512 && kLines * s.nc <= kTlThreads;
+}
+
+size_t tline_matrix_bytes(int n)
+{
+    const TlShape s = tl_shape(n);
+    return 2 * (size_t)s.chunks * s.unit;
+}
+
+// De and Do times scale as seven f16 digits each, laid out as the kernel's
+// shared-memory image ([column chunk][e, o][K chunk][digit][output][8]);
+// returns the binary exponent of the integers (entry = integer 2^-mexp).
+int tline_derivative_matrix(int n, double scale, uint16_t *img)
+{
+    const TlShape s = tl_shape(n);
+    const int h = s.h;
+    std::vector<long double> D(n, 0.0L);   // D(m) = (scale/2) (-1)^m cot(pi m/n), period n
+    for (int m = 1; m < n; ++m) {
+        const long double x = 3.14159265358979323846264338327950288L * (long double)m / (long double)n;
+        D[m] = (long double)scale * 0.5L * ((m & 1) ? -1.0L : 1.0L) * (2 * m == n ? 0.0L : cosl(x) / sinl(x));
+    }
+    long double big = 0.0L;
+    std::vector<long double> c(2 * (size_t)n);     // De(m), Do(m) for m = j - l + h
+    for (int half = 0; half < 2; ++half)
+        for (int m = -h + 1; m < h; ++m) {
+            const long double a = D[(m + n) % n], b = D[(m - h + 2 * n) % n];
+            const long double v = 0.5L * (half ? a - b : a + b);
+            c[(size_t)half * n + m + h] = v;
+            big = std::max(big, fabsl(v));
+        }
+    int e = 0;
+    frexpl(big, &e);                               // big in [2^(e-1), 2^e)
+    const int mexp = 54 - e;                       // integers up to 2^54
+    std::fill(img, img + tline_matrix_bytes(n) / 2, (uint16_t)0);
+    for (int half = 0; half < 2; ++half)
+        for (int j = 0; j < h; ++j) {
+            const int ch = j / (8 * s.g), width = tl_width(s, ch), jj = j - ch * 8 * s.g;
+            uint16_t *base = img + (size_t)(2 * ch + half) * s.unit / 2;
+            for (int l = 0; l < h; ++l) {
+                const long long v = llroundl(ldexpl(c[(size_t)half * n + (j - l) + h], mexp));
+                const uint64_t b = (uint64_t)v + kDigBias;
+                for (int d = 0; d < kDig; ++d) {
+                    const int dig = (int)((b >> (8 * (6 - d))) & 0xff) - 128;
+                    uint16_t f = 0;                // f16 of a small integer: exact
+                    if (dig != 0) {
+                        int a = dig < 0 ? -dig : dig, ex = 0;
+                        while ((a >> ex) > 1) ++ex;
+                        f = (uint16_t)((dig < 0 ? 0x8000 : 0) | ((ex + 15) << 10) | ((a << (10 - ex)) & 0x3ff));
+                    }
+                    base[((size_t)(l / 8) * kDig * width + (size_t)d * width + jj) * 8 + l % 8] = f;
+                }
+            }
+        }
+    return mexp;
+}
+
+cudaError_t tline_smem_limits()
+{
+    return cudaFuncSetAttribute(k_tline, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTlSmemMax);
+}
+
+void launch_tline(const GridInfo &g, const FftAxis *const ax[3], const double *const in[3], float2 *const out[3],
+                  cudaStream_t st)
+{
+    TlJobs jobs{};
+    int blocks = 0, items = 0;
+    uint32_t smem = 0;
+    const long long plane = (long long)g.ny * g.nz;
+    const int n3[3] = {g.nx, g.ny, g.nz};
+    for (int a = 0; a < 3; ++a) {
+        if (!ax[a]) continue;
+        TlJob &j = jobs.job[jobs.count++];
+        j.sh = tl_shape(n3[a]);
+        j.nlines = (int)(g.N / n3[a]);
+        j.tiles = (j.nlines + kLines - 1) / kLines;
+        j.zaxis = a == 2;
+        j.zlen = a == 0 ? (int)plane : (a == 1 ? g.nz : 1);
+        j.ostride = a == 2 ? g.nz : plane;               // (x: one outer index)
+        j.rstride = a == 0 ? plane : (a == 1 ? g.nz : 1);
+        j.mexp = ax[a]->dexp;
+        j.mat = (const unsigned char *)ax[a]->dmat;
+        j.in = in[a];
+        j.out = out[a];
+        blocks += j.tiles;
+        items = std::max(items, kLines * j.sh.nc);
+        smem = std::max(smem, j.sh.smem);
+    }
+    const int threads = items;
+    k_tline<<<blocks, threads + 32, smem, st>>>(jobs);
+}
+
+}  // namespace ofdft
