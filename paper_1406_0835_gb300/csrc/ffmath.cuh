@@ -242,11 +242,11 @@ FF_HD f2 &operator+=(f2 &x, f2 y) { return x = add_s(x, y); }
 FF_HD bool operator>(f2 x, f2 y) { return x.hi > y.hi || (x.hi == y.hi && x.lo > y.lo); }
 
 // Binary64 -> double-float with integer operations only: hi takes the
-// leading 24 significand bits (truncated), lo the next 23 (exact, built with
-// the 2^23 trick); the 6 bits left are dropped (relative error < 2^-46).
+// leading 24 significand bits (truncated), lo the 29 bits left, rounded to
+// binary32 by the integer conversion (relative error < 2^-53).
 // Magnitudes below 2^-126 (and zero) give zero; beyond the binary32 range
 // inf of the same sign, NaN for NaN, with lo = 0.  The result is a
-// valid double-float with |lo| < ulp(hi).
+// valid double-float with |lo| <= ulp(hi).
 FF_HD f2 split_int(double d)
 {
     uint64_t b;
@@ -267,9 +267,8 @@ FF_HD f2 split_int(double d)
         return f2(int_bits_float(nan ? 0x7fc00000u : (sign | 0x7f800000u)), 0.0f);
     }
     const uint32_t hib = sign | ((uint32_t)(E + 127) << 23) | (uint32_t)((b >> 29) & 0x7fffffu);
-    const uint32_t lint = (uint32_t)(b >> 6) & 0x7fffffu;    // significand bits 28..6
-    float lo = fsub(int_bits_float(0x4b000000u | lint), 8388608.0f);   // exact integer < 2^23
-    lo = fmul(fmul(lo, 1.4210854715202004e-14f), pow2i(E));              // * 2^-46 * 2^E
+    float lo = (float)(int32_t)((uint32_t)b & 0x1fffffffu);              // significand bits 28..0
+    lo = fmul(fmul(lo, 2.220446049250313e-16f), pow2i(E));               // * 2^-52 * 2^E
     return f2(int_bits_float(hib), sign ? -lo : lo);
 }
 
@@ -283,26 +282,68 @@ FF_HD f2 fma_step(f2 p, float u, f2 c)
     float w = fadd(s.lo, fadd(ml, c.lo));
     return fast_two_sum(s.hi, w);
 }
+// The same without the final renormalisation (|lo| stays within a few
+// ulp(hi), which the next step's binary32 products with lo carry as well):
+// 11 instead of 14 operations.  Renormalise the last step's result.
+FF_HD f2 fma_step_u(f2 p, float u, f2 c)
+{
+    f2 m = two_prod(p.hi, u);
+    f2 s = two_sum(m.hi, c.hi);
+    return {s.hi, fadd(ffma(p.lo, u, m.lo), fadd(s.lo, c.lo))};
+}
 
+// Binary32 reciprocal and inverse square root to about an ulp: the
+// hardware approximation and one Newton step.
+FF_HD float recip_f(float y)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(y));
+    return ffma(r, ffma(-y, r, 1.0f), r);
+#else
+    return 1.0f / y;
+#endif
+}
+FF_HD float rsqrt_f(float x)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return ffma(0.5f * r, ffma(-fmul(x, r), r, 1.0f), r);
+#else
+    return 1.0f / sqrtf(x);
+#endif
+}
 
-// x / y: binary32 quotient q1, remainder r = x - q1 y in double-float, then
-// q1 + r/y.  Relative error a few u^2.
+// x / y: q1 = x r with the binary32 reciprocal r of y, the remainder
+// x - q1 y (its leading part exact by the FMA), then q1 + r (x - q1 y).
+// Relative error a few u^2.  (With binary32 divisions and a double-float
+// remainder this took four times the instructions.)
 FF_HD f2 div(f2 x, f2 y)
 {
-    float q1 = x.hi / y.hi;
-    f2 r = sub(x, mul(y, q1));
-    float q2 = r.hi / y.hi;
-    return fast_two_sum(q1, q2);
+    const float r = recip_f(y.hi);
+    const float q1 = fmul(x.hi, r);
+    float e = ffma(-q1, y.hi, x.hi);
+    e = ffma(-q1, y.lo, fadd(e, x.lo));
+    return fast_two_sum(q1, fmul(e, r));
 }
-FF_HD f2 recip(f2 y) { return div(f2{1.0f, 0.0f}, y); }
+FF_HD f2 recip(f2 y)
+{
+    const float r = recip_f(y.hi);
+    const float e = ffma(-r, y.lo, ffma(-r, y.hi, 1.0f));
+    return fast_two_sum(r, fmul(e, r));
+}
 FF_HD f2 operator/(f2 x, f2 y) { return div(x, y); }
 
-// sqrt(x), x > 0: s = binary32 root, then s + (x - s^2)/(2 s).
+// sqrt(x), x > 0: s = the binary32 root from the inverse root r and one
+// Newton step, then s + (x - s^2) r / 2.
 FF_HD f2 sqrt(f2 x)
 {
-    float s = sqrtf(x.hi);
-    f2 r = sub(x, two_prod(s, s));
-    return fast_two_sum(s, r.hi / (2.0f * s));
+    const float r = rsqrt_f(x.hi);
+    const float s0 = fmul(x.hi, r);
+    const float s = ffma(ffma(-s0, s0, x.hi), 0.5f * r, s0);
+    const float e = fadd(ffma(-s, s, x.hi), x.lo);
+    return fast_two_sum(s, fmul(e, 0.5f * r));
 }
 
 // e^r - 1 for |r| <= 0.35.  With s = r/8 (|s| <= 0.044) the Taylor series

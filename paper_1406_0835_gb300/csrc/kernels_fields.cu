@@ -59,8 +59,8 @@ template <> __device__ __forceinline__ double2 stc<DD>(ff::cf2 v)
 {
     return make_double2(ff::to_double(v.x), ff::to_double(v.y));
 }
-// Derivative fields between kernels of one evaluation: the double-float
-// kernels keep them as pairs (hi, lo) in the 8 bytes of a binary64, so that
+// Derivative fields and v_part between kernels of one evaluation: the
+// double-float kernels keep them as pairs (hi, lo) in the 8 bytes of a binary64, so that
 // neither side converts.
 template <typename PR> __device__ __forceinline__ typename KT<PR>::R ldp(typename KT<PR>::T x) { return x; }
 template <> __device__ __forceinline__ ff::f2 ldp<DD>(double x)
@@ -220,6 +220,7 @@ __device__ __noinline__ PwF2 pw_dd_fallback(const FuncParams &fp, const double *
     o.eps = ff::f2(b.eps);
     o.vxc = ff::f2(b.vxc);
     for (int a = 0; a < 3; ++a) o.w[a] = ff::f2(b.wc * gd[a]);
+    o.wg = ff::f2(b.wc * (gd[0] * gd[0] + gd[1] * gd[1] + gd[2] * gd[2]));
     return o;
 }
 
@@ -822,6 +823,12 @@ __global__ void OFDFT_FFT_BOUNDS k_dline_ws(GridInfo g, FftAxis fa, const typena
 // Partials: F_s, TS, F_xc, sum(n df/dn - f), sum W.grad n,
 // sum n(v_xc - eps_xc); with STRESS also sum W_a d_b n for ab = xx, yy,
 // zz, xy, xz, yz (the gradient part of Eq. (stressTF_b)) in rows 6..11.
+// The double-float form is bound by instruction issue (74 % of the issue
+// slots at 96^3; 86,000 warp instructions per thousand points, 90 us, before:
+// 96,000 and 123 us): polynomial steps without renormalisation, quotients
+// and roots from one reciprocal (a quarter of the instructions), the PZ81
+// logarithm from a table instead of an exponential, sums of like terms
+// without the cancellation-proof form, W.grad n from s^2.
 // Threads per block of the pointwise kernel and the blocks per SM its
 // register budget is sized for (launch bounds).
 #ifndef OFDFT_PW_THREADS
@@ -862,12 +869,12 @@ __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB) k_pw(GridInfo
             const R ph = ldr<PR>(phit[i]);
             const R n = ph * ph;
             const PwF2 o = pw_dd(fp, tab, tcoef, (double)temp, n, gr, xc);
-            vpart[i] = str<PR>(o.dfdn + o.vxc);
+            vpart[i] = stp<PR>(o.dfdn + o.vxc);
             acc[0] += o.f;
             acc[1] += o.ts;
             acc[2] += n * o.eps;
             acc[3] += n * o.dfdn - o.f;
-            acc[4] += o.w[0] * gr[0] + o.w[1] * gr[1] + o.w[2] * gr[2];
+            acc[4] += o.wg;
             acc[5] += n * (o.vxc - o.eps);
             for (int a = 0; a < 3; ++a) w[a] = o.w[a];
         } else {
@@ -921,8 +928,8 @@ __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB) k_pw(GridInfo
 // transform serves both) and div = d_x U_x + d_y U_y, given as one field or
 // as two (div + div2; div2 may be null).  div may alias vout (each point is
 // read before it is written, by the same thread).  With uz null, d_z U_z is
-// given as the field div3 instead.  div, div2 and div3 are derivative fields
-// (ldp).  Partials
+// given as the field div3 instead.  vpart, div, div2 and div3 are stored as
+// derivative fields are (ldp).  Partials
 // (as k_zfinal's GGA form): rows 0..5 zero, then sum phi^2 v, sum phi^2,
 // sum 2 phi v dphi/dtheta.
 template <typename PR>
@@ -978,7 +985,7 @@ __global__ void OFDFT_FFT_BOUNDS k_zfinal_g(GridInfo g, FftAxis az, int P, const
         const R dr = (rc.r & 1) ? d.y : d.x;
         const R ph = ldr<PR>(phit[rbase + i]);
         const R n = ph * ph;
-        R v = ldr<PR>(vpart[rbase + i]) + dr - ldp<PR>(div[rbase + i]);
+        R v = ldp<PR>(vpart[rbase + i]) + dr - ldp<PR>(div[rbase + i]);
         if (div2 != nullptr) v = v - ldp<PR>(div2[rbase + i]);
         if (uz == nullptr) v = v - ldp<PR>(div3[rbase + i]);
         vout[rbase + i] = str<PR>(v);

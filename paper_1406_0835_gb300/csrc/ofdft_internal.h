@@ -205,9 +205,14 @@ constexpr int kEnEmin = -20;
 constexpr int kEnEmax = 6;
 constexpr int kEnPanels = (kEnEmax - kEnEmin) * kEnSub;
 constexpr int kEnSize = kEnPanels * kEnNc;
+// Logarithm table of the double-float kernels: kLgSub intervals of [1, 2),
+// two pairs each (a binary32 reciprocal, its negative logarithm).
+constexpr int kLgSub = 256;
+constexpr int kLgSize = 2 * kLgSub;
 // Storage of the FP64 field sets' tables, in doubles: the binary64
-// temperature table, its double-float split, the enhancement table's split.
-constexpr int kDdTabSize = 2 * kTfSize + kEnSize;
+// temperature table, its double-float split, the enhancement table's split,
+// the logarithm table.
+constexpr int kDdTabSize = 2 * kTfSize + kEnSize + kLgSize;
 
 // Build the table on the host (FP64 monomial coefficients per panel).
 const std::vector<double> &tfunc_table_host();

@@ -310,8 +310,8 @@ constexpr int kHornerUnroll = OFDFT_HORNER_UNROLL;   // Horner steps unrolled (c
 // the terms of degree >= split in binary32 (their sum, times u^split, is
 // below 2^-24 of the polynomial's smallest value on every panel of the
 // table, so binary32 rounding there stays below the double-float
-// rounding), the rest in double-float.  A split of deg runs every step in
-// double-float.
+// rounding), the rest in double-float, p and dp unnormalised.  A split of
+// deg runs every step in double-float.
 OF_HD void horner_split_f2(const ff::f2 *__restrict__ c, int deg, int split, float uh, ff::f2 &p, ff::f2 &dp,
                            float &d2)
 {
@@ -334,8 +334,8 @@ OF_HD void horner_split_f2(const ff::f2 *__restrict__ c, int deg, int split, flo
 #pragma unroll kHornerUnroll
     for (; j >= 0; --j) {
         d2 = d2 * uh + dp.hi;
-        dp = ff::fma_step(dp, uh, p);
-        p = ff::fma_step(p, uh, c[j]);
+        dp = ff::fma_step_u(dp, uh, p);
+        p = ff::fma_step_u(p, uh, c[j]);
     }
 }
 
@@ -464,9 +464,33 @@ OF_HD void enhance_vt84f_tab(const ff::f2 *__restrict__ etab, ff::f2 x, ff::f2 &
     dF = add(G, mul(x, dG));
 }
 
+// ln x for x > 0 (normal binary32 range): x = 2^e m, the table's binary32
+// reciprocal r of the centre of m's 2^-8-wide interval and its -ln r, then
+// ln m = -ln r + log1p(m r - 1) with |m r - 1| < 2^-8.9: the square in
+// double-float, the terms from the cube on in binary32.  Absolute error a
+// few 2^-48 max(1, |ln x|).
+OF_HD ff::f2 log_tab(const ff::f2 *__restrict__ ltab, ff::f2 x)
+{
+    using namespace ff;
+    int e;
+    float inv2e;
+    const float m = split_pow2(x.hi, e, inv2e);
+    const int i = (int)((m - 1.0f) * (float)kLgSub);
+    const float r = ltab[2 * i].hi;
+    const f2 z = two_prod(m, r);
+    const f2 d = add(f2(fadd(z.hi, -1.0f), z.lo), fmul(fmul(x.lo, inv2e), r));   // z.hi - 1 is exact
+    const float t = d.hi;
+    const f2 sq = two_prod(t, t);
+    const float cube = fmul(t * t, t) * (1.0f / 3.0f + t * (-0.25f + t * (0.2f - t * (1.0f / 6.0f))));
+    const f2 l1 = add(d, f2(-0.5f * sq.hi, ffma(-t, d.lo, -0.5f * sq.lo) + cube));
+    const f2 k = two_prod((float)e, FFC(kLn2).hi);
+    const f2 base = add(f2(k.hi, ffma((float)e, FFC(kLn2).lo, k.lo)), ltab[2 * i + 1]);
+    return add(base, l1);
+}
+
 // PZ81 (same branches and constants as pz81_point) from n, n^(1/3) and
-// y = n^(-1/3) in double-float.
-OF_HD void pz81_f2(ff::f2 c13, ff::f2 y, ff::f2 &eps, ff::f2 &v)
+// y = n^(-1/3) in double-float.  Sums of like terms of one size: add_s.
+OF_HD void pz81_f2(const ff::f2 *__restrict__ ltab, ff::f2 c13, ff::f2 y, ff::f2 &eps, ff::f2 &v)
 {
     using namespace ff;
     const f2 rs = mul(y, FFC(0.62035049089940001667));
@@ -474,25 +498,26 @@ OF_HD void pz81_f2(ff::f2 c13, ff::f2 y, ff::f2 &eps, ff::f2 &v)
     f2 ec, vc;
     if (rs.hi >= 1.0f) {
         const f2 sq = sqrt(rs);
-        const f2 den = recip(add(add(mul(sq, FFC(1.0529)), mul(rs, FFC(0.3334))), 1.0f));
+        const f2 den = recip(add(add_s(mul(sq, FFC(1.0529)), mul(rs, FFC(0.3334))), 1.0f));
         ec = mul(den, FFC(-0.1423));
-        const f2 num = add(add(mul(sq, FFC(7.0 / 6.0 * 1.0529)), mul(rs, FFC(4.0 / 3.0 * 0.3334))), 1.0f);
+        const f2 num = add(add_s(mul(sq, FFC(7.0 / 6.0 * 1.0529)), mul(rs, FFC(4.0 / 3.0 * 0.3334))), 1.0f);
         vc = mul(mul(ec, num), den);
     } else {
-        const f2 lr = log(rs);
-        const f2 rlr = mul(rs, lr);
-        ec = add(add(mul(lr, FFC(0.0311)), FFC(-0.048)), add(mul(rlr, FFC(kPzC)), mul(rs, FFC(kPzD))));
-        vc = add(add(mul(lr, FFC(0.0311)), FFC(-0.048 - 0.0311 / 3.0)),
-                 add(mul(rlr, FFC(2.0 / 3.0 * kPzC)), mul(rs, FFC((2.0 * kPzD - kPzC) / 3.0))));
+        const f2 lr = log_tab(ltab, rs);
+        const f2 rlr = mul(rs, lr), al = mul(lr, FFC(0.0311));
+        ec = add_s(add_s(al, FFC(-0.048)), add_s(mul(rlr, FFC(kPzC)), mul(rs, FFC(kPzD))));
+        vc = add_s(add_s(al, FFC(-0.048 - 0.0311 / 3.0)),
+                   add_s(mul(rlr, FFC(2.0 / 3.0 * kPzC)), mul(rs, FFC((2.0 * kPzD - kPzC) / 3.0))));
     }
-    eps = add(ex, ec);
-    v = add(mul(ex, FFC(4.0 / 3.0)), vc);
+    eps = add_s(ex, ec);
+    v = add_s(mul(ex, FFC(4.0 / 3.0)), vc);
 }
 
 // Double-float outputs of the pointwise functional at one point.
 struct PwF2 {
     ff::f2 f, ts, dfdn, eps, vxc;
     ff::f2 w[3];    // W = d f_s / d(grad n), by component
+    ff::f2 wg;      // W . grad n
 };
 
 // f_s, its derivatives and (xc != 0) PZ81 at one point from n and the
@@ -513,7 +538,6 @@ OF_HD bool pw_core_f2(const FuncParams &fp, const ff::f2 *__restrict__ tab, ff::
     const f2 n23 = mul(c13, c13);
     const f2 rn = mul(y2, y);                                // 1/n
     const f2 tau0 = mul(mul(n, n23), FFC(OF_CTF));           // Eq. (tauTFdefn)
-    const f2 dtau0 = mul(n23, FFC(5.0 / 3.0 * OF_CTF));
     const f2 dtdn = mul(mul(t, rn), FFC(-2.0 / 3.0));
     f2 tf[8];
     if (fp.kind == 0) {                                      // ftTF
@@ -521,12 +545,13 @@ OF_HD bool pw_core_f2(const FuncParams &fp, const ff::f2 *__restrict__ tab, ff::
         const f2 kap = sub(tf[0], tf[1]);
         o.f = mul(tau0, kap);
         o.ts = mul(tau0, tf[1]);
+        const f2 dtau0 = mul(n23, FFC(5.0 / 3.0 * OF_CTF));
         o.dfdn = add(mul(dtau0, kap), mul(mul(tau0, sub(tf[4], tf[5])), dtdn));   // Eq. (vTF)
-        o.w[0] = o.w[1] = o.w[2] = f2(0.0f, 0.0f);
+        o.w[0] = o.w[1] = o.w[2] = o.wg = f2(0.0f, 0.0f);
     } else {
         const f2 rn43 = mul(y2, y2);                         // n^(-4/3)
         const f2 q0 = mul(gr[0], rn43), q1 = mul(gr[1], rn43), q2 = mul(gr[2], rn43);
-        const f2 s2 = mul(add(add(mul(q0, q0), mul(q1, q1)), mul(q2, q2)), FFC(OF_CS));   // Eq. (s_0defn)
+        const f2 s2 = mul(add_s(add_s(mul(q0, q0), mul(q1, q1)), mul(q2, q2)), FFC(OF_CS));   // Eq. (s_0defn)
         if (!(s2.hi <= (float)kPwS2max)) return false;
         tfunc_eval_f2<4>(tab, t, tf);
         const f2 xi = tf[0], ze = tf[1], A = tf[2], B = tf[3];
@@ -543,23 +568,30 @@ OF_HD bool pw_core_f2(const FuncParams &fp, const ff::f2 *__restrict__ tab, ff::
         }
         const f2 Fs = add(neg(Fsg), 2.0f), dFs = neg(dFsg); // F_sigma = 2 - F_tau(s_sigma)
         const f2 kin = mul(tau0, xi), ent = mul(tau0, ze);
-        o.f = sub(mul(kin, Ft), mul(ent, Fs));              // Eq. (FGGA)
-        o.ts = mul(ent, Fs);
+        // (add_s below: the operands carry a few u^2 of their own size, and
+        // every sum is judged against the size of its terms)
+        const f2 eF = mul(ent, Fs);
+        o.f = add_s(mul(kin, Ft), neg(eF));                 // Eq. (FGGA)
+        o.ts = eF;
         const f2 e83 = mul(rn, FFC(-8.0 / 3.0));
         const f2 s2dt = mul(s2, dtdn);
-        // Eq. (vftGGA), first two lines
-        f2 d = mul(dtau0, sub(mul(xi, Ft), mul(ze, Fs)));
-        d = add(d, mul(mul(tau0, dtdn), sub(mul(dxi, Ft), mul(dze, Fs))));
-        d = add(d, mul(mul(kin, dFt), add(mul(e83, xt), mul(s2dt, dA))));
-        d = sub(d, mul(mul(ent, dFs), add(mul(e83, xs), mul(s2dt, dB))));
+        const f2 kF = mul(kin, dFt), sF = mul(ent, dFs);
+        // Eq. (vftGGA), first two lines; dtau0 (xi F_tau - zeta F_sigma) = (5/3) f / n
+        f2 d = mul(div(o.f, n), FFC(5.0 / 3.0));
+        d = add_s(d, mul(mul(tau0, dtdn), add_s(mul(dxi, Ft), neg(mul(dze, Fs)))));
+        d = add_s(d, mul(kF, add_s(mul(e83, xt), mul(s2dt, dA))));
+        d = add_s(d, neg(mul(sF, add_s(mul(e83, xs), mul(s2dt, dB)))));
         o.dfdn = d;
         // last line: W = [tau0 xi F_tau' A - tau0 zeta F_sigma' B] d s^2 / d grad n
-        const f2 wpre = sub(mul(mul(kin, dFt), A), mul(mul(ent, dFs), B));
+        const f2 wpre = add_s(mul(kF, A), neg(mul(sF, B)));
         const f2 wr = mul(mul(wpre, rn43), FFC(2.0 * OF_CS));
-        for (int a = 0; a < 3; ++a) o.w[a] = mul(wr, mul(gr[a], rn43));
+        o.w[0] = mul(wr, q0);
+        o.w[1] = mul(wr, q1);
+        o.w[2] = mul(wr, q2);
+        o.wg = scale(mul(wpre, s2), 2.0f);                  // d s^2/d grad n . grad n = 2 s^2
     }
     if (xc) {
-        pz81_f2(c13, y, o.eps, o.vxc);
+        pz81_f2(tab + kTfSize + kEnSize, c13, y, o.eps, o.vxc);
     } else {
         o.eps = f2(0.0f, 0.0f);
         o.vxc = f2(0.0f, 0.0f);
@@ -596,8 +628,8 @@ inline void tfunc_table_split(const double *tab, float *out, int count = kTfSize
 
 // The FP64 field sets' tables in dst[kDdTabSize]: the binary64 temperature
 // table, its double-float split, the double-float VT84F enhancement table
-// (the split temperature table and the enhancement table are contiguous,
-// as pw_core_f2 reads them).
+// and the logarithm table (the last three contiguous, as pw_core_f2 reads
+// them).
 inline void dd_tables_fill(const double *ttab, double *dst)
 {
     for (int i = 0; i < kTfSize; ++i) dst[i] = ttab[i];
@@ -605,6 +637,15 @@ inline void dd_tables_fill(const double *ttab, double *dst)
     double etab[kEnSize];
     enh_table_fill(etab);
     tfunc_table_split(etab, reinterpret_cast<float *>(dst + 2 * kTfSize), kEnSize);
+    float *lg = reinterpret_cast<float *>(dst + 2 * kTfSize + kEnSize);   // {r, 0}, -ln r per interval
+    for (int i = 0; i < kLgSub; ++i) {
+        const float r = (float)(1.0 / (1.0 + (i + 0.5) / kLgSub));
+        const long double l = -logl((long double)r);
+        lg[4 * i] = r;
+        lg[4 * i + 1] = 0.0f;
+        lg[4 * i + 2] = (float)l;
+        lg[4 * i + 3] = (float)(l - (long double)(float)l);
+    }
 }
 
 }  // namespace ofdft
