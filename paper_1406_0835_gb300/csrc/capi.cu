@@ -1351,14 +1351,17 @@ template <typename T> ofdft_status alloc_fieldset(ofdft_ctx *c, FieldSet &f)
     f.spec_stride = cb / sizeof(cplx<T>);
     // v_ext(G); the Heine-Abarenkov form and triclinic cells append the pressure weights
     CK(cudaMallocAsync((void **)&f.vext, (size_t)((g.lpp || g.tri) ? 2 : 1) * g.NH * sizeof(cplx<T>), c->st));
-    // temperature table; FP64 sets append its double-float split (hi, lo
-    // binary32 pairs) and the double-float VT84F enhancement table for the
-    // double-float pointwise functional
+    // temperature table; FP64 sets append its refined double-float copy (hi,
+    // lo binary32 pairs), the double-float VT84F enhancement table and the
+    // logarithm table for the double-float pointwise functional
     const std::vector<double> &tab = tfunc_table_host();
     std::vector<T> tt(tab.begin(), tab.end());
     if (sizeof(T) == 8) {
-        std::vector<double> dd((size_t)kDdTabSize);
-        dd_tables_fill(tab.data(), dd.data());
+        static const std::vector<double> dd = [&] {   // constants, built once
+            std::vector<double> d((size_t)kDdTabSize);
+            dd_tables_fill(tab.data(), d.data());
+            return d;
+        }();
         tt.assign(dd.begin(), dd.end());
     }
     CK(cudaMallocAsync((void **)&f.tab, tt.size() * sizeof(T), c->st));
@@ -1445,7 +1448,7 @@ double footprint_bytes(const int grid[3], int nat, int precision)
 {
     const double nx = grid[0], ny = grid[1], nz = grid[2];
     const double K = std::floor(nz / 2) + 1, N = nx * ny * nz, NH = nx * ny * K;
-    const double tab = (double)tfunc_table_host().size();
+    const double tab = kDdTabSize;
     auto fieldset = [&](double sz) {
         double cb = std::ceil(NH * 2 * sz / 256.0) * 256.0;
         // v_ext(G) counted twice: the Heine-Abarenkov form adds its pressure weights

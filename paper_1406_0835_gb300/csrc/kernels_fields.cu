@@ -823,12 +823,14 @@ __global__ void OFDFT_FFT_BOUNDS k_dline_ws(GridInfo g, FftAxis fa, const typena
 // Partials: F_s, TS, F_xc, sum(n df/dn - f), sum W.grad n,
 // sum n(v_xc - eps_xc); with STRESS also sum W_a d_b n for ab = xx, yy,
 // zz, xy, xz, yz (the gradient part of Eq. (stressTF_b)) in rows 6..11.
-// The double-float form is bound by instruction issue (74 % of the issue
-// slots at 96^3; 86,000 warp instructions per thousand points, 90 us, before:
-// 96,000 and 123 us): polynomial steps without renormalisation, quotients
-// and roots from one reciprocal (a quarter of the instructions), the PZ81
-// logarithm from a table instead of an exponential, sums of like terms
-// without the cancellation-proof form, W.grad n from s^2.
+// The double-float form is bound by instruction issue (73 % of the issue
+// slots at 96^3, 2,470 instructions a point, 79 us).  From 3,060 and 118 us:
+// polynomial steps without renormalisation, quotients and roots from one
+// reciprocal (a quarter of the instructions), the PZ81 logarithm from a
+// table instead of an exponential, sums of like terms without the
+// cancellation-proof form, W.grad n from s^2 (2,860, 91 us); refined table
+// panels with 20 instead of 32 double-float steps and the polynomials side
+// by side in one rolled loop.
 // Threads per block of the pointwise kernel and the blocks per SM its
 // register budget is sized for (launch bounds).
 #ifndef OFDFT_PW_THREADS

@@ -193,6 +193,19 @@ constexpr int kTfPanels = (kTfEmax - kTfEmin) * kTfSub;
 constexpr int kTfFuncs = 4;                // xi, zeta, A, B
 constexpr int kTfSize = kTfPanels * kTfFuncs * kTfNc;
 
+// The double-float kernels read the same polynomials re-expanded about the
+// centres of kTfRef subpanels: their terms fall off kTfRef times faster per
+// degree, so that those from degree kTfSplit up can be summed in binary32
+// (pointwise.cuh).  Layout per subpanel, in double-float pairs (8 bytes):
+// degrees 0 .. kTfSplit - 1 as pairs [degree][function], then the degrees
+// up to kTfDdDeg as binary32 [degree][function]; 16-byte loads throughout.
+constexpr int kTfRef = 4;
+constexpr int kTfDdSub = kTfSub * kTfRef;
+constexpr int kTfDdDeg = 9;                // the terms of degree 10 are below 3e-16 of their function
+constexpr int kTfSplit = 5;
+constexpr int kTfDdRow = kTfSplit * kTfFuncs + (kTfDdDeg + 1 - kTfSplit) * kTfFuncs / 2;
+constexpr int kTfDdSize = kTfPanels * kTfRef * kTfDdRow;
+
 // VT84F enhancement factor F(x), x = s^2 (Eq. (VT84F)), as a table of
 // G = (F - 1)/x for the double-float kernels: 16 panels per octave of x
 // over [2^-20, 2^6), degree 10 in the panel variable u in [-1, 1) (below:
@@ -205,14 +218,19 @@ constexpr int kEnEmin = -20;
 constexpr int kEnEmax = 6;
 constexpr int kEnPanels = (kEnEmax - kEnEmin) * kEnSub;
 constexpr int kEnSize = kEnPanels * kEnNc;
+// The double-float kernels' copy, per panel: degrees 0 .. kEnSplit - 1 as
+// pairs (padded to an even number), the others in binary32 (padded to 8).
+constexpr int kEnSplit = 5;
+constexpr int kEnDdRow = (kEnSplit + 1) / 2 * 2 + 4;
+constexpr int kEnDdSize = kEnPanels * kEnDdRow;
 // Logarithm table of the double-float kernels: kLgSub intervals of [1, 2),
 // two pairs each (a binary32 reciprocal, its negative logarithm).
 constexpr int kLgSub = 256;
 constexpr int kLgSize = 2 * kLgSub;
 // Storage of the FP64 field sets' tables, in doubles: the binary64
-// temperature table, its double-float split, the enhancement table's split,
-// the logarithm table.
-constexpr int kDdTabSize = 2 * kTfSize + kEnSize + kLgSize;
+// temperature table, its refined double-float copy, the enhancement table's
+// split, the logarithm table.
+constexpr int kDdTabSize = kTfSize + kTfDdSize + kEnDdSize + kLgSize;
 
 // Build the table on the host (FP64 monomial coefficients per panel).
 const std::vector<double> &tfunc_table_host();

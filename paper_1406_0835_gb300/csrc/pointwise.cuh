@@ -294,89 +294,86 @@ template <typename T> struct PwOut {
 
 constexpr double kPwNmin = 1e-18, kPwNmax = 1e18, kPwS2max = 1e10;
 
-#ifndef OFDFT_TF_UNROLL
-#define OFDFT_TF_UNROLL 4
-#endif
-// functions evaluated side by side: fully unrolled, the table values stay
-// in registers (a runtime-indexed out[] would live in local memory)
-constexpr int kTfUnroll = OFDFT_TF_UNROLL;
-#ifndef OFDFT_HORNER_UNROLL
-#define OFDFT_HORNER_UNROLL 2
-#endif
-constexpr int kHornerUnroll = OFDFT_HORNER_UNROLL;   // Horner steps unrolled (code size against loop overhead)
-
-// Horner evaluation of a table polynomial c[0..deg] at the binary32 panel
-// variable uh, with its derivative dp and half its second derivative d2:
-// the terms of degree >= split in binary32 (their sum, times u^split, is
-// below 2^-24 of the polynomial's smallest value on every panel of the
-// table, so binary32 rounding there stays below the double-float
-// rounding), the rest in double-float, p and dp unnormalised.  A split of
-// deg runs every step in double-float.
-OF_HD void horner_split_f2(const ff::f2 *__restrict__ c, int deg, int split, float uh, ff::f2 &p, ff::f2 &dp,
-                           float &d2)
+// The double-float Horner evaluations run several polynomials side by side
+// (the four temperature functions; the enhancement factor at both of its
+// arguments): one rolled loop over the degree, so that the code stays small
+// (instruction fetch) and the chains of one warp overlap.  Each polynomial
+// comes with its derivative dp and half its second derivative d2 at the
+// binary32 panel variable; the terms of degree >= split are summed in
+// binary32: their sum, times u^split, is below 2^-24 of the scale the
+// polynomial enters with on every panel, so binary32 rounding there stays
+// below the double-float rounding.
+struct HornerF2 {
+    ff::f2 p, dp;   // unnormalised
+    float d2;
+};
+OF_HD void horner_lo(HornerF2 &h, float u, float c)
 {
-    d2 = 0.0f;
-    int j = deg - 1;
-    if (split < deg) {
-        float pf = c[deg].hi, dpf = 0.0f;
-#pragma unroll kHornerUnroll
-        for (; j >= split; --j) {
-            d2 = d2 * uh + dpf;
-            dpf = dpf * uh + pf;
-            pf = pf * uh + c[j].hi;
-        }
-        p = {pf, 0.0f};
-        dp = {dpf, 0.0f};
-    } else {
-        p = c[deg];
-        dp = {0.0f, 0.0f};
-    }
-#pragma unroll kHornerUnroll
-    for (; j >= 0; --j) {
-        d2 = d2 * uh + dp.hi;
-        dp = ff::fma_step_u(dp, uh, p);
-        p = ff::fma_step_u(p, uh, c[j]);
-    }
+    h.d2 = h.d2 * u + h.dp.hi;
+    h.dp.hi = h.dp.hi * u + h.p.hi;
+    h.p.hi = h.p.hi * u + c;
+}
+OF_HD void horner_dd(HornerF2 &h, float u, ff::f2 c)
+{
+    h.d2 = h.d2 * u + h.dp.hi;
+    h.dp = ff::fma_step_u(h.dp, u, h.p);
+    h.p = ff::fma_step_u(h.p, u, c);
 }
 
-// Degree from which the temperature table's terms are summed in binary32,
-// per function (xi, zeta, A, B): the largest tails of the fitted
-// polynomials, over every panel and relative to the polynomial's smallest
-// value there, are 3.3e-9 (xi, degree 7 up) and 2.9e-8 (A, degree 8 up).
-// zeta comes close to zero inside some panels, but it enters only beside
-// xi (f = tau0 xi F_tau - tau0 zeta F_sigma): its tail from degree 7 up is
-// 5.1e-9 of the panel's largest |xi|.  B keeps every term in double-float
-// (its monomial coefficients do not decay on the low-t panels).  Against the all-double-float sums the pointwise outputs
-// differ by less than their own double-float rounding (host sweep over
-// every panel, 1e-16 to 1e6 bohr^-3 at 1e4 K and 1e6 K).
-constexpr int kTfSplitXi = 7, kTfSplitZeta = 7, kTfSplitA = 8;
-// The enhancement table of G: tail 1.3e-8 from degree 5 up.
-constexpr int kEnSplit = 5;
-
-// Table polynomials with a double-float table (same layout as tfunc_eval's).
-// The panel variable u = uh + ul: uh is exact in binary32 and the Horner
-// sums run with it; ul (below 5e-7) enters through the first and second
-// derivatives.
+// Table polynomials with the refined double-float table (kTfDdSub panels an
+// octave).  The panel variable u = uh + ul: uh is exact in binary32 and the
+// Horner sums run with it; ul (below 2e-6) enters through the first and
+// second derivatives.  The tails from degree kTfSplit up, over every panel:
+// 6e-10 of xi, 1e-9 of xi for zeta (zeta comes close to zero but enters only
+// beside xi, f = tau0 xi F_tau - tau0 zeta F_sigma), 3e-8 of A and 5e-8 of
+// the larger of B and A xi / zeta (B enters through zeta F(s^2 B) beside
+// xi F(s^2 A)).  With the unrefined panels 7, 7, 8 and all 10 degrees needed
+// double-float: 32 steps instead of 20.
 template <int NF>
 OF_HD void tfunc_eval_f2(const ff::f2 *__restrict__ tab, ff::f2 t, ff::f2 out[8])
 {
+    static_assert(kTfFuncs == 4 && (NF == 2 || NF == 4), "rows of four functions");
     int e;
     float inv2e;
     const float m = split_pow2(t.hi, e, inv2e);
-    const int sub = (int)((m - 1.0f) * 4.0f);
-    const float uh = 8.0f * (m - 1.0f) - (float)(2 * sub + 1);
-    const float ul = 8.0f * t.lo * inv2e;
-    const float dudt = 8.0f * inv2e;
-    const ff::f2 *c = tab + ((size_t)((e - kTfEmin) * kTfSub + sub) * kTfFuncs) * kTfNc;
-#pragma unroll kTfUnroll
+    const int sub = (int)((m - 1.0f) * (float)kTfDdSub);
+    const float uh = (float)(2 * kTfDdSub) * (m - 1.0f) - (float)(2 * sub + 1);
+    const float ul = (float)(2 * kTfDdSub) * t.lo * inv2e;
+    const float dudt = (float)(2 * kTfDdSub) * inv2e;
+    const float4 *c = reinterpret_cast<const float4 *>(tab + (size_t)((e - kTfEmin) * kTfDdSub + sub) * kTfDdRow);
+    const float4 *tail = c + kTfSplit * 2;
+    HornerF2 h[NF];
+    {
+        const float4 a = tail[kTfDdDeg - kTfSplit];
+        h[0] = {{a.x, 0.0f}, {0.0f, 0.0f}, 0.0f};
+        h[1] = {{a.y, 0.0f}, {0.0f, 0.0f}, 0.0f};
+        if (NF == 4) {
+            h[2] = {{a.z, 0.0f}, {0.0f, 0.0f}, 0.0f};
+            h[3] = {{a.w, 0.0f}, {0.0f, 0.0f}, 0.0f};
+        }
+    }
+#pragma unroll 1
+    for (int j = kTfDdDeg - kTfSplit - 1; j >= 0; --j) {
+        const float4 a = tail[j];
+        const float cj[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int q = 0; q < NF; ++q) horner_lo(h[q], uh, cj[q]);
+    }
+#pragma unroll 1
+    for (int j = kTfSplit - 1; j >= 0; --j) {
+        const float4 a = c[2 * j];
+        horner_dd(h[0], uh, ff::f2(a.x, a.y));
+        horner_dd(h[1], uh, ff::f2(a.z, a.w));
+        if (NF == 4) {
+            const float4 b = c[2 * j + 1];
+            horner_dd(h[2], uh, ff::f2(b.x, b.y));
+            horner_dd(h[3], uh, ff::f2(b.z, b.w));
+        }
+    }
+#pragma unroll
     for (int q = 0; q < NF; ++q) {
-        ff::f2 p, dp;
-        float d2;   // half the second derivative
-        horner_split_f2(c + q * kTfNc, kTfDeg, q == 0 ? kTfSplitXi : (q == 1 ? kTfSplitZeta : (q == 2 ? kTfSplitA : kTfDeg)), uh, p, dp, d2);
-        p = ff::add(p, dp.hi * ul);
-        dp = ff::add(dp, 2.0f * d2 * ul);
-        out[q] = p;
-        out[4 + q] = ff::scale(dp, dudt);
+        out[q] = ff::add(h[q].p, h[q].dp.hi * ul);
+        out[4 + q] = ff::scale(ff::add(h[q].dp, 2.0f * h[q].d2 * ul), dudt);
     }
 }
 
@@ -422,12 +419,10 @@ FF_CALL void enhance_f2(const FuncParams &fp, ff::f2 x, ff::f2 &F, ff::f2 &dF)
     }
 }
 
-// VT84F F(x) and dF/dx in double-float from the enhancement table etab of
-// G = (F - 1)/x (kEnSize pairs): F = 1 + x G, dF = G + x G' with G' the
-// polynomial's derivative, so the potential is the exact derivative of the
-// tabulated energy; x < 2^-20: the cubic series (the next terms are below
-// 1e-16 in F and dF), x >= 64: F = 5x/3 + 1/x.
-OF_HD void enhance_vt84f_tab(const ff::f2 *__restrict__ etab, ff::f2 x, ff::f2 &F, ff::f2 &dF)
+// VT84F F(x) and dF/dx in double-float outside the enhancement table's
+// range: x < 2^-20: the cubic series (the next terms are below 1e-16 in F
+// and dF), x >= 64: F = 5x/3 + 1/x.
+FF_CALL void enhance_vt84f_ends(ff::f2 x, ff::f2 &F, ff::f2 &dF)
 {
     using namespace ff;
     if (x.hi < 9.5367431640625e-07f) {
@@ -441,27 +436,60 @@ OF_HD void enhance_vt84f_tab(const ff::f2 *__restrict__ etab, ff::f2 x, ff::f2 &
         dF = add(mul(x, add(mul(x, FFC(3.0 * c3)), FFC(2.0 * c2))), FFC(c1));
         return;
     }
-    if (x.hi >= 64.0f) {
-        const f2 r = recip(x);
-        F = add(mul(x, FFC(5.0 / 3.0)), r);
-        dF = sub(FFC(5.0 / 3.0), mul(r, r));
-        return;
+    const f2 r = recip(x);
+    F = add(mul(x, FFC(5.0 / 3.0)), r);
+    dF = sub(FFC(5.0 / 3.0), mul(r, r));
+}
+
+// VT84F F and dF/dx at two arguments from the enhancement table etab of
+// G = (F - 1)/x: F = 1 + x G, dF = G + x G' with G' the polynomial's
+// derivative, so the potential is the exact derivative of the tabulated
+// energy.  (Tail of G from degree kEnSplit up: 1.3e-8.)
+OF_HD void enhance_vt84f_tab(const ff::f2 *__restrict__ etab, const ff::f2 (&x)[2], ff::f2 (&F)[2], ff::f2 (&dF)[2])
+{
+    using namespace ff;
+    float uh[2], ul[2], dudx[2];
+    const float4 *c[2];
+    bool in[2];
+    HornerF2 h[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        in[k] = x[k].hi >= 9.5367431640625e-07f && x[k].hi < 64.0f;
+        int e;
+        float inv2e;
+        const float m = split_pow2(in[k] ? x[k].hi : 1.0f, e, inv2e);
+        const int sub = (int)((m - 1.0f) * (float)kEnSub);
+        uh[k] = (float)(2 * kEnSub) * (m - 1.0f) - (float)(2 * sub + 1);
+        ul[k] = (float)(2 * kEnSub) * x[k].lo * inv2e;
+        dudx[k] = (float)(2 * kEnSub) * inv2e;
+        c[k] = reinterpret_cast<const float4 *>(etab + (size_t)((e - kEnEmin) * kEnSub + sub) * kEnDdRow);
+        const float4 a = c[k][3], b = c[k][4];   // degrees 5 .. 8, 9 and 10
+        h[k] = {{b.y, 0.0f}, {0.0f, 0.0f}, 0.0f};
+        horner_lo(h[k], uh[k], b.x);
+        horner_lo(h[k], uh[k], a.w);
+        horner_lo(h[k], uh[k], a.z);
+        horner_lo(h[k], uh[k], a.y);
+        horner_lo(h[k], uh[k], a.x);
+        horner_dd(h[k], uh[k], f2(c[k][2].x, c[k][2].y));   // degree 4
     }
-    int e;
-    float inv2e;
-    const float m = split_pow2(x.hi, e, inv2e);
-    const int sub = (int)((m - 1.0f) * (float)kEnSub);
-    const float uh = (float)(2 * kEnSub) * (m - 1.0f) - (float)(2 * sub + 1);
-    const float ul = (float)(2 * kEnSub) * x.lo * inv2e;
-    const float dudx = (float)(2 * kEnSub) * inv2e;
-    const f2 *c = etab + (size_t)((e - kEnEmin) * kEnSub + sub) * kEnNc;
-    f2 p, dp;
-    float d2;   // half the second derivative
-    horner_split_f2(c, kEnDeg, kEnSplit, uh, p, dp, d2);
-    const f2 G = add(p, dp.hi * ul);
-    const f2 dG = scale(add(dp, 2.0f * d2 * ul), dudx);
-    F = add(mul(x, G), 1.0f);
-    dF = add(G, mul(x, dG));
+#pragma unroll 1
+    for (int j = 1; j >= 0; --j)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const float4 a = c[k][j];            // degrees 2 j, 2 j + 1
+            horner_dd(h[k], uh[k], f2(a.z, a.w));
+            horner_dd(h[k], uh[k], f2(a.x, a.y));
+        }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const f2 G = add(h[k].p, h[k].dp.hi * ul[k]);
+        const f2 dG = scale(add(h[k].dp, 2.0f * h[k].d2 * ul[k]), dudx[k]);
+        F[k] = add(mul(x[k], G), 1.0f);
+        dF[k] = add_s(G, mul(x[k], dG));
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if (!in[k]) enhance_vt84f_ends(x[k], F[k], dF[k]);
 }
 
 // ln x for x > 0 (normal binary32 range): x = 2^e m, the table's binary32
@@ -559,9 +587,11 @@ OF_HD bool pw_core_f2(const FuncParams &fp, const ff::f2 *__restrict__ tab, ff::
         const f2 xt = mul(s2, A), xs = mul(s2, B);           // Eq. (s_s)
         f2 Ft, dFt, Fsg, dFsg;
         if (fp.kind == 2) {                                  // VT84F: the enhancement table
-            const f2 *etab = tab + kTfSize;
-            enhance_vt84f_tab(etab, xt, Ft, dFt);
-            enhance_vt84f_tab(etab, xs, Fsg, dFsg);
+            const f2 *etab = tab + kTfDdSize;
+            const f2 xx[2] = {xt, xs};
+            f2 FF[2], dFF[2];
+            enhance_vt84f_tab(etab, xx, FF, dFF);
+            Ft = FF[0], dFt = dFF[0], Fsg = FF[1], dFsg = dFF[1];
         } else {
             enhance_f2(fp, xt, Ft, dFt);
             enhance_f2(fp, xs, Fsg, dFsg);
@@ -591,7 +621,7 @@ OF_HD bool pw_core_f2(const FuncParams &fp, const ff::f2 *__restrict__ tab, ff::
         o.wg = scale(mul(wpre, s2), 2.0f);                  // d s^2/d grad n . grad n = 2 s^2
     }
     if (xc) {
-        pz81_f2(tab + kTfSize + kEnSize, c13, y, o.eps, o.vxc);
+        pz81_f2(tab + kTfDdSize + kEnDdSize, c13, y, o.eps, o.vxc);
     } else {
         o.eps = f2(0.0f, 0.0f);
         o.vxc = f2(0.0f, 0.0f);
@@ -616,28 +646,51 @@ OF_HD PwOut<T> pw_point_native(const FuncParams &fp, const T *__restrict__ tab, 
 }
 
 
-// Double-float table written from the binary64 one (hi, lo per coefficient).
-inline void tfunc_table_split(const double *tab, float *out, int count = kTfSize)
-{
-    for (int i = 0; i < count; ++i) {
-        ff::f2 c = ff::from_double(tab[i]);
-        out[2 * i] = c.hi;
-        out[2 * i + 1] = c.lo;
-    }
-}
-
 // The FP64 field sets' tables in dst[kDdTabSize]: the binary64 temperature
-// table, its double-float split, the double-float VT84F enhancement table
-// and the logarithm table (the last three contiguous, as pw_core_f2 reads
-// them).
+// table, its refined double-float copy, the double-float VT84F enhancement
+// table and the logarithm table (the last three contiguous, as pw_core_f2
+// reads them).
 inline void dd_tables_fill(const double *ttab, double *dst)
 {
     for (int i = 0; i < kTfSize; ++i) dst[i] = ttab[i];
-    tfunc_table_split(ttab, reinterpret_cast<float *>(dst + kTfSize));
+    float *rf = reinterpret_cast<float *>(dst + kTfSize);
+    for (int p = 0; p < kTfPanels; ++p)
+        for (int s = 0; s < kTfRef; ++s)
+            for (int q = 0; q < kTfFuncs; ++q) {
+                // u = ctr + v / kTfRef: Taylor coefficients about ctr by repeated synthetic division
+                const double ctr = (2.0 * s + 1.0 - kTfRef) / kTfRef;
+                double a[kTfNc], sc = 1.0;
+                for (int k = 0; k < kTfNc; ++k) a[k] = ttab[((size_t)p * kTfFuncs + q) * kTfNc + k];
+                for (int k = 0; k < kTfDeg; ++k)
+                    for (int j = kTfDeg - 1; j >= k; --j) a[j] += ctr * a[j + 1];
+                float *row = rf + 2 * (size_t)(p * kTfRef + s) * kTfDdRow;
+                for (int k = 0; k <= kTfDdDeg; ++k, sc /= kTfRef) {
+                    const ff::f2 c = ff::from_double(a[k] * sc);
+                    if (k < kTfSplit) {
+                        row[2 * (k * kTfFuncs + q)] = c.hi;
+                        row[2 * (k * kTfFuncs + q) + 1] = c.lo;
+                    } else {
+                        row[2 * kTfSplit * kTfFuncs + (k - kTfSplit) * kTfFuncs + q] = c.hi;
+                    }
+                }
+            }
+    float *en = reinterpret_cast<float *>(dst + kTfSize + kTfDdSize);
     double etab[kEnSize];
     enh_table_fill(etab);
-    tfunc_table_split(etab, reinterpret_cast<float *>(dst + 2 * kTfSize), kEnSize);
-    float *lg = reinterpret_cast<float *>(dst + 2 * kTfSize + kEnSize);   // {r, 0}, -ln r per interval
+    for (int p = 0; p < kEnPanels; ++p) {
+        float *row = en + 2 * (size_t)p * kEnDdRow;
+        for (int k = 0; k < 2 * kEnDdRow; ++k) row[k] = 0.0f;
+        for (int k = 0; k < kEnNc; ++k) {
+            const ff::f2 c = ff::from_double(etab[(size_t)p * kEnNc + k]);
+            if (k < kEnSplit) {
+                row[2 * k] = c.hi;
+                row[2 * k + 1] = c.lo;
+            } else {
+                row[(kEnSplit + 1) / 2 * 4 + k - kEnSplit] = c.hi;
+            }
+        }
+    }
+    float *lg = en + 2 * kEnDdSize;   // {r, 0}, -ln r per interval
     for (int i = 0; i < kLgSub; ++i) {
         const float r = (float)(1.0 / (1.0 + (i + 0.5) / kLgSub));
         const long double l = -logl((long double)r);
