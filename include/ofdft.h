@@ -416,7 +416,7 @@ void ofdft_destroy(ofdft_ctx *ctx);
  * ofdft_setup + ofdft_energy_potential compute (F_tot and its terms, the
  * pressure terms, v = dF/dn at n = phi^2), in FP64, with the same kernels,
  * but every device scratch buffer is carved from one fixed array compiled
- * into the library: about 2.4 MB that each GPU loading the library holds
+ * into the library: about 3.0 MB that each GPU loading the library holds
  * until the process exits.  The call allocates no memory, on the device or
  * the host.
  *  cell[9], grid[3], nat, ions, Z, T_kelvin, functional: as ofdft_setup,
@@ -431,7 +431,7 @@ void ofdft_destroy(ofdft_ctx *ctx);
  * Limits: each grid edge even, {2,3,5}-smooth and at most 64;
  * nx*ny*nz <= 32768; 1 <= nat <= 64.  Anything larger returns OFDFT_EINVAL,
  * as do Z <= 0, non-finite positions, T or rc.
- * No call may be made on a stream that is being captured (the call copies
+ * No call may be made on a stream that is being captured (the call reads
  * from pageable host memory and synchronises): OFDFT_EINVAL.  The first
  * call on a device does a one-time set-up on the current device (looks up
  * the array's device address, uploads the temperature table).  The set-up

@@ -44,10 +44,25 @@ constexpr size_t kOffPhase = kOffVpart + align256((size_t)kSMaxN * sizeof(double
 constexpr size_t kPhaseBytes = align256((size_t)kSMaxAtoms * (3 * kSMaxEdge) * sizeof(double2));
 constexpr size_t kOffIons = kOffPhase + kPhaseBytes;
 constexpr size_t kOffZ = kOffIons + align256(3 * kSMaxAtoms * sizeof(double));
-constexpr size_t kOffPart = kOffZ + align256(kSMaxAtoms * sizeof(double));
+constexpr size_t kOffFrac = kOffZ + align256(kSMaxAtoms * sizeof(double));
+constexpr size_t kOffPart = kOffFrac + align256(3 * kSMaxAtoms * sizeof(float));
 constexpr size_t kOffScal = kOffPart + align256((size_t)kSMaxPart * sizeof(double));
+// twiddles of every edge the path takes, each as binary64 and double-float pairs
+constexpr int kEdges[] = {8, 10, 12, 16, 18, 20, 24, 30, 32, 36, 40, 48, 50, 54, 60, 64};
+constexpr int tw_offset(int n)   // entries before those of edge n
+{
+    int o = 0;
+    for (int e : kEdges) {
+        if (e == n) return o;
+        o += 2 * e;
+    }
+    return n == 0 ? o : -1;
+}
+constexpr int kTwEntries = tw_offset(0);
 constexpr size_t kOffTw = kOffScal + align256(64 * sizeof(double));
-constexpr size_t kOffTab = kOffTw + align256(3 * kSMaxEdge * 2 * sizeof(double2));   // + double-float copy
+constexpr size_t kOffEwTab = kOffTw + align256(kTwEntries * sizeof(double2));
+constexpr size_t kOffEwPart = kOffEwTab + align256((size_t)kEwTabRows * kSMaxAtoms * sizeof(double2));
+constexpr size_t kOffTab = kOffEwPart + align256(kEwBlocks * sizeof(double));
 constexpr size_t kScratchBytes = kOffTab + align256((size_t)kDdTabSize * sizeof(double));   // + splits
 
 static __device__ __align__(256) unsigned char g_ofdft_scratch[kScratchBytes];
@@ -59,8 +74,43 @@ struct DevState {
 };
 DevState g_dev[kMaxDevices];
 double g_tab_host[kDdTabSize];    // host temperature table + double-float tables, filled once
+double2 g_tw_host[kTwEntries];    // twiddles of every edge, filled once
 bool g_tab_ready = false;
-std::mutex g_setup_mu;            // guards g_dev, g_tab_host and g_tab_ready (locking allocates nothing)
+std::mutex g_setup_mu;            // guards g_dev, g_tab_host, g_tw_host and g_tab_ready (locking allocates nothing)
+
+// exp(-2 pi i m / n) for every edge n, as binary64 and as double-float pairs.
+void twiddles_fill(double2 *tw)
+{
+    for (int n : kEdges)
+        for (int m = 0; m < n; ++m) {
+            const long double ang = -2.0L * 3.14159265358979323846264338327950288L * m / n;
+            const long double cv = cosl(ang), sv = sinl(ang);
+            double2 *d = tw + tw_offset(n) + m;
+            float *f = reinterpret_cast<float *>(d + n);
+            *d = make_double2((double)cv, (double)sv);
+            f[0] = (float)cv;
+            f[1] = (float)(cv - (long double)f[0]);
+            f[2] = (float)sv;
+            f[3] = (float)(sv - (long double)f[2]);
+        }
+}
+
+// The ions of a call, by value in a kernel's arguments: no copy from
+// pageable memory, which would wait for the stream.
+struct Ions {
+    double v[4 * kSMaxAtoms];   // positions, then charges
+    float frac[3 * kSMaxAtoms]; // fractional coordinates in [0, 1]
+};
+__global__ void k_put_ions(int nat, const __grid_constant__ Ions ions, double *R, double *Z, float *frac)
+{
+    const int i = threadIdx.x;
+    if (i < 3 * nat) {
+        R[i] = ions.v[i];
+        frac[i] = ions.frac[i];
+    } else if (i < 4 * nat) {
+        Z[i - 3 * nat] = ions.v[i];
+    }
+}
 
 // Status only: the documented limits say what OFDFT_EINVAL means here.
 ofdft_status serr(ofdft_status s, const char *, cudaError_t = cudaSuccess) { return s; }
@@ -94,10 +144,12 @@ ofdft_status device_setup(int dev, unsigned char **base)
             static double ttab[kTfSize];
             tfunc_table_fill(ttab);
             dd_tables_fill(ttab, g_tab_host);
+            twiddles_fill(g_tw_host);
             g_tab_ready = true;
         }
         SCK(cudaMemcpy(d.base + kOffTab, g_tab_host, sizeof(g_tab_host), cudaMemcpyHostToDevice),
             "temperature table upload failed");
+        SCK(cudaMemcpy(d.base + kOffTw, g_tw_host, sizeof(g_tw_host), cudaMemcpyHostToDevice), "twiddle upload failed");
         int optin = 0;
         SCK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev),
             "device attribute query failed");
@@ -109,8 +161,23 @@ ofdft_status device_setup(int dev, unsigned char **base)
     return OFDFT_OK;
 }
 
-// Textbook Ewald energy on the host, no heap: real-space erfc sum, reciprocal
-// sum over the box of G with |G| < gcut, self and background terms.
+// Self and background terms of the Ewald energy.
+double ewald_consts(const double L[3], int nat, const double *Z)
+{
+    const double pi = 3.14159265358979323846;
+    const double om = L[0] * L[1] * L[2];
+    const double a = 1.2 * sqrt(pi) * pow((double)nat / (om * om), 1.0 / 6.0);
+    double z2 = 0.0, zs = 0.0;
+    for (int I = 0; I < nat; ++I) {
+        z2 += Z[I] * Z[I];
+        zs += Z[I];
+    }
+    return -a / sqrt(pi) * z2 - pi * zs * zs / (2.0 * om * a * a);
+}
+
+// Textbook Ewald sums on the host, no heap: real-space erfc sum and
+// reciprocal sum over the box of G with |G| < gcut (cells too uneven for
+// launch_ewald_energy's tables).
 double ewald_host(const double L[3], int nat, const double *R, const double *Z)
 {
     const double pi = 3.14159265358979323846;
@@ -154,12 +221,7 @@ double ewald_host(const double L[3], int nat, const double *R, const double *Z)
                 }
                 E += 2.0 * pi / om * exp(-g2 / (4.0 * a * a)) / g2 * (sr * sr + si * si);
             }
-    double z2 = 0.0, zs = 0.0;
-    for (int I = 0; I < nat; ++I) {
-        z2 += Z[I] * Z[I];
-        zs += Z[I];
-    }
-    return E - a / sqrt(pi) * z2 - pi * zs * zs / (2.0 * om * a * a);
+    return E;
 }
 
 }  // namespace
@@ -224,34 +286,27 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
     g.dd = 1;   // double-float FFT and pointwise arithmetic, as ofdft_setup's default
     const double T = T_kelvin * 3.166811563e-6;
 
-    // twiddles for the three axes (host stack -> scratch), binary64 then
-    // double-float pairs
-    double2 tw[3][kSMaxEdge];
-    float twf[3][kSMaxEdge][4];
-    int n3[3] = {g.nx, g.ny, g.nz};
-    for (int a = 0; a < 3; ++a)
-        for (int m = 0; m < n3[a]; ++m) {
-            long double ang = -2.0L * 3.14159265358979323846264338327950288L * m / n3[a];
-            long double cv = cosl(ang), sv = sinl(ang);
-            tw[a][m] = make_double2((double)cv, (double)sv);
-            twf[a][m][0] = (float)cv;
-            twf[a][m][1] = (float)(cv - (long double)twf[a][m][0]);
-            twf[a][m][2] = (float)sv;
-            twf[a][m][3] = (float)(sv - (long double)twf[a][m][2]);
-        }
-    double2 *twd = (double2 *)(base + kOffTw);
-    double2 *twfd = twd + 3 * kSMaxEdge;
-    SCK(cudaMemcpyAsync(twd, tw, sizeof(tw), cudaMemcpyHostToDevice, st), "twiddle upload failed");
-    SCK(cudaMemcpyAsync(twfd, twf, sizeof(twf), cudaMemcpyHostToDevice, st), "twiddle upload failed");
-    FftAxis ax = fft_axis(g.nx, twd), ay = fft_axis(g.ny, twd + kSMaxEdge),
-            az = fft_axis(g.nz, twd + 2 * kSMaxEdge, 4);   // the FP64 contexts' z schedule
-    ax.twf = twfd;
-    ay.twf = twfd + kSMaxEdge;
-    az.twf = twfd + 2 * kSMaxEdge;
-    // ions -> phases -> v_ext(G)
+    const double2 *tw = (const double2 *)(base + kOffTw);
+    const double2 *twx = tw + tw_offset(g.nx), *twy = tw + tw_offset(g.ny), *twz = tw + tw_offset(g.nz);
+    FftAxis ax = fft_axis(g.nx, twx), ay = fft_axis(g.ny, twy), az = fft_axis(g.nz, twz, 4);   // the FP64 contexts' z schedule
+    ax.twf = twx + g.nx;
+    ay.twf = twy + g.ny;
+    az.twf = twz + g.nz;
+    // ions -> Ewald sums; phases -> v_ext(G)
     double *Rd = (double *)(base + kOffIons), *Zd = (double *)(base + kOffZ);
-    SCK(cudaMemcpyAsync(Rd, ions, 3 * nat * sizeof(double), cudaMemcpyHostToDevice, st), "ion upload failed");
-    SCK(cudaMemcpyAsync(Zd, Z, nat * sizeof(double), cudaMemcpyHostToDevice, st), "charge upload failed");
+    double *scal = (double *)(base + kOffScal);   // 18 sums of the evaluation, then the Ewald sums
+    Ions arg;
+    memcpy(arg.v, ions, 3 * nat * sizeof(double));
+    memcpy(arg.v + 3 * nat, Z, nat * sizeof(double));
+    float *frac = (float *)(base + kOffFrac);
+    const double L[3] = {g.Lx, g.Ly, g.Lz};
+    for (int i = 0; i < 3 * nat; ++i) {
+        const double f = ions[i] / L[i % 3];
+        arg.frac[i] = (float)(f - floor(f));
+    }
+    k_put_ions<<<1, 4 * kSMaxAtoms, 0, st>>>(nat, arg, Rd, Zd, frac);
+    const bool ewald_dev = launch_ewald_energy(nat, Rd, Zd, frac, L, (double2 *)(base + kOffEwTab), (double *)(base + kOffEwPart),
+                                               scal + 18, st);
     double2 *px = (double2 *)(base + kOffPhase);
     double2 *py = px + (size_t)nat * g.nx, *pz = py + (size_t)nat * g.ny;
     double2 *vext = (double2 *)(base + kOffVext);
@@ -263,8 +318,7 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
     double2 *s0 = (double2 *)(base + kOffSpec), *s1 = s0 + specN, *s2 = s1 + specN, *s3 = s2 + specN;
     const double *tab = (const double *)(base + kOffTab);
     double *vpart = (double *)(base + kOffVpart);
-    double *part = (double *)(base + kOffPart), *scal = (double *)(base + kOffScal);
-    SCK(cudaMemsetAsync(scal, 0, 64 * sizeof(double), st), "scalar clear failed");
+    double *part = (double *)(base + kOffPart);
     const int nbx = xpass_blocks(g);
     const long long npairs = (long long)g.nx * g.ny / 2;
     double *pA = part, *pB = pA + 3 * nbx, *pC = pB + 6 * npairs;
@@ -292,20 +346,19 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
                                         nullptr, v_dev, pC, st);
     }
     launch_reduce_eval(pA, nbx, pB, nbg, pC, nbz, !fttf, scal, st);
-    double h[18];
+    double h[19];
     SCK(cudaMemcpyAsync(h, scal, sizeof(h), cudaMemcpyDeviceToHost, st), "scalar read-back failed");
     SCK(cudaStreamSynchronize(st), "stream synchronisation failed");
     SCK(cudaGetLastError(), "kernel launch failed");
 
     const double *f = fttf ? h + 9 : h + 3;
     const double dV = g.dV, om = g.omega;
-    double L[3] = {g.Lx, g.Ly, g.Lz};
     double Ne = 0.0, zs = 0.0;
     for (int i = 0; i < nat; ++i) {
         Ne += Z[i];
         zs += 3.14159265358979323846 * Z[i] * rc * rc;
     }
-    double E_ion = ewald_host(L, nat, ions, Z);
+    const double E_ion = (ewald_dev ? h[18] : ewald_host(L, nat, ions, Z)) + ewald_consts(L, nat, Z);
     ofdft_energy e;
     memset(&e, 0, sizeof(e));
     e.F_s = dV * f[0];

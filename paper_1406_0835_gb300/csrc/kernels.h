@@ -148,6 +148,15 @@ void launch_ewald_real(int nat, const double *R, const double *Z, const EwCell &
 int launch_ewald_recip(int nat, const double *R, const double *Z, int nG, const double *Gv,
                        const double *wG, double2 *S, double *epart, double *F, cudaStream_t st);
 
+// Ewald energy of an orthorhombic cell (edges L) without its self and
+// background terms, into out[0]; frac: fractional coordinates in [0, 1],
+// binary32, for screening the pairs; tab is scratch of kEwTabRows nat double2,
+// part of kEwBlocks doubles.  False (nothing launched) for cells so uneven
+// that an axis needs more images or reciprocal planes than fit.
+constexpr int kEwTabRows = 256, kEwBlocks = 304;
+bool launch_ewald_energy(int nat, const double *R, const double *Z, const float *frac, const double L[3], double2 *tab, double *part,
+                         double *out, cudaStream_t st);
+
 // MD: half step A (thermostat half, kick, drift) and B (kick, thermostat half).
 void launch_md_a(int nat, const double *m, double *R, double *V, const double *F, double dt,
                  double kT, double Q, int ndof, int thermo, double *nh, cudaStream_t st);

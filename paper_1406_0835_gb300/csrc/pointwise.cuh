@@ -343,14 +343,12 @@ OF_HD void tfunc_eval_f2(const ff::f2 *__restrict__ tab, ff::f2 t, ff::f2 out[8]
     const float4 *c = reinterpret_cast<const float4 *>(tab + (size_t)((e - kTfEmin) * kTfDdSub + sub) * kTfDdRow);
     const float4 *tail = c + kTfSplit * 2;
     HornerF2 h[NF];
-    {
-        const float4 a = tail[kTfDdDeg - kTfSplit];
-        h[0] = {{a.x, 0.0f}, {0.0f, 0.0f}, 0.0f};
-        h[1] = {{a.y, 0.0f}, {0.0f, 0.0f}, 0.0f};
-        if (NF == 4) {
-            h[2] = {{a.z, 0.0f}, {0.0f, 0.0f}, 0.0f};
-            h[3] = {{a.w, 0.0f}, {0.0f, 0.0f}, 0.0f};
-        }
+    const float4 top = tail[kTfDdDeg - kTfSplit];
+    h[0] = {{top.x, 0.0f}, {0.0f, 0.0f}, 0.0f};
+    h[1] = {{top.y, 0.0f}, {0.0f, 0.0f}, 0.0f};
+    if (NF == 4) {
+        h[2] = {{top.z, 0.0f}, {0.0f, 0.0f}, 0.0f};
+        h[3] = {{top.w, 0.0f}, {0.0f, 0.0f}, 0.0f};
     }
 #pragma unroll 1
     for (int j = kTfDdDeg - kTfSplit - 1; j >= 0; --j) {
