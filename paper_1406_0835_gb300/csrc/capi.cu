@@ -47,7 +47,14 @@ struct FieldSet {
     size_t spec_stride = 0;    // elements between spectra
     void *vext = nullptr, *tab = nullptr;
     void *tw[3] = {nullptr, nullptr, nullptr};
-    void *dmat[3] = {nullptr, nullptr, nullptr};   // derivative matrices of the tensor-core passes
+    // tensor-core transforms (double-float sets): matrices per axis (null:
+    // the axis takes FFT passes) in one allocation; real_basis: the Hartree
+    // chain runs in the real Fourier basis too, with v_ext's coefficients
+    // (and the pressure weights') in vre
+    TlAxis tl[3];
+    void *tlmem = nullptr;
+    bool real_basis = false;
+    float2 *vre = nullptr;
     FftAxis ax[3];
     CgState *cs = nullptr;     // device CG state
     cudaGraphExec_t graph = nullptr;
@@ -195,14 +202,95 @@ template <typename T> ofdft_status upload_twiddles(ofdft_ctx *c, FieldSet &f, in
     // butterfly chains between the barriers of the fused z kernels)
     f.ax[axis] = fft_axis(n, f.tw[axis], (sizeof(T) == 8 && axis == 2) ? 4 : 8);
     f.ax[axis].twf = nbf ? (const void *)((const char *)f.tw[axis] + nb) : nullptr;
-    // double-float sets: digits of the derivative matrices
-    if (sizeof(T) == 8 && c->g.dd && !c->g.dws && c->fp.kind != 0 && tline_supported(n)) {
-        std::vector<uint16_t> img(tline_matrix_bytes(n) / 2);
-        f.ax[axis].dexp = tline_derivative_matrix(n, c->g.ds[axis] * n, img.data());
-        CK(cudaMallocAsync((void **)&f.dmat[axis], tline_matrix_bytes(n), c->st));
-        CK(cudaMemcpyAsync(f.dmat[axis], img.data(), tline_matrix_bytes(n), cudaMemcpyHostToDevice, c->st));
-        f.ax[axis].dmat = f.dmat[axis];
+    return OFDFT_OK;
+}
+
+// The derivative passes of a double-float GGA set take the tensor cores along
+// every axis that they support; the Hartree chain does when all three axes
+// are supported and the cell is orthorhombic (4 pi / G^2 is diagonal in
+// products of cosines and sines only there).  ftTF has the chain alone and
+// four kernels more in this form: a solve's evaluation takes 83 us instead of
+// 76 at 48^3, 93 instead of 98 at 60^3 and 155 instead of 204 at 96^3, so
+// smaller ftTF grids keep the FFT passes.  (GGA: 96^3 291 -> 255 us, 48^3
+// 95 -> 92, 32^3 72 -> 73.)
+constexpr long long kRealTfPoints = 160000;
+bool tl_derivatives(const ofdft_ctx *c, int n) { return c->g.dd && !c->g.dws && c->fp.kind != 0 && tline_supported(n); }
+bool tl_real_basis(const ofdft_ctx *c)
+{
+    const GridInfo &g = c->g;
+    return g.dd && !g.dws && !g.tri && (c->fp.kind != 0 || g.N >= kRealTfPoints) && tline_supported(g.nx) &&
+           tline_supported(g.ny) && tline_supported(g.nz);
+}
+
+ofdft_status setup_tline(ofdft_ctx *c, FieldSet &f)
+{
+    const GridInfo &g = c->g;
+    const int n3[3] = {g.nx, g.ny, g.nz};
+    f.real_basis = tl_real_basis(c);
+    size_t bytes = 0;
+    auto place = [&](size_t b) {
+        const size_t at = bytes;
+        bytes += (b + 255) & ~(size_t)255;
+        return at;
+    };
+    // images of axes of one length (and spacing) are shared
+    size_t at[3][4];   // derivative, forward, inverse, (k b)^2
+    for (int a = 0; a < 3; ++a) {
+        for (int k = 0; k < 4; ++k) at[a][k] = (size_t)-1;
+        const size_t mb = tline_supported(n3[a]) ? tline_matrix_bytes(n3[a]) : 0;
+        for (int o = 0; o < a; ++o)
+            if (n3[o] == n3[a]) {
+                at[a][1] = at[o][1];
+                at[a][2] = at[o][2];
+                if (g.ds[o] == g.ds[a]) at[a][0] = at[o][0];
+            }
+        if (tl_derivatives(c, n3[a]) && at[a][0] == (size_t)-1) at[a][0] = place(mb);
+        if (f.real_basis) {
+            if (at[a][1] == (size_t)-1) {
+                at[a][1] = place(mb);
+                at[a][2] = place(mb);
+            }
+            at[a][3] = place(n3[a] * sizeof(float2));
+        }
     }
+    if (bytes == 0) return OFDFT_OK;
+    std::vector<unsigned char> h(bytes);
+    CK(cudaMallocAsync(&f.tlmem, bytes, c->st));
+    unsigned char *dev = (unsigned char *)f.tlmem;
+    const double b3[3] = {g.bx, g.by, g.bz};
+    for (int a = 0; a < 3; ++a) {
+        TlMat *m[3] = {&f.tl[a].der, &f.tl[a].fwd, &f.tl[a].inv};
+        for (int k = 0; k < 3; ++k) {
+            if (at[a][k] == (size_t)-1) continue;
+            m[k]->img = dev + at[a][k];
+            bool made = false;
+            for (int o = 0; o < a; ++o)
+                if (at[o][k] == at[a][k]) {
+                    const TlMat *om[3] = {&f.tl[o].der, &f.tl[o].fwd, &f.tl[o].inv};
+                    m[k]->mexp = om[k]->mexp;
+                    made = true;
+                }
+            if (made) continue;
+            uint16_t *img = (uint16_t *)(h.data() + at[a][k]);
+            m[k]->mexp = k == 0 ? tline_derivative_matrix(n3[a], g.ds[a] * n3[a], img)
+                                : tline_fourier_matrix(n3[a], k == 2, img);
+        }
+        if (at[a][3] != (size_t)-1) {
+            float2 *t = (float2 *)(h.data() + at[a][3]);
+            for (int i = 0; i < n3[a]; ++i) {
+                bool sine;
+                const double k = tline_frequency(n3[a], i, &sine) * b3[a];
+                const ff::f2 x = ff::from_double(k * k);
+                t[i] = make_float2(x.hi, x.lo);
+            }
+            f.tl[a].g2 = (const float2 *)(dev + at[a][3]);
+        }
+        // units of cells beyond any real one would leave binary32's exponents
+        if (f.tl[a].der.img && (f.tl[a].der.mexp > 68 || f.tl[a].der.mexp < -60)) f.tl[a].der = TlMat{};
+    }
+    CK(cudaMemcpyAsync(f.tlmem, h.data(), bytes, cudaMemcpyHostToDevice, c->st));
+    if (f.real_basis)
+        CK(cudaMallocAsync((void **)&f.vre, (size_t)(g.lpp ? 2 : 1) * g.N * sizeof(float2), c->st));
     return OFDFT_OK;
 }
 
@@ -270,13 +358,14 @@ EvalScalars unpack_sums(const double *h, bool fttf)
     return es;
 }
 
-// Kernels of one evaluation (GGA: two launches instead of a pass per axis
-// and half for the axes taken on the tensor cores).
+// Kernels of one evaluation (GGA: two tensor-core launches instead of a pass
+// per axis and half for the axes they take).
 int eval_kernel_count(const ofdft_ctx *c, const FieldSet &f)
 {
+    if (f.real_basis) return c->fp.kind == 0 ? 10 : 12;
     if (c->fp.kind == 0) return 6;
-    const int tc = (f.ax[0].dmat ? 1 : 0) + (f.ax[1].dmat ? 1 : 0);
-    return 11 - 2 * tc + (tc || f.ax[2].dmat ? 2 : 0);
+    const int tc = (f.tl[0].der.img ? 1 : 0) + (f.tl[1].der.img ? 1 : 0);
+    return 11 - 2 * tc + (tc || f.tl[2].der.img ? 2 : 0);
 }
 
 // Enqueue one energy + potential evaluation at ph (or, with phi0 and dh, at the
@@ -296,6 +385,149 @@ int eval_kernel_count(const ofdft_ctx *c, const FieldSet &f)
 //        sum, sums.  Derivatives of double-float sets run on the tensor
 //        cores (one launch for all axes, from the field n that zfwd writes);
 //        other axes take dline along x and y, zfwd and zfinal_gga along z.
+// n(G) for forces and stress: forward z, y, x of n into the second spectrum.
+ofdft_status enqueue_nG(ofdft_ctx *c, FieldSet &f, double *ph, double *part)
+{
+    const GridInfo &g = f.gt;
+    const long long fs = (long long)f.spec_stride;
+    double2 *s1 = (double2 *)f.spec + fs;
+    launch_zfwd<double>(g, f.ax[2], 1, nullptr, ph, nullptr, 0.0, 0.0, nullptr, nullptr, s1, c->st);
+    launch_ypass<double>(g, f.ax[1], false, s1, 1, fs, c->st);
+    launch_xhl<double>(g, f.ax[0], s1, (const double2 *)f.vext, s1, 0, part, c->st);
+    c->launches += 3;
+    DBG("n(G)");
+    return OFDFT_OK;
+}
+
+// Derivatives along the axes that have a matrix, in one launch.
+void launch_derivatives(const GridInfo &g, const FieldSet &f, const double *const in[3], double *const out[3], cudaStream_t st)
+{
+    TlPass p[3];
+    int n = 0;
+    for (int a = 0; a < 3; ++a)
+        if (f.tl[a].der.img)
+            p[n++] = {TlPass::kDerivative, a, &f.tl[a].der, (const float2 *)in[a], (float2 *)out[a]};
+    launch_tline(g, n, p, st);
+}
+
+// Real-basis form (double-float sets, orthorhombic, every axis on the tensor
+// cores): n as a field; its three derivatives and its z transform in one
+// launch; y, x, Hartree and LPP terms and energies, x^-1, y^-1, z^-1 beside
+// the pointwise stage and the divergence's three derivatives; potential and
+// sums.  ftTF: the chain alone, then the pointwise stage.
+ofdft_status enqueue_real(ofdft_ctx *c, FieldSet &f, double *ph, const double *phi0, const double *dh, double cth,
+                          double sth, const double *csd, double *vout, double *sums, double *spart, int *nbg_out)
+{
+    const GridInfo &g = f.gt;
+    cudaStream_t st = c->st;
+    const bool fttf = c->fp.kind == 0;
+    const long long fs = (long long)f.spec_stride, npairs = (long long)g.nx * g.ny / 2;
+    double2 *spec = (double2 *)f.spec;
+    float2 *coef = (float2 *)spec, *nf = (float2 *)f.vpart;
+    double *d[3] = {(double *)(spec + fs), (double *)(spec + 2 * fs), (double *)(spec + 3 * fs)};
+    const double *tab = (const double *)f.tab;
+    double *pA = c->part;
+    {
+        TimerScope ts(c, TM_ZFWD, false);
+        launch_density(g.N, phi0 ? phi0 : ph, phi0 ? dh : nullptr, cth, sth, csd, ph, nf, st);
+    }
+    DBG("k_density");
+    {
+        TimerScope ts(c, TM_DLINE, false);
+        TlPass p[4];
+        int n = 0;
+        if (!fttf)
+            for (int a = 0; a < 3; ++a) p[n++] = {TlPass::kDerivative, a, &f.tl[a].der, nf, (float2 *)d[a]};
+        p[n++] = {TlPass::kForward, 2, &f.tl[2].fwd, nf, coef};
+        launch_tline(g, n, p, st);
+    }
+    DBG("k_tline (grad n, z)");
+    const bool fork = !fttf && c->aux[0] && c->timer_id == 0 && !c->debug_sync;
+    cudaStream_t sh = st;
+    if (fork) {
+        CK(cudaEventRecord(c->fj[0], st));
+        CK(cudaStreamWaitEvent(c->aux[0], c->fj[0], 0));
+        sh = c->aux[0];
+    }
+    {
+        TimerScope ts(c, TM_Y, false);
+        const TlPass p = {TlPass::kForward, 1, &f.tl[1].fwd, coef, coef};
+        launch_tline(g, 1, &p, sh);
+    }
+    DBG("k_tline (y)");
+    int nbx;
+    {
+        TimerScope ts(c, TM_XHL, false);
+        const TlPass fwd = {TlPass::kForward, 0, &f.tl[0].fwd, coef, coef}, inv = {TlPass::kInverse, 0, &f.tl[0].inv, coef, coef};
+        launch_tline(g, 1, &fwd, sh);
+        TlHartree hl{};
+        for (int a = 0; a < 3; ++a) hl.g2[a] = f.tl[a].g2;
+        hl.ve = f.vre;
+        hl.vp = g.lpp ? f.vre + g.N : nullptr;
+        hl.hr = make_float2(g.hr2[0], g.hr2[1]);
+        hl.half_dv = 0.5 * g.dV;
+        hl.dv = g.dV;
+        hl.ploc = g.dV / g.omega * (g.lpp ? 1.0 : 1.0 / 3.0);
+        hl.part = pA;
+        nbx = launch_hartree(g, coef, hl, sh);
+        launch_tline(g, 1, &inv, sh);
+    }
+    DBG("k_tline (x), k_hartree");
+    {
+        TimerScope ts(c, TM_Y, false);
+        const TlPass p = {TlPass::kInverse, 1, &f.tl[1].inv, coef, coef};
+        launch_tline(g, 1, &p, sh);
+    }
+    DBG("k_tline (y^-1)");
+    {
+        TimerScope ts(c, TM_ZFINAL, false);
+        const TlPass p = {TlPass::kInverse, 2, &f.tl[2].inv, coef, coef};
+        launch_tline(g, 1, &p, sh);
+    }
+    DBG("k_tline (z^-1)");
+    if (fork) CK(cudaEventRecord(c->fj[1], sh));
+    double *pB = pA + 3 * nbx, *pC = pB + 6 * npairs;
+    int nbg = 0, nbz;
+    if (fttf) {
+        TimerScope ts(c, TM_PW, false);
+        nbz = launch_ptf(g, coef, ph, phi0, phi0 ? dh : nullptr, cth, sth, csd, c->T, c->fp, tab, c->xc, vout, pC, st);
+    } else {
+        {
+            TimerScope ts(c, TM_PW, false);
+            if (spart) pB = spart;
+            nbg = launch_pw<double>(g, d[0], d[1], d[2], ph, c->T, c->fp, tab, c->xc, (double *)f.vpart, pB,
+                                    spart != nullptr, st);
+            if (nbg_out) *nbg_out = nbg;
+        }
+        DBG("k_pw");
+        {
+            TimerScope ts(c, TM_DLINE, false);
+            launch_derivatives(g, f, d, d, st);
+        }
+        DBG("k_tline (div W)");
+        if (fork) CK(cudaStreamWaitEvent(st, c->fj[1], 0));
+        TimerScope ts(c, TM_ZFINAL, false);
+        TlFinal fin{};
+        fin.vhl = coef;
+        fin.vpart = (const float2 *)f.vpart;
+        for (int a = 0; a < 3; ++a) fin.d[a] = (const float2 *)d[a];
+        fin.phit = ph;
+        fin.phi = phi0;
+        fin.dhat = phi0 ? dh : nullptr;
+        fin.cs = csd;
+        fin.c = cth;
+        fin.s = sth;
+        fin.vout = vout;
+        fin.part = pC;
+        nbz = launch_final(g, fin, st);
+    }
+    DBG("k_final");
+    launch_reduce_eval(pA, nbx, pB, nbg, pC, nbz, !fttf, sums, st);
+    DBG("k_reduce_eval");
+    c->launches += eval_kernel_count(c, f);
+    return OFDFT_OK;
+}
+
 template <typename T>
 ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const T *dh, double cth,
                           double sth, const void *csd, T *vout, bool keep_nG, double *sums,
@@ -315,12 +547,20 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
     const int nbx = xpass_blocks(g);
     const long long npairs = (long long)g.nx * g.ny / 2;
     double *pA = c->part, *pB = pA + 3 * nbx, *pC = pB + 6 * npairs;
+    if constexpr (sizeof(T) == 8) {
+        if (f.real_basis) {
+            ofdft_status r = enqueue_real(c, f, ph, phi0, dh, cth, sth, (const double *)csd, vout, sums, spart, nbg_out);
+            if (r != OFDFT_OK || !keep_nG) return r;
+            return enqueue_nG(c, f, ph, pA);
+        }
+    }
     // the tensor-core derivative passes read n as a field: it waits in the
     // buffer that the pointwise stage overwrites with v_part
-    T *nf = !fttf && (ax.dmat || ay.dmat || az.dmat) ? (T *)f.vpart : nullptr;
+    const bool tcx = f.tl[0].der.img, tcy = f.tl[1].der.img, tcz = f.tl[2].der.img;
+    T *nf = !fttf && (tcx || tcy || tcz) ? (T *)f.vpart : nullptr;
     {
         TimerScope ts(c, TM_ZFWD, sizeof(T) == 4);
-        T *dz = fttf || az.dmat ? nullptr : d2;
+        T *dz = fttf || tcz ? nullptr : d2;
         if (phi0) launch_zfwd<T>(g, az, 2, nullptr, phi0, dh, (T)cth, (T)sth, csd, ph, s0, st, dz, nf);
         else launch_zfwd<T>(g, az, 1, nullptr, ph, nullptr, T(0), T(0), nullptr, nullptr, s0, st, dz, nf);
     }
@@ -363,22 +603,21 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
         cudaStream_t s2nd = fork ? c->aux[1] : st;   // stream of each pair's second pass
         // derivatives along the axes with a digit matrix: one launch on the
         // tensor cores (each pass may write over its input)
-        const FftAxis *const tax[3] = {ax.dmat ? &ax : nullptr, ay.dmat ? &ay : nullptr, az.dmat ? &az : nullptr};
-        auto tline = [&](T *x, T *y, T *z) {
+        auto tline = [&](const T *x, const T *y, const T *z) {
             if constexpr (sizeof(T) == 8) {
                 if (!nf) return;
                 TimerScope ts(c, TM_DLINE, false);
-                const double *const in[3] = {x ? x : nf, y ? y : nf, z ? z : nf};
-                float2 *const out[3] = {(float2 *)d0, (float2 *)d1, (float2 *)d2};
-                launch_tline(g, tax, in, out, st);
+                const double *const in[3] = {x, y, z};
+                double *const out[3] = {d0, d1, d2};
+                launch_derivatives(g, f, in, out, st);
             }
         };
-        tline(nullptr, nullptr, nullptr);
-        if (!ax.dmat) {
+        tline(nf, nf, nf);
+        if (!tcx) {
             TimerScope ts(c, TM_DLINE, sizeof(T) == 4);
             launch_dline<T>(g, ax, 0, nf ? 1 : 0, 0, nf ? nf : ph, d0, st);
         }
-        if (!ay.dmat) {
+        if (!tcy) {
             TimerScope ts(c, TM_DLINE, sizeof(T) == 4);
             launch_dline<T>(g, ay, 1, nf ? 1 : 0, 0, nf ? nf : ph, d1, s2nd);
         }
@@ -406,11 +645,11 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
         // subtracts both (and d_z U_z, which it takes itself unless the
         // tensor-core pass has)
         tline(d0, d1, d2);
-        if (!ay.dmat) {
+        if (!tcy) {
             TimerScope ts(c, TM_DLINE, sizeof(T) == 4);
             launch_dline<T>(g, ay, 1, 1, 0, d1, d1, st);
         }
-        if (!ax.dmat) {
+        if (!tcx) {
             TimerScope ts(c, TM_DLINE, sizeof(T) == 4);
             launch_dline<T>(g, ax, 0, 1, 0, d0, d0, s2nd);
         }
@@ -421,7 +660,7 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
         }
         DBG("k_dline (div W)");
         TimerScope ts(c, TM_ZFINAL, sizeof(T) == 4);
-        nbz = launch_zfinal_gga<T>(g, az, s0, az.dmat ? nullptr : d2, (const T *)f.vpart, d1, d0, d2, ph, phi0, dh,
+        nbz = launch_zfinal_gga<T>(g, az, s0, tcz ? nullptr : d2, (const T *)f.vpart, d1, d0, d2, ph, phi0, dh,
                                    (T)cth, (T)sth, csd, vout, pC, st);
     }
     DBG("k_zfinal");
@@ -429,12 +668,7 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
     DBG("k_reduce_eval");
     c->launches += eval_kernel_count(c, f);
     if (keep_nG && !fttf) {
-        // n(G) for forces and stress: forward z, y, x of n into the second spectrum
-        launch_zfwd<T>(g, az, 1, nullptr, ph, nullptr, T(0), T(0), nullptr, nullptr, s1, st);
-        launch_ypass<T>(g, ay, false, s1, 1, fs, st);
-        launch_xhl<T>(g, ax, s1, vext, s1, 0, pA, st);
-        c->launches += 3;
-        DBG("n(G)");
+        if constexpr (sizeof(T) == 8) return enqueue_nG(c, f, ph, pA);
     }
     return OFDFT_OK;
 }
@@ -557,6 +791,11 @@ ofdft_status update_ions(ofdft_ctx *c)
     const PhaseTablesDD *dd = g.dd ? &c->pdd : nullptr;
     launch_phases(g, c->nat, c->Rd, c->px, c->py, c->pz, dd, st);
     launch_vext(g, c->nat, c->Zd, c->px, c->py, c->pz, dd, (double2 *)c->f[0].vext, st);
+    if (c->f[0].real_basis) {
+        launch_real_coefficients(g, (const double2 *)c->f[0].vext, c->f[0].vre, st);
+        if (g.lpp) launch_real_coefficients(g, (const double2 *)c->f[0].vext + g.NH, c->f[0].vre + g.N, st);
+        c->launches += g.lpp ? 2 : 1;
+    }
     if (c->f[1].valid)
         launch_convert<double, float>(((g.lpp || g.tri) ? 4 : 2) * g.NH, (const double *)c->f[0].vext, (float *)c->f[1].vext,
                                       st);
@@ -1301,7 +1540,7 @@ ofdft_status forces_now(ofdft_ctx *c, EvalScalars &es)
 void free_fieldset(FieldSet &f, cudaStream_t st)
 {
     void *ptrs[] = {f.phi, f.phit, f.dhat, f.g, f.gprev, f.d, f.v, f.vt, f.vpart, f.spec, f.vext, f.tab,
-                    f.tw[0], f.tw[1], f.tw[2], f.dmat[0], f.dmat[1], f.dmat[2], f.cs};
+                    f.tw[0], f.tw[1], f.tw[2], f.tlmem, f.vre, f.cs};
     for (void *p : ptrs)
         if (p) cudaFreeAsync(p, st);
     if (f.graph) cudaGraphExecDestroy(f.graph);
@@ -1369,6 +1608,7 @@ template <typename T> ofdft_status alloc_fieldset(ofdft_ctx *c, FieldSet &f)
     int n3[3] = {g.nx, g.ny, g.nz};
     for (int a = 0; a < 3; ++a)
         if (upload_twiddles<T>(c, f, a, n3[a]) != OFDFT_OK) return OFDFT_EDEVICE;
+    if (sizeof(T) == 8 && setup_tline(c, f) != OFDFT_OK) return OFDFT_EDEVICE;
     CK(cudaMallocAsync((void **)&f.cs, sizeof(CgState), c->st));
     f.gt = c->g;
     CK(cudaMemsetAsync(f.cs, 0, sizeof(CgState), c->st));
@@ -1456,8 +1696,9 @@ double footprint_bytes(const int grid[3], int nat, int precision)
     };
     double b = fieldset(8.0) + (precision == OFDFT_MIXED ? fieldset(4.0) : 0.0);
     b += N * 8;                                                        // phiprev
-    for (int a = 0; a < 3; ++a)                                        // derivative matrices
-        if (tline_supported(grid[a])) b += (double)tline_matrix_bytes(grid[a]);
+    for (int a = 0; a < 3; ++a)                                        // matrices of the tensor-core transforms
+        if (tline_supported(grid[a])) b += 3.0 * tline_matrix_bytes(grid[a]) + 8.0 * grid[a] + 1024;
+    if (tline_supported(grid[0]) && tline_supported(grid[1]) && tline_supported(grid[2])) b += 2 * N * 8;   // v_ext's coefficients
     b += (3 * ny * std::ceil(K / 4) + 15 * (nx * ny / 2) + 64) * 8 + 64 * 8;  // partials, scalars
     b += nat * 11.0 * 8 + 32 + nat * (2 * nx + 2 * ny + 3 * K) * 16.0;  // ions, phase factors (+ double-float)
     b += nat * std::max(1216.0, (double)lpp_force_chunks_dd((long long)(nx * ny), nat)) * 3 * 8 + 16 * 8;   // force partials
@@ -1496,11 +1737,9 @@ struct Tuned {
 // twiddle tables do not depend on the schedule).
 void set_radix(FieldSet &f, int a, int m)
 {
-    const FftAxis old = f.ax[a];
-    f.ax[a] = fft_axis(old.n, old.tw, m);
-    f.ax[a].twf = old.twf;
-    f.ax[a].dmat = old.dmat;
-    f.ax[a].dexp = old.dexp;
+    const void *twf = f.ax[a].twf;
+    f.ax[a] = fft_axis(f.ax[a].n, f.ax[a].tw, m);
+    f.ax[a].twf = twf;
 }
 std::map<TuneKey, Tuned> g_tune;
 
@@ -1532,6 +1771,7 @@ template <typename T> ofdft_status time_evals(ofdft_ctx *c, FieldSet &f, int rep
 template <typename T> ofdft_status autotune_set(ofdft_ctx *c, int k, int reps)
 {
     FieldSet &f = c->f[k];
+    if (f.real_basis) return OFDFT_OK;   // the tensor-core transforms have one shape
     const TuneKey key{c->g.nx, c->g.ny, c->g.nz, (int)sizeof(T)};
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -1600,7 +1840,7 @@ template <typename T> ofdft_status autotune_set(ofdft_ctx *c, int k, int reps)
     }
     // the derivative passes' tile width and threads together (GGA only; the
     // tensor-core form has one shape)
-    if (c->fp.kind != 0 && !(f.ax[0].dmat && f.ax[1].dmat)) {
+    if (c->fp.kind != 0 && !(f.tl[0].der.img && f.tl[1].der.img)) {
         const GridInfo base = best;
         for (int dk : {4, 8, 16})
             for (int th : {64, 128, 256}) {

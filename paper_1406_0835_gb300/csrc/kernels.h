@@ -22,17 +22,64 @@ void launch_zfwd(const GridInfo &g, const FftAxis &az, int mode, const T *in, co
 template <typename T>
 void launch_dline(const GridInfo &g, const FftAxis &fa, int axis, int mode, int acc, const T *in, T *out,
                   cudaStream_t st);
-// Derivatives d f (f = in[a]) along the axes a whose ax[a] is not null, in
-// one launch on the tensor cores, written as double-float pairs; for axes
-// whose digit matrix is set (FftAxis::dmat).  out[a] may be in[a].
-// tline_derivative_matrix fills img (tline_matrix_bytes(n)) with the digits
-// of the derivative matrix times scale and returns its binary exponent.
+// ---- one-axis transforms on the tensor cores (kernels_tline.cu).  Fields
+// and coefficients are double-float pairs (float2).
+// A matrix's digits in device memory and their binary exponent.
+struct TlMat {
+    const void *img = nullptr;
+    int mexp = 0;
+};
+// Matrices of one axis (null: the axis is too long, or not asked for) and
+// (k b)^2 of its real-Fourier coefficients.
+struct TlAxis {
+    TlMat der, fwd, inv;
+    const float2 *g2 = nullptr;
+};
 bool tline_supported(int n);
 size_t tline_matrix_bytes(int n);
+// Fill img (tline_matrix_bytes(n)) and return the exponent: the derivative
+// times scale; the orthonormal real Fourier transform, or its inverse.
 int tline_derivative_matrix(int n, double scale, uint16_t *img);
+int tline_fourier_matrix(int n, bool inverse, uint16_t *img);
+// Frequency of real-Fourier coefficient a and whether it is the sine's.
+int tline_frequency(int n, int a, bool *sine);
 cudaError_t tline_smem_limits();
-void launch_tline(const GridInfo &g, const FftAxis *const ax[3], const double *const in[3], float2 *const out[3],
-                  cudaStream_t st);
+// Up to four transforms, each along one axis, in one launch; out may be in.
+struct TlPass {
+    enum Kind { kDerivative, kForward, kInverse } kind;
+    int axis;
+    const TlMat *mat;
+    const float2 *in;
+    float2 *out;
+};
+void launch_tline(const GridInfo &g, int count, const TlPass *pass, cudaStream_t st);
+// coef: coefficients of n -> of v_HL = 4 pi n / G^2 + v_ext; partials E_H,
+// E_loc, P_loc in three rows of the returned number of columns.
+struct TlHartree {
+    const float2 *g2[3];       // (k b)^2 per coefficient and axis
+    const float2 *ve, *vp;     // v_ext's coefficients; pressure weights or null (Gaussian ion)
+    float2 hr;                 // rc^2 / 2
+    double half_dv, dv, ploc;  // factors of the three sums
+    double *part;
+};
+int launch_hartree(const GridInfo &g, float2 *coef, const TlHartree &hl, cudaStream_t st);
+// v = v_HL + v_part - (d[0] + d[1] + d[2]), partials as launch_zfinal_gga.
+struct TlFinal {
+    const float2 *vhl, *vpart, *d[3];
+    const double *phit, *phi, *dhat, *cs;
+    double c, s, *vout, *part;
+};
+int launch_final(const GridInfo &g, const TlFinal &fin, cudaStream_t st);
+// n = phi^2 (with dhat: of the trial phi c + dhat s, written to phit), as pairs.
+void launch_density(long long n, const double *phi, const double *dhat, double c, double s, const double *cs,
+                    double *phit, float2 *dens, cudaStream_t st);
+// ftTF: v = v_HL + df/dn + v_xc; partials as launch_zfinal's.
+int launch_ptf(const GridInfo &g, const float2 *vhl, const double *phit, const double *phi, const double *dhat, double c,
+               double s, const double *cs, double temp, const FuncParams &fp, const double *tab, int xc, double *vout,
+               double *part, cudaStream_t st);
+// Real-Fourier coefficients (pairs) of the real field whose half spectrum is
+// v (orthorhombic cells; the spectrum's Nyquist planes Hermitian).
+void launch_real_coefficients(const GridInfo &g, const double2 *v, float2 *coef, cudaStream_t st);
 // Pointwise functional + XC: reads phi and the derivatives of n in d0..d2,
 // writes v_part and, over d0..d2, the fields U_j whose derivatives sum to
 // div W.  Partials: 6 rows (12 with stress: sum W_a d_b n in rows 6..11, FP64

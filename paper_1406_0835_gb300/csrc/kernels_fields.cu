@@ -59,8 +59,8 @@ template <> __device__ __forceinline__ double2 stc<DD>(ff::cf2 v)
 {
     return make_double2(ff::to_double(v.x), ff::to_double(v.y));
 }
-// Derivative fields and v_part between kernels of one evaluation: the
-// double-float kernels keep them as pairs (hi, lo) in the 8 bytes of a binary64, so that
+// Fields between the kernels of one evaluation (n, the derivatives of n, U,
+// its derivatives, v_part): the double-float kernels keep them as pairs (hi, lo) in the 8 bytes of a binary64, so that
 // neither side converts.
 template <typename PR> __device__ __forceinline__ typename KT<PR>::R ldp(typename KT<PR>::T x) { return x; }
 template <> __device__ __forceinline__ ff::f2 ldp<DD>(double x)
@@ -319,7 +319,7 @@ __global__ void OFDFT_FFT_BOUNDS k_zfwd(GridInfo g, FftAxis az, int P, const typ
             phit[base + i] = str<PR>(ph);
             val = ph * ph;
         }
-        if (nout != nullptr) nout[base + i] = str<PR>(val);
+        if (nout != nullptr) nout[base + i] = stp<PR>(val);
         R *dstp = reinterpret_cast<R *>(&A[(line >> 1) * nz + e]);
         dstp[line & 1] = val;
     }
@@ -714,7 +714,7 @@ __global__ void OFDFT_FFT_BOUNDS k_dline(GridInfo g, FftAxis fa, const typename 
         const int r = i >> t.tsh, c = i & (t.tk - 1);
         if (c < t.ncol) {
             const T2 v = *reinterpret_cast<const T2 *>(in + t.cbase[c] + r * t.rstride);
-            R a = ldr<PR>(v.x), b = ldr<PR>(v.y);
+            R a = MODE == 0 ? ldr<PR>(v.x) : ldp<PR>(v.x), b = MODE == 0 ? ldr<PR>(v.y) : ldp<PR>(v.y);
             if (MODE == 0) {
                 a = a * a;
                 b = b * b;
@@ -773,7 +773,7 @@ __global__ void OFDFT_FFT_BOUNDS k_dline_ws(GridInfo g, FftAxis fa, const typena
         const int r = i >> t.tsh, c = i & (t.tk - 1);
         if (c < t.ncol) {
             const T2 v = *reinterpret_cast<const T2 *>(in + t.cbase[c] + r * t.rstride);
-            R a = ldr<PR>(v.x), b = ldr<PR>(v.y);
+            R a = MODE == 0 ? ldr<PR>(v.x) : ldp<PR>(v.x), b = MODE == 0 ? ldr<PR>(v.y) : ldp<PR>(v.y);
             if (MODE == 0) {
                 a = a * a;
                 b = b * b;
@@ -902,13 +902,13 @@ __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB) k_pw(GridInfo
             sacc[5] += w[1] * gr[2];
         }
         if constexpr (TRI) {
-            d0[i] = str<PR>(bm[0] * w[0] + bm[1] * w[1] + bm[2] * w[2]);
-            d1[i] = str<PR>(bm[3] * w[0] + bm[4] * w[1] + bm[5] * w[2]);
-            d2[i] = str<PR>(bm[6] * w[0] + bm[7] * w[1] + bm[8] * w[2]);
+            d0[i] = stp<PR>(bm[0] * w[0] + bm[1] * w[1] + bm[2] * w[2]);
+            d1[i] = stp<PR>(bm[3] * w[0] + bm[4] * w[1] + bm[5] * w[2]);
+            d2[i] = stp<PR>(bm[6] * w[0] + bm[7] * w[1] + bm[8] * w[2]);
         } else {
-            d0[i] = str<PR>(w[0]);
-            d1[i] = str<PR>(w[1]);
-            d2[i] = str<PR>(w[2]);
+            d0[i] = stp<PR>(w[0]);
+            d1[i] = stp<PR>(w[1]);
+            d2[i] = stp<PR>(w[2]);
         }
     }
     double tot[6];
@@ -930,8 +930,8 @@ __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB) k_pw(GridInfo
 // transform serves both) and div = d_x U_x + d_y U_y, given as one field or
 // as two (div + div2; div2 may be null).  div may alias vout (each point is
 // read before it is written, by the same thread).  With uz null, d_z U_z is
-// given as the field div3 instead.  vpart, div, div2 and div3 are stored as
-// derivative fields are (ldp).  Partials
+// given as the field div3 instead.  uz, vpart, div, div2 and div3 are pairs
+// (ldp).  Partials
 // (as k_zfinal's GGA form): rows 0..5 zero, then sum phi^2 v, sum phi^2,
 // sum 2 phi v dphi/dtheta.
 template <typename PR>
@@ -967,7 +967,7 @@ __global__ void OFDFT_FFT_BOUNDS k_zfinal_g(GridInfo g, FftAxis az, int P, const
         RowCol rc(nz);
         for (int i = threadIdx.x; i < 2 * nl * nz; i += blockDim.x, rc.next()) {
             R *dst = reinterpret_cast<R *>(&B[(rc.r >> 1) * nz + rc.c]);
-            dst[rc.r & 1] = ldr<PR>(uz[rbase + i]);
+            dst[rc.r & 1] = ldp<PR>(uz[rbase + i]);
         }
         __syncthreads();
         Z = fft_lines<CC, false>(B, B + P * nz, az, nl, nz, 1, false);
@@ -1106,6 +1106,157 @@ void launch_dline(const GridInfo &g, const FftAxis &fa, int axis, int mode, int 
 #undef CALL
 }
 
+// n = phi^2 as pairs, two points a thread (N is even).
+__global__ void k_density(long long pairs, const double2 *__restrict__ phi, const double2 *__restrict__ dhat, double c, double s,
+                          const double *__restrict__ cs, double2 *__restrict__ phit, float4 *__restrict__ dens)
+{
+    if (cs != nullptr) {
+        c = cs[0];
+        s = cs[1];
+    }
+    const ff::f2 cr = ff::split_int(c), sr = ff::split_int(s);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < pairs; i += (long long)gridDim.x * blockDim.x) {
+        const double2 p = phi[i];
+        ff::f2 a = ff::split_int(p.x), b = ff::split_int(p.y);
+        if (dhat != nullptr) {
+            const double2 d = dhat[i];
+            a = cr * a + sr * ff::split_int(d.x);
+            b = cr * b + sr * ff::split_int(d.y);
+            phit[i] = make_double2(ff::to_double(a), ff::to_double(b));
+        }
+        a = a * a;
+        b = b * b;
+        dens[i] = make_float4(a.hi, a.lo, b.hi, b.lo);
+    }
+}
+
+__device__ __forceinline__ ff::f2 f2of(float2 x) { return ff::f2(x.x, x.y); }
+
+// Real-Fourier coefficients of n -> of v_HL = 4 pi n / G^2 + v_ext, with the
+// sums of E_H, E_loc and P_loc.  A kernel of its own: in the transforms'
+// blocks (one to an SM) the same loop waited on memory latency.
+__global__ void __launch_bounds__(256) k_hartree(GridInfo g, float4 *__restrict__ coef, TlHartree hl)
+{
+    constexpr ff::f2 fpi(kFourPi);
+    const ff::f2 hr = f2of(hl.hr), z0(0.0f, 0.0f);
+    ff::f2 acc[3] = {z0, z0, z0};
+    const int hz = g.nz / 2, pairs = (int)(g.N / 2);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += gridDim.x * blockDim.x) {
+        const int ab = i / hz, c = 2 * (i - ab * hz), a = ab / g.ny, b = ab - a * g.ny;
+        const float4 x = coef[i], e = reinterpret_cast<const float4 *>(hl.ve)[i];
+        const float4 gz = reinterpret_cast<const float4 *>(hl.g2[2])[c / 2];
+        float4 p = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (hl.vp) p = reinterpret_cast<const float4 *>(hl.vp)[i];
+        const ff::f2 gxy = ff::add_s(f2of(hl.g2[0][a]), f2of(hl.g2[1][b]));
+        float2 o[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const ff::f2 n = k ? ff::f2(x.z, x.w) : ff::f2(x.x, x.y), ve = k ? ff::f2(e.z, e.w) : ff::f2(e.x, e.y);
+            const ff::f2 g2 = ff::add_s(gxy, k ? ff::f2(gz.z, gz.w) : ff::f2(gz.x, gz.y));
+            o[k] = make_float2(0.0f, 0.0f);
+            if (g2.hi > 0.0f) {
+                const ff::f2 hc = ff::mul(ff::div(fpi, g2), n), cv = ff::mul(n, ve);
+                acc[0] += ff::mul(hc, n);
+                acc[1] += cv;
+                acc[2] += hl.vp ? ff::mul(n, k ? ff::f2(p.z, p.w) : ff::f2(p.x, p.y))
+                                : ff::mul(cv, ff::add(ff::neg(ff::mul(hr, g2)), 1.0f));
+                const ff::f2 w = ff::add_s(hc, ve);
+                o[k] = make_float2(w.hi, w.lo);
+            }
+        }
+        coef[i] = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+    }
+    double tot[3];
+    block_sum_f2<3>(acc, tot);
+    if (threadIdx.x == 0) {
+        hl.part[blockIdx.x] = hl.half_dv * tot[0];
+        hl.part[(size_t)gridDim.x + blockIdx.x] = hl.dv * tot[1];
+        hl.part[(size_t)2 * gridDim.x + blockIdx.x] = hl.ploc * tot[2];
+    }
+}
+
+// GGA potential v = v_HL + v_part - (d_x U_x + d_y U_y + d_z U_z) and the sums
+// of phi^2 v, phi^2 and 2 phi v dphi/dtheta (partials as k_zfinal_g's).
+__global__ void __launch_bounds__(256) k_final(GridInfo g, TlFinal f)
+{
+    double c = f.c, s = f.s;
+    if (f.cs != nullptr) {
+        c = f.cs[0];
+        s = f.cs[1];
+    }
+    const ff::f2 cr = ff::split_int(c), sr = ff::split_int(s), z0(0.0f, 0.0f);
+    ff::f2 acc[3] = {z0, z0, z0};
+    const int pairs = (int)(g.N / 2);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += gridDim.x * blockDim.x) {
+        auto ld = [&](const float2 *p) { return reinterpret_cast<const float4 *>(p)[i]; };
+        auto lr = [&](const double *p) { return reinterpret_cast<const double2 *>(p)[i]; };
+        const float4 vp = ld(f.vpart), dx = ld(f.d[0]), dy = ld(f.d[1]), dz = ld(f.d[2]), vh = ld(f.vhl);
+        const double2 ph = lr(f.phit);
+        double2 p0 = make_double2(0.0, 0.0), dh = p0, out;
+        if (f.dhat != nullptr) {
+            p0 = lr(f.phi);
+            dh = lr(f.dhat);
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            auto of = [&](const float4 &x) { return k ? ff::f2(x.z, x.w) : ff::f2(x.x, x.y); };
+            const ff::f2 div = of(dx) + of(dy) + of(dz), v = of(vp) + of(vh) - div;
+            const ff::f2 p = ff::split_int(k ? ph.y : ph.x), n = p * p;
+            (k ? out.y : out.x) = ff::to_double(v);
+            acc[0] += n * v;
+            acc[1] += n;
+            if (f.dhat != nullptr) {
+                const ff::f2 dphi = cr * ff::split_int(k ? dh.y : dh.x) - sr * ff::split_int(k ? p0.y : p0.x);
+                acc[2] += ff::scale(p * v * dphi, 2.0f);
+            }
+        }
+        reinterpret_cast<double2 *>(f.vout)[i] = out;
+    }
+    double tot[3];
+    block_sum_f2<3>(acc, tot);
+    if (threadIdx.x == 0) {
+        for (int q = 0; q < 6; ++q) f.part[(size_t)q * gridDim.x + blockIdx.x] = 0.0;
+        for (int q = 0; q < 3; ++q) f.part[(size_t)(6 + q) * gridDim.x + blockIdx.x] = tot[q];
+    }
+}
+
+// ftTF pointwise stage: v = v_HL + df/dn + v_xc, partials as k_zfinal's.
+__global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB)
+    k_ptf(GridInfo g, const float2 *__restrict__ vhl, const double *__restrict__ phit, const double *__restrict__ phi,
+          const double *__restrict__ dhat, double c, double s, const double *__restrict__ cs, double temp, FuncParams fp,
+          const double *__restrict__ tab, int xc, double *__restrict__ vout, double *__restrict__ part)
+{
+    if (cs != nullptr) {
+        c = cs[0];
+        s = cs[1];
+    }
+    const ff::f2 cr = ff::split_int(c), sr = ff::split_int(s), z0(0.0f, 0.0f);
+    ff::f2 acc[9] = {z0, z0, z0, z0, z0, z0, z0, z0, z0};
+    const ff::f2 tcoef = ff::f2(2.0 / OF_K23 * temp), gz[3] = {z0, z0, z0};
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < g.N; i += (long long)gridDim.x * blockDim.x) {
+        const ff::f2 ph = ff::split_int(phit[i]), n = ph * ph;
+        const float2 h = vhl[i];
+        const PwF2 o = pw_dd(fp, tab, tcoef, temp, n, gz, xc);
+        const ff::f2 v = o.dfdn + o.vxc + ff::f2(h.x, h.y);
+        vout[i] = ff::to_double(v);
+        acc[0] += o.f;
+        acc[1] += o.ts;
+        acc[2] += n * o.eps;
+        acc[3] += n * o.dfdn - o.f;
+        acc[5] += n * (o.vxc - o.eps);
+        acc[6] += n * v;
+        acc[7] += n;
+        if (dhat != nullptr) {
+            const ff::f2 dphi = cr * ff::split_int(dhat[i]) - sr * ff::split_int(phi[i]);
+            acc[8] += ff::f2(2.0f, 0.0f) * (ph * v) * dphi;
+        }
+    }
+    double tot[9];
+    block_sum_f2<9>(acc, tot);
+    if (threadIdx.x == 0)
+        for (int q = 0; q < 9; ++q) part[(size_t)q * gridDim.x + blockIdx.x] = tot[q];
+}
+
 // Blocks of the pointwise kernel: about eight points a thread (the block
 // sums cost a few hundred instructions a thread), at least one full wave of
 // the GPU's SMs, at most one block per z line pair (the partial-sum rows
@@ -1147,6 +1298,47 @@ int launch_pw(const GridInfo &g, T *d0, T *d1, T *d2, const T *phit, T temp, con
     }
     OFDFT_DISPATCH(T, g, CALL);
 #undef CALL
+    return blocks;
+}
+
+void launch_density(long long n, const double *phi, const double *dhat, double c, double s, const double *cs,
+                    double *phit, float2 *dens, cudaStream_t st)
+{
+    const long long pairs = n / 2;
+    const int blocks = (int)std::min<long long>((pairs + 255) / 256, 1216);
+    k_density<<<blocks, 256, 0, st>>>(pairs, (const double2 *)phi, (const double2 *)dhat, c, s, cs, (double2 *)phit,
+                                      (float4 *)dens);
+}
+
+// Blocks of the elementwise kernels over pairs of points: four pairs a thread
+// at most, at most one block per z line pair (their partial-sum rows).
+int pair_blocks(const GridInfo &g)
+{
+    const long long b = std::min<long long>((g.N / 2 + 255) / 256, std::max<long long>(912, (g.N / 2 + 1023) / 1024));
+    return (int)std::min<long long>(b, (long long)g.nx * g.ny / 2);
+}
+
+int launch_hartree(const GridInfo &g, float2 *coef, const TlHartree &hl, cudaStream_t st)
+{
+    // partial rows of at most one column per four half-spectrum columns of the yz plane
+    const int blocks = std::min(pair_blocks(g), g.ny * ((g.K + 3) / 4));
+    k_hartree<<<blocks, 256, 0, st>>>(g, (float4 *)coef, hl);
+    return blocks;
+}
+
+int launch_final(const GridInfo &g, const TlFinal &fin, cudaStream_t st)
+{
+    const int blocks = pair_blocks(g);
+    k_final<<<blocks, 256, 0, st>>>(g, fin);
+    return blocks;
+}
+
+int launch_ptf(const GridInfo &g, const float2 *vhl, const double *phit, const double *phi, const double *dhat, double c,
+               double s, const double *cs, double temp, const FuncParams &fp, const double *tab, int xc, double *vout,
+               double *part, cudaStream_t st)
+{
+    const int th = OFDFT_PW_THREADS, blocks = pw_blocks(g, th);
+    k_ptf<<<blocks, th, 0, st>>>(g, vhl, phit, phi, dhat, c, s, cs, temp, fp, tab, xc, vout, part);
     return blocks;
 }
 

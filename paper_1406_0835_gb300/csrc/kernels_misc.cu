@@ -3,6 +3,8 @@
 // terms and the MD integrator.  Every reduction writes per-block partial
 // sums that a second kernel adds in a fixed order, so results do not depend
 // on scheduling.
+#include <algorithm>
+
 #include "fft_core.cuh"
 #include "kernels.h"
 
@@ -500,6 +502,56 @@ __global__ void k_vext(GridInfo g, int nat, const double *__restrict__ Z,
             const double wp = lpp_wp_ha(g, k.g2);
             vext[(size_t)g.NH + q] = make_double2(wp * v.x, wp * v.y);
         }
+    }
+}
+
+// Real-Fourier coefficients of a real field from its half spectrum V (v(r) =
+// sum_G V(G) e^{i G.r}): along an axis of n points a cosine of frequency k
+// takes (V(k) + V(-k)) and a sine i (V(k) - V(-k)), each times sqrt(n/2); k
+// = 0 and n/2 take sqrt(n) V(k).  V(-G) = conj V(G).  fx, fy, fz: frequency
+// of each coefficient, negative for a sine (tables of one int per index).
+__device__ __forceinline__ int real_freq(int n, int a, bool &sine)
+{
+    const int h = n / 2;
+    const bool odd = a >= h;
+    const int i = odd ? a - h : a;
+    sine = odd ? (i & 1) != 0 : (i > 0 && (i & 1) == 0);
+    return odd ? 2 * (i / 2) + 1 : 2 * ((i + 1) / 2);
+}
+__global__ void k_real_coefficients(GridInfo g, const double2 *__restrict__ V, float2 *__restrict__ coef)
+{
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < (int)g.N; q += gridDim.x * blockDim.x) {
+        const int c = q % g.nz, ab = q / g.nz, b = ab % g.ny, a = ab / g.ny;
+        bool sx, sy, sz;
+        const int kx = real_freq(g.nx, a, sx), ky = real_freq(g.ny, b, sy), kz = real_freq(g.nz, c, sz);
+        const bool ex = kx == 0 || 2 * kx == g.nx, ey = ky == 0 || 2 * ky == g.ny, ez = kz == 0 || 2 * kz == g.nz;
+        const int mx = ex ? kx : g.nx - kx, my = ey ? ky : g.ny - ky;
+        auto at = [&](int ix, int iy) { return V[((size_t)ix * g.ny + iy) * g.K + kz]; };
+        // z step at the four sign choices of (kx, ky): W = V(s) +- conj V(-s)
+        double2 W[2][2];
+        for (int i = 0; i < 2; ++i)
+            for (int j = 0; j < 2; ++j) {
+                if ((ex && i) || (ey && j)) continue;
+                const double2 p = at(i ? mx : kx, j ? my : ky);
+                if (ez) {
+                    W[i][j] = p;
+                } else {
+                    const double2 m = at(i ? kx : mx, j ? ky : my);
+                    W[i][j] = sz ? make_double2(-(p.y + m.y), p.x - m.x) : make_double2(p.x + m.x, p.y - m.y);
+                }
+            }
+        double2 X[2];
+        for (int i = 0; i < 2; ++i) {
+            if (ex && i) continue;
+            if (ey) X[i] = W[i][0];
+            else if (sy) X[i] = make_double2(-(W[i][0].y - W[i][1].y), W[i][0].x - W[i][1].x);
+            else X[i] = make_double2(W[i][0].x + W[i][1].x, W[i][0].y + W[i][1].y);
+        }
+        const double re = ex ? X[0].x : (sx ? -(X[0].y - X[1].y) : X[0].x + X[1].x);
+        const double f = sqrt((double)g.nx * (ex ? 1.0 : 0.5)) * sqrt((double)g.ny * (ey ? 1.0 : 0.5)) *
+                         sqrt((double)g.nz * (ez ? 1.0 : 0.5));
+        const ff::f2 o = ff::from_double(re * f);
+        coef[q] = make_float2(o.hi, o.lo);
     }
 }
 
@@ -1338,6 +1390,12 @@ __global__ void k_andersen(int nat, const double *m, double *V, double kT, doubl
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
+void launch_real_coefficients(const GridInfo &g, const double2 *v, float2 *coef, cudaStream_t st)
+{
+    const int blocks = (int)std::min<long long>((g.N + 255) / 256, 4864);
+    k_real_coefficients<<<blocks, 256, 0, st>>>(g, v, coef);
+}
+
 bool launch_ewald_energy(int nat, const double *R, const double *Z, const float *frac, const double L[3], double2 *tab, double *part,
                          double *out, cudaStream_t st)
 {

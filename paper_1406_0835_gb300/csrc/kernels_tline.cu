@@ -1,22 +1,27 @@
-// Derivatives along the grid axes on the tensor cores, exact to more than
-// the double-float transforms they replace.
+// One-axis transforms of real fields on the tensor cores, exact to more than
+// the double-float FFT stages they replace: spectral derivatives, and the
+// real Fourier transform (cosines and sines) along an axis and back.
 //
-// The spectral derivative along an axis of n points is a real circulant
-// matrix D (antisymmetric, D(j - l)), so a batch of lines is a contraction.
-// It is taken in integers.  With h = n/2 and the half-length sums and
-// differences s = x_lo + x_hi, d = x_lo - x_hi,
-//   e = De s,  o = Do d,  out_lo = e + o,  out_hi = e - o,
-//   De, Do = (D(j - l) +- D(j - l - h)) / 2      (h x h),
-// each line is scaled by the power of two of its largest magnitude to 53-bit
-// integers (binary64's own last place at that magnitude), the matrices are
-// rounded to 54-bit integers once, and both are cut into seven signed digits
-// of radix 256.  A digit is exact in f16, a product of two is at most 2^14,
+// Each is a real n x n matrix applied to a batch of lines, so a contraction.
+// With h = n/2 it splits into two h x h blocks, e and o, that act on the
+// functions of even and of odd frequency: on a field these are the sums and
+// differences s = x_lo + x_hi, d = x_lo - x_hi of its halves (and back
+// out_lo = e + o, out_hi = e - o); the coefficients of a transformed line
+// are stored even frequencies first, then odd ones.
+//   derivative: e = De s, o = Do d, De, Do = (D(j - l) +- D(j - l - h)) / 2
+//   forward:    the orthonormal cosines and sines of even (odd) frequency
+//   inverse:    their transposes
+//
+// The products are taken in integers.  Each line is scaled by the power of
+// two of its largest magnitude to 53-bit integers, the matrices are rounded
+// to 54-bit integers once, and both are cut into seven signed digits of
+// radix 256.  A digit is exact in f16, a product of two is at most 2^14,
 // and the sums over h <= 128 and up to seven digit pairs (two of them with a
 // leading digit, at most 64) stay below 2^24, so the f32 accumulators of
 // tcgen05.mma (kind::f16) hold exact integers.  Digit products of equal
 // weight share one accumulator: 7 accumulators, 28 products, the first
 // dropped weight about 2^-51 of the line's largest value times the largest
-// matrix entry.
+// matrix entry.  Fields are double-float pairs in memory (8 bytes).
 #include <math.h>
 
 #include <algorithm>
@@ -82,33 +87,42 @@ TlShape tl_shape(int n)
     return s;
 }
 
-// One axis of a launch.
+// One transform of a launch.
 struct TlJob {
     TlShape sh;
     int nlines, tiles, zlen;       // lines; tiles of 64; lines of one outer index (x, y: consecutive in memory)
     int zaxis;                     // lines contiguous in memory
+    int direct_in, direct_out;     // coefficients instead of a field's halves
     long long ostride, rstride;    // between outer indices; between a line's points
     int mexp;
     const unsigned char *mat;
-    const double *in;
+    const float2 *in;
     float2 *out;
 };
-constexpr int kMaxJobs = 3;
+constexpr int kMaxJobs = 4;
 struct TlJobs {
     TlJob job[kMaxJobs];
     int count;
 };
 
-// x as an integer multiple of 2^(E - 52) (truncated towards zero), E the
-// exponent of the line's largest magnitude (at least -100, so that the
-// output's unit is a normal binary32); esh = biased E.
-__device__ __forceinline__ uint64_t to_fixed(double x, int esh)
+// x 2^-E as an integer multiple of 2^-52, plus kFixedOff; u = 2^-E, E the
+// exponent of the line's largest magnitude (|x u| < 2).  Binary32 additions
+// of 1.5 2^23 round the leading word to 2^-20 and 2^-42 and the second to
+// 2^-42; what is left of both, below 2^-42, rounds to 2^-52.  The integers
+// are the low bits of the sums.
+constexpr uint32_t kMagic = 0x4b400000u;   // 1.5 2^23
+constexpr uint64_t kFixedOff = ((uint64_t)kMagic << 32) + 2048ull * kMagic + kMagic;
+__device__ __forceinline__ uint64_t to_fixed(float2 x, float u)
 {
-    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const int sh = min(esh - (int)((hi >> 20) & 0x7ffu), 63);
-    const uint64_t m = (((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32) | lo) >> sh;
-    const int64_t s = (int64_t)((int32_t)hi >> 31);
-    return (m ^ (uint64_t)s) - (uint64_t)s;
+    constexpr float kM = 12582912.0f, k20 = 1048576.0f, k42 = 4398046511104.0f, k52 = 4503599627370496.0f;
+    const float hi = ff::fmul(x.x, u), lo = ff::fmul(x.y, u);
+    const float ta = ff::ffma(hi, k20, kM);
+    const float r = ff::ffma(ff::fsub(ta, kM), -1.0f / k20, hi);
+    const float tb = ff::ffma(r, k42, kM), td = ff::ffma(lo, k42, kM);
+    const float r2 = ff::ffma(ff::fsub(tb, kM), -1.0f / k42, r), l2 = ff::ffma(ff::fsub(td, kM), -1.0f / k42, lo);
+    const float tc = ff::ffma(ff::fadd(r2, l2), k52, kM);
+    const uint64_t low = (uint64_t)(__float_as_uint(tb) + __float_as_uint(td)) * 1024u + __float_as_uint(tc);
+    return low + ((uint64_t)__float_as_uint(ta) << 32);
 }
 
 __device__ __forceinline__ uint32_t digit_pair(uint32_t bytes, uint32_t sel)
@@ -163,6 +177,12 @@ __device__ __forceinline__ ff::f2 combine(const float (&a)[kDig])
         s = t;
     }
     return ff::f2(s, err);
+}
+
+__device__ __forceinline__ float2 scaled(ff::f2 x, float sc)
+{
+    const ff::f2 r = ff::fast_two_sum(x.hi, x.lo);
+    return make_float2(r.hi * sc, r.lo * sc);
 }
 
 // x + sgn y of two such pairs, normalised, times sc (a power of two).
@@ -226,17 +246,38 @@ __device__ __forceinline__ bool issue(const TlShape &sh, const unsigned char *ma
     return good;
 }
 
-// out = d f along each job's axis, one block per tile of 64 lines.  out may
-// be in: a block reads its lines whole before it writes them.
+// Eight consecutive outputs of a line (left: how many lie in the half).
+__device__ __forceinline__ void store_lines(const float2 (&y)[8], float2 *p, long long rstride, int left, bool wide, bool ok)
+{
+    if (!ok) return;
+    if (left >= 8) {
+        if (wide) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                reinterpret_cast<float4 *>(p)[i] = make_float4(y[2 * i].x, y[2 * i].y, y[2 * i + 1].x, y[2 * i + 1].y);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) p[i * rstride] = y[i];
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i < left) p[i * rstride] = y[i];
+    }
+}
+
+// The transforms of a launch's jobs, one block per tile of 64 lines.  out
+// may be in: a block reads its lines whole before it writes them.
 //
 // M = 64 because at 96^3 tiles of 128 lines would leave half the SMs idle
 // (144 tiles of 64 for 152 SMs).  Measured (GB300, in a graph): one axis at
-// 96^3 7.8 us (z 9.5), at 48^3 5.2 us; the double-float transforms took
-// about 19 us a pass at 96^3, of which a GGA evaluation had four and the
-// two z kernels half of theirs.  Of the 12,000 cycles of a tile the MMAs
-// are 6,000 (0.5-0.7 cycles a column, M = 64 runs at half rate), the
-// conversion 2,600, the load 1,500, the read-out 1,700 behind the last MMA;
-// instruction fetch is the largest stall, since each warp runs the code once.
+// 96^3 7.8 us (z 10), three derivatives in one launch 24 us, one axis at
+// 48^3 5.5 us; the double-float FFT passes took about 19 us a derivative and
+// 12-32 us a Fourier pass at 96^3.  Of the 12,000 cycles of a tile the
+// products are 6,000 (0.5-0.7 cycles a column, M = 64 runs at half rate),
+// the conversion 2,800, the load 1,600, the read-out 1,700 behind the last
+// product; instruction fetch is the largest stall, since each warp runs the
+// code once.
 __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_constant__ TlJobs jobs)
 {
     extern __shared__ __align__(1024) unsigned char smraw[];
@@ -251,14 +292,15 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
     const int h = sh.h, nc = sh.nc, zaxis = jb.zaxis;
     const uint32_t a_dig = sh.a_dig;
     unsigned char *A = smraw, *B = smraw + 2 * kDig * (size_t)a_dig;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nconv = blockDim.x - 32;             // the last warp issues the products
     const uint32_t full = tc::smem_addr(s_bar), done = full + 8 * kMaxUnits;
     const uint32_t sa = tc::smem_addr(A), sb = tc::smem_addr(B);
     const long long rstride = jb.rstride;
+    const int nlines = jb.nlines, zlen = jb.zlen;
     if (tid >= nconv) {
         const int units = 2 * sh.chunks;
-        if (tid == nconv) {
+        if (lane == 0) {
             s_bad = 0;
             for (int i = 0; i < 2 * kMaxUnits; ++i) tc::mbar_init(full + 8 * i, 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -294,22 +336,31 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
     const int row = zaxis ? tid / nc : tid & (kLines - 1);
     const int chunk = zaxis ? tid - row * nc : tid >> 6;
     const bool mine = tid < kLines * nc;           // (a shorter job may share the launch)
-    double v[16];
+    // read-out: a warp takes its quarter's 16 lines of e (lanes 0-15) and of o
+    const int half = lane >> 4, quarter = warp & 3, set = warp >> 2, nset = nconv >> 7;
+    const int r = quarter * 16 + (lane & 15);
+    const int ln = tile * kLines + r;
+    const bool w_ok = ln < nlines;
+    const int ou = ln / zlen;
+    const long long ln_off = (w_ok ? ou * jb.ostride + (zaxis ? 0 : ln - ou * zlen) : 0) + (half ? h * rstride : 0);
+    const bool wide = zaxis && (h & 1) == 0;
+    if (tid < kLines) s_max[tid] = 27u << 23;      // 2^-100: the least exponent of the scale
+    float2 v[16];
     if (mine) {
         const int line = tile * kLines + row;
-        const bool ok = line < jb.nlines;
-        const int outer = ok ? line / jb.zlen : 0, left = min(8, h - chunk * 8);
-        const double *src = jb.in + (ok ? outer * jb.ostride + (zaxis ? 0 : line - outer * jb.zlen) : 0) + chunk * 8 * rstride;
-        const double *srh = src + h * rstride;
+        const bool ok = line < nlines;
+        const int outer = ok ? line / zlen : 0, left = min(8, h - chunk * 8);
+        const float2 *src = jb.in + (ok ? outer * jb.ostride + (zaxis ? 0 : line - outer * zlen) : 0) + chunk * 8 * rstride;
+        const float2 *srh = src + h * rstride;
         if (ok && left == 8) {
-            if (zaxis && (h & 1) == 0) {           // 16-byte aligned halves
+            if (wide) {                        // 16-byte aligned halves
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const double2 x = reinterpret_cast<const double2 *>(src)[i], y = reinterpret_cast<const double2 *>(srh)[i];
-                    v[2 * i] = x.x;
-                    v[2 * i + 1] = x.y;
-                    v[8 + 2 * i] = y.x;
-                    v[8 + 2 * i + 1] = y.y;
+                    const float4 x = reinterpret_cast<const float4 *>(src)[i], y = reinterpret_cast<const float4 *>(srh)[i];
+                    v[2 * i] = make_float2(x.x, x.y);
+                    v[2 * i + 1] = make_float2(x.z, x.w);
+                    v[8 + 2 * i] = make_float2(y.x, y.y);
+                    v[8 + 2 * i + 1] = make_float2(y.z, y.w);
                 }
             } else {
 #pragma unroll
@@ -322,30 +373,40 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const bool in_line = ok && i < left;
-                v[i] = in_line ? src[i * rstride] : 0.0;
-                v[8 + i] = in_line ? srh[i * rstride] : 0.0;
+                v[i] = in_line ? src[i * rstride] : make_float2(0.0f, 0.0f);
+                v[8 + i] = in_line ? srh[i * rstride] : make_float2(0.0f, 0.0f);
             }
         }
     }
-    if (tid < kLines) s_max[tid] = 0x39b00000u;    // 2^-100: the least exponent of the scale
-    bar_sync(3, nconv);
+    bar_sync(3, nconv);                            // s_max is set
     if (mine) {
         uint32_t m = 0;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) m = max(m, (uint32_t)__double2hiint(v[i]) & 0x7fffffffu);
-        if (m > 0x39b00000u) atomicMax(&s_max[row], m);
+        for (int i = 0; i < 16; ++i) m = max(m, __float_as_uint(v[i].x) & 0x7fffffffu);
+        if (m > (27u << 23)) atomicMax(&s_max[row], m);
     }
     bar_sync(3, nconv);
-    // digits of s, then of d: the products of e start in between
+    // digits of the first operand (s), then of the second (d): the
+    // products of e start in between
     unsigned char *dsta = A + chunk * kALbo + row * 16;
     uint64_t q[8];
     if (mine) {
-        const int esh = (int)(s_max[row] >> 20);
+        const float u = ff::int_bits_float((254u - (s_max[row] >> 23)) << 23 | (s_max[row] >> 23 == 254u ? 0x400000u : 0u));
+        if (jb.direct_in) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const uint64_t x = to_fixed(v[i], esh), y = to_fixed(v[8 + i], esh);
-            q[i] = x + y + kDigBias;
-            v[i] = __longlong_as_double((long long)(x - y + kDigBias));
+            for (int i = 0; i < 8; ++i) {
+                q[i] = to_fixed(v[i], u) + (kDigBias - kFixedOff);
+                const uint64_t y = to_fixed(v[8 + i], u) + (kDigBias - kFixedOff);
+                v[i] = make_float2(__uint_as_float((uint32_t)y), __uint_as_float((uint32_t)(y >> 32)));
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint64_t x = to_fixed(v[i], u), y = to_fixed(v[8 + i], u);
+                q[i] = x + y + (kDigBias - 2 * kFixedOff);
+                const uint64_t d = x - y + kDigBias;
+                v[i] = make_float2(__uint_as_float((uint32_t)d), __uint_as_float((uint32_t)(d >> 32)));
+            }
         }
         store_digits(q, dsta, a_dig);
     }
@@ -353,7 +414,8 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
     bar_arrive(1, blockDim.x);
     if (mine) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) q[i] = (uint64_t)__double_as_longlong(v[i]);
+        for (int i = 0; i < 8; ++i)
+            q[i] = (uint64_t)__float_as_uint(v[i].x) | (uint64_t)__float_as_uint(v[i].y) << 32;
         store_digits(q, dsta + kDig * a_dig, a_dig);
     }
     tc::fence_async();
@@ -362,30 +424,23 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
     tc::fence_after_sync();
     const uint32_t tmem = s_tmem;
 
-    // read-out: a warp reads its quarter's 16 lines of e and of o
-    const int lane = tid & 31, half = lane >> 4, quarter = warp & 3, set = warp >> 2, nset = nconv >> 7;
-    const int r = quarter * 16 + (lane & 15);
-    const int ln = tile * kLines + r;
-    const bool w_ok = ln < jb.nlines;
-    const int ou = ln / jb.zlen;
-    float2 *dst = jb.out + (w_ok ? ou * jb.ostride + (zaxis ? 0 : ln - ou * jb.zlen) : 0) + (half ? h * rstride : 0);
-    const bool wide = zaxis && (h & 1) == 0;
     const uint32_t m = s_max[r];
     // weight 1 stands for 2^96 times the integers' units 2^(E - 52) and 2^-mexp
-    float sc = ff::pow2i((int)(m >> 20) - 1023 + 44 - jb.mexp);
-    if (m >= 0x47f00000u) sc = __uint_as_float(0x7fc00000u);   // 2^128 and beyond, inf, NaN
+    float sc = ff::pow2i((int)(m >> 23) - 127 + 44 - jb.mexp);
+    if (m >= 0x7f800000u) sc = __uint_as_float(0x7fc00000u);   // inf, NaN
     const float sgn = half ? -1.0f : 1.0f;
+    float2 *dst = jb.out + ln_off;
 #pragma unroll 1
     for (int ch = 0; ch < sh.chunks; ++ch) {
         const int width = tl_width(sh, ch), j0 = ch * sh.g * 8;
         if (!tc::mbar_wait(done + 8 * (2 * ch + 1), 0) || *(volatile int *)&s_bad) sc = __uint_as_float(0x7fc00000u);
         tc::fence_after_sync();
-        const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + j0 * kDig;
+        const uint32_t tacc = tmem + ((uint32_t)(quarter * 32) << 16) + j0 * kDig;
 #pragma unroll 1
         for (int c0 = set * 8; c0 < width; c0 += nset * 8) {
             float a[kDig][8];
 #pragma unroll
-            for (int d = 0; d < kDig; ++d) tc::tmem_ld8(acc + d * width + c0, a[d]);
+            for (int d = 0; d < kDig; ++d) tc::tmem_ld8(tacc + d * width + c0, a[d]);
             tc::tmem_wait_ld();
 #pragma unroll
             for (int d = 0; d < kDig; ++d) tc::pin8(a[d]);
@@ -396,27 +451,17 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
 #pragma unroll
                 for (int d = 0; d < kDig; ++d) t[d] = a[d][i];
                 const ff::f2 own = combine(t);
-                ff::f2 other;
-                other.hi = __shfl_xor_sync(0xffffffffu, own.hi, 16);
-                other.lo = __shfl_xor_sync(0xffffffffu, own.lo, 16);
-                y[i] = butterfly(other, own, sgn, sc);
+                if (jb.direct_out) {
+                    y[i] = scaled(own, sc);
+                } else {
+                    ff::f2 other;
+                    other.hi = __shfl_xor_sync(0xffffffffu, own.hi, 16);
+                    other.lo = __shfl_xor_sync(0xffffffffu, own.lo, 16);
+                    y[i] = butterfly(other, own, sgn, sc);
+                }
             }
             const int j = j0 + c0;
-            float2 *p = dst + j * rstride;
-            if (w_ok && j + 8 <= h) {
-                if (wide) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        reinterpret_cast<float4 *>(p)[i] = make_float4(y[2 * i].x, y[2 * i].y, y[2 * i + 1].x, y[2 * i + 1].y);
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) p[i * rstride] = y[i];
-                }
-            } else if (w_ok) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    if (j + i < h) p[i * rstride] = y[i];
-            }
+            store_lines(y, dst + j * rstride, rstride, h - j, wide, w_ok);
         }
     }
     tc::fence_before_sync();
@@ -437,51 +482,98 @@ size_t tline_matrix_bytes(int n)
     return 2 * (size_t)s.chunks * s.unit;
 }
 
-// De and Do times scale as seven f16 digits each, laid out as the kernel's
-// shared-memory image ([column chunk][e, o][K chunk][digit][output][8]);
-// returns the binary exponent of the integers (entry = integer 2^-mexp).
-int tline_derivative_matrix(int n, double scale, uint16_t *img)
+namespace {
+
+// The matrix blocks e and o (h x h each; at(half, output, input) indexes a
+// table of the distinct entries) times 2^mexp as seven f16 digits each, laid
+// out as the kernel's shared-memory image ([column chunk][e, o][K chunk]
+// [digit][output][8]); returns mexp.
+template <typename F> int pack_matrix(int n, const std::vector<long double> &entry, F at, uint16_t *img)
 {
     const TlShape s = tl_shape(n);
     const int h = s.h;
-    std::vector<long double> D(n, 0.0L);   // D(m) = (scale/2) (-1)^m cot(pi m/n), period n
-    for (int m = 1; m < n; ++m) {
-        const long double x = 3.14159265358979323846264338327950288L * (long double)m / (long double)n;
-        D[m] = (long double)scale * 0.5L * ((m & 1) ? -1.0L : 1.0L) * (2 * m == n ? 0.0L : cosl(x) / sinl(x));
-    }
-    long double big = 0.0L;
-    std::vector<long double> c(2 * (size_t)n);     // De(m), Do(m) for m = j - l + h
-    for (int half = 0; half < 2; ++half)
-        for (int m = -h + 1; m < h; ++m) {
-            const long double a = D[(m + n) % n], b = D[(m - h + 2 * n) % n];
-            const long double v = 0.5L * (half ? a - b : a + b);
-            c[(size_t)half * n + m + h] = v;
-            big = std::max(big, fabsl(v));
+    static const std::vector<uint16_t> digit = [] {   // f16 of -128 .. 127
+        std::vector<uint16_t> d(256);
+        for (int b = 0; b < 256; ++b) {
+            int a = b < 128 ? 128 - b : b - 128, ex = 0;
+            while ((a >> ex) > 1) ++ex;
+            d[b] = a == 0 ? 0 : (uint16_t)((b < 128 ? 0x8000 : 0) | ((ex + 15) << 10) | ((a << (10 - ex)) & 0x3ff));
         }
+        return d;
+    }();
+    long double big = 0.0L;
+    for (long double x : entry) big = std::max(big, fabsl(x));
     int e = 0;
     frexpl(big, &e);                               // big in [2^(e-1), 2^e)
     const int mexp = 54 - e;                       // integers up to 2^54
+    std::vector<uint64_t> fixed(entry.size());
+    for (size_t i = 0; i < entry.size(); ++i) fixed[i] = (uint64_t)llroundl(ldexpl(entry[i], mexp)) + kDigBias;
     std::fill(img, img + tline_matrix_bytes(n) / 2, (uint16_t)0);
     for (int half = 0; half < 2; ++half)
         for (int j = 0; j < h; ++j) {
             const int ch = j / (8 * s.g), width = tl_width(s, ch), jj = j - ch * 8 * s.g;
             uint16_t *base = img + (size_t)(2 * ch + half) * s.unit / 2;
             for (int l = 0; l < h; ++l) {
-                const long long v = llroundl(ldexpl(c[(size_t)half * n + (j - l) + h], mexp));
-                const uint64_t b = (uint64_t)v + kDigBias;
-                for (int d = 0; d < kDig; ++d) {
-                    const int dig = (int)((b >> (8 * (6 - d))) & 0xff) - 128;
-                    uint16_t f = 0;                // f16 of a small integer: exact
-                    if (dig != 0) {
-                        int a = dig < 0 ? -dig : dig, ex = 0;
-                        while ((a >> ex) > 1) ++ex;
-                        f = (uint16_t)((dig < 0 ? 0x8000 : 0) | ((ex + 15) << 10) | ((a << (10 - ex)) & 0x3ff));
-                    }
-                    base[((size_t)(l / 8) * kDig * width + (size_t)d * width + jj) * 8 + l % 8] = f;
-                }
+                const uint64_t b = fixed[at(half, j, l)];
+                uint16_t *p = base + ((size_t)(l / 8) * kDig * width + jj) * 8 + l % 8;
+                for (int d = 0; d < kDig; ++d) p[(size_t)d * width * 8] = digit[(b >> (8 * (6 - d))) & 0xff];
             }
         }
     return mexp;
+}
+
+const long double kTwoPiL = 6.283185307179586476925286766559005768L;
+
+}  // namespace
+
+// D(m) = (scale/2) (-1)^m cot(pi m/n), period n.
+int tline_derivative_matrix(int n, double scale, uint16_t *img)
+{
+    const int h = n / 2;
+    std::vector<long double> D(n, 0.0L), t(2 * (size_t)n);
+    for (int m = 1; m < n; ++m) {
+        const long double x = 0.5L * kTwoPiL * m / n;
+        D[m] = (long double)scale * 0.5L * ((m & 1) ? -1.0L : 1.0L) * (2 * m == n ? 0.0L : cosl(x) / sinl(x));
+    }
+    for (int m = 0; m < n; ++m) {                  // De, Do by m = j - l (mod n)
+        const long double a = D[m], b = D[(m + n - h) % n];
+        t[m] = 0.5L * (a + b);
+        t[n + m] = 0.5L * (a - b);
+    }
+    return pack_matrix(n, t, [&](int half, int j, int l) { return (size_t)half * n + (j - l + n) % n; }, img);
+}
+
+// Coefficients 0 .. n/2 - 1: even frequencies 0, 2 (cosine, sine), 4, ...;
+// the others: odd ones; the Nyquist frequency has a cosine only.
+int tline_frequency(int n, int a, bool *sine)
+{
+    const int h = n / 2;
+    const bool odd = a >= h;
+    const int i = odd ? a - h : a;
+    *sine = odd ? (i & 1) != 0 : (i > 0 && (i & 1) == 0);
+    return odd ? 2 * (i / 2) + 1 : 2 * ((i + 1) / 2);
+}
+
+int tline_fourier_matrix(int n, bool inverse, uint16_t *img)
+{
+    const int h = n / 2;
+    const long double edge = 1.0L / sqrtl((long double)n), mid = sqrtl(2.0L / (long double)n);
+    std::vector<long double> t(3 * (size_t)n);     // cosines, sines, cosines of the end frequencies
+    for (int m = 0; m < n; ++m) {
+        t[m] = mid * cosl(kTwoPiL * m / n);
+        t[n + m] = mid * sinl(kTwoPiL * m / n);
+        t[2 * n + m] = edge * cosl(kTwoPiL * m / n);
+    }
+    std::vector<int> k(n), type(n);
+    for (int a = 0; a < n; ++a) {
+        bool sine;
+        k[a] = tline_frequency(n, a, &sine);
+        type[a] = sine ? 1 : (k[a] == 0 || 2 * k[a] == n ? 2 : 0);
+    }
+    return pack_matrix(n, t, [&](int half, int out, int in) {
+        const int a = (inverse ? in : out) + half * h, j = inverse ? out : in;
+        return (size_t)type[a] * n + (size_t)(k[a] * j) % n;
+    }, img);
 }
 
 cudaError_t tline_smem_limits()
@@ -489,34 +581,46 @@ cudaError_t tline_smem_limits()
     return cudaFuncSetAttribute(k_tline, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTlSmemMax);
 }
 
-void launch_tline(const GridInfo &g, const FftAxis *const ax[3], const double *const in[3], float2 *const out[3],
-                  cudaStream_t st)
+namespace {
+
+TlJob make_job(const GridInfo &g, int axis, const TlMat &m, const float2 *in, float2 *out, int direct_in, int direct_out)
+{
+    const long long plane = (long long)g.ny * g.nz;
+    const int n = axis == 0 ? g.nx : (axis == 1 ? g.ny : g.nz);
+    TlJob j{};
+    j.sh = tl_shape(n);
+    j.nlines = (int)(g.N / n);
+    j.tiles = (j.nlines + kLines - 1) / kLines;
+    j.zaxis = axis == 2;
+    j.zlen = axis == 0 ? (int)plane : (axis == 1 ? g.nz : 1);
+    j.ostride = axis == 2 ? g.nz : plane;                // (x: one outer index)
+    j.rstride = axis == 0 ? plane : (axis == 1 ? g.nz : 1);
+    j.direct_in = direct_in;
+    j.direct_out = direct_out;
+    j.mexp = m.mexp;
+    j.mat = (const unsigned char *)m.img;
+    j.in = in;
+    j.out = out;
+    return j;
+}
+
+}  // namespace
+
+void launch_tline(const GridInfo &g, int count, const TlPass *pass, cudaStream_t st)
 {
     TlJobs jobs{};
     int blocks = 0, items = 0;
     uint32_t smem = 0;
-    const long long plane = (long long)g.ny * g.nz;
-    const int n3[3] = {g.nx, g.ny, g.nz};
-    for (int a = 0; a < 3; ++a) {
-        if (!ax[a]) continue;
+    for (int i = 0; i < count; ++i) {
+        const TlPass &p = pass[i];
         TlJob &j = jobs.job[jobs.count++];
-        j.sh = tl_shape(n3[a]);
-        j.nlines = (int)(g.N / n3[a]);
-        j.tiles = (j.nlines + kLines - 1) / kLines;
-        j.zaxis = a == 2;
-        j.zlen = a == 0 ? (int)plane : (a == 1 ? g.nz : 1);
-        j.ostride = a == 2 ? g.nz : plane;               // (x: one outer index)
-        j.rstride = a == 0 ? plane : (a == 1 ? g.nz : 1);
-        j.mexp = ax[a]->dexp;
-        j.mat = (const unsigned char *)ax[a]->dmat;
-        j.in = in[a];
-        j.out = out[a];
+        j = make_job(g, p.axis, *p.mat, p.in, p.out, p.kind == TlPass::kInverse, p.kind == TlPass::kForward);
         blocks += j.tiles;
         items = std::max(items, kLines * j.sh.nc);
         smem = std::max(smem, j.sh.smem);
     }
-    const int threads = items;
-    k_tline<<<blocks, threads + 32, smem, st>>>(jobs);
+    if (blocks == 0) return;
+    k_tline<<<blocks, items + 32, smem, st>>>(jobs);
 }
 
 }  // namespace ofdft

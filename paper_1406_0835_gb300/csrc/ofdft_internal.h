@@ -53,8 +53,6 @@ struct FftAxis {
     const void *tw;          // cplx<T>[n]
     const void *twf;         // FP64 sets: the same twiddles as double-float pairs (ff::cf2[n])
     int mp;                  // the largest power-of-two radix of the schedule (4 or 8)
-    const void *dmat;        // double-float sets: digits of the derivative matrix (kernels_tline.cu), or null
-    int dexp;                // its binary exponent
 };
 
 // Stockham schedule of one axis: radix-8 stages first, then 4, 2, 3, 5;

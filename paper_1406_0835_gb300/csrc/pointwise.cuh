@@ -344,11 +344,17 @@ OF_HD void tfunc_eval_f2(const ff::f2 *__restrict__ tab, ff::f2 t, ff::f2 out[8]
     const float4 *tail = c + kTfSplit * 2;
     HornerF2 h[NF];
     const float4 top = tail[kTfDdDeg - kTfSplit];
-    h[0] = {{top.x, 0.0f}, {0.0f, 0.0f}, 0.0f};
-    h[1] = {{top.y, 0.0f}, {0.0f, 0.0f}, 0.0f};
+    h[0].p.hi = top.x;
+    h[1].p.hi = top.y;
     if (NF == 4) {
-        h[2] = {{top.z, 0.0f}, {0.0f, 0.0f}, 0.0f};
-        h[3] = {{top.w, 0.0f}, {0.0f, 0.0f}, 0.0f};
+        h[2].p.hi = top.z;
+        h[3].p.hi = top.w;
+    }
+#pragma unroll
+    for (int q = 0; q < NF; ++q) {
+        h[q].p.lo = 0.0f;
+        h[q].dp = ff::f2(0.0f, 0.0f);
+        h[q].d2 = 0.0f;
     }
 #pragma unroll 1
     for (int j = kTfDdDeg - kTfSplit - 1; j >= 0; --j) {

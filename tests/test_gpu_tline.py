@@ -1,4 +1,5 @@
-"""GPU parity of the tensor-core derivative passes (kernels_tline.cu) at the
+"""GPU parity of the tensor-core transforms (kernels_tline.cu: derivatives,
+and the Hartree chain in the real Fourier basis) at the
 sizes where their tiling can go wrong: the smallest edges, odd half lengths,
 edges whose halves are no multiple of the padding, one, two and three column
 chunks, the largest edge they take (144) and the first beyond it (150, which
@@ -44,6 +45,28 @@ def check(grid, cell=None, functional="vt84f"):
                                   (150, 16, 12), (12, 10, 150), (20, 36, 90), (96, 40, 8)])
 def test_evaluation_at_the_edges_of_the_tiling(grid):
     check(grid)
+
+
+@pytest.mark.parametrize("grid", [(60, 54, 50), (144, 36, 40)])
+def test_fttf_grids_large_enough_for_the_real_basis(grid):
+    check(grid, functional="fttf")
+
+
+def test_heine_abarenkov_weights_in_the_real_basis():
+    """Pressure weights and v_ext of Eq. (E4A), odd half lengths on two axes."""
+    cfg = inputs.config_single_point()
+    grid = (18, 20, 30)
+    so = O.System(cfg["L"], grid, cfg["ions"], cfg["Z"], cfg["T"], "sga", lpp="ha")
+    rng = np.random.default_rng(3)
+    phi = so.uniform_phi() * (1.0 + 0.1 * rng.standard_normal(grid))
+    ev = O.evaluate(so, phi)
+    with ofdft.Context(cfg["L"], grid, cfg["ions"], cfg["Z"], cfg["T"], "sga", lpp="ha") as ctx:
+        E, v = ctx.energy_potential(phi)
+    for k in ("F_tot", "E_H", "E_loc"):
+        assert abs(E[k] - ev[k]) <= 1e-10 * abs(ev["F_tot"]), k
+    for k in ("P", "P_H", "P_loc"):
+        assert abs(E[k] - ev[k]) <= 1e-9 * abs(ev["P"]), k
+    assert np.max(np.abs(v - ev["v"])) <= 1e-9 * np.max(np.abs(ev["v"]))
 
 
 def test_sheared_cell():
