@@ -13,6 +13,7 @@
 #include <math.h>
 
 #include "kernels.h"
+#include "pdl.cuh"
 
 namespace ofdft {
 
@@ -31,6 +32,7 @@ __device__ __forceinline__ double e_elec(const CgState *s, const double *ev)
 
 __global__ void k_ctl_norm(CgState *s)
 {
+    pdl_enter();
     double ss = s->rn[0] * s->dV;
     if (!(ss > 0.0) || !isfinite(ss)) {
         s->scale = 1.0;
@@ -43,6 +45,7 @@ __global__ void k_ctl_norm(CgState *s)
 
 __global__ void k_ctl_init(CgState *s)
 {
+    pdl_enter();
     s->mu = s->ev[15] / s->ev[16];
     for (int k = 0; k < 18; ++k) s->ev_acc[k] = s->ev[k];
     s->nevals = 1;
@@ -63,6 +66,7 @@ __global__ void k_ctl_init(CgState *s)
 
 __global__ void k_ctl_grad(CgState *s, int first, cudaGraphConditionalHandle outer, int use)
 {
+    pdl_enter();
     if (first) {
         s->gg = s->rg[0];
         s->have_prev = 0;
@@ -104,6 +108,7 @@ __global__ void k_ctl_grad(CgState *s, int first, cudaGraphConditionalHandle out
 
 __global__ void k_ctl_dir(CgState *s)
 {
+    pdl_enter();
     const double sphd = s->rd[0], sdd = s->rd[1], sdg = s->rd[2], spp = s->rd[3], spg = s->rd[4];
     double c1 = sphd / spp;
     double dg = sdg - c1 * spg;
@@ -120,6 +125,7 @@ __global__ void k_ctl_dir(CgState *s)
 
 __global__ void k_ctl_dhat(CgState *s, cudaGraphConditionalHandle ls, int use)
 {
+    pdl_enter();
     s->D0 = s->dV * s->rh[0];
     s->lo = 0.0;
     s->Dlo = s->D0;
@@ -143,6 +149,7 @@ __global__ void k_ctl_dhat(CgState *s, cudaGraphConditionalHandle ls, int use)
 
 __global__ void k_ctl_ls(CgState *s, cudaGraphConditionalHandle ls, int use)
 {
+    pdl_enter();
     s->nls += 1;
     s->nevals += 1;
     const double D = s->dV * s->ev[17];
@@ -224,20 +231,20 @@ __global__ void k_ctl_ls(CgState *s, cudaGraphConditionalHandle ls, int use)
 
 }  // namespace
 
-void launch_ctl_norm(CgState *s, cudaStream_t st) { k_ctl_norm<<<1, 1, 0, st>>>(s); }
-void launch_ctl_init(CgState *s, cudaStream_t st) { k_ctl_init<<<1, 1, 0, st>>>(s); }
+void launch_ctl_norm(CgState *s, cudaStream_t st) { pdl_launch(k_ctl_norm, 1, 1, 0, st, s); }
+void launch_ctl_init(CgState *s, cudaStream_t st) { pdl_launch(k_ctl_init, 1, 1, 0, st, s); }
 void launch_ctl_grad(CgState *s, int first, cudaGraphConditionalHandle outer, int use_cond, cudaStream_t st)
 {
-    k_ctl_grad<<<1, 1, 0, st>>>(s, first, outer, use_cond);
+    pdl_launch(k_ctl_grad, 1, 1, 0, st, s, first, outer, use_cond);
 }
-void launch_ctl_dir(CgState *s, cudaStream_t st) { k_ctl_dir<<<1, 1, 0, st>>>(s); }
+void launch_ctl_dir(CgState *s, cudaStream_t st) { pdl_launch(k_ctl_dir, 1, 1, 0, st, s); }
 void launch_ctl_dhat(CgState *s, cudaGraphConditionalHandle ls, int use_cond, cudaStream_t st)
 {
-    k_ctl_dhat<<<1, 1, 0, st>>>(s, ls, use_cond);
+    pdl_launch(k_ctl_dhat, 1, 1, 0, st, s, ls, use_cond);
 }
 void launch_ctl_ls(CgState *s, cudaGraphConditionalHandle ls, int use_cond, cudaStream_t st)
 {
-    k_ctl_ls<<<1, 1, 0, st>>>(s, ls, use_cond);
+    pdl_launch(k_ctl_ls, 1, 1, 0, st, s, ls, use_cond);
 }
 
 }  // namespace ofdft

@@ -18,6 +18,7 @@
 
 #include "fft_core.cuh"
 #include "kernels.h"
+#include "pdl.cuh"
 #include "pointwise.cuh"
 
 namespace ofdft {
@@ -289,6 +290,7 @@ __global__ void OFDFT_FFT_BOUNDS k_zfwd(GridInfo g, FftAxis az, int P, const typ
                        typename KT<PR>::T *__restrict__ phit, typename KT<PR>::C *__restrict__ out,
                        typename KT<PR>::T *__restrict__ dzout, typename KT<PR>::T *__restrict__ nout)
 {
+    pdl_enter();
     typedef typename KT<PR>::T T;
     typedef typename KT<PR>::R R;
     typedef typename KT<PR>::CC CC;
@@ -405,6 +407,7 @@ __global__ void k_zfinal(GridInfo g, FftAxis az, int P, const typename KT<PR>::C
                          typename KT<PR>::T temp, FuncParams fp, const typename KT<PR>::T *__restrict__ tab, int xc,
                          typename KT<PR>::T *__restrict__ vout, double *__restrict__ part)
 {
+    pdl_enter();
     typedef typename KT<PR>::T T;
     typedef typename KT<PR>::R R;
     typedef typename KT<PR>::CC CC;
@@ -540,6 +543,7 @@ __device__ __forceinline__ void store_tile(typename KT<PR>::C *__restrict__ dst,
 template <typename PR, bool INV>
 __global__ void OFDFT_FFT_BOUNDS k_ypass(GridInfo g, FftAxis ay, typename KT<PR>::C *__restrict__ data, long long fstride)
 {
+    pdl_enter();
     typedef typename KT<PR>::C C;
     typedef typename KT<PR>::CC CC;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -580,6 +584,7 @@ __global__ void OFDFT_FFT_BOUNDS k_xhl(GridInfo g, FftAxis ax, typename KT<PR>::
                       const typename KT<PR>::C *__restrict__ vext, typename KT<PR>::C *__restrict__ nG_out,
                       int inverse, double *__restrict__ part)
 {
+    pdl_enter();
     typedef typename KT<PR>::R R;
     typedef typename KT<PR>::CC CC;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -701,6 +706,7 @@ template <typename PR, int AX, int MODE, int ACC>
 __global__ void OFDFT_FFT_BOUNDS k_dline(GridInfo g, FftAxis fa, const typename KT<PR>::T *in,
                         typename KT<PR>::T *out)
 {
+    pdl_enter();
     typedef typename KT<PR>::T T;
     typedef typename KT<PR>::R R;
     typedef typename KT<PR>::CC CC;
@@ -759,6 +765,7 @@ template <typename PR, int AX, int MODE, int ACC>
 __global__ void OFDFT_FFT_BOUNDS k_dline_ws(GridInfo g, FftAxis fa, const typename KT<PR>::T *in,
                                             typename KT<PR>::T *out)
 {
+    pdl_enter();
     typedef typename KT<PR>::T T;
     typedef typename KT<PR>::R R;
     typedef typename KT<PR>::CC CC;
@@ -846,6 +853,7 @@ __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB) k_pw(GridInfo
                      typename KT<PR>::T temp, FuncParams fp, const typename KT<PR>::T *__restrict__ tab, int xc,
                      typename KT<PR>::T *__restrict__ vpart, double *__restrict__ part)
 {
+    pdl_enter();
     typedef typename KT<PR>::T T;
     typedef typename KT<PR>::R R;
     typedef typename AccK<PR>::type AC;
@@ -943,6 +951,7 @@ __global__ void OFDFT_FFT_BOUNDS k_zfinal_g(GridInfo g, FftAxis az, int P, const
                            typename KT<PR>::T c, typename KT<PR>::T s, const void *__restrict__ cs,
                            typename KT<PR>::T *vout, double *__restrict__ part)
 {
+    pdl_enter();
     typedef typename KT<PR>::T T;
     typedef typename KT<PR>::R R;
     typedef typename KT<PR>::CC CC;
@@ -1057,9 +1066,9 @@ void launch_zfwd(const GridInfo &g, const FftAxis &az, int mode, const T *in, co
     size_t sm = 2 * (size_t)P * g.nz * sizeof(cplx<T>);
     int th = g.zth > 0 ? g.zth : threads_for(P * g.nz);
 #define CALL(PR)                                                                                              \
-    if (mode == 0) k_zfwd<PR, 0><<<blocks, th, sm, st>>>(g, az, P, in, phi, dhat, c, s, cs, phit, out, dz, nout);     \
-    else if (mode == 1) k_zfwd<PR, 1><<<blocks, th, sm, st>>>(g, az, P, in, phi, dhat, c, s, cs, phit, out, dz, nout); \
-    else k_zfwd<PR, 2><<<blocks, th, sm, st>>>(g, az, P, in, phi, dhat, c, s, cs, phit, out, dz, nout)
+    if (mode == 0) pdl_launch(k_zfwd<PR, 0>, blocks, th, sm, st, g, az, P, in, phi, dhat, c, s, cs, phit, out, dz, nout);     \
+    else if (mode == 1) pdl_launch(k_zfwd<PR, 1>, blocks, th, sm, st, g, az, P, in, phi, dhat, c, s, cs, phit, out, dz, nout); \
+    else pdl_launch(k_zfwd<PR, 2>, blocks, th, sm, st, g, az, P, in, phi, dhat, c, s, cs, phit, out, dz, nout)
     OFDFT_DISPATCH(T, g, CALL);
 #undef CALL
 }
@@ -1071,24 +1080,24 @@ void dline_call(const GridInfo &g, const FftAxis &fa, int axis, int mode, int ac
 {
     if (g.dws && th % 32 == 0 && g.dk % (th / 32) == 0) {   // whole lines for every warp
         if (axis == 0) {
-            if (mode == 0) k_dline_ws<PR, 0, 0, 0><<<blocks, th, sm, st>>>(g, fa, in, out);
-            else if (acc == 0) k_dline_ws<PR, 0, 1, 0><<<blocks, th, sm, st>>>(g, fa, in, out);
-            else k_dline_ws<PR, 0, 1, 1><<<blocks, th, sm, st>>>(g, fa, in, out);
+            if (mode == 0) pdl_launch(k_dline_ws<PR, 0, 0, 0>, blocks, th, sm, st, g, fa, in, out);
+            else if (acc == 0) pdl_launch(k_dline_ws<PR, 0, 1, 0>, blocks, th, sm, st, g, fa, in, out);
+            else pdl_launch(k_dline_ws<PR, 0, 1, 1>, blocks, th, sm, st, g, fa, in, out);
         } else {
-            if (mode == 0) k_dline_ws<PR, 1, 0, 0><<<blocks, th, sm, st>>>(g, fa, in, out);
-            else if (acc == 0) k_dline_ws<PR, 1, 1, 0><<<blocks, th, sm, st>>>(g, fa, in, out);
-            else k_dline_ws<PR, 1, 1, 1><<<blocks, th, sm, st>>>(g, fa, in, out);
+            if (mode == 0) pdl_launch(k_dline_ws<PR, 1, 0, 0>, blocks, th, sm, st, g, fa, in, out);
+            else if (acc == 0) pdl_launch(k_dline_ws<PR, 1, 1, 0>, blocks, th, sm, st, g, fa, in, out);
+            else pdl_launch(k_dline_ws<PR, 1, 1, 1>, blocks, th, sm, st, g, fa, in, out);
         }
         return;
     }
     if (axis == 0) {
-        if (mode == 0) k_dline<PR, 0, 0, 0><<<blocks, th, sm, st>>>(g, fa, in, out);
-        else if (acc == 0) k_dline<PR, 0, 1, 0><<<blocks, th, sm, st>>>(g, fa, in, out);
-        else k_dline<PR, 0, 1, 1><<<blocks, th, sm, st>>>(g, fa, in, out);
+        if (mode == 0) pdl_launch(k_dline<PR, 0, 0, 0>, blocks, th, sm, st, g, fa, in, out);
+        else if (acc == 0) pdl_launch(k_dline<PR, 0, 1, 0>, blocks, th, sm, st, g, fa, in, out);
+        else pdl_launch(k_dline<PR, 0, 1, 1>, blocks, th, sm, st, g, fa, in, out);
     } else {
-        if (mode == 0) k_dline<PR, 1, 0, 0><<<blocks, th, sm, st>>>(g, fa, in, out);
-        else if (acc == 0) k_dline<PR, 1, 1, 0><<<blocks, th, sm, st>>>(g, fa, in, out);
-        else k_dline<PR, 1, 1, 1><<<blocks, th, sm, st>>>(g, fa, in, out);
+        if (mode == 0) pdl_launch(k_dline<PR, 1, 0, 0>, blocks, th, sm, st, g, fa, in, out);
+        else if (acc == 0) pdl_launch(k_dline<PR, 1, 1, 0>, blocks, th, sm, st, g, fa, in, out);
+        else pdl_launch(k_dline<PR, 1, 1, 1>, blocks, th, sm, st, g, fa, in, out);
     }
 }
 }  // namespace
@@ -1110,6 +1119,7 @@ void launch_dline(const GridInfo &g, const FftAxis &fa, int axis, int mode, int 
 __global__ void k_density(long long pairs, const double2 *__restrict__ phi, const double2 *__restrict__ dhat, double c, double s,
                           const double *__restrict__ cs, double2 *__restrict__ phit, float4 *__restrict__ dens)
 {
+    pdl_enter();
     if (cs != nullptr) {
         c = cs[0];
         s = cs[1];
@@ -1137,6 +1147,7 @@ __device__ __forceinline__ ff::f2 f2of(float2 x) { return ff::f2(x.x, x.y); }
 // blocks (one to an SM) the same loop waited on memory latency.
 __global__ void __launch_bounds__(256) k_hartree(GridInfo g, float4 *__restrict__ coef, TlHartree hl)
 {
+    pdl_enter();
     constexpr ff::f2 fpi(kFourPi);
     const ff::f2 hr = f2of(hl.hr), z0(0.0f, 0.0f);
     ff::f2 acc[3] = {z0, z0, z0};
@@ -1179,6 +1190,7 @@ __global__ void __launch_bounds__(256) k_hartree(GridInfo g, float4 *__restrict_
 // of phi^2 v, phi^2 and 2 phi v dphi/dtheta (partials as k_zfinal_g's).
 __global__ void __launch_bounds__(256) k_final(GridInfo g, TlFinal f)
 {
+    pdl_enter();
     double c = f.c, s = f.s;
     if (f.cs != nullptr) {
         c = f.cs[0];
@@ -1226,6 +1238,7 @@ __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB)
           const double *__restrict__ dhat, double c, double s, const double *__restrict__ cs, double temp, FuncParams fp,
           const double *__restrict__ tab, int xc, double *__restrict__ vout, double *__restrict__ part)
 {
+    pdl_enter();
     if (cs != nullptr) {
         c = cs[0];
         s = cs[1];
@@ -1288,13 +1301,13 @@ int launch_pw(const GridInfo &g, T *d0, T *d1, T *d2, const T *phit, T temp, con
 #define CALL(PR)                                                                                              \
     if (stress) {                                                                                             \
         if constexpr (!std::is_same<PR, float>::value) {                                                      \
-            if (g.tri) k_pw<PR, true, true><<<blocks, th, 0, st>>>(g, d0, d1, d2, phit, temp, fp, tab, xc, vpart, part); \
-            else k_pw<PR, true, false><<<blocks, th, 0, st>>>(g, d0, d1, d2, phit, temp, fp, tab, xc, vpart, part);     \
+            if (g.tri) pdl_launch(k_pw<PR, true, true>, blocks, th, 0, st, g, d0, d1, d2, phit, temp, fp, tab, xc, vpart, part); \
+            else pdl_launch(k_pw<PR, true, false>, blocks, th, 0, st, g, d0, d1, d2, phit, temp, fp, tab, xc, vpart, part);     \
         }                                                                                                     \
     } else if (g.tri) {                                                                                       \
-        k_pw<PR, false, true><<<blocks, th, 0, st>>>(g, d0, d1, d2, phit, temp, fp, tab, xc, vpart, part);    \
+        pdl_launch(k_pw<PR, false, true>, blocks, th, 0, st, g, d0, d1, d2, phit, temp, fp, tab, xc, vpart, part);    \
     } else {                                                                                                  \
-        k_pw<PR, false, false><<<blocks, th, 0, st>>>(g, d0, d1, d2, phit, temp, fp, tab, xc, vpart, part);   \
+        pdl_launch(k_pw<PR, false, false>, blocks, th, 0, st, g, d0, d1, d2, phit, temp, fp, tab, xc, vpart, part);   \
     }
     OFDFT_DISPATCH(T, g, CALL);
 #undef CALL
@@ -1306,7 +1319,7 @@ void launch_density(long long n, const double *phi, const double *dhat, double c
 {
     const long long pairs = n / 2;
     const int blocks = (int)std::min<long long>((pairs + 255) / 256, 1216);
-    k_density<<<blocks, 256, 0, st>>>(pairs, (const double2 *)phi, (const double2 *)dhat, c, s, cs, (double2 *)phit,
+    pdl_launch(k_density, blocks, 256, 0, st, pairs, (const double2 *)phi, (const double2 *)dhat, c, s, cs, (double2 *)phit,
                                       (float4 *)dens);
 }
 
@@ -1322,14 +1335,14 @@ int launch_hartree(const GridInfo &g, float2 *coef, const TlHartree &hl, cudaStr
 {
     // partial rows of at most one column per four half-spectrum columns of the yz plane
     const int blocks = std::min(pair_blocks(g), g.ny * ((g.K + 3) / 4));
-    k_hartree<<<blocks, 256, 0, st>>>(g, (float4 *)coef, hl);
+    pdl_launch(k_hartree, blocks, 256, 0, st, g, (float4 *)coef, hl);
     return blocks;
 }
 
 int launch_final(const GridInfo &g, const TlFinal &fin, cudaStream_t st)
 {
     const int blocks = pair_blocks(g);
-    k_final<<<blocks, 256, 0, st>>>(g, fin);
+    pdl_launch(k_final, blocks, 256, 0, st, g, fin);
     return blocks;
 }
 
@@ -1338,7 +1351,7 @@ int launch_ptf(const GridInfo &g, const float2 *vhl, const double *phit, const d
                double *part, cudaStream_t st)
 {
     const int th = OFDFT_PW_THREADS, blocks = pw_blocks(g, th);
-    k_ptf<<<blocks, th, 0, st>>>(g, vhl, phit, phi, dhat, c, s, cs, temp, fp, tab, xc, vout, part);
+    pdl_launch(k_ptf, blocks, th, 0, st, g, vhl, phit, phi, dhat, c, s, cs, temp, fp, tab, xc, vout, part);
     return blocks;
 }
 
@@ -1355,10 +1368,10 @@ int launch_zfinal(const GridInfo &g, const FftAxis &az, bool fttf, const cplx<T>
     int th = g.zth > 0 ? g.zth : threads_for(P * g.nz);
 #define CALL(PR)                                                                                       \
     if (fttf)                                                                                          \
-        k_zfinal<PR, true><<<blocks, th, sm, st>>>(g, az, P, dspec, vpart, phit, phi, dhat, c, s, cs,  \
+        pdl_launch(k_zfinal<PR, true>, blocks, th, sm, st, g, az, P, dspec, vpart, phit, phi, dhat, c, s, cs,  \
                                                    temp, fp, tab, xc, vout, part);                     \
     else                                                                                               \
-        k_zfinal<PR, false><<<blocks, th, sm, st>>>(g, az, P, dspec, vpart, phit, phi, dhat, c, s, cs, \
+        pdl_launch(k_zfinal<PR, false>, blocks, th, sm, st, g, az, P, dspec, vpart, phit, phi, dhat, c, s, cs, \
                                                     temp, fp, tab, xc, vout, part)
     OFDFT_DISPATCH(T, g, CALL);
 #undef CALL
@@ -1376,7 +1389,7 @@ int launch_zfinal_gga(const GridInfo &g, const FftAxis &az, const cplx<T> *dspec
     size_t sm = (uz ? 3 : 2) * (size_t)P * g.nz * sizeof(cplx<T>);
     int th = g.zth > 0 ? g.zth : threads_for(P * g.nz);
 #define CALL(PR) \
-    k_zfinal_g<PR><<<blocks, th, sm, st>>>(g, az, P, dspec, uz, vpart, div, div2, div3, phit, phi, dhat, c, s, cs, vout, \
+    pdl_launch(k_zfinal_g<PR>, blocks, th, sm, st, g, az, P, dspec, uz, vpart, div, div2, div3, phit, phi, dhat, c, s, cs, vout, \
                                            part)
     OFDFT_DISPATCH(T, g, CALL);
 #undef CALL
@@ -1391,8 +1404,8 @@ void launch_ypass(const GridInfo &g, const FftAxis &ay, bool inv, cplx<T> *data,
     size_t sm = 2 * (size_t)g.ny * g.tk * sizeof(cplx<T>);
     int th = g.xth > 0 ? g.xth : threads_for(g.ny * g.tk / 2);
 #define CALL(PR)                                                            \
-    if (inv) k_ypass<PR, true><<<grid, th, sm, st>>>(g, ay, data, fstride); \
-    else k_ypass<PR, false><<<grid, th, sm, st>>>(g, ay, data, fstride)
+    if (inv) pdl_launch(k_ypass<PR, true>, grid, th, sm, st, g, ay, data, fstride); \
+    else pdl_launch(k_ypass<PR, false>, grid, th, sm, st, g, ay, data, fstride)
     OFDFT_DISPATCH(T, g, CALL);
 #undef CALL
 }
@@ -1405,8 +1418,8 @@ int launch_xhl(const GridInfo &g, const FftAxis &ax, cplx<T> *spec, const cplx<T
     size_t sm = 2 * (size_t)g.nx * g.tk * sizeof(cplx<T>);
     int th = g.xth > 0 ? g.xth : threads_for(g.nx * g.tk / 2);
 #define CALL(PR)                                                                             \
-    if (g.tri) k_xhl<PR, true><<<blocks, th, sm, st>>>(g, ax, spec, vext, nG_out, inverse, part); \
-    else k_xhl<PR, false><<<blocks, th, sm, st>>>(g, ax, spec, vext, nG_out, inverse, part)
+    if (g.tri) pdl_launch(k_xhl<PR, true>, blocks, th, sm, st, g, ax, spec, vext, nG_out, inverse, part); \
+    else pdl_launch(k_xhl<PR, false>, blocks, th, sm, st, g, ax, spec, vext, nG_out, inverse, part)
     OFDFT_DISPATCH(T, g, CALL);
 #undef CALL
     return blocks;

@@ -7,6 +7,7 @@
 
 #include "fft_core.cuh"
 #include "kernels.h"
+#include "pdl.cuh"
 
 namespace ofdft {
 
@@ -54,6 +55,7 @@ template <int NQ> __device__ __forceinline__ void block_sum_split(AccF *v, doubl
 
 __global__ void k_reduce(const double *__restrict__ part, int nblk, double *__restrict__ out)
 {
+    pdl_enter();
     double v[1] = {0.0};
     const double *p = part + (size_t)blockIdx.x * nblk;
     for (int i = threadIdx.x; i < nblk; i += blockDim.x) v[0] += p[i];
@@ -68,6 +70,7 @@ __global__ void k_reduce(const double *__restrict__ part, int nblk, double *__re
 __global__ void k_reduce_eval(const double *__restrict__ pA, int na, const double *__restrict__ pB, int nb,
                               const double *__restrict__ pC, int nc, int gga, double *__restrict__ out)
 {
+    pdl_enter();
     const int q = blockIdx.x;
     const double *p;
     int n, o;
@@ -93,6 +96,7 @@ __global__ void k_reduce_eval(const double *__restrict__ pA, int na, const doubl
 
 template <typename T> __global__ void k_fill(long long n, T *x, T val)
 {
+    pdl_enter();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         x[i] = val;
@@ -100,6 +104,7 @@ template <typename T> __global__ void k_fill(long long n, T *x, T val)
 
 template <typename T> __global__ void k_scale(long long n, T *x, double s, const double *sp)
 {
+    pdl_enter();
     if (sp != nullptr) s = *sp;
     const T st = (T)s;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -109,6 +114,7 @@ template <typename T> __global__ void k_scale(long long n, T *x, double s, const
 
 template <typename T, typename U> __global__ void k_convert(long long n, const T *x, U *y)
 {
+    pdl_enter();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         y[i] = (U)x[i];
@@ -116,6 +122,7 @@ template <typename T, typename U> __global__ void k_convert(long long n, const T
 
 template <typename T> __global__ void k_sumsq(long long n, const T *__restrict__ x, double *part)
 {
+    pdl_enter();
     typedef typename AccT<T>::type A;
     typedef typename AccT<T>::term P;
     A v[1] = {A(0)};
@@ -149,6 +156,7 @@ __global__ void k_cg_grad(long long n, const T *__restrict__ phi, const T *__res
                           double mu, const double *mup, T *__restrict__ g,
                           const T *__restrict__ gprev, double *part)
 {
+    pdl_enter();
     if (mup != nullptr) mu = *mup;
     typedef typename AccT<T>::type A;
     typedef typename AccT<T>::term P;
@@ -173,6 +181,7 @@ template <typename T>
 __global__ void k_cg_dir(long long n, const T *__restrict__ g, T *__restrict__ d, double beta,
                          const double *betap, const T *__restrict__ phi, double *part)
 {
+    pdl_enter();
     if (betap != nullptr) beta = *betap;
     typedef typename AccT<T>::type A;
     typedef typename AccT<T>::term P;
@@ -201,6 +210,7 @@ __global__ void k_cg_dhat(long long n, const T *__restrict__ g, T *__restrict__ 
                           const T *__restrict__ phi, const T *__restrict__ v, double c1, double c2,
                           int restart, const double *c12r, T *__restrict__ dhat, double *part)
 {
+    pdl_enter();
     if (c12r != nullptr) {
         c1 = c12r[0];
         c2 = c12r[1];
@@ -255,6 +265,7 @@ __global__ void k_cg_update(long long n, const int *__restrict__ accepted, T *__
                             const T *__restrict__ phit, T *__restrict__ v, const T *__restrict__ vt,
                             const double *mup, T *__restrict__ g, T *__restrict__ gprev, double *part)
 {
+    pdl_enter();
     typedef typename AccT<T>::type A;
     typedef typename AccT<T>::term P;
     const bool acc_t = *accepted != 0;
@@ -1418,7 +1429,7 @@ bool launch_ewald_energy(int nat, const double *R, const double *Z, const float 
     if ((double)(2 * w.ni[0] + 1) * (2 * w.ni[1] + 1) * (2 * w.ni[2] + 1) > 1e6) return false;
     k_ewald_tab<<<(nat * rows + 127) / 128, 128, 0, st>>>(nat, w, R, tab);
     k_ewald_energy<<<kEwBlocks, kEwThreads, 0, st>>>(nat, w, R, Z, frac, tab, part);
-    k_reduce<<<1, 256, 0, st>>>(part, kEwBlocks, out);
+    pdl_launch(k_reduce, 1, 256, 0, st, part, kEwBlocks, out);
     return true;
 }
 
@@ -1430,22 +1441,22 @@ void launch_andersen(int nat, const double *m, double *V, double kT, double prob
 
 void launch_reduce(const double *part, int nblk, int nq, double *out, cudaStream_t st)
 {
-    k_reduce<<<nq, 256, 0, st>>>(part, nblk, out);
+    pdl_launch(k_reduce, nq, 256, 0, st, part, nblk, out);
 }
 
 void launch_reduce_eval(const double *pA, int na, const double *pB, int nb, const double *pC, int nc, bool gga,
                         double *out, cudaStream_t st)
 {
-    k_reduce_eval<<<gga ? 18 : 12, 256, 0, st>>>(pA, na, pB, nb, pC, nc, gga ? 1 : 0, out);
+    pdl_launch(k_reduce_eval, gga ? 18 : 12, 256, 0, st, pA, na, pB, nb, pC, nc, gga ? 1 : 0, out);
 }
 
 template <typename T> void launch_fill(long long n, T *x, T val, cudaStream_t st)
 {
-    k_fill<T><<<vec_blocks(n), kVecThreads, 0, st>>>(n, x, val);
+    pdl_launch(k_fill<T>, vec_blocks(n), kVecThreads, 0, st, n, x, val);
 }
 template <typename T> void launch_scale(long long n, T *x, double s, const double *sp, cudaStream_t st)
 {
-    k_scale<T><<<vec_blocks(n), kVecThreads, 0, st>>>(n, x, s, sp);
+    pdl_launch(k_scale<T>, vec_blocks(n), kVecThreads, 0, st, n, x, s, sp);
 }
 
 template <typename T>
@@ -1453,17 +1464,17 @@ int launch_cg_update(long long n, const int *accepted, T *phi, const T *phit, T 
                      const double *mup, T *g, T *gprev, double *part, cudaStream_t st)
 {
     int b = red_blocks<T>(n);
-    k_cg_update<T><<<b, kVecThreads, 0, st>>>(n, accepted, phi, phit, v, vt, mup, g, gprev, part);
+    pdl_launch(k_cg_update<T>, b, kVecThreads, 0, st, n, accepted, phi, phit, v, vt, mup, g, gprev, part);
     return b;
 }
 template <typename T, typename U> void launch_convert(long long n, const T *x, U *y, cudaStream_t st)
 {
-    k_convert<T, U><<<vec_blocks(n), kVecThreads, 0, st>>>(n, x, y);
+    pdl_launch(k_convert<T, U>, vec_blocks(n), kVecThreads, 0, st, n, x, y);
 }
 template <typename T> int launch_sumsq(long long n, const T *x, double *part, cudaStream_t st)
 {
     int b = red_blocks<T>(n);
-    k_sumsq<T><<<b, kVecThreads, 0, st>>>(n, x, part);
+    pdl_launch(k_sumsq<T>, b, kVecThreads, 0, st, n, x, part);
     return b;
 }
 template <typename T>
@@ -1490,7 +1501,7 @@ int launch_cg_grad(long long n, const T *phi, const T *v, double mu, const doubl
                    const T *gprev, double *part, cudaStream_t st)
 {
     int b = red_blocks<T>(n);
-    k_cg_grad<T><<<b, kVecThreads, 0, st>>>(n, phi, v, mu, mup, g, gprev, part);
+    pdl_launch(k_cg_grad<T>, b, kVecThreads, 0, st, n, phi, v, mu, mup, g, gprev, part);
     return b;
 }
 template <typename T>
@@ -1498,7 +1509,7 @@ int launch_cg_dir(long long n, const T *g, T *d, double beta, const double *beta
                   double *part, cudaStream_t st)
 {
     int b = red_blocks<T>(n);
-    k_cg_dir<T><<<b, kVecThreads, 0, st>>>(n, g, d, beta, betap, phi, part);
+    pdl_launch(k_cg_dir<T>, b, kVecThreads, 0, st, n, g, d, beta, betap, phi, part);
     return b;
 }
 template <typename T>
@@ -1506,7 +1517,7 @@ int launch_cg_dhat(long long n, const T *g, T *d, const T *phi, const T *v, doub
                    int restart, const double *c12r, T *dhat, double *part, cudaStream_t st)
 {
     int b = red_blocks<T>(n);
-    k_cg_dhat<T><<<b, kVecThreads, 0, st>>>(n, g, d, phi, v, c1, c2, restart, c12r, dhat, part);
+    pdl_launch(k_cg_dhat<T>, b, kVecThreads, 0, st, n, g, d, phi, v, c1, c2, restart, c12r, dhat, part);
     return b;
 }
 

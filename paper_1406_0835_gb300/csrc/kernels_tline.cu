@@ -28,6 +28,7 @@
 
 #include "ffmath.cuh"
 #include "kernels.h"
+#include "pdl.cuh"
 #include "tcgen.cuh"
 
 namespace ofdft {
@@ -345,6 +346,7 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
     const long long ln_off = (w_ok ? ou * jb.ostride + (zaxis ? 0 : ln - ou * zlen) : 0) + (half ? h * rstride : 0);
     const bool wide = zaxis && (h & 1) == 0;
     if (tid < kLines) s_max[tid] = 27u << 23;      // 2^-100: the least exponent of the scale
+    pdl_enter();                                   // (the issuing warp reads nothing that another kernel writes)
     float2 v[16];
     if (mine) {
         const int line = tile * kLines + row;
@@ -620,7 +622,7 @@ void launch_tline(const GridInfo &g, int count, const TlPass *pass, cudaStream_t
         smem = std::max(smem, j.sh.smem);
     }
     if (blocks == 0) return;
-    k_tline<<<blocks, items + 32, smem, st>>>(jobs);
+    pdl_launch(k_tline, blocks, items + 32, smem, st, jobs);
 }
 
 }  // namespace ofdft
