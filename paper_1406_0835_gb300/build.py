@@ -13,7 +13,7 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libofdft.so")
 ROOT = os.path.dirname(HERE)
 
-SOURCES = ["kernels_fields.cu", "kernels_misc.cu", "kernels_tline.cu", "cg_control.cu", "capi.cu", "capi_static.cu",
+SOURCES = ["kernels_fields.cu", "kernels_misc.cu", "kernels_tline.cu", "kernels_force.cu", "cg_control.cu", "capi.cu", "capi_static.cu",
            "tfunc_table.cpp", "serve.cpp"]
 NVCC_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo",
               "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",

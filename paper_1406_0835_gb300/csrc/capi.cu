@@ -279,7 +279,7 @@ ofdft_status setup_tline(ofdft_ctx *c, FieldSet &f)
             float2 *t = (float2 *)(h.data() + at[a][3]);
             for (int i = 0; i < n3[a]; ++i) {
                 bool sine;
-                const double k = tline_frequency(n3[a], i, &sine) * b3[a];
+                const double k = real_freq(n3[a], i, sine) * b3[a];
                 const ff::f2 x = ff::from_double(k * k);
                 t[i] = make_float2(x.hi, x.lo);
             }
@@ -1515,7 +1515,9 @@ ofdft_status forces_now(ofdft_ctx *c, EvalScalars &es)
     const GridInfo &g = c->g;
     const double2 *nG = (const double2 *)f.spec + f.spec_stride;
     const PhaseTablesDD *dd = g.dd ? &c->pdd : nullptr;
-    size_t need = (size_t)c->nat * lpp_force_chunks(g, c->nat, dd != nullptr) * 3 + 16;
+    const bool tensor = dd != nullptr && force_tc_takes(g, c->nat);
+    const size_t sums = ((size_t)c->nat * (tensor ? force_tc_chunks(g, c->nat) : lpp_force_chunks(g, c->nat, dd != nullptr)) * 3 + 31) / 32 * 32;
+    const size_t need = sums + (tensor ? force_tc_bytes(g, c->nat) / 8 : 16);
     if (need > c->fpart_len) {
         if (c->fpart) cudaFreeAsync(c->fpart, c->st);
         c->fpart = nullptr;
@@ -1524,7 +1526,15 @@ ofdft_status forces_now(ofdft_ctx *c, EvalScalars &es)
     }
     // the third spectrum is free after an evaluation (ftTF and GGA alike)
     double2 *cn = (double2 *)f.spec + 2 * f.spec_stride;
-    int nchunk = launch_lpp_forces<double>(g, c->nat, c->Zd, c->px, c->py, c->pz, dd, nG, cn, c->fpart, c->st);
+    int nchunk;
+    if (tensor) {
+        launch_force_coefficients(g, nG, (float2 *)cn, c->st);
+        nchunk = launch_force_tc(g, c->nat, c->Zd, c->px, c->py, c->pz, nG, (const float2 *)cn, c->fpart + sums, c->fpart,
+                                 c->st);
+        c->launches++;
+    } else {
+        nchunk = launch_lpp_forces<double>(g, c->nat, c->Zd, c->px, c->py, c->pz, dd, nG, cn, c->fpart, c->st);
+    }
     launch_force_reduce(c->nat, nchunk, c->fpart, c->Fd, 0, c->st);
     c->launches += 3;
     std::vector<double> F(3 * c->nat), Fe(3 * c->nat);
@@ -1661,6 +1671,7 @@ ofdft_status alloc_ctx(ofdft_ctx *c)
     CK(set_field_smem_limits<double>(dyn));
     CK(set_field_smem_limits<float>(dyn));
     CK(tline_smem_limits());
+    CK(force_tc_smem_limits());
     CK(cudaStreamCreateWithFlags(&c->cap2, cudaStreamNonBlocking));
     for (cudaStream_t &a : c->aux) CK(cudaStreamCreateWithFlags(&a, cudaStreamNonBlocking));
     for (cudaEvent_t &e : c->fj) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -1702,6 +1713,11 @@ double footprint_bytes(const int grid[3], int nat, int precision)
     b += (3 * ny * std::ceil(K / 4) + 15 * (nx * ny / 2) + 64) * 8 + 64 * 8;  // partials, scalars
     b += nat * 11.0 * 8 + 32 + nat * (2 * nx + 2 * ny + 3 * K) * 16.0;  // ions, phase factors (+ double-float)
     b += nat * std::max(1216.0, (double)lpp_force_chunks_dd((long long)(nx * ny), nat)) * 3 * 8 + 16 * 8;   // force partials
+    GridInfo fg{};
+    fg.nx = grid[0];
+    fg.ny = grid[1];
+    fg.nz = grid[2];
+    b += (double)force_tc_bytes(fg, nat);                              // digits of the ions' phases
     double km = std::ceil(4.27 * std::pow((double)nat, 1.0 / 6.0)) + 1;
     b += std::pow(2 * km + 1, 3) * 6 * 8 + nat * 4.0 * 8;             // Ewald tables
     return 1.05 * b + 8.0 * (1 << 20);                                 // pool granularity, graphs

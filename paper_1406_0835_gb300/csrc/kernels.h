@@ -5,6 +5,39 @@
 
 namespace ofdft {
 
+// Frequency of real-Fourier coefficient a of an axis of n points, and whether
+// it is the sine's: coefficients 0 .. n/2 - 1 are the even frequencies 0, 2
+// (cosine, sine), 4, ..., the others the odd ones; the Nyquist frequency has
+// a cosine only.
+__host__ __device__ __forceinline__ int real_freq(int n, int a, bool &sine)
+{
+    const int h = n / 2;
+    const bool odd = a >= h;
+    const int i = odd ? a - h : a;
+    sine = odd ? (i & 1) != 0 : (i > 0 && (i & 1) == 0);
+    return odd ? 2 * (i / 2) + 1 : 2 * ((i + 1) / 2);
+}
+
+// Index of the cosine of frequency k (the sine's is the next).
+__host__ __device__ __forceinline__ int real_cosine(int n, int k) { return (k & 1 ? n / 2 : 0) + (k > 0 ? k - 1 : 0); }
+
+#ifdef __CUDACC__
+// Local pseudopotential form factor per unit charge, 0 at G = 0.
+// Gaussian ion: w(G) = -4 pi exp(-G^2 rc^2/4) / (Omega G^2).
+// Heine-Abarenkov, Eq. (E4A), q = |G|, divided by the common charge Z:
+// w(q) = -4 pi/(Omega q^2 Z) [(Z - A rc) cos(q rc) + (A/q) sin(q rc)] exp(-(q/qc)^6).
+__device__ __forceinline__ double lpp_w(const GridInfo &g, double g2)
+{
+    if (!(g2 > 0.0)) return 0.0;
+    if (g.lpp == 0) return -12.566370614359172954 * exp(-0.25 * g2 * g.rc * g.rc) / (g.omega * g2);
+    const double q = sqrt(g2), u = q / g.ha_qc, u2 = u * u;
+    double s, c;
+    sincos(q * g.rc, &s, &c);
+    const double B = (g.ha_Z - g.ha_A * g.rc) * c + g.ha_A * s / q;
+    return -12.566370614359172954 * B * exp(-u2 * u2 * u2) / (g.omega * g2 * g.ha_Z);
+}
+#endif
+
 // ---- grid fields (kernels_fields.cu)
 // z pass, forward: n = phi^2 (mode 1), the trial rotation phi cos + dhat sin
 // written to phit (mode 2) or a plain field (mode 0), R2C along z into the
@@ -41,8 +74,6 @@ size_t tline_matrix_bytes(int n);
 // times scale; the orthonormal real Fourier transform, or its inverse.
 int tline_derivative_matrix(int n, double scale, uint16_t *img);
 int tline_fourier_matrix(int n, bool inverse, uint16_t *img);
-// Frequency of real-Fourier coefficient a and whether it is the sine's.
-int tline_frequency(int n, int a, bool *sine);
 cudaError_t tline_smem_limits();
 // Up to four transforms, each along one axis, in one launch; out may be in.
 struct TlPass {
@@ -149,6 +180,18 @@ int launch_cg_dir(long long n, const T *g, T *d, double beta, const double *beta
 template <typename T>
 int launch_cg_dhat(long long n, const T *g, T *d, const T *phi, const T *v, double c1, double c2,
                    int restart, const double *c12r, T *dhat, double *part, cudaStream_t st);
+
+// Local-pseudopotential forces on the tensor cores (kernels_force.cu): coef
+// from launch_force_coefficients (pairs, N), scratch of force_tc_bytes, part
+// as launch_lpp_forces; returns the chunk count (= force_tc_chunks).  Taken
+// when force_tc_takes.
+bool force_tc_takes(const GridInfo &g, int nat);
+size_t force_tc_bytes(const GridInfo &g, int nat);
+int force_tc_chunks(const GridInfo &g, int nat);
+cudaError_t force_tc_smem_limits();
+void launch_force_coefficients(const GridInfo &g, const double2 *nG, float2 *coef, cudaStream_t st);
+int launch_force_tc(const GridInfo &g, int nat, const double *Z, const double2 *px, const double2 *py, const double2 *pz,
+                    const double2 *nG, const float2 *coef, void *scratch, double *part, cudaStream_t st);
 
 // Double-float copies of the phase tables (16 bytes per complex entry, the
 // size of a double2): xT[ix][I], yT[iy][I], zT[kz][I] (atoms fastest) and

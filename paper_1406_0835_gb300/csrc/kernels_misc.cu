@@ -343,21 +343,6 @@ __device__ __forceinline__ double2 zmul(double2 a, double2 b)
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// Local pseudopotential form factor per unit charge, 0 at G = 0.
-// Gaussian ion: w(G) = -4 pi exp(-G^2 rc^2/4) / (Omega G^2).
-// Heine-Abarenkov, Eq. (E4A), q = |G|, divided by the common charge Z:
-// w(q) = -4 pi/(Omega q^2 Z) [(Z - A rc) cos(q rc) + (A/q) sin(q rc)] exp(-(q/qc)^6).
-__device__ __forceinline__ double lpp_w(const GridInfo &g, double g2)
-{
-    if (!(g2 > 0.0)) return 0.0;
-    if (g.lpp == 0) return -12.566370614359172954 * exp(-0.25 * g2 * g.rc * g.rc) / (g.omega * g2);
-    const double q = sqrt(g2), u = q / g.ha_qc, u2 = u * u;
-    double s, c;
-    sincos(q * g.rc, &s, &c);
-    const double B = (g.ha_Z - g.ha_A * g.rc) * c + g.ha_A * s / q;
-    return -12.566370614359172954 * B * exp(-u2 * u2 * u2) / (g.omega * g2 * g.ha_Z);
-}
-
 // Pressure weight of the Heine-Abarenkov form per unit charge: the LPP
 // pressure is sum_G Re[n*(G) wp(G) sum_I Z_I e^{-iG.R_I}] with
 // wp = w + (q/3) dw/dq (Omega w depends on the cell only through q), i.e.
@@ -519,50 +504,65 @@ __global__ void k_vext(GridInfo g, int nat, const double *__restrict__ Z,
 // Real-Fourier coefficients of a real field from its half spectrum V (v(r) =
 // sum_G V(G) e^{i G.r}): along an axis of n points a cosine of frequency k
 // takes (V(k) + V(-k)) and a sine i (V(k) - V(-k)), each times sqrt(n/2); k
-// = 0 and n/2 take sqrt(n) V(k).  V(-G) = conj V(G).  fx, fy, fz: frequency
-// of each coefficient, negative for a sine (tables of one int per index).
-__device__ __forceinline__ int real_freq(int n, int a, bool &sine)
-{
-    const int h = n / 2;
-    const bool odd = a >= h;
-    const int i = odd ? a - h : a;
-    sine = odd ? (i & 1) != 0 : (i > 0 && (i & 1) == 0);
-    return odd ? 2 * (i / 2) + 1 : 2 * ((i + 1) / 2);
-}
+// = 0 and n/2 take sqrt(n) V(k).  V(-G) = conj V(G).  A thread makes the up
+// to eight coefficients of one (|kx|, |ky|, |kz|) from the four values of V
+// they share.  FORCE: times -Omega w(G) instead of the square roots (the
+// local forces' sum, whose functions are the plain cosines and sines), zero
+// on two or three Nyquist frequencies, which are no product of the axes'
+// functions there, and ordered by frequency.
+template <bool FORCE>
 __global__ void k_real_coefficients(GridInfo g, const double2 *__restrict__ V, float2 *__restrict__ coef)
 {
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < (int)g.N; q += gridDim.x * blockDim.x) {
-        const int c = q % g.nz, ab = q / g.nz, b = ab % g.ny, a = ab / g.ny;
-        bool sx, sy, sz;
-        const int kx = real_freq(g.nx, a, sx), ky = real_freq(g.ny, b, sy), kz = real_freq(g.nz, c, sz);
-        const bool ex = kx == 0 || 2 * kx == g.nx, ey = ky == 0 || 2 * ky == g.ny, ez = kz == 0 || 2 * kz == g.nz;
-        const int mx = ex ? kx : g.nx - kx, my = ey ? ky : g.ny - ky;
-        auto at = [&](int ix, int iy) { return V[((size_t)ix * g.ny + iy) * g.K + kz]; };
-        // z step at the four sign choices of (kx, ky): W = V(s) +- conj V(-s)
-        double2 W[2][2];
+    pdl_enter();
+    const int hx = g.nx / 2, hy = g.ny / 2, hz = g.nz / 2;
+    const int total = (hx + 1) * (hy + 1) * g.K;
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
+        const int kz = q % g.K, xy = q / g.K, ky = xy % (hy + 1), kx = xy / (hy + 1);
+        const bool ex = kx == 0 || kx == hx, ey = ky == 0 || ky == hy, ez = kz == 0 || kz == hz;
+        double f;
+        if (FORCE) {
+            const double gx = kx * g.bx, gy = ky * g.by, gz = kz * g.bz;
+            f = (kx == hx) + (ky == hy) + (kz == hz) > 1 ? 0.0 : -g.omega * lpp_w(g, gx * gx + gy * gy + gz * gz);
+        } else {
+            f = sqrt((double)g.nx * (ex ? 1.0 : 0.5)) * sqrt((double)g.ny * (ey ? 1.0 : 0.5)) *
+                sqrt((double)g.nz * (ez ? 1.0 : 0.5));
+        }
+        double2 v[2][2];                               // V(+-kx, +-ky, kz)
+#pragma unroll
         for (int i = 0; i < 2; ++i)
-            for (int j = 0; j < 2; ++j) {
-                if ((ex && i) || (ey && j)) continue;
-                const double2 p = at(i ? mx : kx, j ? my : ky);
-                if (ez) {
-                    W[i][j] = p;
-                } else {
-                    const double2 m = at(i ? kx : mx, j ? ky : my);
-                    W[i][j] = sz ? make_double2(-(p.y + m.y), p.x - m.x) : make_double2(p.x + m.x, p.y - m.y);
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                v[i][j] = V[((size_t)(i && !ex ? g.nx - kx : kx) * g.ny + (j && !ey ? g.ny - ky : ky)) * g.K + kz];
+        const int a = FORCE ? max(2 * kx - 1, 0) : real_cosine(g.nx, kx), b = FORCE ? max(2 * ky - 1, 0) : real_cosine(g.ny, ky),
+                  c = FORCE ? max(2 * kz - 1, 0) : real_cosine(g.nz, kz);
+#pragma unroll
+        for (int tz = 0; tz < 2; ++tz) {
+            if (tz && ez) continue;
+            double2 W[2][2];                           // z step: V(s) +- conj V(-s)
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const double2 p = v[i][j], m = v[1 - i][1 - j];
+                    W[i][j] = ez ? p : tz ? make_double2(-(p.y + m.y), p.x - m.x) : make_double2(p.x + m.x, p.y - m.y);
+                }
+#pragma unroll
+            for (int ty = 0; ty < 2; ++ty) {
+                if (ty && ey) continue;
+                double2 X[2];
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    X[i] = ey ? W[i][0] : ty ? make_double2(-(W[i][0].y - W[i][1].y), W[i][0].x - W[i][1].x)
+                                             : make_double2(W[i][0].x + W[i][1].x, W[i][0].y + W[i][1].y);
+#pragma unroll
+                for (int tx = 0; tx < 2; ++tx) {
+                    if (tx && ex) continue;
+                    const double re = ex ? X[0].x : tx ? -(X[0].y - X[1].y) : X[0].x + X[1].x;
+                    const ff::f2 o = ff::from_double(re * f);
+                    coef[((size_t)(a + tx) * g.ny + b + ty) * g.nz + c + tz] = make_float2(o.hi, o.lo);
                 }
             }
-        double2 X[2];
-        for (int i = 0; i < 2; ++i) {
-            if (ex && i) continue;
-            if (ey) X[i] = W[i][0];
-            else if (sy) X[i] = make_double2(-(W[i][0].y - W[i][1].y), W[i][0].x - W[i][1].x);
-            else X[i] = make_double2(W[i][0].x + W[i][1].x, W[i][0].y + W[i][1].y);
         }
-        const double re = ex ? X[0].x : (sx ? -(X[0].y - X[1].y) : X[0].x + X[1].x);
-        const double f = sqrt((double)g.nx * (ex ? 1.0 : 0.5)) * sqrt((double)g.ny * (ey ? 1.0 : 0.5)) *
-                         sqrt((double)g.nz * (ez ? 1.0 : 0.5));
-        const ff::f2 o = ff::from_double(re * f);
-        coef[q] = make_float2(o.hi, o.lo);
     }
 }
 
@@ -995,6 +995,7 @@ __global__ void k_lpp_forces_dd(GridInfo g, int nat, int rows_per_block, const d
 // chunks in a fixed pattern, then a fixed shuffle tree.
 __global__ void k_force_reduce_w(int nat, int nchunk, const double *__restrict__ part, double *F, int accumulate)
 {
+    pdl_enter();
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (w >= 3 * nat) return;
     const int I = w / 3, k = w - 3 * I;
@@ -1401,10 +1402,20 @@ __global__ void k_andersen(int nat, const double *m, double *V, double kT, doubl
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
-void launch_real_coefficients(const GridInfo &g, const double2 *v, float2 *coef, cudaStream_t st)
+static int octant_blocks(const GridInfo &g)
 {
-    const int blocks = (int)std::min<long long>((g.N + 255) / 256, 4864);
-    k_real_coefficients<<<blocks, 256, 0, st>>>(g, v, coef);
+    const long long n = (long long)(g.nx / 2 + 1) * (g.ny / 2 + 1) * g.K;
+    return (int)std::min<long long>((n + 127) / 128, 4864);
+}
+
+void launch_real_coefficients(const GridInfo &g, const double2 *V, float2 *coef, cudaStream_t st)
+{
+    pdl_launch(k_real_coefficients<false>, octant_blocks(g), 128, 0, st, g, V, coef);
+}
+
+void launch_force_coefficients(const GridInfo &g, const double2 *nG, float2 *coef, cudaStream_t st)
+{
+    pdl_launch(k_real_coefficients<true>, octant_blocks(g), 128, 0, st, g, nG, coef);
 }
 
 bool launch_ewald_energy(int nat, const double *R, const double *Z, const float *frac, const double L[3], double2 *tab, double *part,
@@ -1612,7 +1623,7 @@ void launch_force_reduce(int nat, int nchunk, const double *part, double *F, int
                          cudaStream_t st)
 {
     const long long threads = 32LL * 3 * nat;
-    k_force_reduce_w<<<(int)((threads + 255) / 256), 256, 0, st>>>(nat, nchunk, part, F, accumulate);
+    pdl_launch(k_force_reduce_w, (int)((threads + 255) / 256), 256, 0, st, nat, nchunk, part, F, accumulate);
 }
 
 void launch_ewald_real(int nat, const double *R, const double *Z, const EwCell &cl, double alpha,

@@ -26,7 +26,7 @@
 
 #include <algorithm>
 
-#include "ffmath.cuh"
+#include "digits.cuh"
 #include "kernels.h"
 #include "pdl.cuh"
 #include "tcgen.cuh"
@@ -36,8 +36,6 @@ namespace ofdft {
 namespace {
 
 constexpr int kLines = 64;    // lines of a tile: the rows of one M = 64 accumulator
-constexpr int kDig = 7;       // digits of radix 256
-constexpr uint64_t kDigBias = 0x0080808080808080ull;   // + 128 per digit
 constexpr int kTlThreads = 640;   // converting and reading-out threads at most; one more warp issues the products
 constexpr int kMaxChunks = 3;     // column chunks of a matrix
 constexpr int kMaxUnits = 2 * kMaxChunks;
@@ -105,86 +103,6 @@ struct TlJobs {
     TlJob job[kMaxJobs];
     int count;
 };
-
-// x 2^-E as an integer multiple of 2^-52, plus kFixedOff; u = 2^-E, E the
-// exponent of the line's largest magnitude (|x u| < 2).  Binary32 additions
-// of 1.5 2^23 round the leading word to 2^-20 and 2^-42 and the second to
-// 2^-42; what is left of both, below 2^-42, rounds to 2^-52.  The integers
-// are the low bits of the sums.
-constexpr uint32_t kMagic = 0x4b400000u;   // 1.5 2^23
-constexpr uint64_t kFixedOff = ((uint64_t)kMagic << 32) + 2048ull * kMagic + kMagic;
-__device__ __forceinline__ uint64_t to_fixed(float2 x, float u)
-{
-    constexpr float kM = 12582912.0f, k20 = 1048576.0f, k42 = 4398046511104.0f, k52 = 4503599627370496.0f;
-    const float hi = ff::fmul(x.x, u), lo = ff::fmul(x.y, u);
-    const float ta = ff::ffma(hi, k20, kM);
-    const float r = ff::ffma(ff::fsub(ta, kM), -1.0f / k20, hi);
-    const float tb = ff::ffma(r, k42, kM), td = ff::ffma(lo, k42, kM);
-    const float r2 = ff::ffma(ff::fsub(tb, kM), -1.0f / k42, r), l2 = ff::ffma(ff::fsub(td, kM), -1.0f / k42, lo);
-    const float tc = ff::ffma(ff::fadd(r2, l2), k52, kM);
-    const uint64_t low = (uint64_t)(__float_as_uint(tb) + __float_as_uint(td)) * 1024u + __float_as_uint(tc);
-    return low + ((uint64_t)__float_as_uint(ta) << 32);
-}
-
-__device__ __forceinline__ uint32_t digit_pair(uint32_t bytes, uint32_t sel)
-{
-    // (b, 0x64) is the f16 1024 + b; minus 1152 gives the digit b - 128 exactly
-    const uint32_t u = __byte_perm(bytes, 0x64646464u, sel);
-    uint32_t r;
-    asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(u), "r"(0xe480e480u));
-    return r;
-}
-
-// The seven digits (most significant first) of eight biased integers as
-// seven 16-byte rows of f16.
-__device__ __forceinline__ void store_digits(const uint64_t (&x)[8], unsigned char *dst, uint32_t dig_bytes)
-{
-    uint32_t w[kDig][4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        const uint32_t l0 = (uint32_t)x[2 * p], l1 = (uint32_t)x[2 * p + 1];
-        const uint32_t h0 = (uint32_t)(x[2 * p] >> 32), h1 = (uint32_t)(x[2 * p + 1] >> 32);
-        const uint32_t t0 = __byte_perm(l0, l1, 0x5140), t1 = __byte_perm(l0, l1, 0x7362);
-        const uint32_t u0 = __byte_perm(h0, h1, 0x5140), u1 = __byte_perm(h0, h1, 0x7362);
-        w[6][p] = digit_pair(t0, 0x4140);
-        w[5][p] = digit_pair(t0, 0x4342);
-        w[4][p] = digit_pair(t1, 0x4140);
-        w[3][p] = digit_pair(t1, 0x4342);
-        w[2][p] = digit_pair(u0, 0x4140);
-        w[1][p] = digit_pair(u0, 0x4342);
-        w[0][p] = digit_pair(u1, 0x4140);
-    }
-#pragma unroll
-    for (int d = 0; d < kDig; ++d)
-        *reinterpret_cast<uint4 *>(dst + d * dig_bytes) = make_uint4(w[d][0], w[d][1], w[d][2], w[d][3]);
-}
-
-// The accumulators (exact integers in f32, below 2^24) summed with their
-// weights 256^-d, as an unnormalised pair (s, rounding errors of the sums of
-// weight 256^-3 and up; those below are under 2^-51 of the full scale).
-// Fast2Sum is exact here although its operands are not ordered: each
-// accumulator is an integer, hence a multiple of the last place of the
-// smaller-weight sum it meets (below 2^16).
-__device__ __forceinline__ ff::f2 combine(const float (&a)[kDig])
-{
-    constexpr float w = 1.0f / 256.0f;
-    float s = ff::ffma(ff::ffma(a[6], w, a[5]), w, a[4]);
-    float err = 0.0f;
-#pragma unroll
-    for (int d = 3; d >= 0; --d) {
-        const float t = ff::ffma(s, w, a[d]);           // w is a power of two: the product is exact
-        const float e = ff::ffma(s, w, -ff::fsub(t, a[d]));
-        err = d == 3 ? e : ff::ffma(err, w, e);
-        s = t;
-    }
-    return ff::f2(s, err);
-}
-
-__device__ __forceinline__ float2 scaled(ff::f2 x, float sc)
-{
-    const ff::f2 r = ff::fast_two_sum(x.hi, x.lo);
-    return make_float2(r.hi * sc, r.lo * sc);
-}
 
 // x + sgn y of two such pairs, normalised, times sc (a power of two).
 __device__ __forceinline__ float2 butterfly(ff::f2 x, ff::f2 y, float sgn, float sc)
@@ -545,17 +463,6 @@ int tline_derivative_matrix(int n, double scale, uint16_t *img)
     return pack_matrix(n, t, [&](int half, int j, int l) { return (size_t)half * n + (j - l + n) % n; }, img);
 }
 
-// Coefficients 0 .. n/2 - 1: even frequencies 0, 2 (cosine, sine), 4, ...;
-// the others: odd ones; the Nyquist frequency has a cosine only.
-int tline_frequency(int n, int a, bool *sine)
-{
-    const int h = n / 2;
-    const bool odd = a >= h;
-    const int i = odd ? a - h : a;
-    *sine = odd ? (i & 1) != 0 : (i > 0 && (i & 1) == 0);
-    return odd ? 2 * (i / 2) + 1 : 2 * ((i + 1) / 2);
-}
-
 int tline_fourier_matrix(int n, bool inverse, uint16_t *img)
 {
     const int h = n / 2;
@@ -569,7 +476,7 @@ int tline_fourier_matrix(int n, bool inverse, uint16_t *img)
     std::vector<int> k(n), type(n);
     for (int a = 0; a < n; ++a) {
         bool sine;
-        k[a] = tline_frequency(n, a, &sine);
+        k[a] = real_freq(n, a, sine);
         type[a] = sine ? 1 : (k[a] == 0 || 2 * k[a] == n ? 2 : 0);
     }
     return pack_matrix(n, t, [&](int half, int out, int in) {
