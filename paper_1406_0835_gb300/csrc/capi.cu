@@ -209,11 +209,12 @@ template <typename T> ofdft_status upload_twiddles(ofdft_ctx *c, FieldSet &f, in
 // every axis that they support; the Hartree chain does when all three axes
 // are supported and the cell is orthorhombic (4 pi / G^2 is diagonal in
 // products of cosines and sines only there).  ftTF has the chain alone and
-// four kernels more in this form: a solve's evaluation takes 83 us instead of
-// 76 at 48^3, 93 instead of 98 at 60^3 and 155 instead of 204 at 96^3, so
-// smaller ftTF grids keep the FFT passes.  (GGA: 96^3 291 -> 255 us, 48^3
-// 95 -> 92, 32^3 72 -> 73.)
-constexpr long long kRealTfPoints = 160000;
+// five kernels more in this form, which on the smallest grids cost more than
+// they save, FFT passes -> here: an evaluation at 8^3 51 -> 56 us, 16^3 62 ->
+// 55, 32^3 64 -> 58, 48^3 73 -> 70, 54^3 86 -> 79, a solve's evaluation at
+// 32^3 119 -> 102 us.  (GGA: 96^3 291 -> 255 us, 48^3 95 -> 92, 32^3 72 -> 73
+// before the launches of a chain overlapped.)
+constexpr long long kRealTfPoints = 2048;
 bool tl_derivatives(const ofdft_ctx *c, int n) { return c->g.dd && !c->g.dws && c->fp.kind != 0 && tline_supported(n); }
 bool tl_real_basis(const ofdft_ctx *c)
 {

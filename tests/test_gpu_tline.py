@@ -83,3 +83,9 @@ def test_a_non_finite_density_is_refused(bad):
         with pytest.raises(ofdft.OfdftError) as e:
             ctx.energy_potential(phi)
         assert e.value.status == -4
+
+
+@pytest.mark.parametrize("grid", [(8, 16, 16), (10, 12, 16), (12, 10, 18), (36, 8, 10)])
+def test_fttf_grids_on_both_sides_of_the_rule(grid):
+    """2048 points and more take the real basis; 1920 keep the FFT passes."""
+    check(grid, functional="fttf")
