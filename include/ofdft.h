@@ -416,15 +416,14 @@ void ofdft_destroy(ofdft_ctx *ctx);
  * ofdft_setup + ofdft_energy_potential compute (F_tot and its terms, the
  * pressure terms, v = dF/dn at n = phi^2), in FP64, with the same kernels,
  * but every device scratch buffer is carved from one fixed array compiled
- * into the library: about 3.0 MB that each GPU loading the library holds
+ * into the library: about 4.2 MB that each GPU loading the library holds
  * until the process exits.  The call allocates no memory, on the device or
- * the host.
+ * (after the set-up below) the host.
  *  cell[9], grid[3], nat, ions, Z, T_kelvin, functional: as ofdft_setup,
  *              but orthorhombic cells only (else OFDFT_EINVAL).
  *  xc, rc: as ofdft_params (Gaussian ion only).
  *  phi_dev  device pointer, N doubles (input; not modified), 16-byte aligned.
- *  v_dev    device pointer, N doubles (output potential), 16-byte aligned;
- *           also the call's scratch for one field before v is written.
+ *  v_dev    device pointer, N doubles (output potential), 16-byte aligned.
  *  E        host output (may be NULL).
  *  stream   cudaStream_t to run on, or NULL for the default stream; the call
  *           returns after the stream has finished its work.
@@ -434,11 +433,11 @@ void ofdft_destroy(ofdft_ctx *ctx);
  * No call may be made on a stream that is being captured (the call reads
  * from pageable host memory and synchronises): OFDFT_EINVAL.  The first
  * call on a device does a one-time set-up on the current device (looks up
- * the array's device address, uploads the temperature table).  The set-up
- * runs under a mutex, so
+ * the array's device address, fills and uploads the tables and matrices).  The
+ * set-up runs under a mutex, so
  * first calls from several host threads are safe on the host.  It is cached
  * for the life of the device's context: after cudaDeviceReset (or a release
- * of the primary context) the cached address and table are stale and the
+ * of the primary context) the cached address and tables are stale and the
  * path must not be called again in that process.  All calls share the array
  * and it keeps the last call's contents: calls that overlap on the GPU (from
  * other threads or streams) race, so serialise them.

@@ -1,16 +1,16 @@
 // Allocation-free energy and potential: ofdft_energy_potential_static.
 //
 // Same arithmetic and kernels as ofdft_setup + ofdft_energy_potential, but all
-// device scratch (half spectra, local potential, phases, reduction partials,
-// twiddles, temperature table) lives in one file-scope __device__ array, so a
-// call allocates nothing.  Callers that cannot allocate device memory (tight
+// device scratch (fields, local potential, phases, reduction partials,
+// transform matrices, temperature table) lives in one file-scope __device__
+// array, so a call allocates nothing.  Callers that cannot allocate device memory (tight
 // loops where cudaMalloc could synchronise the GPU, or programs whose device
 // memory belongs to another allocator) pass their own phi and v buffers.
 //
 // Host code reaches the array only through the address cudaGetSymbolAddress
 // returns for the current device (the symbol itself is a host-side stand-in).
-// The first call on a device does that lookup and uploads the temperature
-// table, under a mutex, so first calls from several host threads do not race
+// The first call on a device does that lookup and uploads the tables
+// and matrices, under a mutex, so first calls from several host threads do not race
 // on the host.  Every call reuses the same array; calls that overlap on the
 // GPU race.
 #include <math.h>
@@ -36,10 +36,9 @@ constexpr long long kSMaxPart = 3LL * kSMaxEdge * 5 + 15LL * (kSMaxN / 16) + 64;
 constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Byte offsets inside the scratch array.
-constexpr size_t kOffSpec = 0;                                              // 4 spectra
-constexpr size_t kSpecBytes = align256((size_t)kSMaxNH * sizeof(double2));
-constexpr size_t kOffVext = kOffSpec + 4 * kSpecBytes;
-constexpr size_t kOffVpart = kOffVext + kSpecBytes;
+constexpr size_t kFieldBytes = align256((size_t)kSMaxN * sizeof(float2));   // a field of pairs: n's coefficients, three derivatives
+constexpr size_t kOffVext = 4 * kFieldBytes;
+constexpr size_t kOffVpart = kOffVext + align256((size_t)kSMaxNH * sizeof(double2));
 constexpr size_t kOffPhase = kOffVpart + align256((size_t)kSMaxN * sizeof(double));
 constexpr size_t kPhaseBytes = align256((size_t)kSMaxAtoms * (3 * kSMaxEdge) * sizeof(double2));
 constexpr size_t kOffIons = kOffPhase + kPhaseBytes;
@@ -47,22 +46,18 @@ constexpr size_t kOffZ = kOffIons + align256(3 * kSMaxAtoms * sizeof(double));
 constexpr size_t kOffFrac = kOffZ + align256(kSMaxAtoms * sizeof(double));
 constexpr size_t kOffPart = kOffFrac + align256(3 * kSMaxAtoms * sizeof(float));
 constexpr size_t kOffScal = kOffPart + align256((size_t)kSMaxPart * sizeof(double));
-// twiddles of every edge the path takes, each as binary64 and double-float pairs
-constexpr int kEdges[] = {8, 10, 12, 16, 18, 20, 24, 30, 32, 36, 40, 48, 50, 54, 60, 64};
-constexpr int tw_offset(int n)   // entries before those of edge n
-{
-    int o = 0;
-    for (int e : kEdges) {
-        if (e == n) return o;
-        o += 2 * e;
-    }
-    return n == 0 ? o : -1;
-}
-constexpr int kTwEntries = tw_offset(0);
-constexpr size_t kOffTw = kOffScal + align256(64 * sizeof(double));
-constexpr size_t kOffEwTab = kOffTw + align256(kTwEntries * sizeof(double2));
+constexpr int kEdges[] = {8, 10, 12, 16, 18, 20, 24, 30, 32, 36, 40, 48, 50, 54, 60, 64};   // the path takes
+constexpr size_t kOffEwTab = kOffScal + align256(64 * sizeof(double));
 constexpr size_t kOffEwPart = kOffEwTab + align256((size_t)kEwTabRows * kSMaxAtoms * sizeof(double2));
-constexpr size_t kOffTab = kOffEwPart + align256(kEwBlocks * sizeof(double));
+// double-float phase tables, v_ext's real-Fourier coefficients and (k b)^2
+constexpr size_t kOffPhaseDD = kOffEwPart + align256(kEwBlocks * sizeof(double));
+constexpr size_t kOffVre = kOffPhaseDD + 2 * kPhaseBytes;
+constexpr size_t kOffG2 = kOffVre + align256((size_t)kSMaxN * sizeof(float2));
+// tensor-core matrices of every edge: derivative per lattice period, forward
+// and inverse real Fourier transform
+constexpr size_t kMatBytes = 768 * 1024;
+constexpr size_t kOffMat = kOffG2 + align256(3 * kSMaxEdge * sizeof(float2));
+constexpr size_t kOffTab = kOffMat + kMatBytes;
 constexpr size_t kScratchBytes = kOffTab + align256((size_t)kDdTabSize * sizeof(double));   // + splits
 
 static __device__ __align__(256) unsigned char g_ofdft_scratch[kScratchBytes];
@@ -74,25 +69,45 @@ struct DevState {
 };
 DevState g_dev[kMaxDevices];
 double g_tab_host[kDdTabSize];    // host temperature table + double-float tables, filled once
-double2 g_tw_host[kTwEntries];    // twiddles of every edge, filled once
+struct EdgeMats {                 // transform matrices, filled once
+    size_t at[3];                 // offsets in the matrices' block
+    int mexp[3];
+} g_mat[sizeof(kEdges) / sizeof(kEdges[0])];
+unsigned char g_mat_host[kMatBytes];
 bool g_tab_ready = false;
-std::mutex g_setup_mu;            // guards g_dev, g_tab_host, g_tw_host and g_tab_ready (locking allocates nothing)
+std::mutex g_setup_mu;            // guards g_dev, g_tab_host, g_mat, g_mat_host and g_tab_ready (locking allocates nothing)
 
-// exp(-2 pi i m / n) for every edge n, as binary64 and as double-float pairs.
-void twiddles_fill(double2 *tw)
-{
-    for (int n : kEdges)
-        for (int m = 0; m < n; ++m) {
-            const long double ang = -2.0L * 3.14159265358979323846264338327950288L * m / n;
-            const long double cv = cosl(ang), sv = sinl(ang);
-            double2 *d = tw + tw_offset(n) + m;
-            float *f = reinterpret_cast<float *>(d + n);
-            *d = make_double2((double)cv, (double)sv);
-            f[0] = (float)cv;
-            f[1] = (float)(cv - (long double)f[0]);
-            f[2] = (float)sv;
-            f[3] = (float)(sv - (long double)f[2]);
+// The matrices of every edge, filled once with the other tables.
+bool matrices_fill()
+try {
+    size_t at = 0;
+    for (size_t i = 0; i < sizeof(kEdges) / sizeof(kEdges[0]); ++i) {
+        const int n = kEdges[i];
+        for (int k = 0; k < 3; ++k) {
+            const size_t b = align256(tline_matrix_bytes(n));
+            if (!tline_supported(n) || at + b > kMatBytes) return false;
+            uint16_t *img = (uint16_t *)(g_mat_host + at);
+            g_mat[i].at[k] = at;
+            g_mat[i].mexp[k] = k == 0 ? tline_derivative_matrix(n, 1.0, img) : tline_fourier_matrix(n, k == 2, img);
+            at += b;
         }
+    }
+    return true;
+} catch (...) {   // no host memory for their fill
+    return false;
+}
+
+TlAxis axis_matrices(int n, unsigned char *dev)
+{
+    TlAxis a;
+    TlMat *m[3] = {&a.der, &a.fwd, &a.inv};
+    for (size_t i = 0; i < sizeof(kEdges) / sizeof(kEdges[0]); ++i)
+        if (kEdges[i] == n)
+            for (int k = 0; k < 3; ++k) {
+                m[k]->img = dev + g_mat[i].at[k];
+                m[k]->mexp = g_mat[i].mexp[k];
+            }
+    return a;
 }
 
 // The ions of a call, by value in a kernel's arguments: no copy from
@@ -101,9 +116,17 @@ struct Ions {
     double v[4 * kSMaxAtoms];   // positions, then charges
     float frac[3 * kSMaxAtoms]; // fractional coordinates in [0, 1]
 };
-__global__ void k_put_ions(int nat, const __grid_constant__ Ions ions, double *R, double *Z, float *frac)
+// Also (k b)^2 of each axis's real-Fourier coefficients.
+__global__ void k_put_ions(GridInfo g, int nat, const __grid_constant__ Ions ions, double *R, double *Z, float *frac, float2 *g2)
 {
     const int i = threadIdx.x;
+    if (i < 3 * kSMaxEdge) {
+        const int a = i / kSMaxEdge, j = i - a * kSMaxEdge, n = a == 0 ? g.nx : (a == 1 ? g.ny : g.nz);
+        bool sine;
+        const double k = real_freq(n, j, sine) * (a == 0 ? g.bx : (a == 1 ? g.by : g.bz));
+        const ff::f2 x = ff::from_double(k * k);
+        if (j < n) g2[i] = make_float2(x.hi, x.lo);
+    }
     if (i < 3 * nat) {
         R[i] = ions.v[i];
         frac[i] = ions.frac[i];
@@ -129,8 +152,7 @@ bool edge_ok(int n)
     return n == 1;
 }
 
-
-// One-time set-up on the current device: scratch address, table, smem limits.
+// One-time set-up on the current device: scratch address, tables, smem limits.
 ofdft_status device_setup(int dev, unsigned char **base)
 {
     if (dev < 0 || dev >= kMaxDevices) return serr(OFDFT_EINVAL, "device ordinal out of range");
@@ -144,17 +166,13 @@ ofdft_status device_setup(int dev, unsigned char **base)
             static double ttab[kTfSize];
             tfunc_table_fill(ttab);
             dd_tables_fill(ttab, g_tab_host);
-            twiddles_fill(g_tw_host);
+            if (!matrices_fill()) return serr(OFDFT_EDEVICE, "no transform matrices");
             g_tab_ready = true;
         }
         SCK(cudaMemcpy(d.base + kOffTab, g_tab_host, sizeof(g_tab_host), cudaMemcpyHostToDevice),
             "temperature table upload failed");
-        SCK(cudaMemcpy(d.base + kOffTw, g_tw_host, sizeof(g_tw_host), cudaMemcpyHostToDevice), "twiddle upload failed");
-        int optin = 0;
-        SCK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev),
-            "device attribute query failed");
-        // leave room for the kernels' static shared memory, as ofdft_setup does
-        SCK(set_field_smem_limits<double>((size_t)optin - 8192), "shared-memory limit set-up failed");
+        SCK(cudaMemcpy(d.base + kOffMat, g_mat_host, sizeof(g_mat_host), cudaMemcpyHostToDevice), "matrix upload failed");
+        SCK(tline_smem_limits(), "shared-memory limit set-up failed");
         d.ready = true;
     }
     *base = d.base;
@@ -283,15 +301,9 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
     g.dV = g.omega / (double)N;
     g.rc = rc;
     grid_reciprocal(g);
-    g.dd = 1;   // double-float FFT and pointwise arithmetic, as ofdft_setup's default
+    g.dd = 1;   // double-float transforms and pointwise arithmetic, as ofdft_setup's default
     const double T = T_kelvin * 3.166811563e-6;
 
-    const double2 *tw = (const double2 *)(base + kOffTw);
-    const double2 *twx = tw + tw_offset(g.nx), *twy = tw + tw_offset(g.ny), *twz = tw + tw_offset(g.nz);
-    FftAxis ax = fft_axis(g.nx, twx), ay = fft_axis(g.ny, twy), az = fft_axis(g.nz, twz, 4);   // the FP64 contexts' z schedule
-    ax.twf = twx + g.nx;
-    ay.twf = twy + g.ny;
-    az.twf = twz + g.nz;
     // ions -> Ewald sums; phases -> v_ext(G)
     double *Rd = (double *)(base + kOffIons), *Zd = (double *)(base + kOffZ);
     double *scal = (double *)(base + kOffScal);   // 18 sums of the evaluation, then the Ewald sums
@@ -304,46 +316,85 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
         const double f = ions[i] / L[i % 3];
         arg.frac[i] = (float)(f - floor(f));
     }
-    k_put_ions<<<1, 4 * kSMaxAtoms, 0, st>>>(nat, arg, Rd, Zd, frac);
+    float2 *g2 = (float2 *)(base + kOffG2);
+    k_put_ions<<<1, 4 * kSMaxAtoms, 0, st>>>(g, nat, arg, Rd, Zd, frac, g2);
     const bool ewald_dev = launch_ewald_energy(nat, Rd, Zd, frac, L, (double2 *)(base + kOffEwTab), (double *)(base + kOffEwPart),
                                                scal + 18, st);
     double2 *px = (double2 *)(base + kOffPhase);
     double2 *py = px + (size_t)nat * g.nx, *pz = py + (size_t)nat * g.ny;
     double2 *vext = (double2 *)(base + kOffVext);
-    launch_phases(g, nat, Rd, px, py, pz, nullptr, st);
-    launch_vext(g, nat, Zd, px, py, pz, nullptr, vext, st);
+    PhaseTablesDD dd;
+    double2 *pd = (double2 *)(base + kOffPhaseDD);
+    dd.xT = pd;
+    dd.yT = pd + (size_t)nat * g.nx;
+    dd.zT = pd + (size_t)nat * (g.nx + g.ny);
+    dd.zd = pd + (size_t)nat * (g.nx + g.ny + g.K);
+    launch_phases(g, nat, Rd, px, py, pz, &dd, st);
+    launch_vext(g, nat, Zd, px, py, pz, &dd, vext, st);
 
-    // evaluation (same kernel sequence as the context path)
-    const size_t specN = kSpecBytes / sizeof(double2);
-    double2 *s0 = (double2 *)(base + kOffSpec), *s1 = s0 + specN, *s2 = s1 + specN, *s3 = s2 + specN;
     const double *tab = (const double *)(base + kOffTab);
     double *vpart = (double *)(base + kOffVpart);
-    double *part = (double *)(base + kOffPart);
-    const int nbx = xpass_blocks(g);
-    const long long npairs = (long long)g.nx * g.ny / 2;
-    double *pA = part, *pB = pA + 3 * nbx, *pC = pB + 6 * npairs;
-    double *ph = const_cast<double *>(phi_dev);
+    double *pA = (double *)(base + kOffPart);
     const bool fttf = fp.kind == 0;
-    // the second to fourth spectra double as real fields (2 NH >= N values):
-    // derivatives of n, then the fields whose derivatives make up div W;
-    // v_dev holds d_x U_x + d_y U_y until the final pass overwrites it with v
-    double *d0 = (double *)s1, *d1 = (double *)s2, *d2 = (double *)s3;
-    launch_zfwd<double>(g, az, 1, nullptr, ph, nullptr, 0.0, 0.0, nullptr, nullptr, s0, st, fttf ? nullptr : d2);
-    launch_ypass<double>(g, ay, false, s0, 1, specN, st);
-    launch_xhl<double>(g, ax, s0, vext, nullptr, 1, pA, st);
-    launch_ypass<double>(g, ay, true, s0, 1, specN, st);
-    int nbz, nbg = 0;   // blocks of the final z pass and of the pointwise stage: their partial sums
+    // The context path's sequence in the real Fourier basis.  The matrices are
+    // those of unit spacing, shared by all cells of an edge: the derivatives
+    // are per lattice period, and the pointwise stage takes them (and gives the
+    // fields of div W) through the reciprocal basis, as in a general cell.
+    unsigned char *mat = base + kOffMat;
+    const TlAxis tl[3] = {axis_matrices(g.nx, mat), axis_matrices(g.ny, mat), axis_matrices(g.nz, mat)};
+    float2 *coef = (float2 *)base, *vre = (float2 *)(base + kOffVre), *nf = (float2 *)vpart;
+    double *d[3];
+    TlPass grad[4], div[3];
+    for (int a = 0; a < 3; ++a) {
+        d[a] = (double *)(base + (a + 1) * kFieldBytes);
+        grad[a] = {TlPass::kDerivative, a, &tl[a].der, nf, (float2 *)d[a]};
+        div[a] = {TlPass::kDerivative, a, &tl[a].der, (float2 *)d[a], (float2 *)d[a]};
+    }
+    const TlPass zf = {TlPass::kForward, 2, &tl[2].fwd, nf, coef};
+    grad[3] = zf;
+    launch_real_coefficients(g, vext, vre, st);
+    launch_density(g.N, phi_dev, nullptr, 1.0, 0.0, nullptr, nullptr, nf, st);
+    launch_tline(g, fttf ? 1 : 4, fttf ? &zf : grad, st);
+    for (int a = 1; a >= 0; --a) {
+        const TlPass fwd = {TlPass::kForward, a, &tl[a].fwd, coef, coef};
+        launch_tline(g, 1, &fwd, st);
+    }
+    TlHartree hl{};
+    for (int a = 0; a < 3; ++a) hl.g2[a] = g2 + a * kSMaxEdge;
+    hl.ve = vre;
+    hl.hr = make_float2(g.hr2[0], g.hr2[1]);
+    hl.half_dv = 0.5 * g.dV;
+    hl.dv = g.dV;
+    hl.ploc = g.dV / g.omega / 3.0;
+    hl.part = pA;
+    const int nbx = launch_hartree(g, coef, hl, st);
+    for (int a = 0; a < 3; ++a) {
+        const TlPass inv = {TlPass::kInverse, a, &tl[a].inv, coef, coef};
+        launch_tline(g, 1, &inv, st);
+    }
+    // partial sums of the Hartree, the pointwise and the final stage
+    double *pB = pA + 3 * nbx, *pC = pB + 6 * ((long long)g.nx * g.ny / 2);
+    int nbg = 0, nbz;
     if (fttf) {
-        nbz = launch_zfinal<double>(g, az, true, s0, nullptr, ph, nullptr, nullptr, 1.0, 0.0, nullptr, T, fp,
-                                    tab, xc, v_dev, pC, st);
+        nbz = launch_ptf(g, coef, phi_dev, nullptr, nullptr, 1.0, 0.0, nullptr, T, fp, tab, xc, v_dev, pC, st);
     } else {
-        launch_dline<double>(g, ax, 0, 0, 0, ph, d0, st);
-        launch_dline<double>(g, ay, 1, 0, 0, ph, d1, st);
-        nbg = launch_pw<double>(g, d0, d1, d2, ph, T, fp, tab, xc, vpart, pB, false, st);
-        launch_dline<double>(g, ax, 0, 1, 0, d0, v_dev, st);
-        launch_dline<double>(g, ay, 1, 1, 1, d1, v_dev, st);
-        nbz = launch_zfinal_gga<double>(g, az, s0, d2, vpart, v_dev, nullptr, nullptr, ph, nullptr, nullptr, 1.0, 0.0,
-                                        nullptr, v_dev, pC, st);
+        GridInfo gp = g;
+        gp.tri = 1;
+        for (int i = 0; i < 9; ++i) gp.Bm[i] = 0.0;
+        gp.Bm[0] = g.bx;
+        gp.Bm[4] = g.by;
+        gp.Bm[8] = g.bz;
+        nbg = launch_pw<double>(gp, d[0], d[1], d[2], phi_dev, T, fp, tab, xc, vpart, pB, false, st);
+        launch_tline(g, 3, div, st);
+        TlFinal fin{};
+        fin.vhl = coef;
+        fin.vpart = nf;
+        for (int a = 0; a < 3; ++a) fin.d[a] = (const float2 *)d[a];
+        fin.phit = phi_dev;
+        fin.c = 1.0;
+        fin.vout = v_dev;
+        fin.part = pC;
+        nbz = launch_final(g, fin, st);
     }
     launch_reduce_eval(pA, nbx, pB, nbg, pC, nbz, !fttf, scal, st);
     double h[19];

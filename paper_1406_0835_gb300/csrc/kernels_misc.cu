@@ -303,6 +303,7 @@ __global__ void k_cg_update(long long n, const int *__restrict__ accepted, T *__
 __global__ void k_phases(GridInfo g, int nat, const double *__restrict__ R, double2 *px,
                          double2 *py, double2 *pz)
 {
+    pdl_enter();
     const int per = g.nx + g.ny + g.K;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nat * per; i += gridDim.x * blockDim.x) {
         const int I = i / per, j = i - I * per;
@@ -754,6 +755,7 @@ __global__ void k_phase_tables_dd(GridInfo g, int nat, const double2 *__restrict
                                   const double2 *__restrict__ py, const double2 *__restrict__ pz,
                                   ff::cf2 *pxT, ff::cf2 *pyT, ff::cf2 *pzT, ff::cf2 *pzd)
 {
+    pdl_enter();
     const int per = g.nx + g.ny + g.K;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nat * per; i += gridDim.x * blockDim.x) {
         const int I = i / per, j = i - I * per;
@@ -851,6 +853,7 @@ __global__ void k_vext_dd(GridInfo g, int nat, const double *__restrict__ Z, con
                           const ff::cf2 *__restrict__ pyT, const ff::cf2 *__restrict__ pzd,
                           double2 *__restrict__ vext)
 {
+    pdl_enter();
     const int ix = blockIdx.x / g.ny, iy = blockIdx.x - ix * g.ny;
     const bool rnyq = (2 * ix == g.nx) || (2 * iy == g.ny);
     double2 sa[2], sb[2];
@@ -1197,6 +1200,7 @@ struct EwBox {
 
 __global__ void k_ewald_tab(int nat, EwBox w, const double *__restrict__ R, double2 *__restrict__ tab)
 {
+    pdl_enter();
     const int rows = w.off[2] + w.km[2] + 1;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nat * rows; i += gridDim.x * blockDim.x) {
         const int row = i / nat, I = i - row * nat;
@@ -1236,6 +1240,7 @@ __global__ void __launch_bounds__(kEwThreads) k_ewald_energy(int nat, EwBox w, c
                                                              const float *__restrict__ frac,
                                                              const double2 *__restrict__ tab, double *__restrict__ part)
 {
+    pdl_enter();
     const int nreal = gridDim.x / 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int kW = kEwThreads / 32;
     double acc[1] = {0.0};
@@ -1438,8 +1443,8 @@ bool launch_ewald_energy(int nat, const double *R, const double *Z, const float 
         rows += w.km[a] + 1;
     }
     if ((double)(2 * w.ni[0] + 1) * (2 * w.ni[1] + 1) * (2 * w.ni[2] + 1) > 1e6) return false;
-    k_ewald_tab<<<(nat * rows + 127) / 128, 128, 0, st>>>(nat, w, R, tab);
-    k_ewald_energy<<<kEwBlocks, kEwThreads, 0, st>>>(nat, w, R, Z, frac, tab, part);
+    pdl_launch(k_ewald_tab, (nat * rows + 127) / 128, 128, 0, st, nat, w, R, tab);
+    pdl_launch(k_ewald_energy, kEwBlocks, kEwThreads, 0, st, nat, w, R, Z, frac, tab, part);
     pdl_launch(k_reduce, 1, 256, 0, st, part, kEwBlocks, out);
     return true;
 }
@@ -1537,10 +1542,10 @@ void launch_phases(const GridInfo &g, int nat, const double *R, double2 *px, dou
 {
     int total = nat * (g.nx + g.ny + g.K);
     int b = (total + 255) / 256;
-    k_phases<<<b, 256, 0, st>>>(g, nat, R, px, py, pz);
+    pdl_launch(k_phases, b, 256, 0, st, g, nat, R, px, py, pz);
     if (dd)
-        k_phase_tables_dd<<<b, 256, 0, st>>>(g, nat, px, py, pz, (ff::cf2 *)dd->xT, (ff::cf2 *)dd->yT,
-                                             (ff::cf2 *)dd->zT, (ff::cf2 *)dd->zd);
+        pdl_launch(k_phase_tables_dd, b, 256, 0, st, g, nat, px, py, pz, (ff::cf2 *)dd->xT, (ff::cf2 *)dd->yT,
+                   (ff::cf2 *)dd->zT, (ff::cf2 *)dd->zd);
 }
 
 void launch_vext(const GridInfo &g, int nat, const double *Z, const double2 *px,
@@ -1549,8 +1554,8 @@ void launch_vext(const GridInfo &g, int nat, const double *Z, const double2 *px,
     int th = 32 * ((g.K + 31) / 32);
     if (th > 128) th = 32 * ((((g.K + 1) / 2) + 31) / 32);    // two columns per thread
     if (dd && g.dd)
-        k_vext_dd<<<g.nx * g.ny, th, 0, st>>>(g, nat, Z, (const ff::cf2 *)dd->xT, (const ff::cf2 *)dd->yT,
-                                               (const ff::cf2 *)dd->zd, vext);
+        pdl_launch(k_vext_dd, g.nx * g.ny, th, 0, st, g, nat, Z, (const ff::cf2 *)dd->xT, (const ff::cf2 *)dd->yT,
+                   (const ff::cf2 *)dd->zd, vext);
     else
         k_vext<<<g.nx * g.ny, th, 0, st>>>(g, nat, Z, px, py, pz, vext);
 }
