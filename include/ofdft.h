@@ -416,7 +416,7 @@ void ofdft_destroy(ofdft_ctx *ctx);
  * ofdft_setup + ofdft_energy_potential compute (F_tot and its terms, the
  * pressure terms, v = dF/dn at n = phi^2), in FP64, with the same kernels,
  * but every device scratch buffer is carved from one fixed array compiled
- * into the library: about 4.2 MB that each GPU loading the library holds
+ * into the library: about 3.4 MB that each GPU loading the library holds
  * until the process exits.  The call allocates no memory, on the device or
  * (after the set-up below) the host.
  *  cell[9], grid[3], nat, ions, Z, T_kelvin, functional: as ofdft_setup,

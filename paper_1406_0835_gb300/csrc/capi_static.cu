@@ -26,22 +26,21 @@ using namespace ofdft;
 namespace {
 
 // Limits of the static path.
-constexpr int kSMaxEdge = 64;
+constexpr int kSMaxEdge = kStaticEdge;
 constexpr long long kSMaxN = 32768;
-constexpr int kSMaxAtoms = 64;
-// half spectrum: nx*ny*(nz/2+1) <= N/2 + nx*ny <= 16384 + 4096 (nz >= 8)
-constexpr long long kSMaxNH = kSMaxN / 2 + kSMaxN / 8;
+constexpr int kSMaxAtoms = kStaticAtoms;
 constexpr long long kSMaxPart = 3LL * kSMaxEdge * 5 + 15LL * (kSMaxN / 16) + 64;
 
 constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Byte offsets inside the scratch array.
 constexpr size_t kFieldBytes = align256((size_t)kSMaxN * sizeof(float2));   // a field of pairs: n's coefficients, three derivatives
-constexpr size_t kOffVext = 4 * kFieldBytes;
-constexpr size_t kOffVpart = kOffVext + align256((size_t)kSMaxNH * sizeof(double2));
-constexpr size_t kOffPhase = kOffVpart + align256((size_t)kSMaxN * sizeof(double));
-constexpr size_t kPhaseBytes = align256((size_t)kSMaxAtoms * (3 * kSMaxEdge) * sizeof(double2));
-constexpr size_t kOffIons = kOffPhase + kPhaseBytes;
+constexpr size_t kOffVre = 4 * kFieldBytes;                                 // v_ext's coefficients
+constexpr size_t kOffVpart = kOffVre + kFieldBytes;                         // n, then v_part
+constexpr size_t kOffT = kOffVpart + kFieldBytes;
+constexpr size_t kOffEg = kOffT + align256((size_t)kSMaxAtoms * (3 * kSMaxEdge + 3) * sizeof(float2));
+constexpr size_t kOffG2 = kOffEg + align256(3 * kSMaxEdge * sizeof(double2));
+constexpr size_t kOffIons = kOffG2 + align256(3 * kSMaxEdge * sizeof(float2));
 constexpr size_t kOffZ = kOffIons + align256(3 * kSMaxAtoms * sizeof(double));
 constexpr size_t kOffFrac = kOffZ + align256(kSMaxAtoms * sizeof(double));
 constexpr size_t kOffPart = kOffFrac + align256(3 * kSMaxAtoms * sizeof(float));
@@ -49,14 +48,10 @@ constexpr size_t kOffScal = kOffPart + align256((size_t)kSMaxPart * sizeof(doubl
 constexpr int kEdges[] = {8, 10, 12, 16, 18, 20, 24, 30, 32, 36, 40, 48, 50, 54, 60, 64};   // the path takes
 constexpr size_t kOffEwTab = kOffScal + align256(64 * sizeof(double));
 constexpr size_t kOffEwPart = kOffEwTab + align256((size_t)kEwTabRows * kSMaxAtoms * sizeof(double2));
-// double-float phase tables, v_ext's real-Fourier coefficients and (k b)^2
-constexpr size_t kOffPhaseDD = kOffEwPart + align256(kEwBlocks * sizeof(double));
-constexpr size_t kOffVre = kOffPhaseDD + 2 * kPhaseBytes;
-constexpr size_t kOffG2 = kOffVre + align256((size_t)kSMaxN * sizeof(float2));
 // tensor-core matrices of every edge: derivative per lattice period, forward
 // and inverse real Fourier transform
 constexpr size_t kMatBytes = 768 * 1024;
-constexpr size_t kOffMat = kOffG2 + align256(3 * kSMaxEdge * sizeof(float2));
+constexpr size_t kOffMat = kOffEwPart + align256(kEwBlocks * sizeof(double));
 constexpr size_t kOffTab = kOffMat + kMatBytes;
 constexpr size_t kScratchBytes = kOffTab + align256((size_t)kDdTabSize * sizeof(double));   // + splits
 
@@ -108,31 +103,6 @@ TlAxis axis_matrices(int n, unsigned char *dev)
                 m[k]->mexp = g_mat[i].mexp[k];
             }
     return a;
-}
-
-// The ions of a call, by value in a kernel's arguments: no copy from
-// pageable memory, which would wait for the stream.
-struct Ions {
-    double v[4 * kSMaxAtoms];   // positions, then charges
-    float frac[3 * kSMaxAtoms]; // fractional coordinates in [0, 1]
-};
-// Also (k b)^2 of each axis's real-Fourier coefficients.
-__global__ void k_put_ions(GridInfo g, int nat, const __grid_constant__ Ions ions, double *R, double *Z, float *frac, float2 *g2)
-{
-    const int i = threadIdx.x;
-    if (i < 3 * kSMaxEdge) {
-        const int a = i / kSMaxEdge, j = i - a * kSMaxEdge, n = a == 0 ? g.nx : (a == 1 ? g.ny : g.nz);
-        bool sine;
-        const double k = real_freq(n, j, sine) * (a == 0 ? g.bx : (a == 1 ? g.by : g.bz));
-        const ff::f2 x = ff::from_double(k * k);
-        if (j < n) g2[i] = make_float2(x.hi, x.lo);
-    }
-    if (i < 3 * nat) {
-        R[i] = ions.v[i];
-        frac[i] = ions.frac[i];
-    } else if (i < 4 * nat) {
-        Z[i - 3 * nat] = ions.v[i];
-    }
 }
 
 // Status only: the documented limits say what OFDFT_EINVAL means here.
@@ -195,7 +165,7 @@ double ewald_consts(const double L[3], int nat, const double *Z)
 
 // Textbook Ewald sums on the host, no heap: real-space erfc sum and
 // reciprocal sum over the box of G with |G| < gcut (cells too uneven for
-// launch_ewald_energy's tables).
+// launch_static_ions's tables).
 double ewald_host(const double L[3], int nat, const double *R, const double *Z)
 {
     const double pi = 3.14159265358979323846;
@@ -304,35 +274,29 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
     g.dd = 1;   // double-float transforms and pointwise arithmetic, as ofdft_setup's default
     const double T = T_kelvin * 3.166811563e-6;
 
-    // ions -> Ewald sums; phases -> v_ext(G)
-    double *Rd = (double *)(base + kOffIons), *Zd = (double *)(base + kOffZ);
-    double *scal = (double *)(base + kOffScal);   // 18 sums of the evaluation, then the Ewald sums
-    Ions arg;
-    memcpy(arg.v, ions, 3 * nat * sizeof(double));
-    memcpy(arg.v + 3 * nat, Z, nat * sizeof(double));
-    float *frac = (float *)(base + kOffFrac);
+    // ions -> tables -> Ewald sums and v_ext
     const double L[3] = {g.Lx, g.Ly, g.Lz};
+    StaticIons arg;
+    memcpy(arg.R, ions, 3 * nat * sizeof(double));
+    memcpy(arg.Z, Z, nat * sizeof(double));
     for (int i = 0; i < 3 * nat; ++i) {
         const double f = ions[i] / L[i % 3];
         arg.frac[i] = (float)(f - floor(f));
     }
-    float2 *g2 = (float2 *)(base + kOffG2);
-    k_put_ions<<<1, 4 * kSMaxAtoms, 0, st>>>(g, nat, arg, Rd, Zd, frac, g2);
-    const bool ewald_dev = launch_ewald_energy(nat, Rd, Zd, frac, L, (double2 *)(base + kOffEwTab), (double *)(base + kOffEwPart),
-                                               scal + 18, st);
-    double2 *px = (double2 *)(base + kOffPhase);
-    double2 *py = px + (size_t)nat * g.nx, *pz = py + (size_t)nat * g.ny;
-    double2 *vext = (double2 *)(base + kOffVext);
-    PhaseTablesDD dd;
-    double2 *pd = (double2 *)(base + kOffPhaseDD);
-    dd.xT = pd;
-    dd.yT = pd + (size_t)nat * g.nx;
-    dd.zT = pd + (size_t)nat * (g.nx + g.ny);
-    dd.zd = pd + (size_t)nat * (g.nx + g.ny + g.K);
-    launch_phases(g, nat, Rd, px, py, pz, &dd, st);
-    launch_vext(g, nat, Zd, px, py, pz, &dd, vext, st);
+    StaticIonTables it;
+    it.R = (double *)(base + kOffIons);
+    it.Z = (double *)(base + kOffZ);
+    it.frac = (float *)(base + kOffFrac);
+    it.t = (float2 *)(base + kOffT);
+    it.eg = (double2 *)(base + kOffEg);
+    it.g2 = (float2 *)(base + kOffG2);
+    it.ewtab = (double2 *)(base + kOffEwTab);
+    it.ewpart = (double *)(base + kOffEwPart);
+    float2 *vre = (float2 *)(base + kOffVre);
+    const int newald = launch_static_ions(g, nat, arg, it, vre, st);
 
     const double *tab = (const double *)(base + kOffTab);
+    double *scal = (double *)(base + kOffScal);   // 18 sums of the evaluation, then the Ewald sum
     double *vpart = (double *)(base + kOffVpart);
     double *pA = (double *)(base + kOffPart);
     const bool fttf = fp.kind == 0;
@@ -342,7 +306,7 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
     // fields of div W) through the reciprocal basis, as in a general cell.
     unsigned char *mat = base + kOffMat;
     const TlAxis tl[3] = {axis_matrices(g.nx, mat), axis_matrices(g.ny, mat), axis_matrices(g.nz, mat)};
-    float2 *coef = (float2 *)base, *vre = (float2 *)(base + kOffVre), *nf = (float2 *)vpart;
+    float2 *coef = (float2 *)base, *nf = (float2 *)vpart;
     double *d[3];
     TlPass grad[4], div[3];
     for (int a = 0; a < 3; ++a) {
@@ -352,7 +316,6 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
     }
     const TlPass zf = {TlPass::kForward, 2, &tl[2].fwd, nf, coef};
     grad[3] = zf;
-    launch_real_coefficients(g, vext, vre, st);
     launch_density(g.N, phi_dev, nullptr, 1.0, 0.0, nullptr, nullptr, nf, st);
     launch_tline(g, fttf ? 1 : 4, fttf ? &zf : grad, st);
     for (int a = 1; a >= 0; --a) {
@@ -360,7 +323,7 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
         launch_tline(g, 1, &fwd, st);
     }
     TlHartree hl{};
-    for (int a = 0; a < 3; ++a) hl.g2[a] = g2 + a * kSMaxEdge;
+    for (int a = 0; a < 3; ++a) hl.g2[a] = it.g2 + a * kSMaxEdge;
     hl.ve = vre;
     hl.hr = make_float2(g.hr2[0], g.hr2[1]);
     hl.half_dv = 0.5 * g.dV;
@@ -396,7 +359,7 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
         fin.part = pC;
         nbz = launch_final(g, fin, st);
     }
-    launch_reduce_eval(pA, nbx, pB, nbg, pC, nbz, !fttf, scal, st);
+    launch_reduce_eval(pA, nbx, pB, nbg, pC, nbz, !fttf, scal, st, it.ewpart, newald);
     double h[19];
     SCK(cudaMemcpyAsync(h, scal, sizeof(h), cudaMemcpyDeviceToHost, st), "scalar read-back failed");
     SCK(cudaStreamSynchronize(st), "stream synchronisation failed");
@@ -409,7 +372,7 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
         Ne += Z[i];
         zs += 3.14159265358979323846 * Z[i] * rc * rc;
     }
-    const double E_ion = (ewald_dev ? h[18] : ewald_host(L, nat, ions, Z)) + ewald_consts(L, nat, Z);
+    const double E_ion = (newald ? h[18] : ewald_host(L, nat, ions, Z)) + ewald_consts(L, nat, Z);
     ofdft_energy e;
     memset(&e, 0, sizeof(e));
     e.F_s = dV * f[0];

@@ -148,9 +148,10 @@ template <typename T> cudaError_t set_field_smem_limits(size_t bytes);
 void launch_reduce(const double *part, int nblk, int nq, double *out, cudaStream_t st);
 // The three reductions of an evaluation in one launch: rows 0..2 of pA (na
 // columns) into out[0..2], rows 0..5 of pB (nb columns, GGA only) into
-// out[3..8], rows 0..8 of pC (nc columns) into out[9..17].
+// out[3..8], rows 0..8 of pC (nc columns) into out[9..17]; with ne also the
+// ne sums of pE into out[18].
 void launch_reduce_eval(const double *pA, int na, const double *pB, int nb, const double *pC, int nc, bool gga,
-                        double *out, cudaStream_t st);
+                        double *out, cudaStream_t st, const double *pE = nullptr, int ne = 0);
 template <typename T> void launch_fill(long long n, T *x, T val, cudaStream_t st);
 template <typename T> void launch_scale(long long n, T *x, double s, const double *sp, cudaStream_t st);
 // if *accepted: phi <- phit, v <- vt, gprev <- g; then g = 2 phi (v - *mup);
@@ -238,14 +239,28 @@ void launch_ewald_real(int nat, const double *R, const double *Z, const EwCell &
 int launch_ewald_recip(int nat, const double *R, const double *Z, int nG, const double *Gv,
                        const double *wG, double2 *S, double *epart, double *F, cudaStream_t st);
 
-// Ewald energy of an orthorhombic cell (edges L) without its self and
-// background terms, into out[0]; frac: fractional coordinates in [0, 1],
-// binary32, for screening the pairs; tab is scratch of kEwTabRows nat double2,
-// part of kEwBlocks doubles.  False (nothing launched) for cells so uneven
-// that an axis needs more images or reciprocal planes than fit.
-constexpr int kEwTabRows = 256, kEwBlocks = 304;
-bool launch_ewald_energy(int nat, const double *R, const double *Z, const float *frac, const double L[3], double2 *tab, double *part,
-                         double *out, cudaStream_t st);
+// The ions of the allocation-free entry point, by value in a kernel's
+// arguments (a copy from pageable memory would wait for the stream), and the
+// tables made of them: t nat (nx + ny + nz + 3), eg and g2 3 kStaticEdge,
+// ewtab kEwTabRows nat, ewpart kEwBlocks entries.
+constexpr int kStaticEdge = 64, kStaticAtoms = 64, kEwTabRows = 256, kEwBlocks = 304;
+struct StaticIons {
+    double R[3 * kStaticAtoms], Z[kStaticAtoms];
+    float frac[3 * kStaticAtoms];   // fractional coordinates in [0, 1], for screening the pairs
+};
+struct StaticIonTables {
+    double *R, *Z;
+    float *frac;
+    float2 *t;
+    double2 *eg;
+    float2 *g2;                     // (k b)^2 of each axis's coefficients, kStaticEdge apart
+    double2 *ewtab;
+    double *ewpart;
+};
+// v_ext's coefficients into vre (N) and the Ewald energy, without its self
+// and background terms, as the returned number of sums in ewpart: 0 for cells
+// so uneven that an axis needs more images or reciprocal planes than fit.
+int launch_static_ions(const GridInfo &g, int nat, const StaticIons &ions, const StaticIonTables &t, float2 *vre, cudaStream_t st);
 
 // MD: half step A (thermostat half, kick, drift) and B (kick, thermostat half).
 void launch_md_a(int nat, const double *m, double *R, double *V, const double *F, double dt,

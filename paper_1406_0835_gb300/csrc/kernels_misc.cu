@@ -68,7 +68,8 @@ __global__ void k_reduce(const double *__restrict__ part, int nblk, double *__re
 // of the final z-pass partials (the rest) into out[q] (ftTF: out[9 + r] for
 // final row r), in the same fixed order as k_reduce.
 __global__ void k_reduce_eval(const double *__restrict__ pA, int na, const double *__restrict__ pB, int nb,
-                              const double *__restrict__ pC, int nc, int gga, double *__restrict__ out)
+                              const double *__restrict__ pC, int nc, int gga, const double *__restrict__ pE, int ne,
+                              double *__restrict__ out)
 {
     pdl_enter();
     const int q = blockIdx.x;
@@ -82,6 +83,10 @@ __global__ void k_reduce_eval(const double *__restrict__ pA, int na, const doubl
         p = pB + (size_t)(q - 3) * nb;
         n = nb;
         o = q;
+    } else if (q >= (gga ? 18 : 12)) {
+        p = pE;
+        n = ne;
+        o = 18;
     } else {
         const int r = q - (gga ? 9 : 3);
         p = pC + (size_t)r * nc;
@@ -1187,29 +1192,21 @@ __global__ void k_ewald_F(int nat, const double *__restrict__ R, const double *_
         for (int k = 0; k < 3; ++k) F[3 * I + k] += acc[k];
 }
 
-// Ewald energy alone, for callers without a G list (the allocation-free
-// entry point; orthorhombic cells).  Summed by one host thread it took 1.9
-// of the 2.1 ms of such a call with 32 ions; the two kernels below take
-// about 10 us.  FP64 throughput (2 lanes a clock and SM) is what both parts
-// are arranged for.
+// The ions of the allocation-free entry point (orthorhombic cells, Gaussian
+// ions, at most kStaticAtoms of them), in two launches: k_static_ions makes
+// every table from the ions in its arguments, k_static_sums the Ewald sums in
+// its first blocks and, beside them, v_ext's real-Fourier coefficients.  As a
+// chain of seven kernels (copies, Ewald table, Ewald sums, their reduction,
+// phases, v_ext's spectrum, its coefficients) they took about 60 us of a
+// 165 us call at 24x30x40; that call now takes 126 us, one at 20^3 (ftTF) 97
+// instead of 126.  The Ewald sums alone took 1.9 ms on a host
+// thread.  FP64 throughput (2 lanes a clock and SM) is what their parts are
+// arranged for.
 struct EwBox {
     double L[3], alpha, rcut, gcut, om;
     int ni[3], km[3];
     int off[3];               // first k of each axis in the phase table, [off + k][ion]
 };
-
-__global__ void k_ewald_tab(int nat, EwBox w, const double *__restrict__ R, double2 *__restrict__ tab)
-{
-    pdl_enter();
-    const int rows = w.off[2] + w.km[2] + 1;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nat * rows; i += gridDim.x * blockDim.x) {
-        const int row = i / nat, I = i - row * nat;
-        const int a = row >= w.off[2] ? 2 : (row >= w.off[1] ? 1 : 0);
-        double s, c;
-        sincos(6.283185307179586477 * (row - w.off[a]) / w.L[a] * R[3 * I + a], &s, &c);
-        tab[i] = make_double2(c, s);
-    }
-}
 
 // One pair term of the real-space sum: pair p of the triangle I <= J, image m.
 __device__ __forceinline__ void ew_pair(const EwBox &w, long long q, int nimg, int &I, int &J, int im[3], float &wt)
@@ -1228,23 +1225,21 @@ __device__ __forceinline__ void ew_pair(const EwBox &w, long long q, int nimg, i
     wt = I == J ? 0.5f : 1.0f;
 }
 
-// Blocks [0, gridDim.x / 2): the real-space pairs.  About one pair image in
+// Blocks [0, nblocks / 2): the real-space pairs.  About one pair image in
 // twenty lies within the cutoff, so a warp first screens 32 of them in
 // binary32 and queues those that pass (in lane order: the sum does not
 // depend on scheduling); the binary64 terms run on full warps of the queue.
 // The other blocks: the reciprocal sum over half the G box (-G gives the
 // same term), eight lanes to a G, each over an eighth of the ions.
 constexpr int kEwThreads = 128;
-__global__ void __launch_bounds__(kEwThreads) k_ewald_energy(int nat, EwBox w, const double *__restrict__ R,
-                                                             const double *__restrict__ Z,
-                                                             const float *__restrict__ frac,
-                                                             const double2 *__restrict__ tab, double *__restrict__ part)
+__device__ void ewald_block(int block, int nblocks, int nat, const EwBox &w, const double *__restrict__ R,
+                            const double *__restrict__ Z, const float *__restrict__ frac, const double2 *__restrict__ tab,
+                            double *__restrict__ part)
 {
-    pdl_enter();
-    const int nreal = gridDim.x / 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nreal = nblocks / 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int kW = kEwThreads / 32;
     double acc[1] = {0.0};
-    if ((int)blockIdx.x < nreal) {
+    if (block < nreal) {
         __shared__ long long queue[kW][64];
         const int nimg = (2 * w.ni[0] + 1) * (2 * w.ni[1] + 1) * (2 * w.ni[2] + 1);
         const long long total = (long long)nat * (nat + 1) / 2 * nimg;
@@ -1264,7 +1259,7 @@ __global__ void __launch_bounds__(kEwThreads) k_ewald_energy(int nat, EwBox w, c
         };
         const float rc2 = (float)(w.rcut * w.rcut) * 1.0001f;
         int held = 0;
-        for (long long q0 = ((long long)blockIdx.x * kW + warp) * 32; q0 < total; q0 += (long long)nreal * kW * 32) {
+        for (long long q0 = ((long long)block * kW + warp) * 32; q0 < total; q0 += (long long)nreal * kW * 32) {
             const long long q = q0 + lane;
             bool near = false;
             if (q < total) {
@@ -1302,8 +1297,8 @@ __global__ void __launch_bounds__(kEwThreads) k_ewald_energy(int nat, EwBox w, c
         const int n1 = 2 * w.km[1] + 1, n2 = 2 * w.km[2] + 1;
         const long long half = ((long long)(2 * w.km[0] + 1) * n1 * n2 - 1) / 2;
         const int sub = lane & 7;
-        const long long step = (long long)(gridDim.x - nreal) * kW * 4;
-        for (long long q0 = ((long long)(blockIdx.x - nreal) * kW + warp) * 4; q0 < half; q0 += step) {
+        const long long step = (long long)(nblocks - nreal) * kW * 4;
+        for (long long q0 = ((long long)(block - nreal) * kW + warp) * 4; q0 < half; q0 += step) {
             const long long q = q0 + (lane >> 3);
             const int k2 = (int)(q % n2) - w.km[2], k1 = (int)(q / n2 % n1) - w.km[1], k0 = (int)(q / n2 / n1) - w.km[0];
             const double twopi = 6.283185307179586477;
@@ -1333,7 +1328,101 @@ __global__ void __launch_bounds__(kEwThreads) k_ewald_energy(int nat, EwBox w, c
         }
     }
     block_sum<1>(acc);
-    if (threadIdx.x == 0) part[blockIdx.x] = acc[0];
+    if (threadIdx.x == 0) part[block] = acc[0];
+}
+
+// Tables of every ion I: t = (cosine or sine of each coefficient's frequency
+// along x, y, z, times Z along x; entry n of an axis: the sine of its Nyquist
+// frequency), the Ewald phases exp(i 2 pi k R / L); and of every coefficient:
+// eg = (its axis's share of Omega w(k) G^2 / -4 pi, times the two functions'
+// weight and norm; (k b)^2), g2 = (k b)^2 as a pair.
+__global__ void k_static_ions(GridInfo g, int nat, const __grid_constant__ StaticIons ions, EwBox w, int ewrows,
+                              StaticIonTables t)
+{
+    pdl_enter();
+    const int n3[3] = {g.nx, g.ny, g.nz};
+    const double b3[3] = {g.bx, g.by, g.bz};
+    const int per = g.nx + g.ny + g.nz + 3, nt = nat * per, ne = nat * ewrows;
+    const int total = nt + ne + 3 * kStaticEdge + 4 * kStaticAtoms;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        double s, c;
+        if (i < nt) {
+            const int I = i / per;
+            int j = i - I * per, a = 0;
+            while (j > n3[a]) j -= n3[a++] + 1;
+            const int n = n3[a];
+            bool sine = true;
+            const int k = j < n ? real_freq(n, j, sine) : n / 2;
+            sincos(k * b3[a] * ions.R[3 * I + a], &s, &c);
+            const double f = sine ? s : c;
+            const ff::f2 x = ff::from_double(a == 0 ? f * ions.Z[I] : f);
+            t.t[i] = make_float2(x.hi, x.lo);
+        } else if (i < nt + ne) {
+            const int q = i - nt, row = q / nat, I = q - row * nat;
+            const int a = row >= w.off[2] ? 2 : (row >= w.off[1] ? 1 : 0);
+            sincos(6.283185307179586477 * (row - w.off[a]) / w.L[a] * ions.R[3 * I + a], &s, &c);
+            t.ewtab[q] = make_double2(c, s);
+        } else if (i < nt + ne + 3 * kStaticEdge) {
+            const int q = i - nt - ne, a = q / kStaticEdge, j = q - a * kStaticEdge, n = n3[a];
+            if (j >= n) continue;
+            bool sine;
+            const int k = real_freq(n, j, sine);
+            const double kb = k * b3[a], k2 = kb * kb;
+            t.eg[q] = make_double2(exp(-0.25 * k2 * g.rc * g.rc) * sqrt((double)n * (k == 0 || 2 * k == n ? 1.0 : 2.0)), k2);
+            const ff::f2 x = ff::from_double(k2);
+            t.g2[q] = make_float2(x.hi, x.lo);
+        } else {
+            const int q = i - nt - ne - 3 * kStaticEdge;
+            if (q < 3 * nat) {
+                t.R[q] = ions.R[q];
+                t.frac[q] = ions.frac[q];
+            } else if (q < 4 * nat) {
+                t.Z[q - 3 * nat] = ions.Z[q - 3 * nat];
+            }
+        }
+    }
+}
+
+// Blocks [0, newald): Ewald.  The others: one coefficient of v_ext a thread,
+// N w(k) sum_I Z f_a f_b f_c over the orthonormal functions' norms.  On two
+// or three Nyquist frequencies, whose v_ext is the mean over G and its
+// partner G', the cosines' product is the cosine of the sum of the phases.
+__global__ void __launch_bounds__(kEwThreads) k_static_sums(GridInfo g, int nat, EwBox w, int newald, StaticIonTables t,
+                                                            float2 *__restrict__ vre)
+{
+    pdl_enter();
+    if ((int)blockIdx.x < newald) {
+        ewald_block(blockIdx.x, newald, nat, w, t.R, t.Z, t.frac, t.ewtab, t.ewpart);
+        return;
+    }
+    const int q = (blockIdx.x - newald) * blockDim.x + threadIdx.x;
+    if (q >= (int)g.N) return;
+    const int c = q % g.nz, ab = q / g.nz, b = ab % g.ny, a = ab / g.ny;
+    const double2 ex = t.eg[a], ey = t.eg[kStaticEdge + b], ez = t.eg[2 * kStaticEdge + c];
+    const double k2 = ex.y + ey.y + ez.y;
+    const int per = g.nx + g.ny + g.nz + 3, oy = g.nx + 1, oz = oy + g.ny + 1;
+    bool s;
+    const bool qx = 2 * real_freq(g.nx, a, s) == g.nx, qy = 2 * real_freq(g.ny, b, s) == g.ny, qz = 2 * real_freq(g.nz, c, s) == g.nz;
+    ff::f2 sum(0.0f, 0.0f);
+    const float2 *p = t.t;
+    if ((int)qx + (int)qy + (int)qz < 2) {
+#pragma unroll 2
+        for (int I = 0; I < nat; ++I, p += per) {
+            const float2 x = p[a], y = p[oy + b], z = p[oz + c];
+            sum = ff::add(sum, ff::mul(ff::mul(ff::f2(x.x, x.y), ff::f2(y.x, y.y)), ff::f2(z.x, z.y)));
+        }
+    } else {
+        const ff::f2 z0(0.0f, 0.0f);
+        auto at = [&](int j, int n, bool nyq) {
+            const float2 u = p[j], v = p[n];
+            return ff::cf2{ff::f2(u.x, u.y), nyq ? ff::f2(v.x, v.y) : z0};
+        };
+        for (int I = 0; I < nat; ++I, p += per)
+            sum = ff::add(sum, ff::cmul(ff::cmul(at(a, g.nx, qx), at(oy + b, oy + g.ny, qy)), at(oz + c, oz + g.nz, qz)).x);
+    }
+    const double v = k2 > 0.0 ? ff::to_double(sum) * ex.x * ey.x * ez.x * (-12.566370614359172954 / (g.omega * k2)) : 0.0;
+    const ff::f2 o = ff::from_double(v);
+    vre[q] = make_float2(o.hi, o.lo);
 }
 
 // ------------------------------------------------------------------- MD
@@ -1423,30 +1512,33 @@ void launch_force_coefficients(const GridInfo &g, const double2 *nG, float2 *coe
     pdl_launch(k_real_coefficients<true>, octant_blocks(g), 128, 0, st, g, nG, coef);
 }
 
-bool launch_ewald_energy(int nat, const double *R, const double *Z, const float *frac, const double L[3], double2 *tab, double *part,
-                         double *out, cudaStream_t st)
+int launch_static_ions(const GridInfo &g, int nat, const StaticIons &ions, const StaticIonTables &t, float2 *vre, cudaStream_t st)
 {
     const double pi = 3.14159265358979323846;
-    EwBox w;
+    const double L[3] = {g.Lx, g.Ly, g.Lz};
+    EwBox w{};
     w.om = L[0] * L[1] * L[2];
     w.alpha = 1.2 * sqrt(pi) * pow((double)nat / (w.om * w.om), 1.0 / 6.0);
     w.rcut = 6.3 / w.alpha;
     w.gcut = 2.0 * w.alpha * 6.3;
     int rows = 0;
-    for (int a = 0; a < 3; ++a) {
+    bool ewald = true;
+    for (int a = 0; a < 3 && ewald; ++a) {
         const double ni = ceil(w.rcut / L[a] + 0.5), km = ceil(w.gcut * L[a] / (2.0 * pi));
-        if (!(ni <= 512.0) || !(km + 1 + rows <= (double)kEwTabRows)) return false;
+        ewald = ni <= 512.0 && km + 1 + rows <= (double)kEwTabRows;
+        if (!ewald) break;
         w.L[a] = L[a];
         w.ni[a] = (int)ni;
         w.km[a] = (int)km;
         w.off[a] = rows;
         rows += w.km[a] + 1;
     }
-    if ((double)(2 * w.ni[0] + 1) * (2 * w.ni[1] + 1) * (2 * w.ni[2] + 1) > 1e6) return false;
-    pdl_launch(k_ewald_tab, (nat * rows + 127) / 128, 128, 0, st, nat, w, R, tab);
-    pdl_launch(k_ewald_energy, kEwBlocks, kEwThreads, 0, st, nat, w, R, Z, frac, tab, part);
-    pdl_launch(k_reduce, 1, 256, 0, st, part, kEwBlocks, out);
-    return true;
+    if (ewald && (double)(2 * w.ni[0] + 1) * (2 * w.ni[1] + 1) * (2 * w.ni[2] + 1) > 1e6) ewald = false;
+    const int ewrows = ewald ? rows : 0, newald = ewald ? kEwBlocks : 0;
+    const int items = nat * (g.nx + g.ny + g.nz + 3 + ewrows) + 3 * kStaticEdge + 4 * kStaticAtoms;
+    pdl_launch(k_static_ions, (items + 127) / 128, 128, 0, st, g, nat, ions, w, ewrows, t);
+    pdl_launch(k_static_sums, newald + (int)((g.N + kEwThreads - 1) / kEwThreads), kEwThreads, 0, st, g, nat, w, newald, t, vre);
+    return newald;
 }
 
 void launch_andersen(int nat, const double *m, double *V, double kT, double prob, const double *u,
@@ -1461,9 +1553,9 @@ void launch_reduce(const double *part, int nblk, int nq, double *out, cudaStream
 }
 
 void launch_reduce_eval(const double *pA, int na, const double *pB, int nb, const double *pC, int nc, bool gga,
-                        double *out, cudaStream_t st)
+                        double *out, cudaStream_t st, const double *pE, int ne)
 {
-    pdl_launch(k_reduce_eval, gga ? 18 : 12, 256, 0, st, pA, na, pB, nb, pC, nc, gga ? 1 : 0, out);
+    pdl_launch(k_reduce_eval, (gga ? 18 : 12) + (ne > 0), 256, 0, st, pA, na, pB, nb, pC, nc, gga ? 1 : 0, pE, ne, out);
 }
 
 template <typename T> void launch_fill(long long n, T *x, T val, cudaStream_t st)
