@@ -207,10 +207,9 @@ template <typename T> ofdft_status upload_twiddles(ofdft_ctx *c, FieldSet &f, in
 
 // The derivative passes of a double-float GGA set take the tensor cores along
 // every axis that they support; the Hartree chain does when all three axes
-// are supported and the cell is orthorhombic (4 pi / G^2 is diagonal in
-// products of cosines and sines only there).  ftTF has the chain alone and
-// five kernels more in this form, which on the smallest grids cost more than
-// they save, FFT passes -> here: an evaluation at 8^3 51 -> 56 us, 16^3 62 ->
+// are supported.  ftTF has the chain alone and five kernels more in this
+// form, which on the smallest grids cost more than they save, FFT passes ->
+// here: an evaluation at 8^3 51 -> 56 us, 16^3 62 ->
 // 55, 32^3 64 -> 58, 48^3 73 -> 70, 54^3 86 -> 79, a solve's evaluation at
 // 32^3 119 -> 102 us.  (GGA: 96^3 291 -> 255 us, 48^3 95 -> 92, 32^3 72 -> 73
 // before the launches of a chain overlapped.)
@@ -219,7 +218,7 @@ bool tl_derivatives(const ofdft_ctx *c, int n) { return c->g.dd && !c->g.dws && 
 bool tl_real_basis(const ofdft_ctx *c)
 {
     const GridInfo &g = c->g;
-    return g.dd && !g.dws && !g.tri && (c->fp.kind != 0 || g.N >= kRealTfPoints) && tline_supported(g.nx) &&
+    return g.dd && !g.dws && (c->fp.kind != 0 || g.N >= kRealTfPoints) && tline_supported(g.nx) &&
            tline_supported(g.ny) && tline_supported(g.nz);
 }
 
@@ -291,7 +290,7 @@ ofdft_status setup_tline(ofdft_ctx *c, FieldSet &f)
     }
     CK(cudaMemcpyAsync(f.tlmem, h.data(), bytes, cudaMemcpyHostToDevice, c->st));
     if (f.real_basis)
-        CK(cudaMallocAsync((void **)&f.vre, (size_t)(g.lpp ? 2 : 1) * g.N * sizeof(float2), c->st));
+        CK(cudaMallocAsync((void **)&f.vre, (size_t)(g.lpp || g.tri ? 2 : 1) * g.N * sizeof(float2), c->st));
     return OFDFT_OK;
 }
 
@@ -464,11 +463,11 @@ ofdft_status enqueue_real(ofdft_ctx *c, FieldSet &f, double *ph, const double *p
         TlHartree hl{};
         for (int a = 0; a < 3; ++a) hl.g2[a] = f.tl[a].g2;
         hl.ve = f.vre;
-        hl.vp = g.lpp ? f.vre + g.N : nullptr;
+        hl.vp = g.lpp || g.tri ? f.vre + g.N : nullptr;
         hl.hr = make_float2(g.hr2[0], g.hr2[1]);
         hl.half_dv = 0.5 * g.dV;
         hl.dv = g.dV;
-        hl.ploc = g.dV / g.omega * (g.lpp ? 1.0 : 1.0 / 3.0);
+        hl.ploc = g.dV / g.omega * (g.lpp || g.tri ? 1.0 : 1.0 / 3.0);
         hl.part = pA;
         nbx = launch_hartree(g, coef, hl, sh);
         launch_tline(g, 1, &inv, sh);
@@ -794,8 +793,8 @@ ofdft_status update_ions(ofdft_ctx *c)
     launch_vext(g, c->nat, c->Zd, c->px, c->py, c->pz, dd, (double2 *)c->f[0].vext, st);
     if (c->f[0].real_basis) {
         launch_real_coefficients(g, (const double2 *)c->f[0].vext, c->f[0].vre, st);
-        if (g.lpp) launch_real_coefficients(g, (const double2 *)c->f[0].vext + g.NH, c->f[0].vre + g.N, st);
-        c->launches += g.lpp ? 2 : 1;
+        if (g.lpp || g.tri) launch_real_coefficients(g, (const double2 *)c->f[0].vext + g.NH, c->f[0].vre + g.N, st);
+        c->launches += g.lpp || g.tri ? 2 : 1;
     }
     if (c->f[1].valid)
         launch_convert<double, float>(((g.lpp || g.tri) ? 4 : 2) * g.NH, (const double *)c->f[0].vext, (float *)c->f[1].vext,

@@ -87,8 +87,8 @@ void launch_tline(const GridInfo &g, int count, const TlPass *pass, cudaStream_t
 // coef: coefficients of n -> of v_HL = 4 pi n / G^2 + v_ext; partials E_H,
 // E_loc, P_loc in three rows of the returned number of columns.
 struct TlHartree {
-    const float2 *g2[3];       // (k b)^2 per coefficient and axis
-    const float2 *ve, *vp;     // v_ext's coefficients; pressure weights or null (Gaussian ion)
+    const float2 *g2[3];       // (k b)^2 per coefficient and axis (orthorhombic cells)
+    const float2 *ve, *vp;     // v_ext's coefficients; pressure weights or null (Gaussian ion, orthorhombic cell)
     float2 hr;                 // rc^2 / 2
     double half_dv, dv, ploc;  // factors of the three sums
     double *part;
@@ -109,7 +109,7 @@ int launch_ptf(const GridInfo &g, const float2 *vhl, const double *phit, const d
                double s, const double *cs, double temp, const FuncParams &fp, const double *tab, int xc, double *vout,
                double *part, cudaStream_t st);
 // Real-Fourier coefficients (pairs) of the real field whose half spectrum is
-// v (orthorhombic cells; the spectrum's Nyquist planes Hermitian).
+// v (its Nyquist planes Hermitian).
 void launch_real_coefficients(const GridInfo &g, const double2 *v, float2 *coef, cudaStream_t st);
 // Pointwise functional + XC: reads phi and the derivatives of n in d0..d2,
 // writes v_part and, over d0..d2, the fields U_j whose derivatives sum to

@@ -1,13 +1,19 @@
 // Grid-field kernels of one energy + potential evaluation.
 //
-// A real field is transformed in three passes: z (real-to-complex, two real
-// lines packed in one complex line), y and x (complex, on column tiles of
-// the half spectrum [ix][iy][kz]).  The G-space work (Hartree, local
-// pseudopotential, i G n(G), i G.W(G)) is fused into the x pass and the
-// pointwise functional into the z pass, so one GGA evaluation is
-//   zfwd(n = phi^2) -> y -> x[grad] -> y^-1 (3) -> z[pointwise, W] -> y (3)
-//   -> x[div] -> y^-1 -> z^-1[potential, reductions]
-// (ftTF: zfwd -> y -> x[v_HL] -> y^-1 -> z^-1[pointwise, potential]).
+// Two forms.  Double-float field sets whose edges the tensor-core transforms
+// take (kernels_tline.cu; up to 144) run in the real Fourier basis, with the
+// elementwise kernels of this file between the transforms:
+//   k_density -> [d_x, d_y, d_z and forward z] -> y -> x -> k_hartree (or
+//   _tri) -> x^-1 -> y^-1 -> z^-1;  k_pw;  [d_x, d_y, d_z of U] -> k_final
+// (ftTF: the chain without derivatives, then k_ptf).
+// FP32 and binary64 sets, longer edges and the smallest ftTF grids take FFT
+// passes: z (real-to-complex, two real lines packed in one complex line), y
+// and x (complex, on column tiles of the half spectrum [ix][iy][kz]), with
+// the G-space work (Hartree, local pseudopotential) fused into the x pass
+// and derivatives along one axis at a time:
+//   k_zfwd (n = phi^2, d_z n) -> k_ypass -> k_xhl -> k_ypass^-1;  k_dline x,
+//   y;  k_pw;  k_dline y, x;  k_zfinal_g (d_z U_z, potential, reductions)
+// (ftTF: k_zfwd -> k_ypass -> k_xhl -> k_ypass^-1 -> k_zfinal).
 //
 // Every kernel is written once for a precision tag PR: float and double
 // compute in their own type; DD keeps the fields in binary64 in memory and
@@ -1186,6 +1192,80 @@ __global__ void __launch_bounds__(256) k_hartree(GridInfo g, float4 *__restrict_
     }
 }
 
+// The same in a general cell.  4 pi / G^2 is not diagonal in products of the
+// axes' cosines and sines there, but it is in the plane waves that the up to
+// eight coefficients of one (|kx|, |ky|, |kz|) span: with K(s_x, s_y) its
+// value at (s_x kx, s_y ky, kz), K = k0 + s_x s_y k1 + s_x s_z k2 + s_y s_z k3
+// for the four sign pairs, and s_x s_y acts on the functions as cos cos <->
+// -sin sin, cos sin <-> sin cos.  A frequency 0 or n/2 has no sine: the sign
+// of its axis averages out, except that on two or three Nyquist axes, where
+// the spectrum takes the mean over G and its partner of opposite Nyquist
+// components, the product of two such signs stays 1.  A thread does one set
+// of eight.  A solve's evaluation in a sheared cell, FFT passes -> with this:
+// GGA 60 x 54 x 72 138 -> 120 us, 96^3 309 -> 259, ftTF 16^3 68 -> 58, 96^3
+// 198 -> 156.
+__global__ void __launch_bounds__(128) k_hartree_tri(GridInfo g, float2 *__restrict__ coef, TlHartree hl)
+{
+    pdl_enter();
+    constexpr ff::f2 fpi(kFourPi);
+    const ff::f2 z0(0.0f, 0.0f);
+    const RecipB<DD, true> rb(g);
+    ff::f2 acc[3] = {z0, z0, z0};
+    const int hx = g.nx / 2, hy = g.ny / 2, hz = g.nz / 2, total = (hx + 1) * (hy + 1) * (hz + 1);
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
+        const int kz = q % (hz + 1), xy = q / (hz + 1), ky = xy % (hy + 1), kx = xy / (hy + 1);
+        const bool ex = kx == 0 || kx == hx, ey = ky == 0 || ky == hy, ez = kz == 0 || kz == hz;
+        const size_t at = ((size_t)real_cosine(g.nx, kx) * g.ny + real_cosine(g.ny, ky)) * g.nz + real_cosine(g.nz, kz);
+        if (q == 0) {
+            coef[at] = make_float2(0.0f, 0.0f);
+            continue;
+        }
+        ff::f2 x[8];                                   // [x][y][z], 0: cosine, 1: sine
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const bool there = !((i & 4) && ex) && !((i & 2) && ey) && !((i & 1) && ez);
+            x[i] = there ? f2of(coef[at + (size_t)(i >> 2) * g.ny * g.nz + (i >> 1 & 1) * g.nz + (i & 1)]) : z0;
+        }
+        ff::f2 K[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float fx = i & 2 ? -(float)kx : (float)kx, fy = i & 1 ? -(float)ky : (float)ky, fz = (float)kz;
+            const ff::f2 gx = ff::mul(rb.b[0], fx) + ff::mul(rb.b[3], fy) + ff::mul(rb.b[6], fz);
+            const ff::f2 gy = ff::mul(rb.b[1], fx) + ff::mul(rb.b[4], fy) + ff::mul(rb.b[7], fz);
+            const ff::f2 gz = ff::mul(rb.b[2], fx) + ff::mul(rb.b[5], fy) + ff::mul(rb.b[8], fz);
+            K[i] = ff::div(fpi, gx * gx + gy * gy + gz * gz);
+        }
+        const ff::f2 s0 = K[0] + K[3], s1 = K[1] + K[2], d0 = K[0] - K[3], d1 = K[1] - K[2];
+        ff::f2 k0 = ff::scale(s0 + s1, 0.25f);
+        const ff::f2 k1 = ff::scale(s0 - s1, 0.25f), k2 = ff::scale(d0 + d1, 0.25f), k3 = ff::scale(d0 - d1, 0.25f);
+        const bool qx = kx == hx, qy = ky == hy, qz = kz == hz;
+        if (qx && qy) k0 = k0 + k1;
+        if (qx && qz) k0 = k0 + k2;
+        if (qy && qz) k0 = k0 + k3;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (((i & 4) && ex) || ((i & 2) && ey) || ((i & 1) && ez)) continue;
+            const bool tx = i >> 2, ty = i >> 1 & 1, tz = i & 1;
+            const ff::f2 a = ff::mul(k1, x[i ^ 6]), b = ff::mul(k2, x[i ^ 5]), c = ff::mul(k3, x[i ^ 3]);
+            const ff::f2 hc = ff::mul(k0, x[i]) + (tx == ty ? ff::neg(a) : a) + (tx == tz ? ff::neg(b) : b) + (ty == tz ? ff::neg(c) : c);
+            const size_t o = at + (size_t)(i >> 2) * g.ny * g.nz + (i >> 1 & 1) * g.nz + (i & 1);
+            const ff::f2 ve = f2of(hl.ve[o]);
+            acc[0] += ff::mul(hc, x[i]);
+            acc[1] += ff::mul(x[i], ve);
+            acc[2] += ff::mul(x[i], f2of(hl.vp[o]));
+            const ff::f2 w = hc + ve;
+            coef[o] = make_float2(w.hi, w.lo);
+        }
+    }
+    double tot[3];
+    block_sum_f2<3>(acc, tot);
+    if (threadIdx.x == 0) {
+        hl.part[blockIdx.x] = hl.half_dv * tot[0];
+        hl.part[(size_t)gridDim.x + blockIdx.x] = hl.dv * tot[1];
+        hl.part[(size_t)2 * gridDim.x + blockIdx.x] = hl.ploc * tot[2];
+    }
+}
+
 // GGA potential v = v_HL + v_part - (d_x U_x + d_y U_y + d_z U_z) and the sums
 // of phi^2 v, phi^2 and 2 phi v dphi/dtheta (partials as k_zfinal_g's).
 __global__ void __launch_bounds__(256) k_final(GridInfo g, TlFinal f)
@@ -1334,6 +1414,12 @@ int pair_blocks(const GridInfo &g)
 int launch_hartree(const GridInfo &g, float2 *coef, const TlHartree &hl, cudaStream_t st)
 {
     // partial rows of at most one column per four half-spectrum columns of the yz plane
+    if (g.tri) {
+        const int total = (g.nx / 2 + 1) * (g.ny / 2 + 1) * g.K;
+        const int blocks = std::min(std::min((total + 127) / 128, 1216), g.ny * ((g.K + 3) / 4));
+        pdl_launch(k_hartree_tri, blocks, 128, 0, st, g, coef, hl);
+        return blocks;
+    }
     const int blocks = std::min(pair_blocks(g), g.ny * ((g.K + 3) / 4));
     pdl_launch(k_hartree, blocks, 256, 0, st, g, (float4 *)coef, hl);
     return blocks;

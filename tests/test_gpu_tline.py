@@ -89,3 +89,24 @@ def test_a_non_finite_density_is_refused(bad):
 def test_fttf_grids_on_both_sides_of_the_rule(grid):
     """2048 points and more take the real basis; 1920 keep the FFT passes."""
     check(grid, functional="fttf")
+
+
+@pytest.mark.parametrize("functional,lpp", [("fttf", "gauss"), ("vt84f", "ha")])
+@pytest.mark.parametrize("grid", [(8, 16, 16), (10, 18, 30), (36, 20, 8), (12, 50, 18)])
+def test_real_basis_in_sheared_cells(grid, functional, lpp):
+    """Every Nyquist plane, line and corner carries weight (rough density) and
+    the cell has no right angle."""
+    cfg = inputs.config_single_point()
+    L = np.array(cfg["L"])
+    cell = np.diag(L) + np.array([[0.0, 0.3, -0.2], [0.8, 0.0, 0.4], [-0.5, 0.9, 0.0]])
+    ions = (cfg["ions"] / L) @ cell
+    so = O.System(None, grid, ions, cfg["Z"], cfg["T"], functional, cell=cell, lpp=lpp)
+    phi = so.uniform_phi() * (1.0 + 0.1 * np.random.default_rng(sum(grid)).standard_normal(grid))
+    ev = O.evaluate(so, phi)
+    with ofdft.Context(None, grid, ions, cfg["Z"], cfg["T"], functional, cell=cell, lpp=lpp) as ctx:
+        E, v = ctx.energy_potential(phi)
+    for k in ("F_tot", "F_s", "F_xc", "E_H", "E_loc"):
+        assert abs(E[k] - ev[k]) <= 1e-10 * abs(ev["F_tot"]), (k, E[k], ev[k])
+    for k in ("P", "P_loc"):
+        assert abs(E[k] - ev[k]) <= 1e-9 * abs(ev["P"]), (k, E[k], ev[k])
+    assert np.max(np.abs(v - ev["v"])) <= 1e-9 * np.max(np.abs(ev["v"]))
