@@ -217,7 +217,7 @@ def kernel_model(name, g, fttf=False):
     if name == "pw":           # pointwise functional: phi, 3 derivatives in; v_part, 3 U out
         flops = POINTWISE_FLOP * N
         byts = 8 * N * 8
-    elif name == "dline":      # one derivative along x or y: forward + inverse line transforms
+    elif name == "dline":      # per axis, as the FFT passes count it: forward + inverse line transforms
         n = (nx + ny) / 2.0
         flops = 2 * (N / 2 / n) * fft_flops(n)
         byts = 8 * N * 2                                   # field in, derivative out

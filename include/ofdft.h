@@ -345,9 +345,11 @@ ofdft_status ofdft_sizes(ofdft_ctx *ctx, long long *N, int *nat);
 /*
  * Diagnostics: record CUDA events around every launch of one kernel class on
  * the context's stream (no extra synchronisation).  id: 0 off,
- * 1 pointwise GGA functional, 2 derivative passes along x and y (gradient of
- * n, divergence of W), 4 y pass, 5 z forward pass, 6 z final pass, 7 x pass
- * of the Hartree and local-pseudopotential potential; id + 8 times only the
+ * 1 pointwise GGA functional, 2 derivative passes (gradient of n, divergence
+ * of W; on the tensor cores one launch of all axes, the gradient's with the
+ * forward z transform), 4 y pass, 5 z forward pass (density), 6 z final pass
+ * (inverse z; potential and sums), 7 x passes of the Hartree and
+ * local-pseudopotential potential; id + 8 times only the
  * class's FP32 launches, id + 16 only its FP64 ones.  ofdft_timer_read
  * synchronises the stream,
  * returns the summed event time (ms) and the launch count, and optionally

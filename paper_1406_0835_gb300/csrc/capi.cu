@@ -410,8 +410,7 @@ void launch_derivatives(const GridInfo &g, const FieldSet &f, const double *cons
     launch_tline(g, n, p, st);
 }
 
-// Real-basis form (double-float sets, orthorhombic, every axis on the tensor
-// cores): n as a field; its three derivatives and its z transform in one
+// Real-basis form (double-float sets with every axis on the tensor cores): n as a field; its three derivatives and its z transform in one
 // launch; y, x, Hartree and LPP terms and energies, x^-1, y^-1, z^-1 beside
 // the pointwise stage and the divergence's three derivatives; potential and
 // sums.  ftTF: the chain alone, then the pointwise stage.
