@@ -837,7 +837,7 @@ __global__ void OFDFT_FFT_BOUNDS k_dline_ws(GridInfo g, FftAxis fa, const typena
 // sum n(v_xc - eps_xc); with STRESS also sum W_a d_b n for ab = xx, yy,
 // zz, xy, xz, yz (the gradient part of Eq. (stressTF_b)) in rows 6..11.
 // The double-float form is bound by instruction issue (73 % of the issue
-// slots at 96^3, 2,470 instructions a point, 79 us).  From 3,060 and 118 us:
+// slots at 96^3, 2,350 instructions a point, 78 us).  From 3,060 and 118 us:
 // polynomial steps without renormalisation, quotients and roots from one
 // reciprocal (a quarter of the instructions), the PZ81 logarithm from a
 // table instead of an exponential, sums of like terms without the
