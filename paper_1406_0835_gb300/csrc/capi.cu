@@ -205,28 +205,12 @@ template <typename T> ofdft_status upload_twiddles(ofdft_ctx *c, FieldSet &f, in
     return OFDFT_OK;
 }
 
-// The derivative passes of a double-float GGA set take the tensor cores along
-// every axis that they support; the Hartree chain does when all three axes
-// are supported.  ftTF has the chain alone and five kernels more in this
-// form, which on the smallest grids cost more than they save, FFT passes ->
-// here: an evaluation at 8^3 51 -> 56 us, 16^3 62 ->
-// 55, 32^3 64 -> 58, 48^3 73 -> 70, 54^3 86 -> 79, a solve's evaluation at
-// 32^3 119 -> 102 us.  (GGA: 96^3 291 -> 255 us, 48^3 95 -> 92, 32^3 72 -> 73
-// before the launches of a chain overlapped.)
-constexpr long long kRealTfPoints = 2048;
-bool tl_derivatives(const ofdft_ctx *c, int n) { return c->g.dd && !c->g.dws && c->fp.kind != 0 && tline_supported(n); }
-bool tl_real_basis(const ofdft_ctx *c)
-{
-    const GridInfo &g = c->g;
-    return g.dd && !g.dws && (c->fp.kind != 0 || g.N >= kRealTfPoints) && tline_supported(g.nx) &&
-           tline_supported(g.ny) && tline_supported(g.nz);
-}
-
 ofdft_status setup_tline(ofdft_ctx *c, FieldSet &f)
 {
     const GridInfo &g = c->g;
     const int n3[3] = {g.nx, g.ny, g.nz};
-    f.real_basis = tl_real_basis(c);
+    const TlPlan plan = tline_plan(g, c->fp.kind != 0);
+    f.real_basis = plan.real_basis;
     size_t bytes = 0;
     auto place = [&](size_t b) {
         const size_t at = bytes;
@@ -244,7 +228,7 @@ ofdft_status setup_tline(ofdft_ctx *c, FieldSet &f)
                 at[a][2] = at[o][2];
                 if (g.ds[o] == g.ds[a]) at[a][0] = at[o][0];
             }
-        if (tl_derivatives(c, n3[a]) && at[a][0] == (size_t)-1) at[a][0] = place(mb);
+        if (plan.der[a] && at[a][0] == (size_t)-1) at[a][0] = place(mb);
         if (f.real_basis) {
             if (at[a][1] == (size_t)-1) {
                 at[a][1] = place(mb);
@@ -285,8 +269,6 @@ ofdft_status setup_tline(ofdft_ctx *c, FieldSet &f)
             }
             f.tl[a].g2 = (const float2 *)(dev + at[a][3]);
         }
-        // units of cells beyond any real one would leave binary32's exponents
-        if (f.tl[a].der.img && (f.tl[a].der.mexp > 68 || f.tl[a].der.mexp < -60)) f.tl[a].der = TlMat{};
     }
     CK(cudaMemcpyAsync(f.tlmem, h.data(), bytes, cudaMemcpyHostToDevice, c->st));
     if (f.real_basis)

@@ -69,6 +69,12 @@ struct TlAxis {
     const float2 *g2 = nullptr;
 };
 bool tline_supported(int n);
+bool tline_derivative_supported(int n, double scale);
+struct TlPlan {
+    bool der[3];        // derivatives along the axis
+    bool real_basis;    // the Hartree chain in the real Fourier basis
+};
+TlPlan tline_plan(const GridInfo &g, bool gga);
 size_t tline_matrix_bytes(int n);
 // Fill img (tline_matrix_bytes(n)) and return the exponent: the derivative
 // times scale; the orthonormal real Fourier transform, or its inverse.

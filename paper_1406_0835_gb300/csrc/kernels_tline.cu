@@ -396,6 +396,39 @@ bool tline_supported(int n)
     return s.nslot >= 2 && kDig * s.np <= 512 && kLines * s.nc <= kTlThreads;
 }
 
+// The derivative matrix's largest entry is scale / (2 sin(2 pi / n)), both
+// blocks' sums of cot and tan; its exponent has to keep a line's scale (2^-100
+// to 2^127, times 2^(44 - mexp)) within binary32.  Grid spacings from 2^14
+// bohr leave that range.
+bool tline_derivative_supported(int n, double scale)
+{
+    if (!tline_supported(n)) return false;
+    int e = 0;
+    frexp(fabs(scale) / (2.0 * sin(6.283185307179586477 / n)), &e);
+    return 54 - e >= -60 && 54 - e <= 68;
+}
+
+// A double-float set's transforms: the derivatives of a GGA take the tensor
+// cores along every axis that they support; the Hartree chain does when all
+// three axes (and for a GGA their derivatives) are supported.  ftTF has the
+// chain alone and five kernels more in this form, which on the smallest grids
+// cost more than they save, FFT passes -> here: an evaluation at 8^3 51 -> 56
+// us, 16^3 62 -> 55, 32^3 64 -> 58, 48^3 73 -> 70, 54^3 86 -> 79, a solve's
+// evaluation at 32^3 119 -> 102 us.  (GGA: 96^3 291 -> 255 us, 48^3 95 -> 92,
+// 32^3 72 -> 73 before the launches of a chain overlapped.)
+constexpr long long kRealTfPoints = 2048;
+TlPlan tline_plan(const GridInfo &g, bool gga)
+{
+    const int n3[3] = {g.nx, g.ny, g.nz};
+    const bool on = g.dd && !g.dws;
+    TlPlan p{{false, false, false}, on && (gga || g.N >= kRealTfPoints)};
+    for (int a = 0; a < 3; ++a) {
+        p.der[a] = on && gga && tline_derivative_supported(n3[a], g.ds[a] * n3[a]);
+        p.real_basis = p.real_basis && (gga ? p.der[a] : tline_supported(n3[a]));
+    }
+    return p;
+}
+
 size_t tline_matrix_bytes(int n)
 {
     const TlShape s = tl_shape(n);
