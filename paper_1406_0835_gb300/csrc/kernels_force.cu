@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kForceThreads, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int group = blockIdx.x / kblocks, kb = blockIdx.x - group * kblocks;
     const int nbt = (g.ny + kRows - 1) / kRows, tiles = g.nx * nbt;
-    pdl_enter();
+    pdl_wait();
     if (tid == 0) {
         s_bad = 0;
         tc::mbar_init(b_a, 1);
@@ -206,6 +206,7 @@ __global__ void __launch_bounds__(kForceThreads, 1)
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
+    pdl_trigger();                                     // the block has its tensor memory: see pdl.cuh
     const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
 
     if (warp < kReadWarps) {

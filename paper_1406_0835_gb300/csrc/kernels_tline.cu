@@ -231,6 +231,7 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
         }
         __syncwarp();
         tc::tmem_alloc(tc::smem_addr(&s_tmem), sh.cols);
+        pdl_trigger();                             // not before: see pdl.cuh
         __syncwarp();
         tc::fence_before_sync();
         bar_arrive(4, blockDim.x);                 // barriers and tensor memory are there
@@ -264,7 +265,7 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
     const long long ln_off = (w_ok ? ou * jb.ostride + (zaxis ? 0 : ln - ou * zlen) : 0) + (half ? h * rstride : 0);
     const bool wide = zaxis && (h & 1) == 0;
     if (tid < kLines) s_max[tid] = 27u << 23;      // 2^-100: the least exponent of the scale
-    pdl_enter();                                   // (the issuing warp reads nothing that another kernel writes)
+    pdl_wait();                                    // (the issuing warp reads nothing that another kernel writes)
     float2 v[16];
     if (mine) {
         const int line = tile * kLines + row;

@@ -4,6 +4,13 @@
 // all earlier ones, since each of them waits too) has finished and its
 // writes are visible, and must not touch global memory that another kernel
 // writes before.  pdl_trigger() lets the next kernel start its own set-up.
+// A kernel that allocates tensor memory triggers only once its block holds its
+// columns: the allocation waits for columns without a limit, and blocks of
+// several launches and contexts share an SM's 512.  A dependent's block is
+// placed when every block before it has triggered, so whoever holds columns
+// while it waits, waits for blocks that hold theirs, and no cycle can form.
+// (Triggered earlier, a dependent could take the columns that its own
+// predecessor was still to get.)
 // The loops of a small-grid minimisation are chains of kernels of a few
 // microseconds, where the gap between dependent kernels (about 1.5 us) counts.
 // Measured (GB300, one evaluation in a captured loop, plain -> dependent):

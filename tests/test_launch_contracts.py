@@ -1,0 +1,87 @@
+"""CPU: what the dependent launches (pdl.cuh) rest on, read from the kernels'
+source.  Every kernel launched dependent waits for its predecessors, and one
+that allocates tensor memory lets the next kernel start only after its block
+holds its columns (a dependent that took them first could wait for its own
+predecessor for ever).  The GPU case runs the shapes of which several blocks
+share an SM (edges 18 to 48) from many contexts at once."""
+import os
+import re
+import threading
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1406_0835_gb300", "csrc")
+
+
+def sources():
+    return {f: re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, f)).read())
+            for f in sorted(os.listdir(CSRC)) if f.endswith((".cu", ".cuh"))}
+
+
+def kernels():
+    """name -> (parameters, body) of every __global__ function."""
+    out = {}
+    for text in sources().values():
+        for m in re.finditer(r"__global__[^{;]*?\b(k_\w+)\s*\(([^{;]*)\)\s*\{", text):
+            depth, i = 1, m.end()
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[i], 0)
+                i += 1
+            out[m.group(1)] = (m.group(2), text[m.end():i])
+    return out
+
+
+def dependent():
+    names = set()
+    for text in sources().values():
+        names |= set(re.findall(r"pdl_launch\(\s*(k_\w+)", text))
+    return names
+
+
+def test_dependent_kernels_wait():
+    k, d = kernels(), dependent()
+    assert len(d) > 30
+    for name in sorted(d):
+        assert re.search(r"\bpdl_(wait|enter)\(\)", k[name][1]), name
+
+
+def test_tensor_memory_is_held_before_the_next_kernel_may_start():
+    k, d = kernels(), dependent()
+    holders = [n for n in d if "tmem_alloc" in k[n][1]]
+    assert sorted(holders) == ["k_force", "k_tline"]
+    for n in holders:
+        body = k[n][1]
+        assert "pdl_enter" not in body, n
+        assert body.count("pdl_trigger()") == 1, n
+        assert body.index("tmem_alloc") < body.index("pdl_trigger()"), n
+
+
+@pytest.mark.gpu
+def test_small_edges_of_many_contexts_share_the_sms():
+    """Eight contexts minimise at once from eight threads, edges of 128 and of
+    256 columns mixed; each result repeats its solo run bit for bit."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1406_0835_gb300 import inputs, ofdft
+    grids = [(18, 32, 128), (32, 30, 96), (24, 48, 60), (32, 32, 32), (30, 64, 32), (20, 24, 120), (48, 50, 18), (32, 20, 144)]
+    ctxs = []
+    for i, grid in enumerate(grids):
+        d = inputs.hydrogen(8, 1.0, 1.0e5, grid, seed=i, functional="vt84f")
+        ctxs.append(ofdft.Context(d["L"], grid, d["ions"], d["Z"], d["T"], "vt84f"))
+    solo, both = [], [None] * len(ctxs)
+    for c in ctxs:
+        c.set_phi()
+        solo.append(c.minimize(gtol=1e-6)[0]["F_tot"])
+
+    def work(i):
+        ctxs[i].set_phi()
+        both[i] = ctxs[i].minimize(gtol=1e-6)[0]["F_tot"]
+    ts = [threading.Thread(target=work, args=(i,)) for i in range(len(ctxs))]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    for c in ctxs:
+        c.close()
+    assert np.array_equal(solo, both)
