@@ -290,11 +290,11 @@ __device__ __forceinline__ CC times_ik(CC x, int e, int n, R s)
 // line transforms it already holds: the forward spectrum times i kt ds_z,
 // transformed back).
 template <typename PR, int MODE>
-__global__ void OFDFT_FFT_BOUNDS k_zfwd(GridInfo g, FftAxis az, int P, const typename KT<PR>::T *__restrict__ in,
-                       const typename KT<PR>::T *__restrict__ phi, const typename KT<PR>::T *__restrict__ dhat,
-                       typename KT<PR>::T c, typename KT<PR>::T s, const void *__restrict__ cs,
-                       typename KT<PR>::T *__restrict__ phit, typename KT<PR>::C *__restrict__ out,
-                       typename KT<PR>::T *__restrict__ dzout, typename KT<PR>::T *__restrict__ nout)
+__global__ void OFDFT_FFT_BOUNDS k_zfwd(GridInfo g, FftAxis az, int P, const typename KT<PR>::T *in,
+                       const typename KT<PR>::T *phi, const typename KT<PR>::T *dhat,
+                       typename KT<PR>::T c, typename KT<PR>::T s, const void *cs,
+                       typename KT<PR>::T *phit, typename KT<PR>::C *out,
+                       typename KT<PR>::T *dzout, typename KT<PR>::T *nout)
 {
     pdl_enter();
     typedef typename KT<PR>::T T;
@@ -406,12 +406,12 @@ __device__ __forceinline__ void unpack_r2c(const typename KT<PR>::CC *X, long lo
 // for the first six): F_s, TS, F_xc, sum(n df/dn - f), 0, sum n(v_xc - eps),
 // then sum phi^2 v, sum phi^2, sum 2 phi v dphi/dtheta.
 template <typename PR, bool FTTF>
-__global__ void k_zfinal(GridInfo g, FftAxis az, int P, const typename KT<PR>::C *__restrict__ dspec,
-                         const typename KT<PR>::T *__restrict__ vpart, const typename KT<PR>::T *__restrict__ phit,
-                         const typename KT<PR>::T *__restrict__ phi, const typename KT<PR>::T *__restrict__ dhat,
-                         typename KT<PR>::T c, typename KT<PR>::T s, const void *__restrict__ cs,
+__global__ void k_zfinal(GridInfo g, FftAxis az, int P, const typename KT<PR>::C *dspec,
+                         const typename KT<PR>::T *vpart, const typename KT<PR>::T *phit,
+                         const typename KT<PR>::T *phi, const typename KT<PR>::T *dhat,
+                         typename KT<PR>::T c, typename KT<PR>::T s, const void *cs,
                          typename KT<PR>::T temp, FuncParams fp, const typename KT<PR>::T *__restrict__ tab, int xc,
-                         typename KT<PR>::T *__restrict__ vout, double *__restrict__ part)
+                         typename KT<PR>::T *vout, double *part)
 {
     pdl_enter();
     typedef typename KT<PR>::T T;
@@ -464,13 +464,13 @@ __global__ void k_zfinal(GridInfo g, FftAxis az, int P, const typename KT<PR>::C
         } else {
             v = ldr<PR>(vpart[rbase + i]) + dr;
         }
-        vout[rbase + i] = str<PR>(v);
         acc[6] += n * v;
         acc[7] += n;
         if (dhat != nullptr) {
             R dphi = -sr * ldr<PR>(phi[rbase + i]) + cr * ldr<PR>(dhat[rbase + i]);
             acc[8] += R(2) * (ph * v) * dphi;
         }
+        vout[rbase + i] = str<PR>(v);
     }
     double tot[9];
     block_total<9, PR>(acc, tot);
@@ -547,7 +547,7 @@ __device__ __forceinline__ void store_tile(typename KT<PR>::C *__restrict__ dst,
 }
 
 template <typename PR, bool INV>
-__global__ void OFDFT_FFT_BOUNDS k_ypass(GridInfo g, FftAxis ay, typename KT<PR>::C *__restrict__ data, long long fstride)
+__global__ void OFDFT_FFT_BOUNDS k_ypass(GridInfo g, FftAxis ay, typename KT<PR>::C *data, long long fstride)
 {
     pdl_enter();
     typedef typename KT<PR>::C C;
@@ -586,9 +586,9 @@ __device__ __forceinline__ typename KT<PR>::R ploc_term(const GridInfo &g, const
 // x pass, ftTF variant: forward x -> energies -> v_HL(G) = 4 pi n/G^2 + v_ext
 // inverse-x, written over the spectrum.  If keep_n, n(G) is also stored in nG_out.
 template <typename PR, bool TRI>
-__global__ void OFDFT_FFT_BOUNDS k_xhl(GridInfo g, FftAxis ax, typename KT<PR>::C *__restrict__ spec,
-                      const typename KT<PR>::C *__restrict__ vext, typename KT<PR>::C *__restrict__ nG_out,
-                      int inverse, double *__restrict__ part)
+__global__ void OFDFT_FFT_BOUNDS k_xhl(GridInfo g, FftAxis ax, typename KT<PR>::C *spec,
+                      const typename KT<PR>::C *vext, typename KT<PR>::C *nG_out,
+                      int inverse, double *part)
 {
     pdl_enter();
     typedef typename KT<PR>::R R;
@@ -854,10 +854,10 @@ __global__ void OFDFT_FFT_BOUNDS k_dline_ws(GridInfo g, FftAxis fa, const typena
 #endif
 
 template <typename PR, bool STRESS, bool TRI>
-__global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB) k_pw(GridInfo g, typename KT<PR>::T *__restrict__ d0, typename KT<PR>::T *__restrict__ d1,
-                     typename KT<PR>::T *__restrict__ d2, const typename KT<PR>::T *__restrict__ phit,
+__global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB) k_pw(GridInfo g, typename KT<PR>::T *d0, typename KT<PR>::T *d1,
+                     typename KT<PR>::T *d2, const typename KT<PR>::T *phit,
                      typename KT<PR>::T temp, FuncParams fp, const typename KT<PR>::T *__restrict__ tab, int xc,
-                     typename KT<PR>::T *__restrict__ vpart, double *__restrict__ part)
+                     typename KT<PR>::T *vpart, double *part)
 {
     pdl_enter();
     typedef typename KT<PR>::T T;
@@ -949,13 +949,13 @@ __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB) k_pw(GridInfo
 // (as k_zfinal's GGA form): rows 0..5 zero, then sum phi^2 v, sum phi^2,
 // sum 2 phi v dphi/dtheta.
 template <typename PR>
-__global__ void OFDFT_FFT_BOUNDS k_zfinal_g(GridInfo g, FftAxis az, int P, const typename KT<PR>::C *__restrict__ dspec,
-                           const typename KT<PR>::T *__restrict__ uz, const typename KT<PR>::T *__restrict__ vpart,
-                           const typename KT<PR>::T *div, const typename KT<PR>::T *__restrict__ div2,
-                           const typename KT<PR>::T *__restrict__ div3, const typename KT<PR>::T *__restrict__ phit,
-                           const typename KT<PR>::T *__restrict__ phi, const typename KT<PR>::T *__restrict__ dhat,
-                           typename KT<PR>::T c, typename KT<PR>::T s, const void *__restrict__ cs,
-                           typename KT<PR>::T *vout, double *__restrict__ part)
+__global__ void OFDFT_FFT_BOUNDS k_zfinal_g(GridInfo g, FftAxis az, int P, const typename KT<PR>::C *dspec,
+                           const typename KT<PR>::T *uz, const typename KT<PR>::T *vpart,
+                           const typename KT<PR>::T *div, const typename KT<PR>::T *div2,
+                           const typename KT<PR>::T *div3, const typename KT<PR>::T *phit,
+                           const typename KT<PR>::T *phi, const typename KT<PR>::T *dhat,
+                           typename KT<PR>::T c, typename KT<PR>::T s, const void *cs,
+                           typename KT<PR>::T *vout, double *part)
 {
     pdl_enter();
     typedef typename KT<PR>::T T;
@@ -1005,13 +1005,13 @@ __global__ void OFDFT_FFT_BOUNDS k_zfinal_g(GridInfo g, FftAxis az, int P, const
         R v = ldp<PR>(vpart[rbase + i]) + dr - ldp<PR>(div[rbase + i]);
         if (div2 != nullptr) v = v - ldp<PR>(div2[rbase + i]);
         if (uz == nullptr) v = v - ldp<PR>(div3[rbase + i]);
-        vout[rbase + i] = str<PR>(v);
         acc[6] += n * v;
         acc[7] += n;
         if (dhat != nullptr) {
             const R dphi = -sr * ldr<PR>(phi[rbase + i]) + cr * ldr<PR>(dhat[rbase + i]);
             acc[8] += R(2) * (ph * v) * dphi;
         }
+        vout[rbase + i] = str<PR>(v);
     }
     double tot[9];
     block_total<9, PR>(acc, tot);
@@ -1122,8 +1122,8 @@ void launch_dline(const GridInfo &g, const FftAxis &fa, int axis, int mode, int 
 }
 
 // n = phi^2 as pairs, two points a thread (N is even).
-__global__ void k_density(long long pairs, const double2 *__restrict__ phi, const double2 *__restrict__ dhat, double c, double s,
-                          const double *__restrict__ cs, double2 *__restrict__ phit, float4 *__restrict__ dens)
+__global__ void k_density(long long pairs, const double2 *phi, const double2 *dhat, double c, double s,
+                          const double *cs, double2 *phit, float4 *dens)
 {
     pdl_enter();
     if (cs != nullptr) {
@@ -1151,7 +1151,7 @@ __device__ __forceinline__ ff::f2 f2of(float2 x) { return ff::f2(x.x, x.y); }
 // Real-Fourier coefficients of n -> of v_HL = 4 pi n / G^2 + v_ext, with the
 // sums of E_H, E_loc and P_loc.  A kernel of its own: in the transforms'
 // blocks (one to an SM) the same loop waited on memory latency.
-__global__ void __launch_bounds__(256) k_hartree(GridInfo g, float4 *__restrict__ coef, TlHartree hl)
+__global__ void __launch_bounds__(256) k_hartree(GridInfo g, float4 *coef, TlHartree hl)
 {
     pdl_enter();
     constexpr ff::f2 fpi(kFourPi);
@@ -1204,7 +1204,7 @@ __global__ void __launch_bounds__(256) k_hartree(GridInfo g, float4 *__restrict_
 // of eight.  A solve's evaluation in a sheared cell, FFT passes -> with this:
 // GGA 60 x 54 x 72 138 -> 120 us, 96^3 309 -> 259, ftTF 16^3 68 -> 58, 96^3
 // 198 -> 156.
-__global__ void __launch_bounds__(128) k_hartree_tri(GridInfo g, float2 *__restrict__ coef, TlHartree hl)
+__global__ void __launch_bounds__(128) k_hartree_tri(GridInfo g, float2 *coef, TlHartree hl)
 {
     pdl_enter();
     constexpr ff::f2 fpi(kFourPi);
@@ -1314,9 +1314,9 @@ __global__ void __launch_bounds__(256) k_final(GridInfo g, TlFinal f)
 
 // ftTF pointwise stage: v = v_HL + df/dn + v_xc, partials as k_zfinal's.
 __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB)
-    k_ptf(GridInfo g, const float2 *__restrict__ vhl, const double *__restrict__ phit, const double *__restrict__ phi,
-          const double *__restrict__ dhat, double c, double s, const double *__restrict__ cs, double temp, FuncParams fp,
-          const double *__restrict__ tab, int xc, double *__restrict__ vout, double *__restrict__ part)
+    k_ptf(GridInfo g, const float2 *vhl, const double *phit, const double *phi,
+          const double *dhat, double c, double s, const double *cs, double temp, FuncParams fp,
+          const double *__restrict__ tab, int xc, double *vout, double *part)
 {
     pdl_enter();
     if (cs != nullptr) {
@@ -1331,7 +1331,6 @@ __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB)
         const float2 h = vhl[i];
         const PwF2 o = pw_dd(fp, tab, tcoef, temp, n, gz, xc);
         const ff::f2 v = o.dfdn + o.vxc + ff::f2(h.x, h.y);
-        vout[i] = ff::to_double(v);
         acc[0] += o.f;
         acc[1] += o.ts;
         acc[2] += n * o.eps;
@@ -1343,6 +1342,7 @@ __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB)
             const ff::f2 dphi = cr * ff::split_int(dhat[i]) - sr * ff::split_int(phi[i]);
             acc[8] += ff::f2(2.0f, 0.0f) * (ph * v) * dphi;
         }
+        vout[i] = ff::to_double(v);
     }
     double tot[9];
     block_sum_f2<9>(acc, tot);

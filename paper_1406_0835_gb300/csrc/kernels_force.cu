@@ -125,10 +125,10 @@ __device__ void corners(const GridInfo &g, int I, const double *__restrict__ Z, 
 // The A images (f_c and f_c' / block_top, times 2^54), eight c
 // a thread, and the pairs (f, f') of the x and y coefficients; the first
 // blocks sum the corners.
-__global__ void k_force_phases(GridInfo g, int nat, int natp, int kblocks, const double *__restrict__ Z,
-                               const double2 *__restrict__ px, const double2 *__restrict__ py,
-                               const double2 *__restrict__ pz, const double2 *__restrict__ nG, unsigned char *image,
-                               float4 *tx, float4 *ty, int nchunk, double *__restrict__ part)
+__global__ void k_force_phases(GridInfo g, int nat, int natp, int kblocks, const double *Z,
+                               const double2 *px, const double2 *py,
+                               const double2 *pz, const double2 *nG, unsigned char *image,
+                               float4 *tx, float4 *ty, int nchunk, double *part)
 {
     pdl_enter();
     const int ncorner = (nat + 3) / 4;
@@ -172,9 +172,9 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 }
 
 __global__ void __launch_bounds__(kForceThreads, 1)
-    k_force(GridInfo g, int nat, int natp, int kblocks, const double *__restrict__ Z, const float2 *__restrict__ coef,
-            const unsigned char *__restrict__ image, const float4 *__restrict__ tx, const float4 *__restrict__ ty,
-            double *__restrict__ part)
+    k_force(GridInfo g, int nat, int natp, int kblocks, const double *Z, const float2 *coef,
+            const unsigned char *image, const float4 *tx, const float4 *ty,
+            double *part)
 {
     extern __shared__ __align__(1024) unsigned char smraw[];
     // A in place; B tile converted, its products done, its accumulators read (per buffer); scales written (four tiles deep)
@@ -219,6 +219,7 @@ __global__ void __launch_bounds__(kForceThreads, 1)
         int it = 0;
         for (int t = blockIdx.y; t < tiles && good; t += gridDim.y, ++it) {
             const int a = t / nbt, b0 = (t - a * nbt) * kRows, buf = it & 1;
+            const float4 fa = tx[(size_t)a * natp + I];
             good = tc::mbar_wait(b_scale + 8 * (it & 3), (it >> 2) & 1) && tc::mbar_wait(b_done + 8 * buf, (it >> 1) & 1);
             tc::fence_after_sync();
             ff::f2 S1 = z0, S2 = z0;
@@ -249,9 +250,8 @@ __global__ void __launch_bounds__(kForceThreads, 1)
             __syncwarp();
             if (lane == 0) mbar_arrive(b_read + 8 * buf);
             // x force: f_a' sum f_b T; y: f_a sum f_b' T; z: f_a sum f_b T'
-            const float4 f = tx[(size_t)a * natp + I];
-            F1 += ff::mul(half ? ff::f2(f.x, f.y) : ff::f2(f.z, f.w), S1);
-            F2 += ff::mul(ff::f2(f.x, f.y), S2);
+            F1 += ff::mul(half ? ff::f2(fa.x, fa.y) : ff::f2(fa.z, fa.w), S1);
+            F2 += ff::mul(ff::f2(fa.x, fa.y), S2);
         }
         if (!good) s_bad = 1;
         __syncthreads();

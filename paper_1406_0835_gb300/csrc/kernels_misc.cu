@@ -53,7 +53,7 @@ template <int NQ> __device__ __forceinline__ void block_sum_split(const double *
 }
 template <int NQ> __device__ __forceinline__ void block_sum_split(AccF *v, double *tot) { block_sum<NQ>(v, tot); }
 
-__global__ void k_reduce(const double *__restrict__ part, int nblk, double *__restrict__ out)
+__global__ void k_reduce(const double *part, int nblk, double *out)
 {
     pdl_enter();
     double v[1] = {0.0};
@@ -67,9 +67,9 @@ __global__ void k_reduce(const double *__restrict__ part, int nblk, double *__re
 // x-pass partials (q < 3), of the pointwise partials (GGA, 3 <= q < 9) or
 // of the final z-pass partials (the rest) into out[q] (ftTF: out[9 + r] for
 // final row r), in the same fixed order as k_reduce.
-__global__ void k_reduce_eval(const double *__restrict__ pA, int na, const double *__restrict__ pB, int nb,
-                              const double *__restrict__ pC, int nc, int gga, const double *__restrict__ pE, int ne,
-                              double *__restrict__ out)
+__global__ void k_reduce_eval(const double *pA, int na, const double *pB, int nb,
+                              const double *pC, int nc, int gga, const double *pE, int ne,
+                              double *out)
 {
     pdl_enter();
     const int q = blockIdx.x;
@@ -125,7 +125,7 @@ template <typename T, typename U> __global__ void k_convert(long long n, const T
         y[i] = (U)x[i];
 }
 
-template <typename T> __global__ void k_sumsq(long long n, const T *__restrict__ x, double *part)
+template <typename T> __global__ void k_sumsq(long long n, const T *x, double *part)
 {
     pdl_enter();
     typedef typename AccT<T>::type A;
@@ -157,9 +157,9 @@ __global__ void k_extrap(long long n, const T *__restrict__ x, const T *__restri
 }
 
 template <typename T>
-__global__ void k_cg_grad(long long n, const T *__restrict__ phi, const T *__restrict__ v,
-                          double mu, const double *mup, T *__restrict__ g,
-                          const T *__restrict__ gprev, double *part)
+__global__ void k_cg_grad(long long n, const T *phi, const T *v,
+                          double mu, const double *mup, T *g,
+                          const T *gprev, double *part)
 {
     pdl_enter();
     if (mup != nullptr) mu = *mup;
@@ -170,9 +170,9 @@ __global__ void k_cg_grad(long long n, const T *__restrict__ phi, const T *__res
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         T gi = T(2) * phi[i] * (v[i] - mut);
-        g[i] = gi;
         acc[0] += (P)gi * (P)gi;
         if (gprev != nullptr) acc[1] += (P)gi * (P)gprev[i];
+        g[i] = gi;
     }
     double tot[2];
     block_sum_split<2>(acc, tot);
@@ -183,8 +183,8 @@ __global__ void k_cg_grad(long long n, const T *__restrict__ phi, const T *__res
 }
 
 template <typename T>
-__global__ void k_cg_dir(long long n, const T *__restrict__ g, T *__restrict__ d, double beta,
-                         const double *betap, const T *__restrict__ phi, double *part)
+__global__ void k_cg_dir(long long n, const T *g, T *d, double beta,
+                         const double *betap, const T *phi, double *part)
 {
     pdl_enter();
     if (betap != nullptr) beta = *betap;
@@ -195,9 +195,9 @@ __global__ void k_cg_dir(long long n, const T *__restrict__ g, T *__restrict__ d
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         T gi = g[i];
+        P p = (P)phi[i];
         T di = (beta == 0.0) ? -gi : (T)(-(P)gi + ba * (P)d[i]);
         d[i] = di;
-        P p = (P)phi[i];
         acc[0] += p * (P)di;
         acc[1] += (P)di * (P)di;
         acc[2] += (P)di * (P)gi;
@@ -211,9 +211,9 @@ __global__ void k_cg_dir(long long n, const T *__restrict__ g, T *__restrict__ d
 }
 
 template <typename T>
-__global__ void k_cg_dhat(long long n, const T *__restrict__ g, T *__restrict__ d,
-                          const T *__restrict__ phi, const T *__restrict__ v, double c1, double c2,
-                          int restart, const double *c12r, T *__restrict__ dhat, double *part)
+__global__ void k_cg_dhat(long long n, const T *g, T *d,
+                          const T *phi, const T *v, double c1, double c2,
+                          int restart, const double *c12r, T *dhat, double *part)
 {
     pdl_enter();
     if (c12r != nullptr) {
@@ -227,11 +227,12 @@ __global__ void k_cg_dhat(long long n, const T *__restrict__ g, T *__restrict__ 
     A acc[1] = {A(0)};
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
-        P di = restart ? -(P)g[i] : (P)d[i] - c1a * (P)phi[i];
+        const P p = (P)phi[i], vi = (P)v[i];
+        P di = restart ? -(P)g[i] : (P)d[i] - c1a * p;
         d[i] = (T)di;
         T dh = (T)(c2a * di);
         dhat[i] = dh;
-        acc[0] += P(2) * (P)phi[i] * (P)v[i] * (P)dh;
+        acc[0] += P(2) * p * vi * (P)dh;
     }
     double tot[1];
     block_sum_split<1>(acc, tot);
@@ -266,9 +267,9 @@ __global__ void k_axpby(long long n, double alpha, const T *x, double beta, cons
 // sum g.g_prev.  Each element is read once (the accepted trial's phi and v
 // feed the gradient directly).
 template <typename T>
-__global__ void k_cg_update(long long n, const int *__restrict__ accepted, T *__restrict__ phi,
-                            const T *__restrict__ phit, T *__restrict__ v, const T *__restrict__ vt,
-                            const double *mup, T *__restrict__ g, T *__restrict__ gprev, double *part)
+__global__ void k_cg_update(long long n, const int *accepted, T *phi,
+                            const T *phit, T *v, const T *vt,
+                            const double *mup, T *g, T *gprev, double *part)
 {
     pdl_enter();
     typedef typename AccT<T>::type A;
@@ -305,7 +306,7 @@ __global__ void k_cg_update(long long n, const int *__restrict__ accepted, T *__
 }
 
 // ------------------------------------------------ structure factor, forces
-__global__ void k_phases(GridInfo g, int nat, const double *__restrict__ R, double2 *px,
+__global__ void k_phases(GridInfo g, int nat, const double *R, double2 *px,
                          double2 *py, double2 *pz)
 {
     pdl_enter();
@@ -517,7 +518,7 @@ __global__ void k_vext(GridInfo g, int nat, const double *__restrict__ Z,
 // on two or three Nyquist frequencies, which are no product of the axes'
 // functions there, and ordered by frequency.
 template <bool FORCE>
-__global__ void k_real_coefficients(GridInfo g, const double2 *__restrict__ V, float2 *__restrict__ coef)
+__global__ void k_real_coefficients(GridInfo g, const double2 *V, float2 *coef)
 {
     pdl_enter();
     const int hx = g.nx / 2, hy = g.ny / 2, hz = g.nz / 2;
@@ -756,8 +757,8 @@ __global__ void k_lpp_forces(GridInfo g, int nat, const double *__restrict__ Z,
 // Double-float copies of the axis phase tables: pxT[ix][I], pyT[iy][I],
 // pzT[kz][I] (atoms fastest, for the force kernel's one-thread-per-atom
 // loads) and pzd[I][kz] (for v_ext's one-thread-per-kz loads).
-__global__ void k_phase_tables_dd(GridInfo g, int nat, const double2 *__restrict__ px,
-                                  const double2 *__restrict__ py, const double2 *__restrict__ pz,
+__global__ void k_phase_tables_dd(GridInfo g, int nat, const double2 *px,
+                                  const double2 *py, const double2 *pz,
                                   ff::cf2 *pxT, ff::cf2 *pyT, ff::cf2 *pzT, ff::cf2 *pzd)
 {
     pdl_enter();
@@ -854,9 +855,9 @@ __device__ __forceinline__ void row_sf_dd(const GridInfo &g, int nat, const doub
 
 // v_ext(G) as k_vext (same Nyquist handling and outputs), with the sums
 // over atoms in double-float (row_sf_dd).
-__global__ void k_vext_dd(GridInfo g, int nat, const double *__restrict__ Z, const ff::cf2 *__restrict__ pxT,
-                          const ff::cf2 *__restrict__ pyT, const ff::cf2 *__restrict__ pzd,
-                          double2 *__restrict__ vext)
+__global__ void k_vext_dd(GridInfo g, int nat, const double *Z, const ff::cf2 *pxT,
+                          const ff::cf2 *pyT, const ff::cf2 *pzd,
+                          double2 *vext)
 {
     pdl_enter();
     const int ix = blockIdx.x / g.ny, iy = blockIdx.x - ix * g.ny;
@@ -1001,7 +1002,7 @@ __global__ void k_lpp_forces_dd(GridInfo g, int nat, int rows_per_block, const d
 
 // Sum of force partials: one warp per (atom, component), lanes over the
 // chunks in a fixed pattern, then a fixed shuffle tree.
-__global__ void k_force_reduce_w(int nat, int nchunk, const double *__restrict__ part, double *F, int accumulate)
+__global__ void k_force_reduce_w(int nat, int nchunk, const double *part, double *F, int accumulate)
 {
     pdl_enter();
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -1388,7 +1389,7 @@ __global__ void k_static_ions(GridInfo g, int nat, const __grid_constant__ Stati
 // or three Nyquist frequencies, whose v_ext is the mean over G and its
 // partner G', the cosines' product is the cosine of the sum of the phases.
 __global__ void __launch_bounds__(kEwThreads) k_static_sums(GridInfo g, int nat, EwBox w, int newald, StaticIonTables t,
-                                                            float2 *__restrict__ vre)
+                                                            float2 *vre)
 {
     pdl_enter();
     if ((int)blockIdx.x < newald) {

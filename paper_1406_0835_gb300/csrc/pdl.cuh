@@ -4,6 +4,12 @@
 // all earlier ones, since each of them waits too) has finished and its
 // writes are visible, and must not touch global memory that another kernel
 // writes before.  pdl_trigger() lets the next kernel start its own set-up.
+// Pointers to what other kernels write are not __restrict__ parameters of a
+// kernel so launched: that would promise that nothing, the wait included,
+// changes what they point to while the kernel runs, and allow their loads
+// before the wait or through the non-coherent path, whose lines an earlier
+// kernel's blocks may have fetched before the data were there.  (Tables laid
+// out at set-up may be.)  The kernels load a point's values before they store.
 // A kernel that allocates tensor memory triggers only once its block holds its
 // columns: the allocation waits for columns without a limit, and blocks of
 // several launches and contexts share an SM's 512.  A dependent's block is

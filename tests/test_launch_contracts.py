@@ -1,6 +1,7 @@
 """CPU: what the dependent launches (pdl.cuh) rest on, read from the kernels'
-source.  Every kernel launched dependent waits for its predecessors, and one
-that allocates tensor memory lets the next kernel start only after its block
+source.  Every kernel launched dependent waits for its predecessors and does
+not promise the compiler that their outputs stay unchanged; one that
+allocates tensor memory lets the next kernel start only after its block
 holds its columns (a dependent that took them first could wait for its own
 predecessor for ever).  The GPU case runs the shapes of which several blocks
 share an SM (edges 18 to 48) from many contexts at once."""
@@ -55,6 +56,15 @@ def test_tensor_memory_is_held_before_the_next_kernel_may_start():
         assert "pdl_enter" not in body, n
         assert body.count("pdl_trigger()") == 1, n
         assert body.index("tmem_alloc") < body.index("pdl_trigger()"), n
+
+
+def test_dependent_kernels_restrict_only_tables():
+    """A __restrict__ parameter tells the compiler that nothing changes what it
+    points to while the kernel runs, so that its loads need not stay behind the
+    wait; only the functional's table, written at set-up, may be one."""
+    k = kernels()
+    for name in sorted(dependent()):
+        assert set(re.findall(r"__restrict__\s+(\w+)", k[name][0])) <= {"tab"}, name
 
 
 @pytest.mark.gpu
