@@ -123,7 +123,10 @@ bool edge_ok(int n)
 }
 
 // One-time set-up on the current device: scratch address, tables, smem limits.
-ofdft_status device_setup(int dev, unsigned char **base)
+// The uploads run on the caller's stream and are waited for: a copy from
+// pageable memory may return before its data have arrived, and a later call
+// may come on any stream.
+ofdft_status device_setup(int dev, cudaStream_t st, unsigned char **base)
 {
     if (dev < 0 || dev >= kMaxDevices) return serr(OFDFT_EINVAL, "device ordinal out of range");
     std::lock_guard<std::mutex> lk(g_setup_mu);
@@ -139,9 +142,11 @@ ofdft_status device_setup(int dev, unsigned char **base)
             if (!matrices_fill()) return serr(OFDFT_EDEVICE, "no transform matrices");
             g_tab_ready = true;
         }
-        SCK(cudaMemcpy(d.base + kOffTab, g_tab_host, sizeof(g_tab_host), cudaMemcpyHostToDevice),
+        SCK(cudaMemcpyAsync(d.base + kOffTab, g_tab_host, sizeof(g_tab_host), cudaMemcpyHostToDevice, st),
             "temperature table upload failed");
-        SCK(cudaMemcpy(d.base + kOffMat, g_mat_host, sizeof(g_mat_host), cudaMemcpyHostToDevice), "matrix upload failed");
+        SCK(cudaMemcpyAsync(d.base + kOffMat, g_mat_host, sizeof(g_mat_host), cudaMemcpyHostToDevice, st),
+            "matrix upload failed");
+        SCK(cudaStreamSynchronize(st), "table upload failed");
         SCK(tline_smem_limits(), "shared-memory limit set-up failed");
         d.ready = true;
     }
@@ -254,7 +259,7 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
     int dev = 0;
     SCK(cudaGetDevice(&dev), "cudaGetDevice failed");
     unsigned char *base = nullptr;
-    ofdft_status s = device_setup(dev, &base);
+    ofdft_status s = device_setup(dev, st, &base);
     if (s != OFDFT_OK) return s;
 
     GridInfo g{};

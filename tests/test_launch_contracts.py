@@ -67,6 +67,48 @@ def test_dependent_kernels_restrict_only_tables():
         assert set(re.findall(r"__restrict__\s+(\w+)", k[name][0])) <= {"tab"}, name
 
 
+def test_the_static_entry_waits_for_its_tables():
+    """A copy from pageable memory may return before the data have arrived, and
+    the caller's stream need not follow the default stream: the one-time
+    uploads run on the caller's stream and are waited for."""
+    text = sources()["capi_static.cu"]
+    setup = text[text.index("device_setup("):text.index("d.ready = true")]
+    assert "cudaMemcpy(" not in setup
+    copies = re.findall(r"cudaMemcpyAsync\([^;]*?(\w+)\)\s*,", setup)
+    assert copies == ["st", "st"]
+    assert setup.index("cudaStreamSynchronize(st)") > setup.rindex("cudaMemcpyAsync")
+
+
+FIRST_CALL = """
+import numpy as np, torch
+from paper_1406_0835_gb300 import inputs, ofdft
+d = inputs.hydrogen(8, 1.0, 1.0e5, (24, 20, 30), seed=3, functional="vt84f")
+N = 24 * 20 * 30
+p = torch.full((N,), float(np.sqrt(8.0 / np.prod(d["L"]))), dtype=torch.float64, device="cuda")
+p *= 1.0 + 0.1 * torch.cos(torch.arange(N, device="cuda", dtype=torch.float64))
+torch.cuda.synchronize()
+s, out = torch.cuda.Stream(), []
+for _ in range(2):
+    v = torch.zeros_like(p)
+    torch.cuda.synchronize()
+    E = ofdft.ofdft_energy_potential_static(np.diag(d["L"]), d["grid"], d["ions"], d["Z"], d["T"], "vt84f",
+                                            p.data_ptr(), v.data_ptr(), stream=s.cuda_stream)
+    out.append((E["F_tot"], v.cpu().numpy()))
+assert out[0][0] == out[1][0] and np.array_equal(out[0][1], out[1][1]) and np.all(out[0][1] != 0.0)
+"""
+
+
+@pytest.mark.gpu
+def test_first_static_call_on_a_non_blocking_stream():
+    """In a process of its own; the second call repeats the first bit for bit."""
+    import subprocess
+    import sys
+    import __graft_entry__
+    __graft_entry__.build()
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", FIRST_CALL], cwd=root, check=True, timeout=600)
+
+
 @pytest.mark.gpu
 def test_small_edges_of_many_contexts_share_the_sms():
     """Eight contexts minimise at once from eight threads, edges of 128 and of
