@@ -124,18 +124,26 @@ __device__ __forceinline__ void bar_sync(int id, int count) { asm volatile("bar.
 // the tensor memory, o in lanes 16-31.  KS: 16-wide K steps; unrolled, so
 // that the descriptors are built in uniform registers (with run-time loops
 // the products of n = 96 took 9,400 cycles to issue, from a single thread
-// 19,100; so they run at the tensor cores' rate, 0.46 cycles a column).
+// 19,100; so they run at the tensor cores' rate, 0.46 cycles a column).  A
+// wait that runs out raises *bad before the products that it stood for are
+// committed: whoever sees them done sees *bad.
 template <int KS>
-__device__ __forceinline__ bool issue(const TlShape &sh, const unsigned char *mat, uint32_t full, uint32_t done, uint32_t sa,
-                                      uint32_t sb, uint32_t tmem, int nthreads)
+__device__ __forceinline__ void issue(const TlShape &sh, const unsigned char *mat, uint32_t full, uint32_t done, uint32_t sa,
+                                      uint32_t sb, uint32_t tmem, int nthreads, volatile int *bad)
 {
     const int units = 2 * sh.chunks;
     const uint32_t a_dig = sh.a_dig;
-    bool good = true;
+    auto wait = [&](uint32_t bar) {
+        if (!tc::mbar_wait(bar, 0)) {
+            *bad = 1;
+            __threadfence_block();
+        }
+        __syncwarp();
+    };
 #pragma unroll 1
     for (int u = 0; u < units; ++u) {
         const int c = u >> 1, width = tl_width(sh, c);
-        good = tc::mbar_wait(full + 8 * u, 0) && good;
+        wait(full + 8 * u);
         if (u < 2) bar_sync(1 + u, nthreads);     // the digits of s (u = 0), of d (u = 1)
         tc::fence_after_sync();
         const uint32_t blb = (uint32_t)(kDig * width) * 16;
@@ -153,7 +161,7 @@ __device__ __forceinline__ bool issue(const TlShape &sh, const unsigned char *ma
         tc::mma_commit(done + 8 * u);
         const int next = u - 1 + sh.nslot;        // the unit that takes over slot (u - 1)
         if (u >= 1 && next < units) {
-            good = tc::mbar_wait(done + 8 * (u - 1), 0) && good;
+            wait(done + 8 * (u - 1));
             if ((threadIdx.x & 31) == 0) {
                 const uint32_t bytes = tl_unit_bytes(sh, next >> 1);
                 tc::mbar_expect(full + 8 * next, bytes);
@@ -162,7 +170,6 @@ __device__ __forceinline__ bool issue(const TlShape &sh, const unsigned char *ma
             __syncwarp();
         }
     }
-    return good;
 }
 
 // Eight consecutive outputs of a line (left: how many lie in the half).
@@ -236,15 +243,13 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
         tc::fence_before_sync();
         bar_arrive(4, blockDim.x);                 // barriers and tensor memory are there
         const uint32_t tmem = __shfl_sync(0xffffffffu, *(volatile uint32_t *)&s_tmem, 0);
-        bool good;
         switch (nc / 2) {
-        case 1: good = issue<1>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x); break;
-        case 2: good = issue<2>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x); break;
-        case 3: good = issue<3>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x); break;
-        case 4: good = issue<4>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x); break;
-        default: good = issue<5>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x); break;
+        case 1: issue<1>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x, &s_bad); break;
+        case 2: issue<2>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x, &s_bad); break;
+        case 3: issue<3>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x, &s_bad); break;
+        case 4: issue<4>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x, &s_bad); break;
+        default: issue<5>(sh, jb.mat, full, done, sa, sb, tmem, blockDim.x, &s_bad); break;
         }
-        if (!good) s_bad = 1;
         __syncthreads();                           // every accumulator has been read
         tc::fence_after_sync();
         tc::tmem_dealloc(tmem, sh.cols);

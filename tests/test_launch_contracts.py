@@ -79,6 +79,18 @@ def test_the_static_entry_waits_for_its_tables():
     assert setup.index("cudaStreamSynchronize(st)") > setup.rindex("cudaMemcpyAsync")
 
 
+def test_a_wait_that_runs_out_is_flagged_before_its_products_are_committed():
+    """k_tline's readers look at s_bad once a unit's products are done, so the
+    issuing warp has to have raised it before it commits them."""
+    text = sources()["kernels_tline.cu"]
+    body = text[text.index("void issue("):text.index("store_lines(")]
+    waits = re.findall(r"[^;{}]*mbar_wait\([^;]*", body)
+    assert len(waits) == 1 and waits[0].strip().startswith("if (!tc::mbar_wait(bar, 0))")
+    raised = body.index("*bad = 1;")
+    assert raised < body.index("__threadfence_block()", raised) < body.index("mma_commit")
+    assert re.search(r"wait\(full[^;]*;.*mma_commit", body, re.S)
+
+
 FIRST_CALL = """
 import numpy as np, torch
 from paper_1406_0835_gb300 import inputs, ofdft
