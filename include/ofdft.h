@@ -420,7 +420,7 @@ void ofdft_destroy(ofdft_ctx *ctx);
  * but every device scratch buffer is carved from one fixed array compiled
  * into the library: about 3.4 MB that each GPU loading the library holds
  * until the process exits.  The call allocates no memory, on the device or
- * (after the set-up below) the host.
+ * the host.
  *  cell[9], grid[3], nat, ions, Z, T_kelvin, functional: as ofdft_setup,
  *              but orthorhombic cells only (else OFDFT_EINVAL).
  *  xc, rc: as ofdft_params (Gaussian ion only).
@@ -432,8 +432,8 @@ void ofdft_destroy(ofdft_ctx *ctx);
  * Limits: each grid edge even, {2,3,5}-smooth and at most 64;
  * nx*ny*nz <= 32768; 1 <= nat <= 64.  Anything larger returns OFDFT_EINVAL,
  * as do Z <= 0, non-finite positions, T or rc.
- * No call may be made on a stream that is being captured (the call reads
- * from pageable host memory and synchronises): OFDFT_EINVAL.  The first
+ * No call may be made on a stream that is being captured (the call copies
+ * to host memory and synchronises): OFDFT_EINVAL.  The first
  * call on a device does a one-time set-up on the current device (looks up
  * the array's device address, fills and uploads the tables and matrices).  The
  * set-up runs under a mutex, so

@@ -74,7 +74,7 @@ std::mutex g_setup_mu;            // guards g_dev, g_tab_host, g_mat, g_mat_host
 
 // The matrices of every edge, filled once with the other tables.
 bool matrices_fill()
-try {
+{
     size_t at = 0;
     for (size_t i = 0; i < sizeof(kEdges) / sizeof(kEdges[0]); ++i) {
         const int n = kEdges[i];
@@ -88,8 +88,6 @@ try {
         }
     }
     return true;
-} catch (...) {   // no host memory for their fill
-    return false;
 }
 
 TlAxis axis_matrices(int n, unsigned char *dev)
@@ -250,8 +248,7 @@ extern "C" ofdft_status ofdft_energy_potential_static(const double cell[9], cons
     if (fp.kind < 0) return serr(OFDFT_EINVAL, "unknown functional");
     cudaStream_t st = (cudaStream_t)stream;
     {
-        // the call copies from pageable host memory and synchronises: not
-        // capturable
+        // the call copies to host memory and synchronises: not capturable
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
             return serr(OFDFT_EINVAL, "the stream is being captured");

@@ -16,7 +16,7 @@
 // two of its largest magnitude to 53-bit integers, the matrices are rounded
 // to 54-bit integers once, and both are cut into seven signed digits of
 // radix 256.  A digit is exact in f16, a product of two is at most 2^14,
-// and the sums over h <= 128 and up to seven digit pairs (two of them with a
+// and the sums over h <= 72 and up to seven digit pairs (two of them with a
 // leading digit, at most 64) stay below 2^24, so the f32 accumulators of
 // tcgen05.mma (kind::f16) hold exact integers.  Digit products of equal
 // weight share one accumulator: 7 accumulators, 28 products, the first
@@ -447,26 +447,32 @@ namespace {
 // table of the distinct entries) times 2^mexp as seven f16 digits each, laid
 // out as the kernel's shared-memory image ([column chunk][e, o][K chunk]
 // [digit][output][8]); returns mexp.
-template <typename F> int pack_matrix(int n, const std::vector<long double> &entry, F at, uint16_t *img)
-{
-    const TlShape s = tl_shape(n);
-    const int h = s.h;
-    static const std::vector<uint16_t> digit = [] {   // f16 of -128 .. 127
-        std::vector<uint16_t> d(256);
+// On fixed arrays: the allocation-free entry point's first call fills its
+// matrices too.
+constexpr int kTlMaxEdge = 2 * (512 / kDig / 8 * 8);   // tline_supported: the accumulators of np <= 72
+struct DigitF16 {
+    uint16_t f[256];                               // f16 of -128 .. 127
+    constexpr DigitF16() : f{}
+    {
         for (int b = 0; b < 256; ++b) {
             int a = b < 128 ? 128 - b : b - 128, ex = 0;
             while ((a >> ex) > 1) ++ex;
-            d[b] = a == 0 ? 0 : (uint16_t)((b < 128 ? 0x8000 : 0) | ((ex + 15) << 10) | ((a << (10 - ex)) & 0x3ff));
+            f[b] = a == 0 ? 0 : (uint16_t)((b < 128 ? 0x8000 : 0) | ((ex + 15) << 10) | ((a << (10 - ex)) & 0x3ff));
         }
-        return d;
-    }();
+    }
+};
+template <typename F> int pack_matrix(int n, const long double *entry, int entries, F at, uint16_t *img)
+{
+    const TlShape s = tl_shape(n);
+    const int h = s.h;
+    static constexpr DigitF16 digit;
     long double big = 0.0L;
-    for (long double x : entry) big = std::max(big, fabsl(x));
+    for (int i = 0; i < entries; ++i) big = std::max(big, fabsl(entry[i]));
     int e = 0;
     frexpl(big, &e);                               // big in [2^(e-1), 2^e)
     const int mexp = 54 - e;                       // integers up to 2^54
-    std::vector<uint64_t> fixed(entry.size());
-    for (size_t i = 0; i < entry.size(); ++i) fixed[i] = (uint64_t)llroundl(ldexpl(entry[i], mexp)) + kDigBias;
+    uint64_t fixed[3 * kTlMaxEdge];
+    for (int i = 0; i < entries; ++i) fixed[i] = (uint64_t)llroundl(ldexpl(entry[i], mexp)) + kDigBias;
     std::fill(img, img + tline_matrix_bytes(n) / 2, (uint16_t)0);
     for (int half = 0; half < 2; ++half)
         for (int j = 0; j < h; ++j) {
@@ -475,7 +481,7 @@ template <typename F> int pack_matrix(int n, const std::vector<long double> &ent
             for (int l = 0; l < h; ++l) {
                 const uint64_t b = fixed[at(half, j, l)];
                 uint16_t *p = base + ((size_t)(l / 8) * kDig * width + jj) * 8 + l % 8;
-                for (int d = 0; d < kDig; ++d) p[(size_t)d * width * 8] = digit[(b >> (8 * (6 - d))) & 0xff];
+                for (int d = 0; d < kDig; ++d) p[(size_t)d * width * 8] = digit.f[(b >> (8 * (6 - d))) & 0xff];
             }
         }
     return mexp;
@@ -489,7 +495,7 @@ const long double kTwoPiL = 6.283185307179586476925286766559005768L;
 int tline_derivative_matrix(int n, double scale, uint16_t *img)
 {
     const int h = n / 2;
-    std::vector<long double> D(n, 0.0L), t(2 * (size_t)n);
+    long double D[kTlMaxEdge] = {}, t[2 * kTlMaxEdge];
     for (int m = 1; m < n; ++m) {
         const long double x = 0.5L * kTwoPiL * m / n;
         D[m] = (long double)scale * 0.5L * ((m & 1) ? -1.0L : 1.0L) * (2 * m == n ? 0.0L : cosl(x) / sinl(x));
@@ -499,26 +505,26 @@ int tline_derivative_matrix(int n, double scale, uint16_t *img)
         t[m] = 0.5L * (a + b);
         t[n + m] = 0.5L * (a - b);
     }
-    return pack_matrix(n, t, [&](int half, int j, int l) { return (size_t)half * n + (j - l + n) % n; }, img);
+    return pack_matrix(n, t, 2 * n, [&](int half, int j, int l) { return (size_t)half * n + (j - l + n) % n; }, img);
 }
 
 int tline_fourier_matrix(int n, bool inverse, uint16_t *img)
 {
     const int h = n / 2;
     const long double edge = 1.0L / sqrtl((long double)n), mid = sqrtl(2.0L / (long double)n);
-    std::vector<long double> t(3 * (size_t)n);     // cosines, sines, cosines of the end frequencies
+    long double t[3 * kTlMaxEdge];                 // cosines, sines, cosines of the end frequencies
     for (int m = 0; m < n; ++m) {
         t[m] = mid * cosl(kTwoPiL * m / n);
         t[n + m] = mid * sinl(kTwoPiL * m / n);
         t[2 * n + m] = edge * cosl(kTwoPiL * m / n);
     }
-    std::vector<int> k(n), type(n);
+    int k[kTlMaxEdge], type[kTlMaxEdge];
     for (int a = 0; a < n; ++a) {
         bool sine;
         k[a] = real_freq(n, a, sine);
         type[a] = sine ? 1 : (k[a] == 0 || 2 * k[a] == n ? 2 : 0);
     }
-    return pack_matrix(n, t, [&](int half, int out, int in) {
+    return pack_matrix(n, t, 3 * n, [&](int half, int out, int in) {
         const int a = (inverse ? in : out) + half * h, j = inverse ? out : in;
         return (size_t)type[a] * n + (size_t)(k[a] * j) % n;
     }, img);

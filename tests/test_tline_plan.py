@@ -3,7 +3,8 @@
 set takes the real-basis form only with all three derivative matrices: a grid
 spacing whose matrix leaves the exponent range keeps that axis, and with it
 the Hartree chain, on the FFT passes, and axes of one length never share a
-matrix that is not there.  The GPU case evaluates such a cell."""
+matrix that is not there.  Laying out matrices takes no host memory (the
+allocation-free entry point does it on its first call).  The GPU case evaluates such a cell."""
 import os
 import subprocess
 
@@ -18,9 +19,19 @@ LIBDIR = os.path.join(ROOT, "paper_1406_0835_gb300", "_build")
 SRC = r"""
 #include <cstdio>
 #include <cstdlib>
+#include <new>
 #include <vector>
 #include "kernels.h"
 using namespace ofdft;
+static long long news = 0;             // also counts the library's
+void *operator new(size_t n)
+{
+    ++news;
+    if (void *p = malloc(n)) return p;
+    throw std::bad_alloc();
+}
+void operator delete(void *p) noexcept { free(p); }
+void operator delete(void *p, size_t) noexcept { free(p); }
 int main(int, char **v)
 {
     GridInfo g{};
@@ -38,9 +49,14 @@ int main(int, char **v)
         int e = 999;
         if (tline_supported(n3[a])) {
             std::vector<uint16_t> img(tline_matrix_bytes(n3[a]) / 2);
+            const long long before = news;
             e = tline_derivative_matrix(n3[a], g.ds[a] * n3[a], img.data());
+            for (int inv = 0; inv < 2; ++inv) tline_fourier_matrix(n3[a], inv, img.data());
+            news -= before;
+        } else {
+            news = 0;
         }
-        printf(" %d", e);
+        printf(" %d %lld", e, news);
     }
     return 0;
 }
@@ -59,7 +75,7 @@ def plan(tmp_path_factory):
 
     def run(grid, L, gga):
         out = subprocess.check_output([str(exe)] + [str(x) for x in (*grid, *L, int(gga))]).split()
-        return [x == b"1" for x in out[:3]], out[3] == b"1", [int(x) for x in out[4:]]
+        return [x == b"1" for x in out[:3]], out[3] == b"1", [int(x) for x in out[4::2]], [int(x) for x in out[5::2]]
     return run
 
 
@@ -68,10 +84,11 @@ def plan(tmp_path_factory):
                                      (1.0e5, 0.3, 0.3), (1.0e-40, 1.0, 1.0)])
 def test_a_set_takes_the_form_its_matrices_allow(plan, grid, spacing):
     L = [n * s for n, s in zip(grid, spacing)]
-    der, real, mexp = plan(grid, L, True)
+    der, real, mexp, news = plan(grid, L, True)
     assert der == [-60 <= e <= 68 for e in mexp]
     assert real == all(der)
-    der, real, _ = plan(grid, L, False)
+    assert news == [0, 0, 0]
+    der, real, _, _ = plan(grid, L, False)
     assert der == [False] * 3
     assert real == all(n <= 144 for n in grid)
 
