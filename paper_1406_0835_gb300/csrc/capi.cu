@@ -342,31 +342,14 @@ EvalScalars unpack_sums(const double *h, bool fttf)
 
 // Kernels of one evaluation (GGA: two tensor-core launches instead of a pass
 // per axis and half for the axes they take).
-int eval_kernel_count(const ofdft_ctx *c, const FieldSet &f)
+int eval_kernel_count(const ofdft_ctx *c, const FieldSet &f, bool real)
 {
-    if (f.real_basis) return c->fp.kind == 0 ? 10 : 12;
+    if (real) return c->fp.kind == 0 ? 10 : 12;
     if (c->fp.kind == 0) return 6;
     const int tc = (f.tl[0].der.img ? 1 : 0) + (f.tl[1].der.img ? 1 : 0);
     return 11 - 2 * tc + (tc || f.tl[2].der.img ? 2 : 0);
 }
 
-// Enqueue one energy + potential evaluation at ph (or, with phi0 and dh, at the
-// trial phi0 cos + dh sin written into ph; angles from csd (two T values in
-// device memory) if given).  Sums go to sums[0..17].  With keep_nG, n(G) is
-// left in the second spectrum (forces, stress).  With spart (FP64 GGA sets),
-// the pointwise stage also writes the gradient stress sums: spart holds 12
-// partial rows of *nbg_out columns.  No synchronisation.
-//
-// ftTF:  zfwd (n, R2C z) -> y -> x [Hartree, LPP, energies, v_HL(G), x^-1]
-//        -> y^-1 -> zfinal [C2R z, pointwise, potential, sums].
-// GGA:   the same Hartree path, and the gradient and divergence one axis at
-//        a time (the derivative along axis j needs transforms along j only):
-//        d_x n, d_y n, d_z n into the second to fourth spectra, used as real
-//        fields; pointwise: v_part and U_j over the derivatives; d_x U_x,
-//        d_y U_y, d_z U_z in place; zfinal_gga: v = v_HL + v_part - their
-//        sum, sums.  Derivatives of double-float sets run on the tensor
-//        cores (one launch for all axes, from the field n that zfwd writes);
-//        other axes take dline along x and y, zfwd and zfinal_gga along z.
 // n(G) for forces and stress: forward z, y, x of n into the second spectrum.
 ofdft_status enqueue_nG(ofdft_ctx *c, FieldSet &f, double *ph, double *part)
 {
@@ -505,10 +488,31 @@ ofdft_status enqueue_real(ofdft_ctx *c, FieldSet &f, double *ph, const double *p
     DBG("k_final");
     launch_reduce_eval(pA, nbx, pB, nbg, pC, nbz, !fttf, sums, st);
     DBG("k_reduce_eval");
-    c->launches += eval_kernel_count(c, f);
+    c->launches += eval_kernel_count(c, f, true);
     return OFDFT_OK;
 }
 
+// Enqueue one energy + potential evaluation at ph (or, with phi0 and dh, at the
+// trial phi0 cos + dh sin written into ph; angles from csd (two T values in
+// device memory) if given).  Sums go to sums[0..17].  With keep_nG, n(G) is
+// left in the second spectrum (forces, stress).  With spart (FP64 GGA sets),
+// the pointwise stage also writes the gradient stress sums: spart holds 12
+// partial rows of *nbg_out columns.  No synchronisation.
+//
+// ftTF:  zfwd (n, R2C z) -> y -> x [Hartree, LPP, energies, v_HL(G), x^-1]
+//        -> y^-1 -> zfinal [C2R z, pointwise, potential, sums].
+// GGA:   the same Hartree path, and the gradient and divergence one axis at
+//        a time (the derivative along axis j needs transforms along j only):
+//        d_x n, d_y n, d_z n into the second to fourth spectra, used as real
+//        fields; pointwise: v_part and U_j over the derivatives; d_x U_x,
+//        d_y U_y, d_z U_z in place; zfinal_gga: v = v_HL + v_part - their
+//        sum, sums.  Derivatives of double-float sets run on the tensor
+//        cores (one launch for all axes, from the field n that zfwd writes);
+//        other axes take dline along x and y, zfwd and zfinal_gga along z.
+// Sets in the real basis take enqueue_real, but for ftTF with keep_nG: there
+// n(G) falls out of the FFT form's x pass, where the real basis needs three
+// passes more.  ftTF forces in one call, real basis -> here (us): 16^3 139 ->
+// 125, 32^3 153 -> 138, 48^3 186 -> 160, 96^3 317 -> 305, 144^3 977 -> 845.
 template <typename T>
 ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const T *dh, double cth,
                           double sth, const void *csd, T *vout, bool keep_nG, double *sums,
@@ -529,7 +533,7 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
     const long long npairs = (long long)g.nx * g.ny / 2;
     double *pA = c->part, *pB = pA + 3 * nbx, *pC = pB + 6 * npairs;
     if constexpr (sizeof(T) == 8) {
-        if (f.real_basis) {
+        if (f.real_basis && !(fttf && keep_nG)) {
             ofdft_status r = enqueue_real(c, f, ph, phi0, dh, cth, sth, (const double *)csd, vout, sums, spart, nbg_out);
             if (r != OFDFT_OK || !keep_nG) return r;
             return enqueue_nG(c, f, ph, pA);
@@ -647,7 +651,7 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
     DBG("k_zfinal");
     launch_reduce_eval(pA, nbx, pB, nbg, pC, nbz, !fttf, sums, st);
     DBG("k_reduce_eval");
-    c->launches += eval_kernel_count(c, f);
+    c->launches += eval_kernel_count(c, f, false);
     if (keep_nG && !fttf) {
         if constexpr (sizeof(T) == 8) return enqueue_nG(c, f, ph, pA);
     }
@@ -1087,8 +1091,8 @@ ofdft_status minimize_start(ofdft_ctx *c, double gtol, int maxit)
 // (direction + update), per line-search trial (evaluation + controller).
 long long graph_launches(const ofdft_ctx *c, const FieldSet &f, const CgState &h)
 {
-    return 8 + eval_kernel_count(c, f) + (long long)h.nouter * 9 +
-           (long long)(h.nevals - 1) * (eval_kernel_count(c, f) + 1);
+    const int k = eval_kernel_count(c, f, f.real_basis);
+    return 8 + k + (long long)h.nouter * 9 + (long long)(h.nevals - 1) * (k + 1);
 }
 
 ofdft_status finish_minimize(ofdft_ctx *c, bool graph, ofdft_stats &stats, EvalScalars &es);
