@@ -238,7 +238,6 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
         }
         __syncwarp();
         tc::tmem_alloc(tc::smem_addr(&s_tmem), sh.cols);
-        pdl_trigger();                             // not before: see pdl.cuh
         __syncwarp();
         tc::fence_before_sync();
         bar_arrive(4, blockDim.x);                 // barriers and tensor memory are there
@@ -270,7 +269,11 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
     const long long ln_off = (w_ok ? ou * jb.ostride + (zaxis ? 0 : ln - ou * zlen) : 0) + (half ? h * rstride : 0);
     const bool wide = zaxis && (h & 1) == 0;
     if (tid < kLines) s_max[tid] = 27u << 23;      // 2^-100: the least exponent of the scale
+    bar_sync(4, blockDim.x);
+    tc::fence_after_sync();
+    const uint32_t tmem = s_tmem;
     pdl_wait();                                    // (the issuing warp reads nothing that another kernel writes)
+    pdl_trigger();                                 // the block has its tensor memory: see pdl.cuh
     float2 v[16];
     if (mine) {
         const int line = tile * kLines + row;
@@ -346,9 +349,6 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
     }
     tc::fence_async();
     bar_arrive(2, blockDim.x);
-    bar_sync(4, blockDim.x);
-    tc::fence_after_sync();
-    const uint32_t tmem = s_tmem;
 
     const uint32_t m = s_max[r];
     // weight 1 stands for 2^96 times the integers' units 2^(E - 52) and 2^-mexp

@@ -55,7 +55,10 @@ def test_tensor_memory_is_held_before_the_next_kernel_may_start():
         body = k[n][1]
         assert "pdl_enter" not in body, n
         assert body.count("pdl_trigger()") == 1, n
-        assert body.index("tmem_alloc") < body.index("pdl_trigger()"), n
+        # the allocating warp's barrier lies between the two
+        known = re.search(r"bar_arrive\(4,.*?bar_sync\(4,|__syncthreads\(\)", body[body.index("tmem_alloc"):], re.S)
+        assert body.index("tmem_alloc") + known.end() < body.index("pdl_trigger()"), n
+        assert body.index("pdl_wait()") < body.index("pdl_trigger()"), n
 
 
 def test_dependent_kernels_restrict_only_tables():
