@@ -1721,9 +1721,10 @@ ofdft_status busy(ofdft_ctx *c)
 // ------------------------------------------------------------ autotuner
 struct TuneKey {
     int nx, ny, nz, prec;
+    bool real_basis;   // tuned by the passes that such a set takes
     bool operator<(const TuneKey &o) const
     {
-        return std::tie(nx, ny, nz, prec) < std::tie(o.nx, o.ny, o.nz, o.prec);
+        return std::tie(nx, ny, nz, prec, real_basis) < std::tie(o.nx, o.ny, o.nz, o.prec, o.real_basis);
     }
 };
 std::mutex g_tune_mu;
@@ -1744,16 +1745,22 @@ void set_radix(FieldSet &f, int a, int m)
 }
 std::map<TuneKey, Tuned> g_tune;
 
-// Mean time of `reps` evaluations of field set f at its current phi.
+// Mean time of `reps` evaluations of field set f at its current phi; of a set
+// in the real basis, whose evaluations have one shape, of the FFT passes that
+// its forces and stress take: n(G) (ftTF: the evaluation that yields it).
 template <typename T> ofdft_status time_evals(ofdft_ctx *c, FieldSet &f, int reps, float &ms)
 {
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    ofdft_status r = enqueue_eval<T>(c, f, (T *)f.phi, nullptr, nullptr, 1.0, 0.0, nullptr, (T *)f.vt, false, c->scal);
+    auto run = [&]() -> ofdft_status {
+        if constexpr (sizeof(T) == 8)
+            if (f.real_basis && c->fp.kind != 0) return enqueue_nG(c, f, (double *)f.phi, c->part);
+        return enqueue_eval<T>(c, f, (T *)f.phi, nullptr, nullptr, 1.0, 0.0, nullptr, (T *)f.vt, f.real_basis, c->scal);
+    };
+    ofdft_status r = run();
     cudaEventRecord(e0, c->st);
-    for (int i = 0; i < reps && r == OFDFT_OK; ++i)
-        r = enqueue_eval<T>(c, f, (T *)f.phi, nullptr, nullptr, 1.0, 0.0, nullptr, (T *)f.vt, false, c->scal);
+    for (int i = 0; i < reps && r == OFDFT_OK; ++i) r = run();
     cudaEventRecord(e1, c->st);
     cudaError_t e = cudaEventSynchronize(e1);
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
@@ -1765,15 +1772,14 @@ template <typename T> ofdft_status time_evals(ofdft_ctx *c, FieldSet &f, int rep
     return OFDFT_OK;
 }
 
-// Pick the launch shapes by timing whole evaluations: tile width and
+// Pick the launch shapes by timing whole evaluations (time_evals): tile width and
 // threads of the y/x passes together, then line pairs per block and threads
 // of the z passes, then tile width and threads of the derivative passes,
 // then each axis's radix schedule.
 template <typename T> ofdft_status autotune_set(ofdft_ctx *c, int k, int reps)
 {
     FieldSet &f = c->f[k];
-    if (f.real_basis) return OFDFT_OK;   // the tensor-core transforms have one shape
-    const TuneKey key{c->g.nx, c->g.ny, c->g.nz, (int)sizeof(T)};
+    const TuneKey key{c->g.nx, c->g.ny, c->g.nz, (int)sizeof(T), f.real_basis};
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune.find(key);

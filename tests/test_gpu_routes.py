@@ -40,3 +40,18 @@ def test_fttf_forces_take_n_of_G_from_the_evaluation(grid):
         n, (E, _) = launches(ctx, lambda: ctx.energy_potential(None, want_v=False))
         assert n == 10                      # the real-basis form
     assert abs(P - E["P"]) <= 1e-12 * (abs(E["P_s"]) + abs(E["P_H"]) + abs(E["P_loc"]) + abs(E["P_ion"]))
+
+
+# (grids of their own: the shapes found are kept per grid for the process)
+@pytest.mark.parametrize("functional,grid", [("fttf", (30, 24, 36)), ("vt84f", (36, 24, 30))])
+def test_autotune_times_the_passes_that_are_left(functional, grid):
+    with context(functional, grid) as a, context(functional, grid) as b:
+        n, _ = launches(a, lambda: a.autotune(reps=2))
+        assert n > 0
+        E, Ea = b.energy_potential(None, want_v=False)[0], a.energy_potential(None, want_v=False)[0]
+        assert E == Ea                      # real-basis evaluations have one shape
+        (F, _), (Fa, _) = b.forces(), a.forces()
+        assert np.max(np.abs(F - Fa)) <= 1e-12 * np.max(np.abs(F))
+        a.set_phi()
+        b.set_phi()
+        assert a.minimize(gtol=1e-6)[0]["F_tot"] == b.minimize(gtol=1e-6)[0]["F_tot"]
