@@ -194,14 +194,19 @@ constexpr int kTfSize = kTfPanels * kTfFuncs * kTfNc;
 // The double-float kernels read the same polynomials re-expanded about the
 // centres of kTfRef subpanels: their terms fall off kTfRef times faster per
 // degree, so that those from degree kTfSplit up can be summed in binary32
-// (pointwise.cuh).  Layout per subpanel, in double-float pairs (8 bytes):
-// degrees 0 .. kTfSplit - 1 as pairs [degree][function], then the degrees
-// up to kTfDdDeg as binary32 [degree][function]; 16-byte loads throughout.
+// (pointwise.cuh).  A and B, whose coefficients fall off slowest, keep one
+// degree more as pairs and one degree more in all (the terms of degree 10 are
+// below 4e-18 of xi; of A and B they would be 2e-13 of the t-derivative).
+// Layout per subpanel, in rows of 16 bytes: degrees 0 .. kTfSplit - 1 as
+// pairs, two functions a row; A and B of degree kTfSplit as pairs; degrees
+// kTfSplit + 1 .. kTfDdDeg in binary32, four functions a row; and (xi, zeta
+// of degree kTfSplit, A, B of degree 10).
 constexpr int kTfRef = 4;
 constexpr int kTfDdSub = kTfSub * kTfRef;
-constexpr int kTfDdDeg = 9;                // the terms of degree 10 are below 3e-16 of their function
+constexpr int kTfDdDeg = 9;
 constexpr int kTfSplit = 5;
-constexpr int kTfDdRow = kTfSplit * kTfFuncs + (kTfDdDeg + 1 - kTfSplit) * kTfFuncs / 2;
+constexpr int kTfDdRows = 2 * kTfSplit + 1 + (kTfDdDeg - kTfSplit) + 1;   // 256 bytes
+constexpr int kTfDdRow = 2 * kTfDdRows;
 constexpr int kTfDdSize = kTfPanels * kTfRef * kTfDdRow;
 
 // VT84F enhancement factor F(x), x = s^2 (Eq. (VT84F)), as a table of

@@ -304,7 +304,7 @@ constexpr double kPwNmin = 1e-18, kPwNmax = 1e18, kPwS2max = 1e10;
 // polynomial enters with on every panel, so binary32 rounding there stays
 // below the double-float rounding.
 struct HornerF2 {
-    ff::f2 p, dp;   // unnormalised
+    ff::f2 p, dp;
     float d2;
 };
 OF_HD void horner_lo(HornerF2 &h, float u, float c)
@@ -316,19 +316,22 @@ OF_HD void horner_lo(HornerF2 &h, float u, float c)
 OF_HD void horner_dd(HornerF2 &h, float u, ff::f2 c)
 {
     h.d2 = h.d2 * u + h.dp.hi;
-    h.dp = ff::fma_step_u(h.dp, u, h.p);
-    h.p = ff::fma_step_u(h.p, u, c);
+    h.dp = ff::fma_step(h.dp, u, h.p);
+    h.p = ff::fma_step(h.p, u, c);
 }
 
 // Table polynomials with the refined double-float table (kTfDdSub panels an
 // octave).  The panel variable u = uh + ul: uh is exact in binary32 and the
 // Horner sums run with it; ul (below 2e-6) enters through the first and
-// second derivatives.  The tails from degree kTfSplit up, over every panel:
-// 6e-10 of xi, 1e-9 of xi for zeta (zeta comes close to zero but enters only
-// beside xi, f = tau0 xi F_tau - tau0 zeta F_sigma), 3e-8 of A and 5e-8 of
-// the larger of B and A xi / zeta (B enters through zeta F(s^2 B) beside
-// xi F(s^2 A)).  With the unrefined panels 7, 7, 8 and all 10 degrees needed
-// double-float: 32 steps instead of 20.
+// second derivatives.  The tails in binary32 cost, over every panel, at most
+// 4e-17 of xi, 8e-17 of xi for zeta (zeta comes close to zero but enters only
+// beside xi, f = tau0 xi F_tau - tau0 zeta F_sigma), 5e-17 of A and 8e-17 of
+// the larger of B and A xi / zeta (B enters through zeta F(s^2 B) beside xi
+// F(s^2 A)); of the derivatives per ln t, which the potential takes, 6e-15,
+// 1.3e-14, 9e-15 and 1.6e-14.  (A and B from degree 5 up in binary32 and
+// without degree 10 put 8e-13 into df/dn where s^2 is large.)  With the
+// unrefined panels 7, 7, 8 and all 10 degrees needed double-float: 32 steps
+// instead of 22.
 template <int NF>
 OF_HD void tfunc_eval_f2(const ff::f2 *__restrict__ tab, ff::f2 t, ff::f2 out[8])
 {
@@ -341,14 +344,14 @@ OF_HD void tfunc_eval_f2(const ff::f2 *__restrict__ tab, ff::f2 t, ff::f2 out[8]
     const float ul = (float)(2 * kTfDdSub) * t.lo * inv2e;
     const float dudt = (float)(2 * kTfDdSub) * inv2e;
     const float4 *c = reinterpret_cast<const float4 *>(tab + (size_t)((e - kTfEmin) * kTfDdSub + sub) * kTfDdRow);
-    const float4 *tail = c + kTfSplit * 2;
+    const float4 *tail = c + 2 * kTfSplit;               // tail[k]: degree kTfSplit + k (k = 0: A and B, pairs)
+    const float4 ends = c[kTfDdRows - 1], top = tail[kTfDdDeg - kTfSplit];
     HornerF2 h[NF];
-    const float4 top = tail[kTfDdDeg - kTfSplit];
     h[0].p.hi = top.x;
     h[1].p.hi = top.y;
     if (NF == 4) {
-        h[2].p.hi = top.z;
-        h[3].p.hi = top.w;
+        h[2].p.hi = ends.z;
+        h[3].p.hi = ends.w;
     }
 #pragma unroll
     for (int q = 0; q < NF; ++q) {
@@ -356,12 +359,23 @@ OF_HD void tfunc_eval_f2(const ff::f2 *__restrict__ tab, ff::f2 t, ff::f2 out[8]
         h[q].dp = ff::f2(0.0f, 0.0f);
         h[q].d2 = 0.0f;
     }
+    if (NF == 4) {
+        horner_lo(h[2], uh, top.z);
+        horner_lo(h[3], uh, top.w);
+    }
 #pragma unroll 1
-    for (int j = kTfDdDeg - kTfSplit - 1; j >= 0; --j) {
+    for (int j = kTfDdDeg - kTfSplit - 1; j >= 1; --j) {
         const float4 a = tail[j];
         const float cj[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
         for (int q = 0; q < NF; ++q) horner_lo(h[q], uh, cj[q]);
+    }
+    horner_lo(h[0], uh, ends.x);
+    horner_lo(h[1], uh, ends.y);
+    if (NF == 4) {
+        const float4 a = tail[0];
+        horner_dd(h[2], uh, ff::f2(a.x, a.y));
+        horner_dd(h[3], uh, ff::f2(a.z, a.w));
     }
 #pragma unroll 1
     for (int j = kTfSplit - 1; j >= 0; --j) {
@@ -570,6 +584,7 @@ OF_HD bool pw_core_f2(const FuncParams &fp, const ff::f2 *__restrict__ tab, ff::
     const f2 n23 = mul(c13, c13);
     const f2 rn = mul(y2, y);                                // 1/n
     const f2 tau0 = mul(mul(n, n23), FFC(OF_CTF));           // Eq. (tauTFdefn)
+    const f2 dtau0 = mul(n23, FFC(5.0 / 3.0 * OF_CTF));
     const f2 dtdn = mul(mul(t, rn), FFC(-2.0 / 3.0));
     f2 tf[8];
     if (fp.kind == 0) {                                      // ftTF
@@ -577,7 +592,6 @@ OF_HD bool pw_core_f2(const FuncParams &fp, const ff::f2 *__restrict__ tab, ff::
         const f2 kap = sub(tf[0], tf[1]);
         o.f = mul(tau0, kap);
         o.ts = mul(tau0, tf[1]);
-        const f2 dtau0 = mul(n23, FFC(5.0 / 3.0 * OF_CTF));
         o.dfdn = add(mul(dtau0, kap), mul(mul(tau0, sub(tf[4], tf[5])), dtdn));   // Eq. (vTF)
         o.w[0] = o.w[1] = o.w[2] = o.wg = f2(0.0f, 0.0f);
     } else {
@@ -610,8 +624,8 @@ OF_HD bool pw_core_f2(const FuncParams &fp, const ff::f2 *__restrict__ tab, ff::
         const f2 e83 = mul(rn, FFC(-8.0 / 3.0));
         const f2 s2dt = mul(s2, dtdn);
         const f2 kF = mul(kin, dFt), sF = mul(ent, dFs);
-        // Eq. (vftGGA), first two lines; dtau0 (xi F_tau - zeta F_sigma) = (5/3) f / n
-        f2 d = mul(div(o.f, n), FFC(5.0 / 3.0));
+        // Eq. (vftGGA), first two lines
+        f2 d = mul(dtau0, add_s(mul(xi, Ft), neg(mul(ze, Fs))));
         d = add_s(d, mul(mul(tau0, dtdn), add_s(mul(dxi, Ft), neg(mul(dze, Fs)))));
         d = add_s(d, mul(kF, add_s(mul(e83, xt), mul(s2dt, dA))));
         d = add_s(d, neg(mul(sF, add_s(mul(e83, xs), mul(s2dt, dB)))));
@@ -668,13 +682,18 @@ inline void dd_tables_fill(const double *ttab, double *dst)
                 for (int k = 0; k < kTfDeg; ++k)
                     for (int j = kTfDeg - 1; j >= k; --j) a[j] += ctr * a[j + 1];
                 float *row = rf + 2 * (size_t)(p * kTfRef + s) * kTfDdRow;
-                for (int k = 0; k <= kTfDdDeg; ++k, sc /= kTfRef) {
+                for (int k = 0; k <= kTfDeg; ++k, sc /= kTfRef) {
                     const ff::f2 c = ff::from_double(a[k] * sc);
-                    if (k < kTfSplit) {
-                        row[2 * (k * kTfFuncs + q)] = c.hi;
-                        row[2 * (k * kTfFuncs + q) + 1] = c.lo;
-                    } else {
-                        row[2 * kTfSplit * kTfFuncs + (k - kTfSplit) * kTfFuncs + q] = c.hi;
+                    if (k < kTfSplit || (k == kTfSplit && q >= 2)) {
+                        float *pair = row + (k < kTfSplit ? 2 * (k * kTfFuncs + q) : 8 * kTfSplit + 2 * (q - 2));
+                        pair[0] = c.hi;
+                        pair[1] = c.lo;
+                    } else if (k == kTfSplit) {
+                        row[4 * (kTfDdRows - 1) + q] = c.hi;
+                    } else if (k <= kTfDdDeg) {
+                        row[4 * (k + kTfSplit) + q] = c.hi;
+                    } else if (q >= 2) {
+                        row[4 * (kTfDdRows - 1) + q] = c.hi;
                     }
                 }
             }
