@@ -304,7 +304,7 @@ constexpr double kPwNmin = 1e-18, kPwNmax = 1e18, kPwS2max = 1e10;
 // polynomial enters with on every panel, so binary32 rounding there stays
 // below the double-float rounding.
 struct HornerF2 {
-    ff::f2 p, dp;
+    ff::f2 p, dp;   // unnormalised but for the last step
     float d2;
 };
 OF_HD void horner_lo(HornerF2 &h, float u, float c)
@@ -314,6 +314,21 @@ OF_HD void horner_lo(HornerF2 &h, float u, float c)
     h.p.hi = h.p.hi * u + c;
 }
 OF_HD void horner_dd(HornerF2 &h, float u, ff::f2 c)
+{
+    h.d2 = h.d2 * u + h.dp.hi;
+    h.dp = ff::fma_step_u(h.dp, u, h.p);
+    h.p = ff::fma_step_u(h.p, u, c);
+}
+// The step from a binary32 tail to its first pair (the derivative, one degree
+// behind, stays in binary32), and the last step.
+OF_HD void horner_first(HornerF2 &h, float u, ff::f2 c)
+{
+    h.d2 = h.d2 * u + h.dp.hi;
+    h.dp.hi = h.dp.hi * u + h.p.hi;
+    const ff::f2 m = ff::two_prod(h.p.hi, u), s = ff::two_sum(m.hi, c.hi);
+    h.p = ff::f2(s.hi, ff::fadd(m.lo, ff::fadd(s.lo, c.lo)));
+}
+OF_HD void horner_last(HornerF2 &h, float u, ff::f2 c)
 {
     h.d2 = h.d2 * u + h.dp.hi;
     h.dp = ff::fma_step(h.dp, u, h.p);
@@ -374,11 +389,11 @@ OF_HD void tfunc_eval_f2(const ff::f2 *__restrict__ tab, ff::f2 t, ff::f2 out[8]
     horner_lo(h[1], uh, ends.y);
     if (NF == 4) {
         const float4 a = tail[0];
-        horner_dd(h[2], uh, ff::f2(a.x, a.y));
-        horner_dd(h[3], uh, ff::f2(a.z, a.w));
+        horner_first(h[2], uh, ff::f2(a.x, a.y));
+        horner_first(h[3], uh, ff::f2(a.z, a.w));
     }
 #pragma unroll 1
-    for (int j = kTfSplit - 1; j >= 0; --j) {
+    for (int j = kTfSplit - 1; j >= 1; --j) {
         const float4 a = c[2 * j];
         horner_dd(h[0], uh, ff::f2(a.x, a.y));
         horner_dd(h[1], uh, ff::f2(a.z, a.w));
@@ -387,6 +402,14 @@ OF_HD void tfunc_eval_f2(const ff::f2 *__restrict__ tab, ff::f2 t, ff::f2 out[8]
             horner_dd(h[2], uh, ff::f2(b.x, b.y));
             horner_dd(h[3], uh, ff::f2(b.z, b.w));
         }
+    }
+    const float4 a0 = c[0];
+    horner_last(h[0], uh, ff::f2(a0.x, a0.y));
+    horner_last(h[1], uh, ff::f2(a0.z, a0.w));
+    if (NF == 4) {
+        const float4 b0 = c[1];
+        horner_last(h[2], uh, ff::f2(b0.x, b0.y));
+        horner_last(h[3], uh, ff::f2(b0.z, b0.w));
     }
 #pragma unroll
     for (int q = 0; q < NF; ++q) {
@@ -584,7 +607,6 @@ OF_HD bool pw_core_f2(const FuncParams &fp, const ff::f2 *__restrict__ tab, ff::
     const f2 n23 = mul(c13, c13);
     const f2 rn = mul(y2, y);                                // 1/n
     const f2 tau0 = mul(mul(n, n23), FFC(OF_CTF));           // Eq. (tauTFdefn)
-    const f2 dtau0 = mul(n23, FFC(5.0 / 3.0 * OF_CTF));
     const f2 dtdn = mul(mul(t, rn), FFC(-2.0 / 3.0));
     f2 tf[8];
     if (fp.kind == 0) {                                      // ftTF
@@ -592,6 +614,7 @@ OF_HD bool pw_core_f2(const FuncParams &fp, const ff::f2 *__restrict__ tab, ff::
         const f2 kap = sub(tf[0], tf[1]);
         o.f = mul(tau0, kap);
         o.ts = mul(tau0, tf[1]);
+        const f2 dtau0 = mul(n23, FFC(5.0 / 3.0 * OF_CTF));
         o.dfdn = add(mul(dtau0, kap), mul(mul(tau0, sub(tf[4], tf[5])), dtdn));   // Eq. (vTF)
         o.w[0] = o.w[1] = o.w[2] = o.wg = f2(0.0f, 0.0f);
     } else {
@@ -624,8 +647,8 @@ OF_HD bool pw_core_f2(const FuncParams &fp, const ff::f2 *__restrict__ tab, ff::
         const f2 e83 = mul(rn, FFC(-8.0 / 3.0));
         const f2 s2dt = mul(s2, dtdn);
         const f2 kF = mul(kin, dFt), sF = mul(ent, dFs);
-        // Eq. (vftGGA), first two lines
-        f2 d = mul(dtau0, add_s(mul(xi, Ft), neg(mul(ze, Fs))));
+        // Eq. (vftGGA), first two lines; dtau0 (xi F_tau - zeta F_sigma) = (5/3) f / n
+        f2 d = mul(div(o.f, n), FFC(5.0 / 3.0));
         d = add_s(d, mul(mul(tau0, dtdn), add_s(mul(dxi, Ft), neg(mul(dze, Fs)))));
         d = add_s(d, mul(kF, add_s(mul(e83, xt), mul(s2dt, dA))));
         d = add_s(d, neg(mul(sF, add_s(mul(e83, xs), mul(s2dt, dB)))));
