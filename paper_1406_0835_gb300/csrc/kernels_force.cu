@@ -76,9 +76,9 @@ __device__ __forceinline__ void ion_phase(int c, const double2 *__restrict__ p, 
 // f_c' enters divided by the block's highest frequency and times 7/4 (below
 // 2^55: the leading digit still fits).  The fixed-point errors of T' are
 // relative to that frequency while its sum comes from lower ones, so T' keeps
-// the products of one weight more than T (B's digit 7 is zero and clears
-// their accumulator): 64 ions at 64^3, error of the forces along x, y, z in
-// Ha/bohr 2, 2, 8e-15 without, 2.5, 2.3, 3.7e-15 with; the double-float kernel 2.6, 3.0, 3.1e-15.
+// the products of one weight more than T, and rows of g an eighth digit (in
+// units of 2^-60 of the row's largest value, which is often the coefficient of
+// frequency 0, whose f' is zero).
 __host__ __device__ __forceinline__ double block_top(int nz, int kb) { return 0.5 * min((kb + 1) * kKc, nz) / 1.75; }
 
 // The coefficients on two or three Nyquist frequencies, whose phases do not
@@ -272,10 +272,6 @@ __global__ void __launch_bounds__(kForceThreads, 1)
         const int ct = tid - kReadWarps * 32, row = ct >> 2, part4 = ct & 3;
         bool good = true;
         int it = 0;
-#pragma unroll
-        for (int h = 0; h < 4; ++h)                    // digit 7 of the thread's row and chunks, both buffers
-            *reinterpret_cast<uint4 *>(B + (h >> 1) * kBBuf + (part4 * 2 + (h & 1)) * kBLbo + (kDig * kRows + row) * 16) =
-                make_uint4(0, 0, 0, 0);
         for (int t = blockIdx.y; t < tiles && good; t += gridDim.y, ++it) {
             const int a = t / nbt, b = (t - a * nbt) * kRows + row, buf = it & 1;
             const int c0 = kb * kKc + part4 * 16;
@@ -308,8 +304,8 @@ __global__ void __launch_bounds__(kForceThreads, 1)
             for (int h = 0; h < 2; ++h) {
                 uint64_t q[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) q[i] = to_fixed(v[8 * h + i], u) + (kDigBias - kFixedOff);
-                store_digits(q, dst + h * kBLbo, kRows * 16);
+                for (int i = 0; i < 8; ++i) q[i] = to_fixed<60>(v[8 * h + i], u) + (kDigBias8 - fixed_off<60>());
+                store_digits<8>(q, dst + h * kBLbo, kRows * 16);
             }
             tc::fence_async();
             mbar_arrive(b_full + 8 * buf);

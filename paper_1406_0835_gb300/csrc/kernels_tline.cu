@@ -324,15 +324,15 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
         if (jb.direct_in) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                q[i] = to_fixed(v[i], u) + (kDigBias - kFixedOff);
-                const uint64_t y = to_fixed(v[8 + i], u) + (kDigBias - kFixedOff);
+                q[i] = to_fixed(v[i], u) + (kDigBias - fixed_off<52>());
+                const uint64_t y = to_fixed(v[8 + i], u) + (kDigBias - fixed_off<52>());
                 v[i] = make_float2(__uint_as_float((uint32_t)y), __uint_as_float((uint32_t)(y >> 32)));
             }
         } else {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const uint64_t x = to_fixed(v[i], u), y = to_fixed(v[8 + i], u);
-                q[i] = x + y + (kDigBias - 2 * kFixedOff);
+                q[i] = x + y + (kDigBias - 2 * fixed_off<52>());
                 const uint64_t d = x - y + kDigBias;
                 v[i] = make_float2(__uint_as_float((uint32_t)d), __uint_as_float((uint32_t)(d >> 32)));
             }
