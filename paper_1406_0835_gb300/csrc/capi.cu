@@ -600,11 +600,11 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
         tline(nf, nf, nf);
         if (!tcx) {
             TimerScope ts(c, TM_DLINE, sizeof(T) == 4);
-            launch_dline<T>(g, ax, 0, nf ? 1 : 0, 0, nf ? nf : ph, d0, st);
+            launch_dline<T>(g, ax, 0, nf ? 1 : 0, nf ? nf : ph, d0, st);
         }
         if (!tcy) {
             TimerScope ts(c, TM_DLINE, sizeof(T) == 4);
-            launch_dline<T>(g, ay, 1, nf ? 1 : 0, 0, nf ? nf : ph, d1, s2nd);
+            launch_dline<T>(g, ay, 1, nf ? 1 : 0, nf ? nf : ph, d1, s2nd);
         }
         if (fork) {
             CK(cudaEventRecord(c->fj[2], s2nd));
@@ -632,11 +632,11 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
         tline(d0, d1, d2);
         if (!tcy) {
             TimerScope ts(c, TM_DLINE, sizeof(T) == 4);
-            launch_dline<T>(g, ay, 1, 1, 0, d1, d1, st);
+            launch_dline<T>(g, ay, 1, 1, d1, d1, st);
         }
         if (!tcx) {
             TimerScope ts(c, TM_DLINE, sizeof(T) == 4);
-            launch_dline<T>(g, ax, 0, 1, 0, d0, d0, s2nd);
+            launch_dline<T>(g, ax, 0, 1, d0, d0, s2nd);
         }
         if (fork) {
             CK(cudaEventRecord(c->fj[4], s2nd));
@@ -645,7 +645,7 @@ ofdft_status enqueue_eval(ofdft_ctx *c, FieldSet &f, T *ph, const T *phi0, const
         }
         DBG("k_dline (div W)");
         TimerScope ts(c, TM_ZFINAL, sizeof(T) == 4);
-        nbz = launch_zfinal_gga<T>(g, az, s0, tcz ? nullptr : d2, (const T *)f.vpart, d1, d0, d2, ph, phi0, dh,
+        nbz = launch_zfinal_gga<T>(g, az, s0, tcz ? nullptr : d2, (const T *)f.vpart, d0, d1, d2, ph, phi0, dh,
                                    (T)cth, (T)sth, csd, vout, pC, st);
     }
     DBG("k_zfinal");

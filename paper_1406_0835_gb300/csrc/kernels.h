@@ -48,12 +48,12 @@ void launch_zfwd(const GridInfo &g, const FftAxis &az, int mode, const T *in, co
                  const T *dhat, T c, T s, const void *cs, T *phit, cplx<T> *out, cudaStream_t st,
                  T *dz = nullptr, T *nout = nullptr);
 // Derivative of a real field along grid axis 0 (x) or 1 (y) by 1-D
-// transforms along that axis: out (= or, acc != 0, +=) d f, f = phi^2 for
-// mode 0 and f = in for mode 1 (scale GridInfo::ds).  Derivative fields
-// (this out, zfwd's dz, zfinal_gga's div*) are double-float pairs in a
+// transforms along that axis: out = d f, f = phi^2 for mode 0 and f = in for
+// mode 1 (scale GridInfo::ds).  Derivative fields (this out, zfwd's dz,
+// zfinal_gga's dx, dy, dz) are double-float pairs in a
 // double-float grid (two binary32 words in a double's place).
 template <typename T>
-void launch_dline(const GridInfo &g, const FftAxis &fa, int axis, int mode, int acc, const T *in, T *out,
+void launch_dline(const GridInfo &g, const FftAxis &fa, int axis, int mode, const T *in, T *out,
                   cudaStream_t st);
 // ---- one-axis transforms on the tensor cores (kernels_tline.cu).  Fields
 // and coefficients are double-float pairs (float2).
@@ -130,11 +130,11 @@ int launch_zfinal(const GridInfo &g, const FftAxis &az, bool fttf, const cplx<T>
                   const T *vpart, const T *phit, const T *phi, const T *dhat, T c, T s,
                   const void *cs, T temp, const FuncParams &fp, const T *tab, int xc, T *vout,
                   double *part, cudaStream_t st);
-// z pass, final (GGA): v = v_HL - d_z U_z + v_part - div - div2 (div may
-// alias vout; div2 may be null); with uz null, div3 stands for d_z U_z.
+// z pass, final (GGA): v = v_HL + v_part - dx - dy - d_z U_z; with uz null, dz
+// is that last term.
 template <typename T>
 int launch_zfinal_gga(const GridInfo &g, const FftAxis &az, const cplx<T> *dspec, const T *uz, const T *vpart,
-                      const T *div, const T *div2, const T *div3, const T *phit, const T *phi, const T *dhat, T c,
+                      const T *dx, const T *dy, const T *dz, const T *phit, const T *phi, const T *dhat, T c,
                       T s, const void *cs, T *vout, double *part, cudaStream_t st);
 template <typename T>
 void launch_ypass(const GridInfo &g, const FftAxis &ay, bool inv, cplx<T> *data, int nfields,

@@ -705,10 +705,10 @@ template <typename T> struct Pair2;
 template <> struct Pair2<double> { typedef double2 type; };
 template <> struct Pair2<float> { typedef float2 type; };
 
-// out (= or +=) d_j f along grid axis AX for f = phi^2 (MODE 0) or f = in
-// (MODE 1); ACC 1 adds to out.  out may be in (each block reads its columns
-// whole before it writes them, and no other block touches them).
-template <typename PR, int AX, int MODE, int ACC>
+// out = d_j f along grid axis AX for f = phi^2 (MODE 0) or f = in (MODE 1).
+// out may be in (each block reads its columns whole before it writes them, and
+// no other block touches them).
+template <typename PR, int AX, int MODE>
 __global__ void OFDFT_FFT_BOUNDS k_dline(GridInfo g, FftAxis fa, const typename KT<PR>::T *in,
                         typename KT<PR>::T *out)
 {
@@ -749,14 +749,8 @@ __global__ void OFDFT_FFT_BOUNDS k_dline(GridInfo g, FftAxis fa, const typename 
         T2 *p = reinterpret_cast<T2 *>(out + t.cbase[c] + r * t.rstride);
         const CC y = Y[i];
         T2 o;
-        if (ACC) {
-            const T2 q = *p;
-            o.x = stp<PR>(ldp<PR>(q.x) + y.x);
-            o.y = stp<PR>(ldp<PR>(q.y) + y.y);
-        } else {
-            o.x = stp<PR>(y.x);
-            o.y = stp<PR>(y.y);
-        }
+        o.x = stp<PR>(y.x);
+        o.y = stp<PR>(y.y);
         *p = o;
     }
 }
@@ -767,7 +761,7 @@ __global__ void OFDFT_FFT_BOUNDS k_dline(GridInfo g, FftAxis fa, const typename 
 // back-transforms lines [w L, (w + 1) L), L = tile width / warps, with
 // warp-level synchronisation between stages; the block synchronises only
 // after the load and before the store.
-template <typename PR, int AX, int MODE, int ACC>
+template <typename PR, int AX, int MODE>
 __global__ void OFDFT_FFT_BOUNDS k_dline_ws(GridInfo g, FftAxis fa, const typename KT<PR>::T *in,
                                             typename KT<PR>::T *out)
 {
@@ -814,14 +808,8 @@ __global__ void OFDFT_FFT_BOUNDS k_dline_ws(GridInfo g, FftAxis fa, const typena
         T2 *p = reinterpret_cast<T2 *>(out + t.cbase[c] + r * t.rstride);
         const CC y = Y[c * ls + r];
         T2 o;
-        if (ACC) {
-            const T2 q = *p;
-            o.x = stp<PR>(ldp<PR>(q.x) + y.x);
-            o.y = stp<PR>(ldp<PR>(q.y) + y.y);
-        } else {
-            o.x = stp<PR>(y.x);
-            o.y = stp<PR>(y.y);
-        }
+        o.x = stp<PR>(y.x);
+        o.y = stp<PR>(y.y);
         *p = o;
     }
 }
@@ -937,22 +925,19 @@ __global__ void __launch_bounds__(OFDFT_PW_THREADS, OFDFT_PW_MINB) k_pw(GridInfo
     }
 }
 
-// Final stage of a GGA evaluation: v = v_HL - d_z U_z + v_part - div, with
-// v_HL from the half spectrum dspec (Hartree + LPP after the inverse x and
-// y passes), d_z U_z from the pair-packed lines of U_z (forward z transform,
-// times i kt ds_z, added to the packed spectrum of v_HL, so one inverse
-// transform serves both) and div = d_x U_x + d_y U_y, given as one field or
-// as two (div + div2; div2 may be null).  div may alias vout (each point is
-// read before it is written, by the same thread).  With uz null, d_z U_z is
-// given as the field div3 instead.  uz, vpart, div, div2 and div3 are pairs
-// (ldp).  Partials
-// (as k_zfinal's GGA form): rows 0..5 zero, then sum phi^2 v, sum phi^2,
-// sum 2 phi v dphi/dtheta.
+// Final stage of a GGA evaluation: v = v_HL + v_part - (d_x U_x + d_y U_y +
+// d_z U_z), with v_HL from the half spectrum dspec (Hartree + LPP after the
+// inverse x and y passes), the x and y terms given as the fields dx and dy, and
+// d_z U_z from the pair-packed lines of uz (forward z transform, times i kt
+// ds_z, added to the packed spectrum of v_HL, so one inverse transform serves
+// both) or, with uz null, given as the field dz.  uz, vpart, dx, dy and dz are
+// pairs (ldp).  Partials (as k_zfinal's GGA form): rows 0..5 zero, then sum
+// phi^2 v, sum phi^2, sum 2 phi v dphi/dtheta.
 template <typename PR>
 __global__ void OFDFT_FFT_BOUNDS k_zfinal_g(GridInfo g, FftAxis az, int P, const typename KT<PR>::C *dspec,
                            const typename KT<PR>::T *uz, const typename KT<PR>::T *vpart,
-                           const typename KT<PR>::T *div, const typename KT<PR>::T *div2,
-                           const typename KT<PR>::T *div3, const typename KT<PR>::T *phit,
+                           const typename KT<PR>::T *dx, const typename KT<PR>::T *dy,
+                           const typename KT<PR>::T *dz, const typename KT<PR>::T *phit,
                            const typename KT<PR>::T *phi, const typename KT<PR>::T *dhat,
                            typename KT<PR>::T c, typename KT<PR>::T s, const void *cs,
                            typename KT<PR>::T *vout, double *part)
@@ -1002,9 +987,8 @@ __global__ void OFDFT_FFT_BOUNDS k_zfinal_g(GridInfo g, FftAxis az, int P, const
         const R dr = (rc.r & 1) ? d.y : d.x;
         const R ph = ldr<PR>(phit[rbase + i]);
         const R n = ph * ph;
-        R v = ldp<PR>(vpart[rbase + i]) + dr - ldp<PR>(div[rbase + i]);
-        if (div2 != nullptr) v = v - ldp<PR>(div2[rbase + i]);
-        if (uz == nullptr) v = v - ldp<PR>(div3[rbase + i]);
+        R v = ldp<PR>(vpart[rbase + i]) + dr - ldp<PR>(dy[rbase + i]) - ldp<PR>(dx[rbase + i]);
+        if (uz == nullptr) v = v - ldp<PR>(dz[rbase + i]);
         acc[6] += n * v;
         acc[7] += n;
         if (dhat != nullptr) {
@@ -1081,42 +1065,38 @@ void launch_zfwd(const GridInfo &g, const FftAxis &az, int mode, const T *in, co
 
 namespace {
 template <typename PR>
-void dline_call(const GridInfo &g, const FftAxis &fa, int axis, int mode, int acc, const typename KT<PR>::T *in,
+void dline_call(const GridInfo &g, const FftAxis &fa, int axis, int mode, const typename KT<PR>::T *in,
                 typename KT<PR>::T *out, int blocks, int th, size_t sm, cudaStream_t st)
 {
     if (g.dws && th % 32 == 0 && g.dk % (th / 32) == 0) {   // whole lines for every warp
         if (axis == 0) {
-            if (mode == 0) pdl_launch(k_dline_ws<PR, 0, 0, 0>, blocks, th, sm, st, g, fa, in, out);
-            else if (acc == 0) pdl_launch(k_dline_ws<PR, 0, 1, 0>, blocks, th, sm, st, g, fa, in, out);
-            else pdl_launch(k_dline_ws<PR, 0, 1, 1>, blocks, th, sm, st, g, fa, in, out);
+            if (mode == 0) pdl_launch(k_dline_ws<PR, 0, 0>, blocks, th, sm, st, g, fa, in, out);
+            else pdl_launch(k_dline_ws<PR, 0, 1>, blocks, th, sm, st, g, fa, in, out);
         } else {
-            if (mode == 0) pdl_launch(k_dline_ws<PR, 1, 0, 0>, blocks, th, sm, st, g, fa, in, out);
-            else if (acc == 0) pdl_launch(k_dline_ws<PR, 1, 1, 0>, blocks, th, sm, st, g, fa, in, out);
-            else pdl_launch(k_dline_ws<PR, 1, 1, 1>, blocks, th, sm, st, g, fa, in, out);
+            if (mode == 0) pdl_launch(k_dline_ws<PR, 1, 0>, blocks, th, sm, st, g, fa, in, out);
+            else pdl_launch(k_dline_ws<PR, 1, 1>, blocks, th, sm, st, g, fa, in, out);
         }
         return;
     }
     if (axis == 0) {
-        if (mode == 0) pdl_launch(k_dline<PR, 0, 0, 0>, blocks, th, sm, st, g, fa, in, out);
-        else if (acc == 0) pdl_launch(k_dline<PR, 0, 1, 0>, blocks, th, sm, st, g, fa, in, out);
-        else pdl_launch(k_dline<PR, 0, 1, 1>, blocks, th, sm, st, g, fa, in, out);
+        if (mode == 0) pdl_launch(k_dline<PR, 0, 0>, blocks, th, sm, st, g, fa, in, out);
+        else pdl_launch(k_dline<PR, 0, 1>, blocks, th, sm, st, g, fa, in, out);
     } else {
-        if (mode == 0) pdl_launch(k_dline<PR, 1, 0, 0>, blocks, th, sm, st, g, fa, in, out);
-        else if (acc == 0) pdl_launch(k_dline<PR, 1, 1, 0>, blocks, th, sm, st, g, fa, in, out);
-        else pdl_launch(k_dline<PR, 1, 1, 1>, blocks, th, sm, st, g, fa, in, out);
+        if (mode == 0) pdl_launch(k_dline<PR, 1, 0>, blocks, th, sm, st, g, fa, in, out);
+        else pdl_launch(k_dline<PR, 1, 1>, blocks, th, sm, st, g, fa, in, out);
     }
 }
 }  // namespace
 
 template <typename T>
-void launch_dline(const GridInfo &g, const FftAxis &fa, int axis, int mode, int acc, const T *in, T *out,
+void launch_dline(const GridInfo &g, const FftAxis &fa, int axis, int mode, const T *in, T *out,
                   cudaStream_t st)
 {
     const int n = axis == 0 ? g.nx : g.ny;
     const int blocks = pair_tiles_of(g, axis);
     const size_t sm = 2 * (size_t)(g.dws ? n + 1 : n) * g.dk * sizeof(cplx<T>);
     const int th = g.dth > 0 ? g.dth : threads_for(n * g.dk / 2);   // warp-owned lines: dk a multiple of th / 32
-#define CALL(PR) dline_call<PR>(g, fa, axis, mode, acc, in, out, blocks, th, sm, st)
+#define CALL(PR) dline_call<PR>(g, fa, axis, mode, in, out, blocks, th, sm, st)
     OFDFT_DISPATCH(T, g, CALL);
 #undef CALL
 }
@@ -1466,7 +1446,7 @@ int launch_zfinal(const GridInfo &g, const FftAxis &az, bool fttf, const cplx<T>
 
 template <typename T>
 int launch_zfinal_gga(const GridInfo &g, const FftAxis &az, const cplx<T> *dspec, const T *uz, const T *vpart,
-                      const T *div, const T *div2, const T *div3, const T *phit, const T *phi, const T *dhat, T c,
+                      const T *dx, const T *dy, const T *dz, const T *phit, const T *phi, const T *dhat, T c,
                       T s, const void *cs, T *vout, double *part, cudaStream_t st)
 {
     int P = zpairs_light(g);
@@ -1475,7 +1455,7 @@ int launch_zfinal_gga(const GridInfo &g, const FftAxis &az, const cplx<T> *dspec
     size_t sm = (uz ? 3 : 2) * (size_t)P * g.nz * sizeof(cplx<T>);
     int th = g.zth > 0 ? g.zth : threads_for(P * g.nz);
 #define CALL(PR) \
-    pdl_launch(k_zfinal_g<PR>, blocks, th, sm, st, g, az, P, dspec, uz, vpart, div, div2, div3, phit, phi, dhat, c, s, cs, vout, \
+    pdl_launch(k_zfinal_g<PR>, blocks, th, sm, st, g, az, P, dspec, uz, vpart, dx, dy, dz, phit, phi, dhat, c, s, cs, vout, \
                                            part)
     OFDFT_DISPATCH(T, g, CALL);
 #undef CALL
@@ -1541,18 +1521,14 @@ template <typename PR> cudaError_t smem_limits(int b)
         cudaFuncSetAttribute(k_ypass<PR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
         cudaFuncSetAttribute(k_xhl<PR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
         cudaFuncSetAttribute(k_xhl<PR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
-        cudaFuncSetAttribute(k_dline<PR, 0, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
-        cudaFuncSetAttribute(k_dline<PR, 0, 1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
-        cudaFuncSetAttribute(k_dline<PR, 0, 1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
-        cudaFuncSetAttribute(k_dline<PR, 1, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
-        cudaFuncSetAttribute(k_dline<PR, 1, 1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
-        cudaFuncSetAttribute(k_dline<PR, 1, 1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
-        cudaFuncSetAttribute(k_dline_ws<PR, 0, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
-        cudaFuncSetAttribute(k_dline_ws<PR, 0, 1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
-        cudaFuncSetAttribute(k_dline_ws<PR, 0, 1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
-        cudaFuncSetAttribute(k_dline_ws<PR, 1, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
-        cudaFuncSetAttribute(k_dline_ws<PR, 1, 1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
-        cudaFuncSetAttribute(k_dline_ws<PR, 1, 1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b)};
+        cudaFuncSetAttribute(k_dline<PR, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
+        cudaFuncSetAttribute(k_dline<PR, 0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
+        cudaFuncSetAttribute(k_dline<PR, 1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
+        cudaFuncSetAttribute(k_dline<PR, 1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
+        cudaFuncSetAttribute(k_dline_ws<PR, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
+        cudaFuncSetAttribute(k_dline_ws<PR, 0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
+        cudaFuncSetAttribute(k_dline_ws<PR, 1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b),
+        cudaFuncSetAttribute(k_dline_ws<PR, 1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b)};
     for (cudaError_t x : e)
         if (x != cudaSuccess) return x;
     return cudaSuccess;
@@ -1569,7 +1545,7 @@ template <typename T> cudaError_t set_field_smem_limits(size_t bytes)
 #define OFDFT_INST(T)                                                                              \
     template void launch_zfwd<T>(const GridInfo &, const FftAxis &, int, const T *, const T *,     \
                                  const T *, T, T, const void *, T *, cplx<T> *, cudaStream_t, T *, T *); \
-    template void launch_dline<T>(const GridInfo &, const FftAxis &, int, int, int, const T *, T *, \
+    template void launch_dline<T>(const GridInfo &, const FftAxis &, int, int, const T *, T *, \
                                   cudaStream_t);                                                  \
     template int launch_pw<T>(const GridInfo &, T *, T *, T *, const T *, T, const FuncParams &,   \
                               const T *, int, T *, double *, bool, cudaStream_t);                 \

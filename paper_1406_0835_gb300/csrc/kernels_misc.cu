@@ -42,7 +42,7 @@ template <typename T> int red_blocks(long long n)
 
 // Block sum of binary64 per-thread partials through the double-float warp
 // stage (block_sum_f2): each partial is split into a double-float pair with
-// integer operations (split_int, relative error < 2^-46), so the shuffles and
+// integer operations (split_int, relative error < 2^-53), so the shuffles and
 // adds run on the integer and FP32 units instead of the FP64 ones.
 template <int NQ> __device__ __forceinline__ void block_sum_split(const double *v, double *tot)
 {
