@@ -284,7 +284,7 @@ FF_HD f2 fma_step(f2 p, float u, f2 c)
 }
 // The same without the final renormalisation (|lo| stays within a few
 // ulp(hi), which the next step's binary32 products with lo carry as well):
-// 11 instead of 14 operations.  The last step of a polynomial takes fma_step.
+// 11 instead of 14 operations.  Renormalise the last step's result.
 FF_HD f2 fma_step_u(f2 p, float u, f2 c)
 {
     f2 m = two_prod(p.hi, u);

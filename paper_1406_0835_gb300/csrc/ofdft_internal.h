@@ -194,19 +194,13 @@ constexpr int kTfSize = kTfPanels * kTfFuncs * kTfNc;
 // The double-float kernels read the same polynomials re-expanded about the
 // centres of kTfRef subpanels: their terms fall off kTfRef times faster per
 // degree, so that those from degree kTfSplit up can be summed in binary32
-// (pointwise.cuh).  A and B, whose coefficients fall off slowest, keep one
-// degree more as pairs and one degree more in all (the terms of degree 10 are
-// below 4e-18 of xi; of A and B they would be 2e-13 of the t-derivative).
-// Layout per subpanel, in rows of 16 bytes: degrees 0 .. kTfSplit - 1 as
-// pairs, two functions a row; A and B of degree kTfSplit as pairs; degrees
-// kTfSplit + 1 .. kTfDdDeg in binary32, four functions a row; and (xi, zeta
-// of degree kTfSplit, A, B of degree 10).
+// (pointwise.cuh).  Layout per subpanel, in rows of 16 bytes: degrees 0 ..
+// kTfSplit - 1 as pairs, two functions a row, then the degrees up to kTfDeg in
+// binary32, four functions a row.
 constexpr int kTfRef = 4;
 constexpr int kTfDdSub = kTfSub * kTfRef;
-constexpr int kTfDdDeg = 9;
-constexpr int kTfSplit = 5;
-constexpr int kTfDdRows = 2 * kTfSplit + 1 + (kTfDdDeg - kTfSplit) + 1;   // 256 bytes
-constexpr int kTfDdRow = 2 * kTfDdRows;
+constexpr int kTfSplit = 6;
+constexpr int kTfDdRow = 2 * (2 * kTfSplit + kTfDeg + 1 - kTfSplit);   // 272 bytes
 constexpr int kTfDdSize = kTfPanels * kTfRef * kTfDdRow;
 
 // VT84F enhancement factor F(x), x = s^2 (Eq. (VT84F)), as a table of

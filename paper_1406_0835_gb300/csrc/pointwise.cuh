@@ -304,7 +304,7 @@ constexpr double kPwNmin = 1e-18, kPwNmax = 1e18, kPwS2max = 1e10;
 // polynomial enters with on every panel, so binary32 rounding there stays
 // below the double-float rounding.
 struct HornerF2 {
-    ff::f2 p, dp;   // unnormalised but for the last step
+    ff::f2 p, dp;   // unnormalised
     float d2;
 };
 OF_HD void horner_lo(HornerF2 &h, float u, float c)
@@ -319,8 +319,9 @@ OF_HD void horner_dd(HornerF2 &h, float u, ff::f2 c)
     h.dp = ff::fma_step_u(h.dp, u, h.p);
     h.p = ff::fma_step_u(h.p, u, c);
 }
-// The step from a binary32 tail to its first pair (the derivative, one degree
-// behind, stays in binary32), and the last step.
+
+// The step from a binary32 tail to its first pair: the derivative, one degree
+// behind, stays in binary32.
 OF_HD void horner_first(HornerF2 &h, float u, ff::f2 c)
 {
     h.d2 = h.d2 * u + h.dp.hi;
@@ -328,25 +329,19 @@ OF_HD void horner_first(HornerF2 &h, float u, ff::f2 c)
     const ff::f2 m = ff::two_prod(h.p.hi, u), s = ff::two_sum(m.hi, c.hi);
     h.p = ff::f2(s.hi, ff::fadd(m.lo, ff::fadd(s.lo, c.lo)));
 }
-OF_HD void horner_last(HornerF2 &h, float u, ff::f2 c)
-{
-    h.d2 = h.d2 * u + h.dp.hi;
-    h.dp = ff::fma_step(h.dp, u, h.p);
-    h.p = ff::fma_step(h.p, u, c);
-}
 
 // Table polynomials with the refined double-float table (kTfDdSub panels an
 // octave).  The panel variable u = uh + ul: uh is exact in binary32 and the
 // Horner sums run with it; ul (below 2e-6) enters through the first and
-// second derivatives.  The tails in binary32 cost, over every panel, at most
-// 4e-17 of xi, 8e-17 of xi for zeta (zeta comes close to zero but enters only
-// beside xi, f = tau0 xi F_tau - tau0 zeta F_sigma), 5e-17 of A and 8e-17 of
-// the larger of B and A xi / zeta (B enters through zeta F(s^2 B) beside xi
-// F(s^2 A)); of the derivatives per ln t, which the potential takes, 6e-15,
-// 1.3e-14, 9e-15 and 1.6e-14.  (A and B from degree 5 up in binary32 and
-// without degree 10 put 8e-13 into df/dn where s^2 is large.)  With the
-// unrefined panels 7, 7, 8 and all 10 degrees needed double-float: 32 steps
-// instead of 22.
+// second derivatives.  The tails in binary32 (degrees 6 to 10) cost, over
+// every panel, at most 8e-19 of xi, 2e-18 of xi for zeta (zeta comes close to
+// zero but enters only beside xi, f = tau0 xi F_tau - tau0 zeta F_sigma),
+// 5e-17 of A and 8e-17 of the larger of B and A xi / zeta (B enters through
+// zeta F(s^2 B) beside xi F(s^2 A)); of the derivatives per ln t, which the
+// potential takes, 2e-16, 3e-16, 9e-15 and 1.6e-14.  (From degree 5 up in
+// binary32 and without degree 10, A and B put 9.6e-13 into df/dn where s^2 is
+// large.)  With the unrefined panels 7, 7, 8 and all 10 degrees needed
+// double-float: 32 steps instead of 24.
 template <int NF>
 OF_HD void tfunc_eval_f2(const ff::f2 *__restrict__ tab, ff::f2 t, ff::f2 out[8])
 {
@@ -359,14 +354,14 @@ OF_HD void tfunc_eval_f2(const ff::f2 *__restrict__ tab, ff::f2 t, ff::f2 out[8]
     const float ul = (float)(2 * kTfDdSub) * t.lo * inv2e;
     const float dudt = (float)(2 * kTfDdSub) * inv2e;
     const float4 *c = reinterpret_cast<const float4 *>(tab + (size_t)((e - kTfEmin) * kTfDdSub + sub) * kTfDdRow);
-    const float4 *tail = c + 2 * kTfSplit;               // tail[k]: degree kTfSplit + k (k = 0: A and B, pairs)
-    const float4 ends = c[kTfDdRows - 1], top = tail[kTfDdDeg - kTfSplit];
+    const float4 *tail = c + 2 * kTfSplit;               // tail[k]: degree kTfSplit + k
     HornerF2 h[NF];
+    const float4 top = tail[kTfDeg - kTfSplit];
     h[0].p.hi = top.x;
     h[1].p.hi = top.y;
     if (NF == 4) {
-        h[2].p.hi = ends.z;
-        h[3].p.hi = ends.w;
+        h[2].p.hi = top.z;
+        h[3].p.hi = top.w;
     }
 #pragma unroll
     for (int q = 0; q < NF; ++q) {
@@ -374,26 +369,25 @@ OF_HD void tfunc_eval_f2(const ff::f2 *__restrict__ tab, ff::f2 t, ff::f2 out[8]
         h[q].dp = ff::f2(0.0f, 0.0f);
         h[q].d2 = 0.0f;
     }
-    if (NF == 4) {
-        horner_lo(h[2], uh, top.z);
-        horner_lo(h[3], uh, top.w);
-    }
 #pragma unroll 1
-    for (int j = kTfDdDeg - kTfSplit - 1; j >= 1; --j) {
+    for (int j = kTfDeg - kTfSplit - 1; j >= 0; --j) {
         const float4 a = tail[j];
         const float cj[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
         for (int q = 0; q < NF; ++q) horner_lo(h[q], uh, cj[q]);
     }
-    horner_lo(h[0], uh, ends.x);
-    horner_lo(h[1], uh, ends.y);
-    if (NF == 4) {
-        const float4 a = tail[0];
-        horner_first(h[2], uh, ff::f2(a.x, a.y));
-        horner_first(h[3], uh, ff::f2(a.z, a.w));
+    {
+        const float4 a = c[2 * kTfSplit - 2];
+        horner_first(h[0], uh, ff::f2(a.x, a.y));
+        horner_first(h[1], uh, ff::f2(a.z, a.w));
+        if (NF == 4) {
+            const float4 b = c[2 * kTfSplit - 1];
+            horner_first(h[2], uh, ff::f2(b.x, b.y));
+            horner_first(h[3], uh, ff::f2(b.z, b.w));
+        }
     }
 #pragma unroll 1
-    for (int j = kTfSplit - 1; j >= 1; --j) {
+    for (int j = kTfSplit - 2; j >= 0; --j) {
         const float4 a = c[2 * j];
         horner_dd(h[0], uh, ff::f2(a.x, a.y));
         horner_dd(h[1], uh, ff::f2(a.z, a.w));
@@ -403,18 +397,12 @@ OF_HD void tfunc_eval_f2(const ff::f2 *__restrict__ tab, ff::f2 t, ff::f2 out[8]
             horner_dd(h[3], uh, ff::f2(b.z, b.w));
         }
     }
-    const float4 a0 = c[0];
-    horner_last(h[0], uh, ff::f2(a0.x, a0.y));
-    horner_last(h[1], uh, ff::f2(a0.z, a0.w));
-    if (NF == 4) {
-        const float4 b0 = c[1];
-        horner_last(h[2], uh, ff::f2(b0.x, b0.y));
-        horner_last(h[3], uh, ff::f2(b0.z, b0.w));
-    }
 #pragma unroll
     for (int q = 0; q < NF; ++q) {
-        out[q] = ff::add(h[q].p, h[q].dp.hi * ul);
-        out[4 + q] = ff::scale(ff::add(h[q].dp, 2.0f * h[q].d2 * ul), dudt);
+        // normalised first: the sums round at the size of the low words
+        const ff::f2 p = ff::fast_two_sum(h[q].p.hi, h[q].p.lo), dp = ff::fast_two_sum(h[q].dp.hi, h[q].dp.lo);
+        out[q] = ff::add(p, dp.hi * ul);
+        out[4 + q] = ff::scale(ff::add(dp, 2.0f * h[q].d2 * ul), dudt);
     }
 }
 
@@ -707,16 +695,11 @@ inline void dd_tables_fill(const double *ttab, double *dst)
                 float *row = rf + 2 * (size_t)(p * kTfRef + s) * kTfDdRow;
                 for (int k = 0; k <= kTfDeg; ++k, sc /= kTfRef) {
                     const ff::f2 c = ff::from_double(a[k] * sc);
-                    if (k < kTfSplit || (k == kTfSplit && q >= 2)) {
-                        float *pair = row + (k < kTfSplit ? 2 * (k * kTfFuncs + q) : 8 * kTfSplit + 2 * (q - 2));
-                        pair[0] = c.hi;
-                        pair[1] = c.lo;
-                    } else if (k == kTfSplit) {
-                        row[4 * (kTfDdRows - 1) + q] = c.hi;
-                    } else if (k <= kTfDdDeg) {
-                        row[4 * (k + kTfSplit) + q] = c.hi;
-                    } else if (q >= 2) {
-                        row[4 * (kTfDdRows - 1) + q] = c.hi;
+                    if (k < kTfSplit) {
+                        row[2 * (k * kTfFuncs + q)] = c.hi;
+                        row[2 * (k * kTfFuncs + q) + 1] = c.lo;
+                    } else {
+                        row[2 * kTfSplit * kTfFuncs + (k - kTfSplit) * kTfFuncs + q] = c.hi;
                     }
                 }
             }
