@@ -19,9 +19,9 @@
 // and the sums over h <= 72 and up to seven digit pairs (two of them with a
 // leading digit, at most 64) stay below 2^24, so the f32 accumulators of
 // tcgen05.mma (kind::f16) hold exact integers.  Digit products of equal
-// weight share one accumulator: 7 accumulators, 28 products, the first
-// dropped weight about 2^-51 of the line's largest value times the largest
-// matrix entry.  Fields are double-float pairs in memory (8 bytes).
+// weight share one accumulator: 7 accumulators, 28 products; the first
+// products dropped, six for each term, are each at most about 2^-51 of the
+// line's largest value times the largest matrix entry.  Fields are double-float pairs in memory (8 bytes).
 #include <math.h>
 
 #include <algorithm>
@@ -269,11 +269,7 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
     const long long ln_off = (w_ok ? ou * jb.ostride + (zaxis ? 0 : ln - ou * zlen) : 0) + (half ? h * rstride : 0);
     const bool wide = zaxis && (h & 1) == 0;
     if (tid < kLines) s_max[tid] = 27u << 23;      // 2^-100: the least exponent of the scale
-    bar_sync(4, blockDim.x);
-    tc::fence_after_sync();
-    const uint32_t tmem = s_tmem;
     pdl_wait();                                    // (the issuing warp reads nothing that another kernel writes)
-    pdl_trigger();                                 // the block has its tensor memory: see pdl.cuh
     float2 v[16];
     if (mine) {
         const int line = tile * kLines + row;
@@ -307,7 +303,10 @@ __global__ void __launch_bounds__(kTlThreads + 32, 1) k_tline(const __grid_const
             }
         }
     }
-    bar_sync(3, nconv);                            // s_max is set
+    bar_sync(4, blockDim.x);                       // s_max is set too; the loads are under way
+    tc::fence_after_sync();
+    const uint32_t tmem = s_tmem;
+    pdl_trigger();                                 // the block has its tensor memory: see pdl.cuh
     if (mine) {
         uint32_t m = 0;
 #pragma unroll
