@@ -193,11 +193,11 @@ def fft_flops(n):
 POINTWISE_FLOP = 200.0
 # Issued warp instructions and DRAM bytes per grid point of one k_pw<DD>
 # launch (the FP64 contexts' pointwise kernel, VT84F at an MD density, 96^3),
-# from the ncu capture summarised in profiles/k_pw_dd_96.md (64,904,760
-# warp instructions, 29.95 MB per launch).  Valid for that kernel only: set
+# from the ncu capture summarised in profiles/k_pw_dd_96.md (67,088,952
+# warp instructions, 29.96 MB per launch).  Valid for that kernel only: set
 # to None when it changes until the capture is repeated.
-PW_DD_WARP_INST_PER_POINT = 64904760.0 / 96 ** 3
-PW_DD_TRAFFIC_PER_POINT = (28.410368e6 + 1.537024e6) / 96 ** 3
+PW_DD_WARP_INST_PER_POINT = 67088952.0 / 96 ** 3
+PW_DD_TRAFFIC_PER_POINT = (28.412032e6 + 1.549440e6) / 96 ** 3
 # FP32-unit instructions per FP64-equivalent flop of the double-float
 # arithmetic in the cost model of the FFT and pointwise work: a sum
 # (two_sum + tail + fast_two_sum) takes 11, a product (two_prod + two FMAs
@@ -205,25 +205,46 @@ PW_DD_TRAFFIC_PER_POINT = (28.410368e6 + 1.537024e6) / 96 ** 3
 DD_INSTR_PER_FLOP = (2 * 11 + 9) / 3.0
 
 
-def kernel_model(name, g, fttf=False):
-    """Algorithmic FLOPs and HBM bytes of one launch (FP64 fields) of a timed
-    kernel class: FFT flops 5 n log2 n per complex line (two real lines
-    travel as one complex line), plus the pointwise functional; bytes =
-    fields read + written once."""
+def kernel_model(name, g, fttf=False, real_basis=False):
+    """Algorithmic FLOPs and HBM bytes of one timed launch (FP64 fields) of a
+    kernel class: transforms as FFTs, 5 n log2 n per complex line (two real
+    lines travel as one complex line), plus the pointwise functional; bytes =
+    fields read + written once.  real_basis: the classes of the tensor-core
+    form (edges up to 144), where a class of two launches of different kinds
+    counts their mean."""
     nx, ny, nz = g
     K = nz // 2 + 1
     N = nx * ny * nz
     NH = nx * ny * K
+
+    def real(n):               # one transform of a real field along an axis of n points
+        return N / (2.0 * n) * fft_flops(n)
+
     if name == "pw":           # pointwise functional: phi, 3 derivatives in; v_part, 3 U out
         flops = POINTWISE_FLOP * N
         byts = 8 * N * 8
-    elif name == "dline":      # per axis, as the FFT passes count it: forward + inverse line transforms
-        n = (nx + ny) / 2.0
-        flops = 2 * (N / 2 / n) * fft_flops(n)
+    elif real_basis and name == "dline":   # n -> 3 derivatives and z coefficients; 3 U -> their derivatives
+        three = 2 * (real(nx) + real(ny) + real(nz))
+        flops = real(nz) if fttf else three + real(nz) / 2
+        byts = 8 * N * (2 if fttf else 5.5)
+    elif real_basis and name == "ypass":   # y forward or inverse: coefficients in and out
+        flops = real(ny)
+        byts = 8 * N * 2
+    elif real_basis and name == "xhl":     # x forward, Hartree and local terms, x inverse
+        flops = 2 * real(nx)
+        byts = 8 * N * 3
+    elif real_basis and name == "zfwd":    # density: phi in, n out
+        flops = N
+        byts = 8 * N * 2
+    elif real_basis and name == "zfinal":  # z inverse; GGA also v from v_HL, v_part, 3 derivatives, phi
+        flops = real(nz) if fttf else real(nz) / 2
+        byts = 8 * N * (2 if fttf else 4.5)
+    elif name == "dline":      # one derivative along x or y: forward + inverse line transforms
+        flops = real(nx) + real(ny)
         byts = 8 * N * 2                                   # field in, derivative out
     elif name == "zfinal":     # GGA: U_z forward + one inverse; ftTF: inverse + pointwise
         # GGA fields: U_z, v_part, d_y U_y, d_x U_x, phi in; v out
-        flops = (nx * ny / 2) * fft_flops(nz) * (1 if fttf else 2) + (POINTWISE_FLOP * N if fttf else 0)
+        flops = real(nz) * (1 if fttf else 2) + (POINTWISE_FLOP * N if fttf else 0)
         byts = 16 * NH + 8 * N * (3 if fttf else 6)
     elif name == "ypass":
         flops = nx * K * fft_flops(ny)
@@ -292,7 +313,7 @@ def roofline_entry(dominant, grid, kms, kcount, clk, peaks, precision="fp64"):
     beside it: FP64-equivalent TFLOP/s of the algorithmic flops (FFT flops +
     200 flop per point for the pointwise functional) against the issue rate
     over DD_INSTR_PER_FLOP, and against the FP64 units' peak."""
-    flops, byts = kernel_model(dominant, grid)
+    flops, byts = kernel_model(dominant, grid, real_basis=precision == "fp64" and max(grid) <= 144)
     avg_s = (kms / 1e3) / max(kcount, 1)
     sm_mhz = clk.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
     issue = 152 * 128 * (sm_mhz * 1e6)                      # thread instructions / s

@@ -825,13 +825,13 @@ __global__ void OFDFT_FFT_BOUNDS k_dline_ws(GridInfo g, FftAxis fa, const typena
 // sum n(v_xc - eps_xc); with STRESS also sum W_a d_b n for ab = xx, yy,
 // zz, xy, xz, yz (the gradient part of Eq. (stressTF_b)) in rows 6..11.
 // The double-float form is bound by instruction issue (73 % of the issue
-// slots at 96^3, 2,350 instructions a point, 78 us).  From 3,060 and 118 us:
+// slots at 96^3, 2,430 instructions a point, 80 us).  From 3,060 and 118 us:
 // polynomial steps without renormalisation, quotients and roots from one
 // reciprocal (a quarter of the instructions), the PZ81 logarithm from a
 // table instead of an exponential, sums of like terms without the
 // cancellation-proof form, W.grad n from s^2 (2,860, 91 us); refined table
-// panels with 20 instead of 32 double-float steps and the polynomials side
-// by side in one rolled loop.
+// panels with 24 instead of 32 double-float steps and the polynomials side
+// by side in rolled loops.
 // Threads per block of the pointwise kernel and the blocks per SM its
 // register budget is sized for (launch bounds).
 #ifndef OFDFT_PW_THREADS

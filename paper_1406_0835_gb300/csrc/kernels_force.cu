@@ -78,7 +78,9 @@ __device__ __forceinline__ void ion_phase(int c, const double2 *__restrict__ p, 
 // relative to that frequency while its sum comes from lower ones, so T' keeps
 // the products of one weight more than T, and rows of g an eighth digit (in
 // units of 2^-60 of the row's largest value, which is often the coefficient of
-// frequency 0, whose f' is zero).
+// frequency 0, whose f' is zero).  Error of the forces along x, y, z in 1e-15
+// Ha/bohr rms, 64 ions at 64^3: 1.9, 1.6, 1.7; with seven digits 1.9, 1.6,
+// 2.5; the double-float kernel 2.1, 1.8, 2.0.
 __host__ __device__ __forceinline__ double block_top(int nz, int kb) { return 0.5 * min((kb + 1) * kKc, nz) / 1.75; }
 
 // The coefficients on two or three Nyquist frequencies, whose phases do not
